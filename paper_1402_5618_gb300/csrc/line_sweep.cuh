@@ -5,20 +5,15 @@
 // memory and runs, in order:
 //   load     cell averages of the segment plus a two-cell halo (ghost cells
 //            from the boundary condition at the line ends);
-//   weights  WENO-Z weights of every cell for both sides (Sec. 2.2, eq.
-//            (weight)), kept in shared memory for the two passes below;
 //   solve    for each conserved variable the minus and plus compact-WENO
-//            systems (eq. (CWENO-FV)) by Thomas elimination in the stable
-//            order (minus left to right, plus right to left), parallelised
-//            exactly: every thread owns a chunk of M rows, the forward
-//            elimination of a chunk is a projective map of the state (c', d')
-//            carried in from the previous rows ((P, Q, D) with c' = P/Q,
-//            d' = D/Q evolves linearly), the maps are composed by
-//            warp-shuffle scans, across warps in shared memory and across the
-//            cluster's CTAs through distributed shared memory; the back
-//            substitution is an affine map per chunk, scanned the same way.
-//            Periodic lines add the second right-hand side of the
-//            Sherman-Morrison correction to the same sweep.
+//            systems (eq. (CWENO-FV)), exactly and in partitioned form
+//            (compact_solve.cuh): every thread eliminates a chunk of M rows of
+//            one variable in both systems, one or two warps combine the
+//            chunks of the segment, eight to a lane and then across lanes,
+//            and the segments of the cluster through distributed shared
+//            memory; the solution at the run ends goes back the same way and
+//            every thread substitutes back in its chunk.  A periodic line is
+//            the same with the ring closed where the segments combine.
 //   limit    Zhang-Shu limiter per cell (Sec. 2.4);
 //   flux     HLLC at every face of the segment (the two segment-end faces
 //            read the neighbour CTA's limited face value);
@@ -39,14 +34,13 @@
 #include <stdint.h>
 
 #include "batch_lines.cuh"
+#include "compact_solve.cuh"
 #include "dfloat.cuh"
 #include "physics.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace ppk {
-
-constexpr int SEGC = 512;       // cells per CTA segment (all chunk lengths)
 
 // device-side control block of one problem (time, dt, reductions, flags)
 struct Ctl {
@@ -158,181 +152,9 @@ __device__ __forceinline__ void bind_line(SweepArgs &a, long long &line) {
   }
 }
 
-// ---------------------------------------------------------------- maps
-// Forward elimination map of a run of rows acting on the projective state
-// (P, Q, D, Z): c' = P/Q, d' = D/Q and, on periodic lines, z' = Z/Q for the
-// second right-hand side.  The map has the block form
-//   [P;Q]' = G [P;Q],  D' = dP P + dQ Q + mu D,  Z' = zP P + zQ Q + mu Z.
-template <typename real>
-struct Fwd {
-  real g00, g01, g10, g11, dP, dQ, mu, zP, zQ;
-};
-
-template <typename real>
-__device__ __forceinline__ Fwd<real> fwd_identity() {
-  Fwd<real> f;
-  f.g00 = real(1); f.g01 = real(0); f.g10 = real(0); f.g11 = real(1);
-  f.dP = real(0); f.dQ = real(0); f.mu = real(1); f.zP = real(0); f.zQ = real(0);
-  return f;
-}
-
-// Y o X (X first)
-template <typename real, bool PER>
-__device__ __forceinline__ Fwd<real> fwd_compose(const Fwd<real> &Y, const Fwd<real> &X) {
-  Fwd<real> f;
-  f.g00 = Y.g00 * X.g00 + Y.g01 * X.g10;
-  f.g01 = Y.g00 * X.g01 + Y.g01 * X.g11;
-  f.g10 = Y.g10 * X.g00 + Y.g11 * X.g10;
-  f.g11 = Y.g10 * X.g01 + Y.g11 * X.g11;
-  f.dP = Y.dP * X.g00 + Y.dQ * X.g10 + Y.mu * X.dP;
-  f.dQ = Y.dP * X.g01 + Y.dQ * X.g11 + Y.mu * X.dQ;
-  f.mu = Y.mu * X.mu;
-  if (PER) {
-    f.zP = Y.zP * X.g00 + Y.zQ * X.g10 + Y.mu * X.zP;
-    f.zQ = Y.zP * X.g01 + Y.zQ * X.g11 + Y.mu * X.zQ;
-  } else {
-    f.zP = real(0); f.zQ = real(0);
-  }
-  return f;
-}
-
-// row first, then the accumulated map (left multiplication by the row)
-template <typename real, bool PER>
-__device__ __forceinline__ void fwd_push_left(Fwd<real> &f, const Row<real> &w, real u) {
-  Fwd<real> o = f;
-  f.g00 = w.c * o.g10;
-  f.g01 = w.c * o.g11;
-  f.g10 = -w.a * o.g00 + w.b * o.g10;
-  f.g11 = -w.a * o.g01 + w.b * o.g11;
-  f.dP = w.r * o.g10 - w.a * o.dP;
-  f.dQ = w.r * o.g11 - w.a * o.dQ;
-  if (PER) {
-    f.zP = u * o.g10 - w.a * o.zP;
-    f.zQ = u * o.g11 - w.a * o.zQ;
-  }
-  f.mu = -w.a * o.mu;
-}
-
-// accumulated map first, then the row (right multiplication by the row)
-template <typename real, bool PER>
-__device__ __forceinline__ void fwd_push_right(Fwd<real> &f, const Row<real> &w, real u) {
-  Fwd<real> o = f;
-  f.g00 = -w.a * o.g01;
-  f.g01 = w.c * o.g00 + w.b * o.g01;
-  f.g10 = -w.a * o.g11;
-  f.g11 = w.c * o.g10 + w.b * o.g11;
-  f.dP = -w.a * o.dQ;
-  f.dQ = w.c * o.dP + w.b * o.dQ + o.mu * w.r;
-  if (PER) {
-    f.zP = -w.a * o.zQ;
-    f.zQ = w.c * o.zP + w.b * o.zQ + o.mu * u;
-  }
-  f.mu = -w.a * o.mu;
-}
-
-// power of two near 1/m (exact scaling, no division): 2^-(exponent of m)
-__device__ __forceinline__ float pow2_inv(float m) {
-  int e = (__float_as_int(m) >> 23) & 0xff;
-  return (e > 0 && e < 254) ? __int_as_float((254 - e) << 23) : 1.0f;
-}
-__device__ __forceinline__ double pow2_inv(double m) {
-  long long e = (__double_as_longlong(m) >> 52) & 0x7ff;
-  return (e > 0 && e < 2046) ? __longlong_as_double((2046 - e) << 52) : 1.0;
-}
-
-// FP64 WENO-Z weights (w0, w2) of the minus side and (v0, v2) of the plus
-// side (eq. (weight), linear weights 0.2, 0.5, 0.3, the plus side on the
-// mirrored indicators) with one division for both: with d_k = beta_k + eps
-// and D = d0 d1 d2, alpha_k D^2 = c_k (D^2 + tau^2 (D / d_k)^2), a common
-// factor of each side's weights, and one reciprocal of the product of the
-// two sides' sums normalises both.  (d, tau) are first scaled by a power of
-// two near 1/max d (exact, the weights are homogeneous in them) so that the
-// sixth powers stay in range.
-__device__ __forceinline__ void zweights_both_fp64(double um2, double um1, double u0, double up1,
-                                                   double up2, double eps, double &w0, double &w2,
-                                                   double &v0, double &v2) {
-  const double c13 = 13.0 / 12.0;
-  const double b0 = c13 * sqr(um2 - 2.0 * um1 + u0) + 0.25 * sqr(um2 - 4.0 * um1 + 3.0 * u0);
-  const double b1 = c13 * sqr(um1 - 2.0 * u0 + up1) + 0.25 * sqr(um1 - up1);
-  const double b2 = c13 * sqr(u0 - 2.0 * up1 + up2) + 0.25 * sqr(3.0 * u0 - 4.0 * up1 + up2);
-  double tau = fabs(b2 - b0);
-  double d0 = b0 + eps, d1 = b1 + eps, d2 = b2 + eps;
-  const double sc = pow2_inv(fmax(fmax(d0, d1), d2));
-  d0 *= sc; d1 *= sc; d2 *= sc; tau *= sc;
-  const double p01 = d0 * d1, p02 = d0 * d2, p12 = d1 * d2;
-  const double D2 = sqr(p01 * d2), t2 = tau * tau;
-  const double e0 = t2 * sqr(p12), e1 = t2 * sqr(p02), e2 = t2 * sqr(p01);
-  // minus: (c0, c1, c2) on (e0, e1, e2); plus: the same c on (e2, e1, e0)
-  const double am0 = 0.2 * (D2 + e0), am1 = 0.5 * (D2 + e1), am2 = 0.3 * (D2 + e2);
-  const double ap0 = 0.2 * (D2 + e2), ap2 = 0.3 * (D2 + e0);
-  const double sm = am0 + am1 + am2, sp = ap0 + am1 + ap2;
-  const double inv = 1.0 / (sm * sp);
-  const double ism = sp * inv, isp = sm * inv;
-  w0 = am0 * ism;
-  w2 = am2 * ism;
-  v0 = ap0 * isp;
-  v2 = ap2 * isp;
-}
-
-// rescale the map (its projective action is unchanged) so that the largest
-// entry of G lies in [1, 2)
-template <typename real>
-__device__ __forceinline__ void fwd_normalise(Fwd<real> &f) {
-  real m = fmax(fmax(fabs(f.g00), fabs(f.g01)), fmax(fabs(f.g10), fabs(f.g11)));
-  if (m > real(0)) {
-    real s = pow2_inv(m);
-    f.g00 *= s; f.g01 *= s; f.g10 *= s; f.g11 *= s;
-    f.dP *= s; f.dQ *= s; f.mu *= s; f.zP *= s; f.zQ *= s;
-  }
-}
-
-// state (c', d', z') -> map -> state, renormalised to Q = 1
-template <typename real, bool PER>
-__device__ __forceinline__ void fwd_apply(const Fwd<real> &f, real &cp, real &dp, real &zp) {
-  real P = f.g00 * cp + f.g01;
-  real Q = f.g10 * cp + f.g11;
-  real D = f.dP * cp + f.dQ + f.mu * dp;
-  real Z = PER ? f.zP * cp + f.zQ + f.mu * zp : real(0);
-  real iq = real(1) / Q;
-  cp = P * iq;
-  dp = D * iq;
-  if (PER) zp = Z * iq;
-}
-
-template <typename real>
-__device__ __forceinline__ real shfl_up_r(real v, int d, int width = 32) {
-  return __shfl_up_sync(0xffffffffu, v, d, width);
-}
 template <typename real>
 __device__ __forceinline__ real shfl_down_r(real v, int d, int width = 32) {
   return __shfl_down_sync(0xffffffffu, v, d, width);
-}
-
-template <typename real, bool PER, bool UP>
-__device__ __forceinline__ Fwd<real> fwd_shfl(const Fwd<real> &f, int d, int width = 32) {
-  Fwd<real> o;
-#define PPK_SH(x) o.x = UP ? shfl_up_r(f.x, d, width) : shfl_down_r(f.x, d, width)
-  PPK_SH(g00); PPK_SH(g01); PPK_SH(g10); PPK_SH(g11); PPK_SH(dP); PPK_SH(dQ); PPK_SH(mu);
-  if (PER) { PPK_SH(zP); PPK_SH(zQ); } else { o.zP = real(0); o.zQ = real(0); }
-#undef PPK_SH
-  return o;
-}
-
-// back-substitution map of a run: x_first = A + B x_after (z alike, same B)
-template <typename real>
-struct Bwd {
-  real A, B, Az;
-};
-
-// the run X followed (in back-substitution order) by the run Y:
-// x_first(X) = X.A + X.B (Y.A + Y.B x_after(Y))
-template <typename real>
-__device__ __forceinline__ Bwd<real> bwd_compose(const Bwd<real> &X, const Bwd<real> &Y) {
-  Bwd<real> r;
-  r.A = X.A + X.B * Y.A;
-  r.Az = X.Az + X.B * Y.Az;
-  r.B = X.B * Y.B;
-  return r;
 }
 
 // split cluster barrier: arrive (release this CTA's shared-memory writes to
@@ -348,119 +170,10 @@ __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory");
 }
 
-// ---------------------------------------------------------------- pairs
-// The mixed form advances the minus (.x) and plus (.y) systems together with
-// paired FP32 instructions (one instruction, two lanes' worth of FP32 work;
-// each component rounds as the scalar fused multiply-add does).
-__device__ __forceinline__ float2 p_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 p_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 p_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 p_neg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 p_set(float a) { return make_float2(a, a); }
-
-// forward maps of both systems
-struct Fwd2 {
-  float2 g00, g01, g10, g11, dP, dQ, mu, zP, zQ;
-};
-
-__device__ __forceinline__ Fwd2 fwd2_pack(const Fwd<float> &m, const Fwd<float> &p) {
-  Fwd2 f;
-  f.g00 = make_float2(m.g00, p.g00); f.g01 = make_float2(m.g01, p.g01);
-  f.g10 = make_float2(m.g10, p.g10); f.g11 = make_float2(m.g11, p.g11);
-  f.dP = make_float2(m.dP, p.dP); f.dQ = make_float2(m.dQ, p.dQ);
-  f.mu = make_float2(m.mu, p.mu); f.zP = make_float2(m.zP, p.zP); f.zQ = make_float2(m.zQ, p.zQ);
-  return f;
-}
-
-__device__ __forceinline__ void fwd2_unpack(const Fwd2 &f, Fwd<float> &m, Fwd<float> &p) {
-  m.g00 = f.g00.x; m.g01 = f.g01.x; m.g10 = f.g10.x; m.g11 = f.g11.x;
-  m.dP = f.dP.x; m.dQ = f.dQ.x; m.mu = f.mu.x; m.zP = f.zP.x; m.zQ = f.zQ.x;
-  p.g00 = f.g00.y; p.g01 = f.g01.y; p.g10 = f.g10.y; p.g11 = f.g11.y;
-  p.dP = f.dP.y; p.dQ = f.dQ.y; p.mu = f.mu.y; p.zP = f.zP.y; p.zQ = f.zQ.y;
-}
-
-// Y o X (X first), both systems
-template <bool PER>
-__device__ __forceinline__ Fwd2 fwd2_compose(const Fwd2 &Y, const Fwd2 &X) {
-  Fwd2 f;
-  f.g00 = p_fma(Y.g01, X.g10, p_mul(Y.g00, X.g00));
-  f.g01 = p_fma(Y.g01, X.g11, p_mul(Y.g00, X.g01));
-  f.g10 = p_fma(Y.g11, X.g10, p_mul(Y.g10, X.g00));
-  f.g11 = p_fma(Y.g11, X.g11, p_mul(Y.g10, X.g01));
-  f.dP = p_fma(Y.mu, X.dP, p_fma(Y.dQ, X.g10, p_mul(Y.dP, X.g00)));
-  f.dQ = p_fma(Y.mu, X.dQ, p_fma(Y.dQ, X.g11, p_mul(Y.dP, X.g01)));
-  f.mu = p_mul(Y.mu, X.mu);
-  if (PER) {
-    f.zP = p_fma(Y.mu, X.zP, p_fma(Y.zQ, X.g10, p_mul(Y.zP, X.g00)));
-    f.zQ = p_fma(Y.mu, X.zQ, p_fma(Y.zQ, X.g11, p_mul(Y.zP, X.g01)));
-  } else {
-    f.zP = p_set(0.0f); f.zQ = p_set(0.0f);
-  }
-  return f;
-}
-
-__device__ __forceinline__ void fwd2_normalise(Fwd2 &f) {
-  float mx = fmaxf(fmaxf(fabsf(f.g00.x), fabsf(f.g01.x)), fmaxf(fabsf(f.g10.x), fabsf(f.g11.x)));
-  float my = fmaxf(fmaxf(fabsf(f.g00.y), fabsf(f.g01.y)), fmaxf(fabsf(f.g10.y), fabsf(f.g11.y)));
-  const float2 sc = make_float2(pow2_inv(mx), pow2_inv(my));   // 1 for 0, inf, nan
-  f.g00 = p_mul(f.g00, sc); f.g01 = p_mul(f.g01, sc); f.g10 = p_mul(f.g10, sc);
-  f.g11 = p_mul(f.g11, sc); f.dP = p_mul(f.dP, sc); f.dQ = p_mul(f.dQ, sc);
-  f.mu = p_mul(f.mu, sc); f.zP = p_mul(f.zP, sc); f.zQ = p_mul(f.zQ, sc);
-}
-
-// back-substitution maps of both systems
-struct Bwd2 {
-  float2 A, B, Az;
-};
-
-__device__ __forceinline__ Bwd2 bwd2_compose(const Bwd2 &X, const Bwd2 &Y) {
-  Bwd2 r;
-  r.A = p_fma(X.B, Y.A, X.A);
-  r.Az = p_fma(X.B, Y.Az, X.Az);
-  r.B = p_mul(X.B, Y.B);
-  return r;
-}
-
-// WENO-Z weights w0, w2 of the minus side (ratios q0, q1, q2, linear weights
-// 0.2, 0.5, 0.3) and v0, v2 of the plus side (the same ratios reversed), in
-// paired FP32; the middle term is common to both
-__device__ __forceinline__ void zweights_pair(float q0, float q1, float q2, float one, float &w0,
-                                              float &w2, float &v0, float &v2) {
-  const float2 o2 = p_set(one);
-  const float2 a0 = p_mul(p_set(0.2f), p_add(o2, make_float2(q0, q2)));
-  const float a1 = 0.5f * (one + q1);
-  const float2 a2 = p_mul(p_set(0.3f), p_add(o2, make_float2(q2, q0)));
-  const float2 sum = p_add(p_add(a0, a2), p_set(a1));
-  const float2 is = make_float2(1.0f / sum.x, 1.0f / sum.y);
-  const float2 W0 = p_mul(a0, is), W2 = p_mul(a2, is);
-  w0 = W0.x;
-  w2 = W2.x;
-  v0 = W0.y;
-  v2 = W2.y;
-}
-
-// the compact row of both systems from their (w0, w2) and neighbour averages
-__device__ __forceinline__ void row2(float2 w0, float2 w2, float2 up, float2 u0, float2 un,
-                                     float2 &a, float2 &b, float2 &c, float2 &r) {
-  const float2 th = p_set(1.0f / 3.0f), sx = p_set(1.0f / 6.0f);
-  a = p_mul(p_add(p_set(1.0f), p_add(w0, p_neg(w2))), th);
-  b = p_mul(p_add(p_set(2.0f), p_neg(w0)), th);
-  c = p_mul(w2, th);
-  const float2 k0 = p_fma(p_set(-4.0f), w2, p_set(5.0f));                 // 5 - 4 w2
-  const float2 k1 = p_fma(p_set(4.0f), w2, p_add(p_set(1.0f), p_neg(w0)));  // 1 - w0 + 4 w2
-  r = p_mul(p_fma(k1, un, p_fma(k0, u0, p_mul(w0, up))), sx);
-}
-
 // ---------------------------------------------------------------- smem
-template <typename real, int NV, int WPV>
+template <typename real, int NV>
 struct Exch {
-  Fwd<real> warp_fwd[NV][2][WPV];
-  real warp_in[NV][2][WPV][3];   // incoming (c', d', z') of each warp
-  Fwd<real> seg_fwd[NV][2];
-  Bwd<real> warp_bwd[NV][2][WPV];
-  real warp_xn[NV][2][WPV][2];   // x, z after each warp
-  Bwd<real> seg_bwd[NV][2];
-  double sm[NV][2][6];           // y_f, z_f, y_l, z_l, -a0/b0 (periodic)
+  Run<real> seg[2 * NV];         // this segment as a run, per variable and side
   // mixed form, the line's reference state R (difference form): per
   // variable the hi / lo pair of the median of five sampled cells, R in
   // FP32, the reference fluxes F(R), (u_R, v_R, p_R, E_R + p_R), whether
@@ -476,27 +189,36 @@ struct Exch {
 // warp then hit distinct banks both when each lane walks its own chunk of M
 // cells (lane stride M) and when consecutive lanes take consecutive cells;
 // a chunk (M divides 128 bytes) never straddles a pad word.
-template <typename real, int NV, int M>
+template <typename real, int NV, int M, int KCHUNK>
 struct Smem {
-  static constexpr int KC = SEGC / M;     // chunks per conserved variable
-  static constexpr int WPV = KC / 32;     // warps per conserved variable
-  static constexpr int SEG = SEGC;
+  static constexpr int KC = KCHUNK;       // chunks per conserved variable
+  static constexpr int SEG = M * KC;      // cells per CTA segment
+  static constexpr int LPS = KC / 8;      // lanes that combine a system's chunks, eight each
   static constexpr int PSH = sizeof(real) == 4 ? 5 : 4;
   __host__ __device__ static constexpr int pad(int c) { return c + (c >> PSH); }
   static constexpr int UH = 3;                         // pad(-2) = -3
   static constexpr int UWP = UH + pad(SEG + 1) + 1;    // cells -2 .. SEG+1
   static constexpr int WP = pad(SEG - 1) + 1;          // cells 0 .. SEG-1
   static_assert(((32 * 4 / (int)sizeof(real)) % M) == 0, "a chunk must not straddle a pad word");
+  static_assert(KC % 32 == 0, "whole warps per variable");
+  // per system: six run values per chunk, and the last unknown of every chunk
+  // in walk order (entry 0: the unknown before the segment); one pad entry
+  // per eight, so that lanes walking eight chunks each hit distinct banks
+  static constexpr int KCP = KC + KC / 8;
+  static constexpr int XP = KC + 1 + KC / 8;
   static constexpr size_t u_off = 0;                                     // real Us[NV][UWP]
-  static constexpr size_t w_off = u_off + sizeof(real) * NV * UWP;       // real Wt[NV][4][WP]
-  static constexpr size_t fm_off = w_off + sizeof(real) * NV * 4 * WP;
-  static constexpr size_t fp_off = fm_off + sizeof(real) * NV * WP;      // real Fm, Fp[NV][WP]
-  static constexpr size_t fl_off = fp_off + sizeof(real) * NV * WP;      // real Fl[NV][SEG+2]
-  static constexpr size_t rm_off = fl_off + sizeof(real) * NV * (SEG + 2);  // remote stencils
-  static constexpr size_t ex_off = (rm_off + sizeof(real) * NV * 2 * 6 + 15) / 16 * 16;
+  static constexpr size_t fm_off = u_off + sizeof(real) * NV * UWP;      // real Fm, Fp[NV][WP]
+  static constexpr size_t fp_off = fm_off + sizeof(real) * NV * WP;
+  static constexpr size_t zm_off = fp_off + sizeof(real) * NV * WP;      // real Zm, Zp[NV][WP]
+  static constexpr size_t zp_off = zm_off + sizeof(real) * NV * WP;
+  static constexpr size_t fl_off = zm_off;     // real Fl[NV][SEG+2], after Zm and Zp are done with
+  static_assert(NV * (SEG + 2) <= 2 * NV * WP, "the fluxes must fit the two planes they reuse");
+  static constexpr size_t cr_off = zp_off + sizeof(real) * NV * WP;      // real Cr[2 NV][6][KCP]
+  static constexpr size_t xs_off = cr_off + sizeof(real) * 2 * NV * 6 * KCP;   // real Xs[2 NV][XP]
+  static constexpr size_t ex_off = (xs_off + sizeof(real) * 2 * NV * XP + 15) / 16 * 16;
   // mixed form: one byte per cell (its face values stored in full, not as
   // differences from R) and one per face (its flux stored as F - F(R))
-  static constexpr size_t cf_off = ex_off + sizeof(Exch<real, NV, WPV>);
+  static constexpr size_t cf_off = ex_off + sizeof(Exch<real, NV>);
   static constexpr size_t ff_off = cf_off + SEG;
   static constexpr size_t bytes = (ff_off + SEG + 2 + 15) / 16 * 16;
 };
@@ -524,35 +246,23 @@ __device__ __forceinline__ void atomic_min_bits(unsigned long long *w, unsigned 
 }
 
 // ---------------------------------------------------------------- kernel
-// Resident CTAs per SM the kernel is compiled for: the mixed form is bound by
-// latency, so it asks for three at M = 8 (85 registers a thread; the shared
-// memory of three segments fits) and two at M = 16; the FP64 form is bound by
-// the FP64 pipe and its shared memory allows one.
-#ifndef PPK_MIXED_CTAS_M8
-#define PPK_MIXED_CTAS_M8 3
-#endif
+// Resident CTAs per SM the kernel is compiled for (CTAS_*): see sweeps.cuh.
 // PRE: the face values come from another kernel (args.Fm_pre / Fp_pre) and
 // the reconstruction phases are compiled out.
-template <typename real, int NV, int M, bool PER, int MODE, bool PRE>
-__global__ void __launch_bounds__(NV * (SEGC / M),
-                                  sizeof(real) == 4 ? (M == 8 ? PPK_MIXED_CTAS_M8 : 2) : 1)
-    line_sweep(SweepArgs args_in) {
+template <typename real, int NV, int M, int KC, int MODE, bool PRE, int CTAS>
+__global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
   constexpr bool MIXED = sizeof(real) == 4;
-  using S = Smem<real, NV, M>;
+  using S = Smem<real, NV, M, KC>;
   constexpr int SEG = S::SEG;
-  constexpr int KC = S::KC;
-  constexpr int WPV = S::WPV;
   constexpr int T = NV * KC;
   constexpr int UW = SEG + 4;            // cells -2 .. SEG+1
   constexpr int UH = S::UH, UWP = S::UWP, WP = S::WP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   real *Us = reinterpret_cast<real *>(smem_raw + S::u_off);
-  real *Wt = reinterpret_cast<real *>(smem_raw + S::w_off);
   real *Fm = reinterpret_cast<real *>(smem_raw + S::fm_off);
   real *Fp = reinterpret_cast<real *>(smem_raw + S::fp_off);
   real *Fl = reinterpret_cast<real *>(smem_raw + S::fl_off);
-  real *Rm = reinterpret_cast<real *>(smem_raw + S::rm_off);
-  Exch<real, NV, WPV> &ex = *reinterpret_cast<Exch<real, NV, WPV> *>(smem_raw + S::ex_off);
+  Exch<real, NV> &ex = *reinterpret_cast<Exch<real, NV> *>(smem_raw + S::ex_off);
 
   cg::cluster_group cluster = cg::this_cluster();
   SweepArgs args = args_in;
@@ -572,7 +282,7 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
   const int v = tid / KC;
   const int k = tid % KC;
   const int lane = tid & 31;
-  const int w = k >> 5;
+  const bool per = args.bclo == 0;
   Ctl *ctl = args.ctl;
 
   // a finished problem skips the launch (uniform over the grid)
@@ -628,8 +338,8 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
     int g = gvar(kv, NV, args.vn, args.vt);
     neg = false;
     if (i < 0 || i >= n) {
-      if (PER) {
-        i = (i % n + n) % n;
+      if (per) {
+        i = i < 0 ? i + n : i - n;
       } else {
         int bc = i < 0 ? args.bclo : args.bchi;
         if (bc == 1) {
@@ -681,15 +391,6 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
       int kv = idx / UW, j = idx % UW;
       int i = lo - 2 + j;
       Us[kv * UWP + UH + S::pad(j - 2)] = (i < hi + 2) ? cell_val(kv, i) : real(0);
-    }
-  }
-  if (PER) {
-    // stencils of the two "position 0" cells (minus: cell 0, plus: cell n-1)
-    // for the Sherman-Morrison row at the far end of each system
-    for (int idx = tid; idx < NV * 2 * 5; idx += T) {
-      int kv = idx / 10, s = (idx / 5) % 2, j = idx % 5;
-      int c0 = s == 0 ? 0 : n - 1;
-      Rm[(kv * 2 + s) * 6 + j] = cell_val(kv, c0 - 2 + j);
     }
   }
 
@@ -800,16 +501,6 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
       } else {
         for (int idx = tid; idx < NV * UW; idx += T) conv_cell(idx / UW, idx % UW);
       }
-      if (PER) {
-        for (int idx = tid; idx < NV * 2 * 5; idx += T) {
-          const int kv = idx / 10, s = (idx / 5) % 2, j = idx % 5;
-          bool neg;
-          const long long a = cell_addr(kv, (s == 0 ? 0 : n - 1) - 2 + j, neg);
-          const float l = args.Ul[a];
-          const int o = (kv * 2 + s) * 6 + j;
-          Rm[o] = (Rm[o] - ex.rh[kv]) + ((neg ? -l : l) - ex.rl[kv]);
-        }
-      }
       __syncthreads();
     }
   }
@@ -837,671 +528,183 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
       Fp[kv * WP + S::pad(c)] = pp[o];
     }
   } else {
-    // ---------------------------------------------------------------- rows
+    // ---------------------------------------------------------------- solve
+    // this thread's chunk: cells lo + k M .. of variable v
+    real *Zm = reinterpret_cast<real *>(smem_raw + S::zm_off);
+    real *Zp = reinterpret_cast<real *>(smem_raw + S::zp_off);
+    real *Cr = reinterpret_cast<real *>(smem_raw + S::cr_off);
+    real *Xs = reinterpret_cast<real *>(smem_raw + S::xs_off);
     const real *uv = Us + v * UWP + UH;         // u of segment cell c at uv[pad(c)], c in [-2, SEG+2)
-    real *wt = Wt + v * 4 * WP;                 // wt[q*WP + pad(c)]: w0-, w2-, w0+, w2+
-    const int s0 = lo + k * M;                  // first cell of this thread's chunk
-    const int len = max(0, min(M, hi - s0));
     const int cb = S::pad(k * M);               // padded offset of the chunk's first cell
-    const bool bounded = !PER;
-    auto u_at = [&](int i) -> real { return uv[S::pad(i - lo)]; };
-
-    // the chunk's cells with a two-cell halo, from shared memory into registers
-    auto load_window = [&](real *win) {
-      win[0] = uv[S::pad(k * M - 2)];
-      win[1] = uv[S::pad(k * M - 1)];
-  #pragma unroll
-      for (int q = 0; q < M; ++q) win[q + 2] = uv[cb + q];
-      win[M + 2] = uv[S::pad(k * M + M)];
-      win[M + 3] = uv[S::pad(k * M + M + 1)];
-    };
-
-    // a, b of the unmodified position-0 row of side 0 (cell 0) or 1 (cell n-1),
-    // needed by the Sherman-Morrison row at the far end of a periodic system
-    auto far_row = [&](int side, real &a0, real &b0) {
-      const real *y = Rm + (v * 2 + side) * 6 + 2;
-      real q0, q1, q2, one, w0, w1, w2;
-      zratios_any(y[-2], y[-1], y[0], y[1], y[2], eps_v, q0, q1, q2, one);
-      if (side == 0) zweights(real(0.2), real(0.5), real(0.3), q0, q1, q2, w0, w1, w2, one);
-      else zweights(real(0.2), real(0.5), real(0.3), q2, q1, q0, w0, w1, w2, one);
-      Row<real> r = compact_row02(w0, w2, real(0), real(0), real(0));
-      a0 = r.a;
-      b0 = r.b;
-    };
-
-    // row of the periodic end cell i (0 or n-1), side 0 (minus) or 1 (plus),
-    // from the stored weights; zr = the Sherman-Morrison right-hand side entry
-    auto per_row = [&](int i, int side, real &zr) -> Row<real> {
-      const real *o = wt + 2 * side * WP + S::pad(i - lo);
-      const real xm = u_at(i - 1), x0 = u_at(i), xp = u_at(i + 1);
-      Row<real> r = side == 0 ? compact_row02(o[0], o[WP], xm, x0, xp)
-                              : compact_row02(o[0], o[WP], xp, x0, xm);
-      const int first = side == 0 ? 0 : n - 1, last = side == 0 ? n - 1 : 0;
-      zr = real(0);
-      if (i == first) {          // T = A - u v^T with g = -b at position 0
-        zr = -r.b;
-        r.b = r.b + r.b;
-        r.a = real(0);
-      } else if (i == last) {    // corner removed, b reduced by c a0 / g
-        real a0, b0;
-        far_row(side, a0, b0);
-        zr = r.c;
-        r.b = r.b + r.c * a0 / b0;
-        r.c = real(0);
-      }
-      return r;
-    };
-
-    // ------------------------------------------- weights + chunk maps (F1)
-    // weights are stored for the elimination pass (F5); the rows come from the
-    // register window.  The bounded closure cells store their explicit
-    // WENO5-Z face values in the w0 slots instead (rows 0 x + 1 x + 0 x = f).
-    Fwd<real> fm = fwd_identity<real>(), fp = fwd_identity<real>();
-    {
-      real win[M + 4];
-      load_window(win);
-  #pragma unroll
-      for (int j = 0; j < M; ++j) {
-        if (j < len) {
-          const int i = s0 + j;
-          real zm = real(0), zp = real(0);
-          Row<real> rm, rp;
-          if (bounded && (i == 0 || i == n - 1)) {
-            real fmv = weno5z_face(win[j], win[j + 1], win[j + 2], win[j + 3], win[j + 4], eps_v);
-            real fpv = weno5z_face(win[j + 4], win[j + 3], win[j + 2], win[j + 1], win[j], eps_v);
-            wt[cb + j] = fmv;
-            wt[2 * WP + cb + j] = fpv;
-            rm.a = real(0); rm.b = real(1); rm.c = real(0); rm.r = fmv;
-            rp.a = real(0); rp.b = real(1); rp.c = real(0); rp.r = fpv;
-          } else {
-            real w0, w2, v0, v2;
-            if constexpr (MIXED) {
-              real q0, q1, q2, one;
-              zratios_any(win[j], win[j + 1], win[j + 2], win[j + 3], win[j + 4], eps_v, q0, q1, q2,
-                          one);
-              zweights_pair(q0, q1, q2, one, w0, w2, v0, v2);
-            } else {
-              zweights_both_fp64(win[j], win[j + 1], win[j + 2], win[j + 3], win[j + 4], eps_v, w0,
-                                 w2, v0, v2);
-            }
-            wt[cb + j] = w0;
-            wt[WP + cb + j] = w2;
-            wt[2 * WP + cb + j] = v0;
-            wt[3 * WP + cb + j] = v2;
-            if (PER && (i == 0 || i == n - 1)) {
-              rm = per_row(i, 0, zm);
-              rp = per_row(i, 1, zp);
-            } else {
-              rm = compact_row02(w0, w2, win[j + 1], win[j + 2], win[j + 3]);
-              rp = compact_row02(v0, v2, win[j + 3], win[j + 2], win[j + 1]);
-            }
-          }
-          fwd_push_left<real, PER>(fm, rm, zm);
-          fwd_push_right<real, PER>(fp, rp, zp);
-        }
-      }
-    }
-    fwd_normalise(fm);
-    fwd_normalise(fp);
-
-    // ------------------------------------------- warp inclusive scans (F2)
-    // minus maps accumulate from the lower lanes, plus maps from the higher
-    if constexpr (MIXED) {
-      Fwd2 f2 = fwd2_pack(fm, fp);
-      const float2 one2 = p_set(1.0f), zero2 = p_set(0.0f);
-  #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const bool am = lane >= d, ap = lane + d < 32;
-        Fwd2 o;
-        // every lane executes both shuffles; the select comes after
-  #define PPK_SH2(fld, idv)                                                    \
-    {                                                                          \
-      const float tm_ = __shfl_up_sync(0xffffffffu, f2.fld.x, d);              \
-      const float tp_ = __shfl_down_sync(0xffffffffu, f2.fld.y, d);            \
-      o.fld.x = am ? tm_ : idv.x;                                              \
-      o.fld.y = ap ? tp_ : idv.y;                                              \
-    }
-        PPK_SH2(g00, one2); PPK_SH2(g01, zero2); PPK_SH2(g10, zero2); PPK_SH2(g11, one2);
-        PPK_SH2(dP, zero2); PPK_SH2(dQ, zero2); PPK_SH2(mu, one2);
-        if (PER) { PPK_SH2(zP, zero2); PPK_SH2(zQ, zero2); } else { o.zP = zero2; o.zQ = zero2; }
-  #undef PPK_SH2
-        f2 = fwd2_compose<PER>(f2, o);   // with the identity where a lane has no partner
-        fwd2_normalise(f2);
-      }
-      fwd2_unpack(f2, fm, fp);
-    } else {
-  #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        Fwd<real> o = fwd_shfl<real, PER, true>(fm, d);
-        if (lane >= d) { fm = fwd_compose<real, PER>(fm, o); fwd_normalise(fm); }
-        Fwd<real> q = fwd_shfl<real, PER, false>(fp, d);
-        if (lane + d < 32) { fp = fwd_compose<real, PER>(fp, q); fwd_normalise(fp); }
-      }
-    }
-    if (lane == 31) ex.warp_fwd[v][0][w] = fm;
-    if (lane == 0) ex.warp_fwd[v][1][w] = fp;
-    __syncthreads();
-
-    // ------------------------------------------- CTA segment maps (F3)
-    if (tid < 2 * NV) {
-      int vv = tid >> 1, sd = tid & 1;
-      Fwd<real> sg = fwd_identity<real>();
-      for (int ww = 0; ww < WPV; ++ww) {
-        int wi = sd == 0 ? ww : WPV - 1 - ww;
-        sg = fwd_compose<real, PER>(ex.warp_fwd[vv][sd][wi], sg);
-        fwd_normalise(sg);
-      }
-      ex.seg_fwd[vv][sd] = sg;
-    }
-    cluster.sync();
-
-    // ------------------------------------------- incoming states (F4)
-    // The segment maps of the CTAs ahead of this one on each side (minus: the
-    // lower ranks, applied in rank order; plus: the higher ranks, from the
-    // last one down) applied to the zero state that enters a line end.
-    // Mixed form (latency bound): composed by a tree over 16 lanes, lane q
-    // holding rank q's map (the identity where rank q is not ahead), so the
-    // remote reads happen at once.  FP64 form (bound by the FP64 pipe): one
-    // thread per side and variable applies them in turn, the fewest FP64
-    // operations.
-    real cin = real(0), din = real(0), zin = real(0);
-    int fvv = -1, fsd = 0;
-    if constexpr (MIXED) {
-      if (tid < 2 * NV * 16) {   // whole warps: T >= 2 NV 16 for M <= 16
-        const int grp = tid >> 4, q = tid & 15;
-        const int vv = grp >> 1, sd = grp & 1;
-        Fwd<real> mq = fwd_identity<real>();
-        if (q < R && (sd == 0 ? q < rank : q > rank)) {
-          Exch<real, NV, WPV> *rx = cluster.map_shared_rank(&ex, q);
-          mq = rx->seg_fwd[vv][sd];
-        }
-  #pragma unroll
-        for (int d = 1; d < 16; d <<= 1) {
-          Fwd<real> o = fwd_shfl<real, PER, false>(mq, d, 16);   // ranks q + d ...
-          if ((q & (2 * d - 1)) == 0) {
-            mq = sd == 0 ? fwd_compose<real, PER>(o, mq) : fwd_compose<real, PER>(mq, o);
-            fwd_normalise(mq);
-          }
-        }
-        if (q == 0) {
-          fwd_apply<real, PER>(mq, cin, din, zin);
-          fvv = vv;
-          fsd = sd;
-        }
-      }
-    } else {
-      if (tid < 2 * NV) {
-        const int vv = tid >> 1, sd = tid & 1;
-        if (sd == 0) {
-          for (int q = 0; q < rank; ++q) {
-            Exch<real, NV, WPV> *rx = cluster.map_shared_rank(&ex, q);
-            fwd_apply<real, PER>(rx->seg_fwd[vv][0], cin, din, zin);
-          }
-        } else {
-          for (int q = R - 1; q > rank; --q) {
-            Exch<real, NV, WPV> *rx = cluster.map_shared_rank(&ex, q);
-            fwd_apply<real, PER>(rx->seg_fwd[vv][1], cin, din, zin);
-          }
-        }
-        fvv = vv;
-        fsd = sd;
-      }
-    }
-    if (fvv >= 0) {   // the state entering each warp of this segment
-      for (int ww = 0; ww < WPV; ++ww) {
-        int wi = fsd == 0 ? ww : WPV - 1 - ww;
-        ex.warp_in[fvv][fsd][wi][0] = cin;
-        ex.warp_in[fvv][fsd][wi][1] = din;
-        ex.warp_in[fvv][fsd][wi][2] = zin;
-        fwd_apply<real, PER>(ex.warp_fwd[fvv][fsd][wi], cin, din, zin);
-      }
-    }
-    __syncthreads();
-
-    // the state after each lane's chunk (its inclusive map applied to the
-    // warp's incoming state), handed to the next lane in elimination order
-    real cpm, dpm, zpm, cpp, dpp, zpp;
-    {
-      const real cw = ex.warp_in[v][0][w][0], dw = ex.warp_in[v][0][w][1], zw = ex.warp_in[v][0][w][2];
-      real c = cw, d = dw, z = zw;
-      fwd_apply<real, PER>(fm, c, d, z);
-      cpm = shfl_up_r(c, 1);
-      dpm = shfl_up_r(d, 1);
-      zpm = PER ? shfl_up_r(z, 1) : real(0);
-      if (lane == 0) { cpm = cw; dpm = dw; zpm = zw; }
-    }
-    {
-      const real cw = ex.warp_in[v][1][w][0], dw = ex.warp_in[v][1][w][1], zw = ex.warp_in[v][1][w][2];
-      real c = cw, d = dw, z = zw;
-      fwd_apply<real, PER>(fp, c, d, z);
-      cpp = shfl_down_r(c, 1);
-      dpp = shfl_down_r(d, 1);
-      zpp = PER ? shfl_down_r(z, 1) : real(0);
-      if (lane == 31) { cpp = cw; dpp = dw; zpp = zw; }
-    }
-
-    // ------------------------------------------- chunk elimination (F5)
-    // Thomas elimination of the chunk from the incoming state, and the chunk's
-    // back-substitution map x_first = A + B x_after accumulated in the same
-    // pass: A = sum_j (prod_{l<j} -c'_l) d'_j, B = prod_l -c'_l.  The minus
-    // system runs over the chunk's cells left to right, the plus system right
-    // to left.  c', d' of a cell overwrite its two weights (read just before by
-    // the same thread); z' stays in registers (periodic lines).
-    // Mixed form: the recurrence runs on the projective state (P, Q, D, Z),
-    // c' = P/Q, d' = D/Q, z' = Z/Q, mapped linearly by a row (P <- c Q,
-    // Q <- b Q - a P, D <- r Q - a D), so consecutive rows depend on each other
-    // through two multiply-adds and the reciprocals 1/Q are off that chain
-    // (over one chunk Q changes by at most M factors b - a c': no rescaling).
-    // FP64 form: the plain recurrence with one division per row, the fewest
-    // FP64 operations.
-    real zmv[PER ? M : 1], zpv[PER ? M : 1];
-    Bwd<real> bm, bp;
-    // a full chunk without a line-end cell: every row is a plain compact row
-    const bool plain = len == M && s0 > 0 && s0 + M < n;
-    bool done5 = false;
-    if constexpr (MIXED) {
-      if (plain) {   // both systems together in paired FP32, no guards
-        float win[M + 4];
-        load_window(win);
-        float *om = wt + cb, *op = wt + 2 * WP + cb;
-        float2 P = make_float2(cpm, cpp), Q = p_set(1.0f), D = make_float2(dpm, dpp);
-        float2 Z = make_float2(zpm, zpp);
-        float2 pi = p_set(1.0f), A = p_set(0.0f), Az = p_set(0.0f);
-  #pragma unroll
-        for (int jj = 0; jj < M; ++jj) {
-          const int jm = jj, jp = M - 1 - jj;    // minus left to right, plus right to left
-          float2 a, b, c, r;
-          row2(make_float2(om[jm], op[jp]), make_float2(om[WP + jm], op[WP + jp]),
-               make_float2(win[jm + 1], win[jp + 3]), make_float2(win[jm + 2], win[jp + 2]),
-               make_float2(win[jm + 3], win[jp + 1]), a, b, c, r);
-          const float2 na = p_neg(a);
-          const float2 nq = p_fma(na, P, p_mul(b, Q));
-          D = p_fma(na, D, p_mul(r, Q));
-          if (PER) Z = p_mul(na, Z);            // zero right-hand side away from the ends
-          P = p_mul(c, Q);
-          Q = nq;
-          const float2 iq = make_float2(1.0f / Q.x, 1.0f / Q.y);
-          const float2 co = p_mul(P, iq), dd = p_mul(D, iq);
-          om[jm] = co.x;
-          om[WP + jm] = dd.x;
-          op[jp] = co.y;
-          op[WP + jp] = dd.y;
-          A = p_fma(pi, dd, A);
-          if (PER) {
-            const float2 zz = p_mul(Z, iq);
-            zmv[jm] = zz.x;
-            zpv[jp] = zz.y;
-            Az = p_fma(pi, zz, Az);
-          }
-          pi = p_mul(pi, p_neg(co));
-        }
-        bm.A = A.x; bm.Az = Az.x; bm.B = pi.x;
-        bp.A = A.y; bp.Az = Az.y; bp.B = pi.y;
-        done5 = true;
-      }
-    }
-    if (!done5) {
-      real win[M + 4];
-      load_window(win);
-      // projective state (mixed) or (c', -, d', z') (FP64) of each side
-      real Pm = cpm, Qm = real(1), Dm = dpm, Zm = zpm;
-      real Pp = cpp, Qp = real(1), Dp = dpp, Zp = zpp;
-      real pim = real(1), Am = real(0), Azm = real(0);
-      real pip = real(1), Ap = real(0), Azp = real(0);
-      (void)Qm; (void)Qp;   // the FP64 chains carry no Q
-      auto elim = [&](const Row<real> &r, real zr, real &P, real &Qs, real &D, real &Z,
-                      real &co, real &dout, real &zo) {
-        if constexpr (MIXED) {
-          real nq = r.b * Qs - r.a * P;
-          D = r.r * Qs - r.a * D;
-          if (PER) Z = zr * Qs - r.a * Z;
-          P = r.c * Qs;
-          Qs = nq;
-          real iq = real(1) / Qs;
-          co = P * iq;
-          dout = D * iq;
-          zo = PER ? Z * iq : real(0);
-        }
-      };
-      // the row of cell s0 + j of side sd (0 minus, 1 plus) and its z entry
-      auto row_of = [&](int sd, int j, real &zr) -> Row<real> {
-        const int i = s0 + j;
-        const real *o = wt + 2 * sd * WP + cb + j;
-        Row<real> r;
-        zr = real(0);
-        if (bounded && (i == 0 || i == n - 1)) {
-          r.a = real(0); r.b = real(1); r.c = real(0); r.r = o[0];
-        } else if (PER && (i == 0 || i == n - 1)) {
-          r = per_row(i, sd, zr);
-        } else if (sd == 0) {
-          r = compact_row02(o[0], o[WP], win[j + 1], win[j + 2], win[j + 3]);
-        } else {
-          r = compact_row02(o[0], o[WP], win[j + 3], win[j + 2], win[j + 1]);
-        }
-        return r;
-      };
-      // c', d' (and z') of a row stored over its weights; the back map grows
-      auto finish = [&](int sd, int j, real co, real dd, real zz) {
-        real *o = wt + 2 * sd * WP + cb + j;
-        o[0] = co;
-        o[WP] = dd;
-        if (sd == 0) {
-          if (PER) zmv[j] = zz;
-          Am += pim * dd;
-          if (PER) Azm += pim * zz;
-          pim *= -co;
-        } else {
-          if (PER) zpv[j] = zz;
-          Ap += pip * dd;
-          if (PER) Azp += pip * zz;
-          pip *= -co;
-        }
-      };
-  #pragma unroll
-      for (int jj = 0; jj < M; ++jj) {
-        const int jm = jj, jp = M - 1 - jj;    // minus left to right, plus right to left
-        const bool am = jm < len, ap = jp < len;
-        if constexpr (MIXED) {
-          if (am) {
-            real zr, co, dd, zz;
-            const Row<real> r = row_of(0, jm, zr);
-            elim(r, zr, Pm, Qm, Dm, Zm, co, dd, zz);
-            finish(0, jm, co, dd, zz);
-          }
-          if (ap) {
-            real zr, co, dd, zz;
-            const Row<real> r = row_of(1, jp, zr);
-            elim(r, zr, Pp, Qp, Dp, Zp, co, dd, zz);
-            finish(1, jp, co, dd, zz);
-          }
-        } else {
-          // FP64: one division for the pivots of both chains,
-          // 1/(q_m q_p) times q_p and q_m
-          real zrm = real(0), zrp = real(0);
-          Row<real> rm, rp;
-          rm.a = rm.c = rm.r = rp.a = rp.c = rp.r = real(0);
-          rm.b = rp.b = real(1);
-          if (am) rm = row_of(0, jm, zrm);
-          if (ap) rp = row_of(1, jp, zrp);
-          const real qm = am ? rm.b - rm.a * Pm : real(1);
-          const real qp = ap ? rp.b - rp.a * Pp : real(1);
-          const real inv = real(1) / (qm * qp);
-          if (am) {
-            const real ip = qp * inv;
-            Dm = (rm.r - rm.a * Dm) * ip;
-            if (PER) Zm = (zrm - rm.a * Zm) * ip;
-            Pm = rm.c * ip;
-            finish(0, jm, Pm, Dm, Zm);
-          }
-          if (ap) {
-            const real ip = qm * inv;
-            Dp = (rp.r - rp.a * Dp) * ip;
-            if (PER) Zp = (zrp - rp.a * Zp) * ip;
-            Pp = rp.c * ip;
-            finish(1, jp, Pp, Dp, Zp);
-          }
-        }
-      }
-      bm.A = Am; bm.Az = Azm; bm.B = pim;
-      bp.A = Ap; bp.Az = Azp; bp.B = pip;
-    }
-
-    // ------------------------------------------- backward scans (F6)
-    // minus back maps accumulate from the higher lanes (its back substitution
-    // runs right to left), plus maps from the lower lanes
-    Bwd<real> bm_in = bm, bp_in = bp;
-    if constexpr (MIXED) {
-      Bwd2 b2;
-      b2.A = make_float2(bm.A, bp.A);
-      b2.B = make_float2(bm.B, bp.B);
-      b2.Az = make_float2(bm.Az, bp.Az);
-  #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const bool am = lane + d < 32, ap = lane >= d;
-        Bwd2 o;
+    const int w0 = lo + (k & ~31) * M;          // first cell of the warp's chunks
+    const bool wlive = w0 < n;                  // (uniform over the warp)
+    typename Pair<real>::t cs[M - 1];
+    if (wlive) {
+      Run<real> rm, rp;
+      {
+        real D[M + 3], S0[M], S1[M], S2[M];
         {
-          float tm = __shfl_down_sync(0xffffffffu, b2.A.x, d), tp = __shfl_up_sync(0xffffffffu, b2.A.y, d);
-          o.A = make_float2(am ? tm : 0.0f, ap ? tp : 0.0f);
+          real win[M + 4];   // the chunk's cells with a two-cell halo
+          win[0] = uv[S::pad(k * M - 2)];
+          win[1] = uv[S::pad(k * M - 1)];
+#pragma unroll
+          for (int q = 0; q < M; ++q) win[q + 2] = uv[cb + q];
+          win[M + 2] = uv[S::pad(k * M + M)];
+          win[M + 3] = uv[S::pad(k * M + M + 1)];
+          chunk_weights<real, M>(win, eps_v, D, S0, S1, S2);
         }
-        {
-          float tm = __shfl_down_sync(0xffffffffu, b2.B.x, d), tp = __shfl_up_sync(0xffffffffu, b2.B.y, d);
-          o.B = make_float2(am ? tm : 1.0f, ap ? tp : 1.0f);
-        }
-        if (PER) {
-          float tm = __shfl_down_sync(0xffffffffu, b2.Az.x, d), tp = __shfl_up_sync(0xffffffffu, b2.Az.y, d);
-          o.Az = make_float2(am ? tm : 0.0f, ap ? tp : 0.0f);
-        } else {
-          o.Az = p_set(0.0f);
-        }
-        b2 = bwd2_compose(b2, o);   // with the identity where a lane has no partner
+        const EdgeInfo e = {lo + k * M, n, per};
+        real *dm = Fm + v * WP + cb, *dp = Fp + v * WP + cb;
+        real *zm = Zm + v * WP + cb, *zp = Zp + v * WP + cb;
+        // a warp without a line end skips the edge rows' tests
+        if (w0 + 32 * M >= n || (w0 == 0 && !per))
+          chunk_eliminate<real, M, true>(D, S0, S1, S2, e, dm, zm, dp, zp, cs, rm, rp);
+        else
+          chunk_eliminate<real, M, false>(D, S0, S1, S2, e, dm, zm, dp, zp, cs, rm, rp);
       }
-      bm_in.A = b2.A.x; bm_in.B = b2.B.x; bm_in.Az = b2.Az.x;
-      bp_in.A = b2.A.y; bp_in.B = b2.B.y; bp_in.Az = b2.Az.y;
-    } else {
-  #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        Bwd<real> o;
-        o.A = shfl_down_r(bm_in.A, d); o.B = shfl_down_r(bm_in.B, d);
-        o.Az = PER ? shfl_down_r(bm_in.Az, d) : real(0);
-        if (lane + d < 32) bm_in = bwd_compose(bm_in, o);
-        Bwd<real> q;
-        q.A = shfl_up_r(bp_in.A, d); q.B = shfl_up_r(bp_in.B, d);
-        q.Az = PER ? shfl_up_r(bp_in.Az, d) : real(0);
-        if (lane >= d) bp_in = bwd_compose(bp_in, q);
-      }
+      real *cm = Cr + (2 * v) * 6 * S::KCP + k + (k >> 3), *cp = cm + 6 * S::KCP;
+      cm[0] = rm.A; cm[S::KCP] = rm.B; cm[2 * S::KCP] = rm.G;
+      cm[3 * S::KCP] = rm.D; cm[4 * S::KCP] = rm.F; cm[5 * S::KCP] = rm.C;
+      cp[0] = rp.A; cp[S::KCP] = rp.B; cp[2 * S::KCP] = rp.G;
+      cp[3 * S::KCP] = rp.D; cp[4 * S::KCP] = rp.F; cp[5 * S::KCP] = rp.C;
     }
-    if (lane == 0) ex.warp_bwd[v][0][w] = bm_in;
-    if (lane == 31) ex.warp_bwd[v][1][w] = bp_in;
     __syncthreads();
 
-    // ------------------------------------------- segment back maps (F7)
-    if (tid < 2 * NV) {
-      int vv = tid >> 1, sd = tid & 1;
-      Bwd<real> sg;
-      sg.A = real(0); sg.B = real(1); sg.Az = real(0);
-      // minus: first cell of the segment = warp 0 o warp 1 o ...; plus: the
-      // last warp's map is applied first
-      for (int ww = WPV - 1; ww >= 0; --ww) {
-        int wi = sd == 0 ? ww : WPV - 1 - ww;
-        sg = bwd_compose(ex.warp_bwd[vv][sd][wi], sg);
-      }
-      ex.seg_bwd[vv][sd] = sg;
-    }
-    cluster.sync();
-    // back substitution entering this segment from the far side: the back maps
-    // of the CTAs behind it in that order (minus: the higher ranks, the last
-    // acting first; plus: the lower ranks, rank 0 acting first); x = 0 after
-    // the line end.  Mixed form: a tree over 16 lanes as in F4; FP64 form: one
-    // thread per side and variable.
-    {
-      real xb = real(0), zb = real(0);
-      int bvv = -1, bsd = 0;
-      if constexpr (MIXED) {
-        if (tid < 2 * NV * 16) {
-          const int grp = tid >> 4, q = tid & 15;
-          const int vv = grp >> 1, sd = grp & 1;
-          Bwd<real> bq;
-          bq.A = real(0); bq.B = real(1); bq.Az = real(0);
-          if (q < R && (sd == 0 ? q > rank : q < rank)) {
-            Exch<real, NV, WPV> *rx = cluster.map_shared_rank(&ex, q);
-            bq = rx->seg_bwd[vv][sd];
-          }
-  #pragma unroll
-          for (int d = 1; d < 16; d <<= 1) {
-            Bwd<real> o;
-            o.A = shfl_down_r(bq.A, d, 16);
-            o.B = shfl_down_r(bq.B, d, 16);
-            o.Az = PER ? shfl_down_r(bq.Az, d, 16) : real(0);
-            if ((q & (2 * d - 1)) == 0) bq = sd == 0 ? bwd_compose(bq, o) : bwd_compose(o, bq);
-          }
-          if (q == 0) {
-            xb = bq.A;
-            zb = bq.Az;
-            bvv = vv;
-            bsd = sd;
-          }
+    // ------------------------------------------- the segment's chunks
+    // LPS lanes per system (variable and side), eight chunks each in walk
+    // order.  Within a lane the chunks' last unknowns l_q are eliminated one
+    // after another, l_q = Dt - Ft X_in - Ct l_{q+1}; the lanes' runs are
+    // joined by a butterfly, every lane keeping the meeting points on its
+    // path, so that the way down needs no exchange.  Serial work on one or
+    // two warps (the other CTAs of the SM fill the pipes meanwhile): a
+    // parallel cyclic reduction over the 32 chunks of a warp would take 4
+    // times the instructions.  Chunks beyond the line end (the last segment's)
+    // are left out: q0 .. q1 are the lane's chunks with cells; a lane without
+    // any is the empty run.
+    constexpr int LPS = S::LPS;
+    constexpr int NCOMB = (2 * NV * LPS + 31) / 32 * 32;
+    const bool comb = tid < NCOMB;
+    const bool on = tid < 2 * NV * LPS;
+    const int sys = on ? tid / LPS : 0, cl = tid % LPS, sd = sys & 1;
+    real Dt[7], Ft[7], Ct[7];
+    Run<real> run = run_empty<real>(), seg;
+    Cut<real> cut[3];
+    const int nlive = (hi - lo + M - 1) / M;
+    const int q0 = sd ? max(0, KC - nlive - 8 * cl) : 0;
+    const int q1 = sd ? 7 : min(8, nlive - 8 * cl) - 1;
+    if (comb) {
+      const real *cr = Cr + sys * 6 * S::KCP;
+      real al = real(0), be = real(0), ga = real(-1);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (q < q0 || q > q1) continue;
+        const int kw = 8 * cl + q, kk = sd ? KC - 1 - kw : kw;
+        const real *c = cr + kk + (kk >> 3);
+        const real cA = c[0], cB = c[S::KCP], cG = c[2 * S::KCP];
+        const real cD = c[3 * S::KCP], cF = c[4 * S::KCP], cC = c[5 * S::KCP];
+        if (q == q0) {
+          run.D = cD; run.F = cF; run.C = cC;
+          al = cA; be = cB; ga = cG;
+        } else {
+          const real i1 = rcp(fma(-run.C, cB, real(1)));
+          const real dt_ = fma(-run.C, cA, run.D) * i1, ft = run.F * i1, ct = -(run.C * cG) * i1;
+          if (q > 0) { Dt[q - 1] = dt_; Ft[q - 1] = ft; Ct[q - 1] = ct; }
+          al = fma(-ga, dt_, al);
+          be = fma(-ga, ft, be);
+          ga = -(ga * ct);
+          const real i2 = rcp(fma(-cF, ct, real(1)));
+          run.D = fma(-cF, dt_, cD) * i2;
+          run.F = -(cF * ft) * i2;
+          run.C = cC * i2;
         }
+      }
+      if (q0 <= q1) {
+        run.A = fma(-ga, run.D, al);
+        run.B = fma(-ga, run.F, be);
+        run.G = -(ga * run.C);
+      }
+      seg = run;
+#pragma unroll
+      for (int d = 1, h = 0; d < LPS; d <<= 1, ++h) {
+        const Run<real> o = run_shfl_xor(seg, d, LPS);
+        const bool rt = cl & d;
+        seg = run_join(rt ? o : seg, rt ? seg : o, cut[h]);
+      }
+      if (on && cl == 0) ex.seg[sys] = seg;
+    }
+    if (R > 1) cluster.sync();
+    if (comb) {
+      // the rest of the line as seen from this segment: l_rest = Dr - Fr
+      // X_last - Cr X_first before it, f_rest = Ar - Br X_last - Gr X_first
+      // after it.  Bounded: lane 0 joins the segments before, lane 1 those
+      // after; periodic: lane 0 joins all others around the ring.
+      Run<real> rest = run_empty<real>();
+      {
+        const int wpos = sd ? R - 1 - rank : rank;
+        const int cnt = per ? (cl == 0 ? R - 1 : 0) : (cl == 0 ? wpos : (cl == 1 ? R - 1 - wpos : 0));
+        int at = (per || cl) ? wpos + 1 : 0;
+        Cut<real> unused;
+#pragma unroll 1
+        for (int q = 0; q < cnt; ++q, ++at) {
+          if (at >= R) at -= R;
+          const Exch<real, NV> *rx = cluster.map_shared_rank(&ex, sd ? R - 1 - at : at);
+          const Run<real> o = rx->seg[sys];
+          rest = run_join(rest, o, unused);
+        }
+      }
+      const Run<real> r0 = run_shfl(rest, 0, LPS), r1 = run_shfl(rest, 1, LPS);
+      real xl, xr;   // the unknowns before and after the segment
+      if (per) {
+        // the ring's closure in FP64 (both forms): 2 x 2
+        const double A = seg.A, B = seg.B, G = seg.G, D = seg.D, F = seg.F, C = seg.C;
+        const double Ar = r0.A, Br = r0.B, Gr = r0.G, Dr = r0.D, Fr = r0.F, Cq = r0.C;
+        const double a11 = 1.0 - Fr * F - Cq * B, a12 = Fr * C + Cq * G;
+        const double a21 = Br * F + Gr * B, a22 = 1.0 - Br * C - Gr * G;
+        const double b1 = Dr - Fr * D - Cq * A, b2 = Ar - Br * D - Gr * A;
+        const double idet = rcp(a11 * a22 - a12 * a21);
+        xl = real((b1 * a22 + a12 * b2) * idet);
+        xr = real((a11 * b2 + a21 * b1) * idet);
       } else {
-        if (tid < 2 * NV) {
-          const int vv = tid >> 1, sd = tid & 1;
-          if (sd == 0) {
-            for (int q = R - 1; q > rank; --q) {
-              Exch<real, NV, WPV> *rx = cluster.map_shared_rank(&ex, q);
-              Bwd<real> b = rx->seg_bwd[vv][0];
-              xb = b.A + b.B * xb;
-              zb = b.Az + b.B * zb;
-            }
-          } else {
-            for (int q = 0; q < rank; ++q) {
-              Exch<real, NV, WPV> *rx = cluster.map_shared_rank(&ex, q);
-              Bwd<real> b = rx->seg_bwd[vv][1];
-              xb = b.A + b.B * xb;
-              zb = b.Az + b.B * zb;
-            }
-          }
-          bvv = vv;
-          bsd = sd;
+        const real a11 = fma(-r0.C, seg.B, real(1)), a12 = r0.C * seg.G;
+        const real a21 = r1.B * seg.F, a22 = fma(-r1.B, seg.C, real(1));
+        const real b1 = fma(-r0.C, seg.A, r0.D), b2 = fma(-r1.B, seg.D, r1.A);
+        const real idet = rcp(fma(a11, a22, -(a12 * a21)));
+        xl = fma(b1, a22, a12 * b2) * idet;
+        xr = fma(a11, b2, a21 * b1) * idet;
+      }
+      if (on && cl == 0) Xs[sys * S::XP] = xl;
+#pragma unroll
+      for (int h = 2; h >= 0; --h) {
+        if ((1 << h) < LPS) {
+          const Cut<real> &c = cut[h];
+          const real l = fma(c.q, xr, fma(-c.p, xl, c.u)), f = fma(-c.s, xr, fma(c.r, xl, c.v));
+          if (cl & (1 << h)) xl = l;
+          else xr = f;
         }
       }
-      if (bvv >= 0) {
-        for (int ww = 0; ww < WPV; ++ww) {
-          int wi = bsd == 0 ? WPV - 1 - ww : ww;
-          ex.warp_xn[bvv][bsd][wi][0] = xb;
-          ex.warp_xn[bvv][bsd][wi][1] = zb;
-          Bwd<real> b = ex.warp_bwd[bvv][bsd][wi];
-          xb = b.A + b.B * xb;
-          zb = b.Az + b.B * zb;
-        }
+      real x = fma(-run.C, xr, fma(-run.F, xl, run.D));
+      real *xs = Xs + sys * S::XP;
+#pragma unroll
+      for (int q = 7; q >= 0; --q) {
+        if (q < 7 && q < q1 && q >= q0) x = fma(-Ct[q], x, fma(-Ft[q], xl, Dt[q]));
+        if (q < q0) x = xl;   // what the first chunk with cells sees before it
+        const int pos = 8 * cl + q + 1;
+        if (on) xs[pos + (pos >> 3)] = x;
       }
     }
     __syncthreads();
 
-    // ------------------------------------------- back substitution (F8)
-    // minus from the chunk's last cell down, plus from its first cell up; c', d'
-    // come from the weight slots, the solution goes to Fm / Fp.  The value
-    // entering a chunk is the value leaving the neighbouring lane's chunk (its
-    // inclusive back map applied to the warp's entering value).
-    real xm, zm_, xp, zp_;
-    {
-      const real xn = ex.warp_xn[v][0][w][0], zn = ex.warp_xn[v][0][w][1];
-      const real xo = bm_in.A + bm_in.B * xn, zo = bm_in.Az + bm_in.B * zn;
-      xm = shfl_down_r(xo, 1);
-      zm_ = PER ? shfl_down_r(zo, 1) : real(0);
-      if (lane == 31) { xm = xn; zm_ = zn; }
-    }
-    {
-      const real xn = ex.warp_xn[v][1][w][0], zn = ex.warp_xn[v][1][w][1];
-      const real xo = bp_in.A + bp_in.B * xn, zo = bp_in.Az + bp_in.B * zn;
-      xp = shfl_up_r(xo, 1);
-      zp_ = PER ? shfl_up_r(zo, 1) : real(0);
-      if (lane == 0) { xp = xn; zp_ = zn; }
-    }
-    real zmo[PER ? M : 1], zpo[PER ? M : 1];
-    bool done8 = false;
-    if constexpr (MIXED) {
-      if (plain) {   // both systems together, no guards
-        const float *om = wt + cb, *op = wt + 2 * WP + cb;
-        float *dm = Fm + v * WP + cb, *dp = Fp + v * WP + cb;
-        float2 x2 = make_float2(xm, xp), z2 = make_float2(zm_, zp_);
-  #pragma unroll
-        for (int jj = 0; jj < M; ++jj) {
-          const int jm = M - 1 - jj, jp = jj;
-          const float2 nc = make_float2(-om[jm], -op[jp]);
-          x2 = p_fma(nc, x2, make_float2(om[WP + jm], op[WP + jp]));
-          dm[jm] = x2.x;
-          dp[jp] = x2.y;
-          if (PER) {
-            z2 = p_fma(nc, z2, make_float2(zmv[jm], zpv[jp]));
-            zmo[jm] = z2.x;
-            zpo[jp] = z2.y;
-          }
-        }
-        done8 = true;
-      }
-    }
-    if (!done8) {
-      {
-        const real *o = wt + cb;
-        real *dst = Fm + v * WP + cb;
-        real x = xm, z = zm_;
-  #pragma unroll
-        for (int jj = 0; jj < M; ++jj) {
-          const int j = M - 1 - jj;
-          if (j < len) {
-            const real c = o[j];
-            x = o[WP + j] - c * x;
-            dst[j] = x;
-            if (PER) {
-              z = zmv[j] - c * z;
-              zmo[j] = z;
-            }
-          }
-        }
-      }
-      {
-        const real *o = wt + 2 * WP + cb;
-        real *dst = Fp + v * WP + cb;
-        real x = xp, z = zp_;
-  #pragma unroll
-        for (int j = 0; j < M; ++j) {
-          if (j < len) {
-            const real c = o[j];
-            x = o[WP + j] - c * x;
-            dst[j] = x;
-            if (PER) {
-              z = zpv[j] - c * z;
-              zpo[j] = z;
-            }
-          }
-        }
-      }
-    }
-
-    if (PER) {
-      // Sherman-Morrison correction x = y - (v.y)/(1 + v.z) z, with
-      // v = e_first + (corner_first / g) e_last and corner_first / g = -a0/b0
-      // of the unmodified position-0 row; the scalars in FP64.  zmo, zpo are
-      // indexed by the chunk's cells.
-      real zm_last = real(0), zp_last = real(0);
-  #pragma unroll
-      for (int j = 0; j < M; ++j) {
-        if (j == len - 1) { zm_last = zmo[j]; zp_last = zpo[j]; }
-      }
-      if (len > 0 && s0 == 0) {              // cell 0: minus first, plus last
-        real a0, b0;
-        far_row(0, a0, b0);
-        ex.sm[v][0][4] = -(double)a0 / (double)b0;
-        ex.sm[v][0][0] = Fm[v * WP + 0];
-        ex.sm[v][0][1] = zmo[0];
-        ex.sm[v][1][2] = Fp[v * WP + 0];
-        ex.sm[v][1][3] = zpo[0];
-      }
-      if (len > 0 && s0 + len == n) {        // cell n-1: plus first, minus last
-        real a0, b0;
-        far_row(1, a0, b0);
-        ex.sm[v][1][4] = -(double)a0 / (double)b0;
-        ex.sm[v][1][0] = Fp[v * WP + S::pad(n - 1 - lo)];
-        ex.sm[v][1][1] = zp_last;
-        ex.sm[v][0][2] = Fm[v * WP + S::pad(n - 1 - lo)];
-        ex.sm[v][0][3] = zm_last;
-      }
-      cluster.sync();
-      {
-        Exch<real, NV, WPV> *r0 = cluster.map_shared_rank(&ex, 0);
-        Exch<real, NV, WPV> *rl = cluster.map_shared_rank(&ex, R - 1);
-        double facm = (r0->sm[v][0][0] + r0->sm[v][0][4] * rl->sm[v][0][2]) /
-                      (1.0 + r0->sm[v][0][1] + r0->sm[v][0][4] * rl->sm[v][0][3]);
-        double facp = (rl->sm[v][1][0] + rl->sm[v][1][4] * r0->sm[v][1][2]) /
-                      (1.0 + rl->sm[v][1][1] + rl->sm[v][1][4] * r0->sm[v][1][3]);
-        real fm_ = real(facm), fp_ = real(facp);
-  #pragma unroll
-        for (int j = 0; j < M; ++j) {
-          if (j < len) {
-            Fm[v * WP + cb + j] -= fm_ * zmo[j];
-            Fp[v * WP + cb + j] -= fp_ * zpo[j];
-          }
-        }
-      }
+    // ------------------------------------------- back substitution
+    if (wlive) {
+      const real *xm = Xs + (2 * v) * S::XP, *xp = xm + S::XP;
+      const int m0 = k, m1 = k + 1, p0 = KC - 1 - k, p1 = KC - k;
+      const typename Pair<real>::t xin = p_set(xm[m0 + (m0 >> 3)], xp[p0 + (p0 >> 3)]);
+      const typename Pair<real>::t xown = p_set(xm[m1 + (m1 >> 3)], xp[p1 + (p1 >> 3)]);
+      const int o = v * WP + cb, len = n - (lo + k * M);
+      if (w0 + 32 * M > n)
+        chunk_back<real, M, true>(uv + cb, Fm + o, Zm + o, Fp + o, Zp + o, cs, xin, xown, len);
+      else
+        chunk_back<real, M, false>(uv + cb, Fm + o, Zm + o, Fp + o, Zp + o, cs, xin, xown, len);
     }
   }
   __syncthreads();
@@ -1533,9 +736,9 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
       float ub[NV], a[NV], b[NV];
 #pragma unroll
       for (int kv = 0; kv < NV; ++kv) {
-        ub[kv] = float(Us[kv * UWP + UH + S::pad(c)]) + rf[kv];
-        a[kv] = float(Fm[kv * WP + S::pad(c)]) + rf[kv];
-        b[kv] = float(Fp[kv * WP + S::pad(c)]) + rf[kv];
+        ub[kv] = to_f32(Us[kv * UWP + UH + S::pad(c)]) + rf[kv];
+        a[kv] = to_f32(Fm[kv * WP + S::pad(c)]) + rf[kv];
+        b[kv] = to_f32(Fp[kv * WP + S::pad(c)]) + rf[kv];
       }
       if (limit_need_mixed<NV>(ub, a, b, wgl_f, inv12_f, eps_f)) mask |= 1u << q;
     }
@@ -1595,7 +798,7 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
     int il = 0, ir = 0;
     // left state: U^- of cell f-1
     if (f == 0) {
-      if (PER) {
+      if (per) {
         srcL = cluster.map_shared_rank(Fm, R - 1); il = (n - 1) - (R - 1) * SEG;
         cfL = cluster.map_shared_rank(cfull, R - 1);
       }
@@ -1605,7 +808,7 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
     } else { srcL = Fm; il = f - 1 - lo; }
     // right state: U^+ of cell f
     if (f == n) {
-      if (PER) {
+      if (per) {
         srcR = cluster.map_shared_rank(Fp, 0); ir = 0;
         cfR = cluster.map_shared_rank(cfull, 0);
       }
@@ -1679,8 +882,8 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
       if (args.bchi == 2) Ur[1] = -Ur[1];
     }
     if (args.flux) llf<real, NV>(Ul, Ur, gam, F, sf);
-    else hllc<real, NV>(Ul, Ur, gam, F, sf);
-    if (sf > fsmax || sf != sf) fsmax = sf;   // a NaN speed stays
+    else hllc<real, NV>(Ul, Ur, gam, F, sf, MIXED || args.fcheck);
+    if ((MIXED || args.fcheck) && (sf > fsmax || sf != sf)) fsmax = sf;   // a NaN speed stays
 #pragma unroll
     for (int kv = 0; kv < NV; ++kv) Fl[kv * (SEG + 2) + (f - lo)] = F[kv];
   };
@@ -1690,7 +893,7 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
     // any of this CTA's cells holds its face values in full
     anyfull = __syncthreads_or(anyfull);
     cluster_arrive();   // this CTA's limited face values, for the neighbours
-    const bool lo_remote = PER || lo > 0, hi_remote = PER || hi < n;
+    const bool lo_remote = per || lo > 0, hi_remote = per || hi < n;
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {   // one call site of the face code
       int f, fend;
@@ -1722,6 +925,8 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
   unsigned long long firstbad = ~0ull;
   const real ih = MIXED ? real(args.ih_f) : real(args.ih);
   const double dt = (MODE == MODE_FINAL) ? ctl->dt : 0.0;
+  const double gg1 = MIXED ? 0.0 : args.gamma * (args.gamma - 1.0);
+  (void)gg1;
   const real *Din = reinterpret_cast<const real *>(args.Din);
   for (int c = tid; c < hi - lo; c += T) {
     int i = lo + c;
@@ -1769,15 +974,15 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
       double mx = NV == 4 && args.vn != 1 ? Ut[2] : Ut[1];
       double my = NV == 4 ? (args.vn != 1 ? Ut[1] : Ut[2]) : 0.0;
       // one division per cell: 1/rho (1/h from the host)
-      const double irho = 1.0 / rho;
+      const double irho = rcp(rho);
       double e = (E - 0.5 * (mx * mx + my * my) * irho) * irho;
-      bool ok = (rho > 0.0) && (e > 0.0) && isfinite(E) && isfinite(mx) && isfinite(my);
+      bool ok = positive(rho) && positive(e) && finite(E) && finite(mx) && finite(my);
       if (!ok) {
         ++nbad;
         firstbad = min(firstbad, (unsigned long long)addr);
       } else {
-        mymin = fmin(mymin, rho);
-        double a = sqrt(args.gamma * (args.gamma - 1.0) * e);
+        mymin = less(rho, mymin) ? rho : mymin;
+        double a = root(gg1 * e);
         double rate;
         if (NV == 4) {
           const double ihx = args.vn == 1 ? args.ih : args.ih_other;
@@ -1786,7 +991,7 @@ __global__ void __launch_bounds__(NV * (SEGC / M),
         } else {
           rate = (fabs(mx) * irho + a) * args.ih;
         }
-        mymax = fmax(mymax, rate);
+        mymax = less(mymax, rate) ? rate : mymax;
       }
     } else {
       // mixed form: compensated stage combination on hi + lo pairs

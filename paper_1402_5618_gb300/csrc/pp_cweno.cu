@@ -811,12 +811,11 @@ void fill_state(const pp_cweno_s *h, SweepArgs &a, const void *Uin, const void *
   }
 }
 
-cudaError_t dispatch(const pp_cweno_s *h, int mode, bool periodic, const SweepArgs &a,
+cudaError_t dispatch(const pp_cweno_s *h, int mode, const SweepArgs &a,
                      long long nlines, bool attrs_only, cudaStream_t st_override = nullptr) {
   LaunchCfg c;
   c.precision = h->cfg.precision;
   c.nv = h->nv;
-  c.periodic = periodic;
   c.mode = mode;
   c.attrs_only = attrs_only;
   c.m = h->m;
@@ -996,7 +995,7 @@ cudaError_t launch(const pp_cweno_s *h, int mode, bool xdir, const void *Uin, co
     cudaError_t e = launch_char(h, a, is_mixed(h) ? (const void *)a.Uh : (const void *)a.U, nlines);
     if (e != cudaSuccess) return e;
   }
-  return dispatch(h, mode, a.bclo == PP_BC_PERIODIC, a, nlines, attrs_only);
+  return dispatch(h, mode, a, nlines, attrs_only);
 }
 
 // Batched launch of one line group.  eps_fixed > 0 with ctl: a measurement
@@ -1032,7 +1031,7 @@ cudaError_t launch_group(const pp_cweno_s *h, const LineGroup &g, int mode, cons
                                       st ? st : h->stream);
     if (e != cudaSuccess) return e;
   }
-  return dispatch(h, mode, g.periodic, a, g.nlines, attrs_only, st);
+  return dispatch(h, mode, a, g.nlines, attrs_only, st);
 }
 
 // y sweep of the mixed 2-D form over the transposed hi planes: a row sweep
@@ -1061,7 +1060,7 @@ cudaError_t launch_ysweep_t(const pp_cweno_s *h, int stage, bool char_done = fal
     cudaError_t e = launch_char(h, a, h->UT, h->nx);   // rows of the transposed planes
     if (e != cudaSuccess) return e;
   }
-  return dispatch(h, MODE_XSWEEP, a.bclo == PP_BC_PERIODIC, a, h->nx, false);
+  return dispatch(h, MODE_XSWEEP, a, h->nx, false);
 }
 
 // the y direction's characteristic-wise face values of the stage input on
@@ -1424,12 +1423,10 @@ int finish_create(pp_cweno_s *h) {
     h->m = mm;
     for (int m = 0; m < 3 && e == cudaSuccess; ++m) {
       if (h->nv == 3 && modes[m] == MODE_XSWEEP) continue;
-      for (int per = 0; per < 2 && e == cudaSuccess; ++per) {
-        SweepArgs a;
-        memset(&a, 0, sizeof(a));
-        a.R = 1;
-        e = dispatch(h, modes[m], per != 0, a, 0, true);
-      }
+      SweepArgs a;
+      memset(&a, 0, sizeof(a));
+      a.R = 1;
+      e = dispatch(h, modes[m], a, 0, true);
     }
   }
   h->m = keep_m;
@@ -2199,12 +2196,10 @@ int pp_cweno_operator_noalloc(const pp_cweno_config *cfg, const double *U_dev, d
         t.nv = ndim == 2 ? 4 : 3;
         for (int m = 0; m < 3; ++m) {
           if (t.nv == 3 && modes[m] == MODE_XSWEEP) continue;
-          for (int per = 0; per < 2; ++per) {
-            SweepArgs a;
-            memset(&a, 0, sizeof(a));
-            a.R = 1;
-            if (dispatch(&t, modes[m], per != 0, a, 0, true) != cudaSuccess) return PP_ERR_CUDA;
-          }
+          SweepArgs a;
+          memset(&a, 0, sizeof(a));
+          a.R = 1;
+          if (dispatch(&t, modes[m], a, 0, true) != cudaSuccess) return PP_ERR_CUDA;
         }
       }
       g_noalloc_ptr[dev] = ptr;

@@ -8,12 +8,19 @@
 
 namespace ppk {
 
-constexpr int SEG_CELLS = SEGC;   // cells per CTA of a line's cluster
+constexpr int SEG_CELLS = 512;    // cells per CTA of a line's cluster
+
+// thread layout by chunk length: 512 cells per CTA, one warp per variable at
+// M = 16 and two at M = 8, and the resident CTAs per SM asked for
+template <typename real, int M>
+struct Layout {
+  static constexpr int KC = SEG_CELLS / M;
+  static constexpr int CTAS = sizeof(real) == 4 ? (M == 8 ? 3 : 4) : (M == 8 ? 1 : 2);
+};
 
 struct LaunchCfg {
   int precision;   // 0 fp64, 1 mixed (fp32 line arithmetic)
   int nv;          // 3 or 4
-  bool periodic;
   int mode;        // MODE_*
   bool attrs_only; // set the kernel's attributes, launch nothing
   int m;           // rows per thread chunk: 8 or 16 (picked by the autotuner)
@@ -40,10 +47,11 @@ inline cudaError_t launch_sweep(const LaunchCfg &c, const SweepArgs &a, long lon
   return m16 ? launch_sweep_f32_m16(c, a, nlines, st) : launch_sweep_f32_m8(c, a, nlines, st);
 }
 
-template <typename real, int NV, int M, bool PER, int MODE, bool PRE>
+template <typename real, int NV, int M, int MODE, bool PRE>
 cudaError_t launch_m(const SweepArgs &a, long long nlines, cudaStream_t st, bool attrs_only) {
-  using S = Smem<real, NV, M>;
-  auto kern = line_sweep<real, NV, M, PER, MODE, PRE>;
+  constexpr int KC = Layout<real, M>::KC;
+  using S = Smem<real, NV, M, KC>;
+  auto kern = line_sweep<real, NV, M, KC, MODE, PRE, Layout<real, M>::CTAS>;
   if (attrs_only) {   // called at handle creation, outside any stream capture
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)S::bytes);
@@ -72,17 +80,17 @@ cudaError_t launch_m(const SweepArgs &a, long long nlines, cudaStream_t st, bool
 
 // the reconstructing kernel, or (M = 8 only) the one taking precomputed
 // face values; attrs_only sets the attributes of both
-template <typename real, int NV, int M, bool PER, int MODE>
+template <typename real, int NV, int M, int MODE>
 cudaError_t launch_pre(const LaunchCfg &c, const SweepArgs &a, long long nlines, cudaStream_t st) {
   if constexpr (M == 8) {
     if (c.attrs_only) {
-      cudaError_t e = launch_m<real, NV, M, PER, MODE, true>(a, nlines, st, true);
+      cudaError_t e = launch_m<real, NV, M, MODE, true>(a, nlines, st, true);
       if (e != cudaSuccess) return e;
     } else if (a.Fm_pre) {
-      return launch_m<real, NV, M, PER, MODE, true>(a, nlines, st, false);
+      return launch_m<real, NV, M, MODE, true>(a, nlines, st, false);
     }
   }
-  return launch_m<real, NV, M, PER, MODE, false>(a, nlines, st, c.attrs_only);
+  return launch_m<real, NV, M, MODE, false>(a, nlines, st, c.attrs_only);
 }
 
 template <typename real, int M>
@@ -90,23 +98,18 @@ cudaError_t launch_dispatch(const LaunchCfg &c, const SweepArgs &a, long long nl
                             cudaStream_t st) {
   if (c.nv == 3) {
     if (c.mode == MODE_FINAL)
-      return c.periodic ? launch_pre<real, 3, M, true, MODE_FINAL>(c, a, nlines, st)
-                        : launch_pre<real, 3, M, false, MODE_FINAL>(c, a, nlines, st);
+      return launch_pre<real, 3, M, MODE_FINAL>(c, a, nlines, st);
     if (c.mode == MODE_OPERATOR)
-      return c.periodic ? launch_pre<real, 3, M, true, MODE_OPERATOR>(c, a, nlines, st)
-                        : launch_pre<real, 3, M, false, MODE_OPERATOR>(c, a, nlines, st);
+      return launch_pre<real, 3, M, MODE_OPERATOR>(c, a, nlines, st);
     return cudaErrorInvalidValue;
   }
   if (c.nv == 4) {
     if (c.mode == MODE_XSWEEP)
-      return c.periodic ? launch_pre<real, 4, M, true, MODE_XSWEEP>(c, a, nlines, st)
-                        : launch_pre<real, 4, M, false, MODE_XSWEEP>(c, a, nlines, st);
+      return launch_pre<real, 4, M, MODE_XSWEEP>(c, a, nlines, st);
     if (c.mode == MODE_FINAL)
-      return c.periodic ? launch_pre<real, 4, M, true, MODE_FINAL>(c, a, nlines, st)
-                        : launch_pre<real, 4, M, false, MODE_FINAL>(c, a, nlines, st);
+      return launch_pre<real, 4, M, MODE_FINAL>(c, a, nlines, st);
     if (c.mode == MODE_OPERATOR)
-      return c.periodic ? launch_pre<real, 4, M, true, MODE_OPERATOR>(c, a, nlines, st)
-                        : launch_pre<real, 4, M, false, MODE_OPERATOR>(c, a, nlines, st);
+      return launch_pre<real, 4, M, MODE_OPERATOR>(c, a, nlines, st);
   }
   return cudaErrorInvalidValue;
 }
