@@ -19,4 +19,15 @@ struct LineRef {
   int prob, line;
 };
 
+// the same line as the line kernels read it, one record instead of a chain of
+// two: offset of its problem's block, first cell in a plane, cell stride,
+// plane size, length, boundaries, inverse cell sizes along and across
+struct LineDesc {
+  long long off, base, ncell;
+  double ih, ih_other;
+  float ih_f, ih_other_f;   // FP32 copies (a conversion takes a slot of the FP64 pipe)
+  int n, cs, prob;
+  short bclo, bchi;
+};
+
 }  // namespace ppk

@@ -105,52 +105,56 @@ struct SweepArgs {
   // arithmetic in the state's layout); nullptr: the kernel reconstructs them
   const void *Fm_pre, *Fp_pre;
   Ctl *ctl;
-  // batched launch: line table and problem descriptors (nullptr: one problem)
-  const LineRef *lines;
-  const ProbDesc *probs;
-  int xdir;           // batched launch: 1 x lines, 0 y lines, 2 rows of the transposed planes
-  long long nvals;    // batched mixed form: values per hi block (lo block follows)
+  // batched launch: line table (nullptr: one problem)
+  const LineDesc *lines;
 };
 
 // resolve the line a cluster works on: for a batched launch, take the
-// problem's grid, boundaries, control block and its slice of every buffer
-template <typename real, int NV>
-__device__ __forceinline__ void bind_line(SweepArgs &a, long long &line) {
-  if (!a.lines) return;
-  LineRef lr = a.lines[line];
-  const ProbDesc pd = a.probs[lr.prob];
-  line = lr.line;
-  a.ctl = a.ctl + lr.prob;
-  a.ncell = pd.ncell;
-  if (a.xdir == 1) {
-    a.n = pd.nx; a.cell_stride = 1; a.line_stride = pd.nx;
-    a.bclo = pd.bc[0]; a.bchi = pd.bc[1];
-    a.h = pd.dx; a.h_other = NV == 4 ? pd.dy : 0.0; a.ih = pd.idx; a.ih_other = NV == 4 ? pd.idy : 0.0;
-    a.ih_f = (float)a.ih; a.ih_other_f = (float)a.ih_other;
-  } else if (a.xdir == 2) {   // a row of the problem's transposed planes: a y line
-    a.n = pd.ny; a.cell_stride = 1; a.line_stride = pd.ny;
-    a.bclo = pd.bc[2]; a.bchi = pd.bc[3];
-    a.h = pd.dy; a.h_other = pd.dx; a.ih = pd.idy; a.ih_other = pd.idx;
-    a.ih_f = (float)a.ih; a.ih_other_f = (float)a.ih_other;
-  } else {
-    a.n = pd.ny; a.cell_stride = pd.nx; a.line_stride = 1;
-    a.bclo = pd.bc[2]; a.bchi = pd.bc[3];
-    a.h = pd.dy; a.h_other = pd.dx; a.ih = pd.idy; a.ih_other = pd.idx;
-    a.ih_f = (float)a.ih; a.ih_other_f = (float)a.ih_other;
-  }
-  const long long o = pd.off;
+// problem's grid, boundaries, control block and its slice of every buffer.
+// Returns the offset of the line's first cell in a plane.
+template <typename real>
+__device__ __forceinline__ long long bind_line(SweepArgs &a, long long line) {
+  if (!a.lines) return line * a.line_stride;
+  const LineDesc d = a.lines[line];
+  a.ctl = a.ctl + d.prob;
+  a.ncell = d.ncell;
+  a.n = d.n;
+  a.cell_stride = d.cs;
+  a.bclo = d.bclo;
+  a.bchi = d.bchi;
+  a.ih = d.ih;
+  a.ih_other = d.ih_other;
+  a.ih_f = d.ih_f;
+  a.ih_other_f = d.ih_other_f;
+  const long long o = d.off;
   if (a.U) a.U += o;
   if (a.U0) a.U0 += o;
   if (a.Uout) a.Uout += o;
-  if (a.Uh) { a.Uh += o; a.Ul = a.Uh + a.nvals; }
-  if (a.U0h) { a.U0h += o; a.U0l = a.U0h + a.nvals; }
-  if (a.Uoh) { a.Uoh += o; a.Uol = a.Uoh + a.nvals; }
+  if (a.Uh) a.Uh += o;
+  if (a.Ul) a.Ul += o;
+  if (a.U0h) { a.U0h += o; a.U0l += o; }
+  if (a.Uoh) { a.Uoh += o; a.Uol += o; }
   if (a.Lout) a.Lout += o;
+  if (a.Din) a.Din = reinterpret_cast<const real *>(a.Din) + o;
+  if (a.Dout) a.Dout = reinterpret_cast<real *>(a.Dout) + o;
   if (a.Fm_pre) {   // face values of the characteristic-wise reconstruction, same layout
     a.Fm_pre = reinterpret_cast<const real *>(a.Fm_pre) + o;
     a.Fp_pre = reinterpret_cast<const real *>(a.Fp_pre) + o;
   }
+  return d.base;
 }
+
+// asynchronous copy of one value global -> shared: a thread's loads of a
+// segment are all in flight together, whatever the line's alignment
+template <typename real>
+__device__ __forceinline__ void load_async(real *dst, const real *src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  if constexpr (sizeof(real) == 4)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void load_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 template <typename real>
 __device__ __forceinline__ real shfl_down_r(real v, int d, int width = 32) {
@@ -268,13 +272,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
   SweepArgs args = args_in;
   const int R = args.R;
   const int rank = (int)cluster.block_rank();
-  long long line = blockIdx.x / R;
-  bind_line<real, NV>(args, line);
-  if (args.lines) {   // D buffers follow the state layout of the batch
-    const long long o = args.probs[args_in.lines[blockIdx.x / R].prob].off;
-    if (args.Din) args.Din = reinterpret_cast<const real *>(args.Din) + o;
-    if (args.Dout) args.Dout = reinterpret_cast<real *>(args.Dout) + o;
-  }
+  const long long lbase = bind_line<real>(args, blockIdx.x / R);
   const int n = args.n;
   const int lo = rank * SEG;
   const int hi = min(lo + SEG, n);
@@ -308,13 +306,12 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
     else eps_pos = real(fmin(ctl->eps_pos, bits_double(ctl->minrho[args.stage - 1])));
   }
 
-  const long long lbase = line * args.line_stride;
   const long long cs = args.cell_stride;
   unsigned char *cfull = smem_raw + S::cf_off;   // mixed: cell's faces stored in full
   unsigned char *fdel = smem_raw + S::ff_off;    // mixed: face flux stored as F - F(R)
 
-  // difference form possible: the reference samples load with the hi parts;
-  // the lo parts, and the differences, only for lines that take the form
+  // difference form possible: the reference samples and the lo parts load
+  // with the hi parts
   const bool two = MIXED && !PRE && args.Ul != nullptr;
   float sh[5], sl[5];
   if constexpr (MIXED && !PRE) {
@@ -352,45 +349,38 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
     }
     return g * args.ncell + lbase + (long long)i * cs;
   };
-  auto cell_val = [&](int kv, int i) -> real {
-    bool neg;
-    const long long a = cell_addr(kv, i, neg);
-    real x;
-    if constexpr (MIXED) x = args.Uh[a];
-    else x = args.U[a];
-    return neg ? -x : x;
-  };
-
-  bool vec = false;
-  int nq = 0;
-  if constexpr (MIXED) {
-    // contiguous line with 16-byte aligned segments: the segment's cells
-    // come in as float4, only the halo and a ragged tail cell by cell
-    vec = cs == 1 && !args.lines && ((lbase + lo) & 3) == 0 && (args.ncell & 3) == 0 &&
-          ((reinterpret_cast<unsigned long long>(args.Uh) & 15) == 0);
-    if (vec) {
-      nq = (hi - lo) >> 2;
-      for (int idx = tid; idx < NV * nq; idx += T) {
-        int kv = idx / nq, q = idx - kv * nq;
-        int g = gvar(kv, NV, args.vn, args.vt);
-        const float4 x = *reinterpret_cast<const float4 *>(args.Uh + g * args.ncell + lbase + lo + 4 * q);
-        real *d = Us + kv * UWP + UH + S::pad(4 * q);
-        d[0] = x.x; d[1] = x.y; d[2] = x.z; d[3] = x.w;
+  // thread (v, k) brings in cells lo - 2 + k, + KC, ... of variable v; the
+  // lo parts go to the planes the face values take later
+  float *Ls = reinterpret_cast<float *>(Fm);
+  static_assert(!MIXED || UWP <= 2 * WP, "the lo parts must fit the face-value planes");
+  {
+    const long long plane = gvar(v, NV, args.vn, args.vt) * args.ncell + lbase;
+    const real *src;
+    if constexpr (MIXED) src = args.Uh + plane;
+    else src = args.U + plane;
+    const float *srl = two ? args.Ul + plane : nullptr;
+    real *dst = Us + v * UWP + UH;
+#pragma unroll 4
+    for (int j = k; j < UW; j += KC) {
+      const int i = lo - 2 + j, c = S::pad(j - 2);
+      if (i >= 0 && i < n) {
+        load_async(dst + c, src + (long long)i * cs);
+        if constexpr (MIXED) {
+          if (two) load_async(Ls + v * UWP + UH + c, srl + (long long)i * cs);
+        }
+      } else if (i < hi + 2) {   // ghost cell
+        bool neg;
+        const long long a = cell_addr(v, i, neg) - plane;
+        dst[c] = neg ? -src[a] : src[a];
+        if constexpr (MIXED) {
+          if (two) Ls[v * UWP + UH + c] = neg ? -srl[a] : srl[a];
+        }
+      } else {
+        dst[c] = real(0);
+        if constexpr (MIXED) {
+          if (two) Ls[v * UWP + UH + c] = 0.0f;
+        }
       }
-      const int nr = UW - 4 * nq;
-      for (int idx = tid; idx < NV * nr; idx += T) {
-        int kv = idx / nr, r = idx - kv * nr;
-        int j = r < 2 ? r : 4 * nq + r;
-        int i = lo - 2 + j;
-        Us[kv * UWP + UH + S::pad(j - 2)] = (i < hi + 2) ? cell_val(kv, i) : real(0);
-      }
-    }
-  }
-  if (!vec) {
-    for (int idx = tid; idx < NV * UW; idx += T) {
-      int kv = idx / UW, j = idx % UW;
-      int i = lo - 2 + j;
-      Us[kv * UWP + UH + S::pad(j - 2)] = (i < hi + 2) ? cell_val(kv, i) : real(0);
     }
   }
 
@@ -440,6 +430,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
       ex.rspread[kv] = spread;
     }
   }
+  load_async_wait();
   __syncthreads();
   if constexpr (MIXED) eps_pos = ex.epsf;
   if constexpr (MIXED && !PRE) {
@@ -472,34 +463,13 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
     }
     if (dlt) {
       // (hi - R_hi) + (lo - R_lo), exact where hi and R_hi are within a
-      // factor of two of each other: each thread brings in the lo parts of
-      // the cells it loaded (the same loops) and replaces their hi parts
-      auto conv = [&](int kv, int slot, float l) {
-        Us[slot] = (Us[slot] - ex.rh[kv]) + (l - ex.rl[kv]);
-      };
-      auto conv_cell = [&](int kv, int j) {
-        const int i = lo - 2 + j;
-        if (i >= hi + 2) return;
-        bool neg;
-        const long long a = cell_addr(kv, i, neg);
-        const float l = args.Ul[a];
-        conv(kv, kv * UWP + UH + S::pad(j - 2), neg ? -l : l);
-      };
-      if (vec) {
-        for (int idx = tid; idx < NV * nq; idx += T) {
-          const int kv = idx / nq, q = idx - kv * nq;
-          const int g = gvar(kv, NV, args.vn, args.vt);
-          const float4 y = *reinterpret_cast<const float4 *>(args.Ul + g * args.ncell + lbase + lo + 4 * q);
-          const int b = kv * UWP + UH + S::pad(4 * q);
-          conv(kv, b, y.x); conv(kv, b + 1, y.y); conv(kv, b + 2, y.z); conv(kv, b + 3, y.w);
-        }
-        const int nr = UW - 4 * nq;
-        for (int idx = tid; idx < NV * nr; idx += T) {
-          const int kv = idx / nr, r = idx - kv * nr;
-          conv_cell(kv, r < 2 ? r : 4 * nq + r);
-        }
-      } else {
-        for (int idx = tid; idx < NV * UW; idx += T) conv_cell(idx / UW, idx % UW);
+      // factor of two of each other
+      const float rh = ex.rh[v], rl = ex.rl[v];
+      real *dst = Us + v * UWP + UH;
+      const float *lsp = Ls + v * UWP + UH;
+      for (int j = k; j < UW; j += KC) {
+        const int c = S::pad(j - 2);
+        if (lo - 2 + j < hi + 2) dst[c] = (dst[c] - rh) + (lsp[c] - rl);
       }
       __syncthreads();
     }
@@ -976,7 +946,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
       // one division per cell: 1/rho (1/h from the host)
       const double irho = rcp(rho);
       double e = (E - 0.5 * (mx * mx + my * my) * irho) * irho;
-      bool ok = positive(rho) && positive(e) && finite(E) && finite(mx) && finite(my);
+      bool ok = positive(rho) && positive(e) && is_finite(E) && is_finite(mx) && is_finite(my);
       if (!ok) {
         ++nbad;
         firstbad = min(firstbad, (unsigned long long)addr);

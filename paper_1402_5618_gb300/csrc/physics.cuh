@@ -57,8 +57,8 @@ __device__ __forceinline__ bool less(double a, double b) {
   q ^= (q >> 63) & 0x7fffffffffffffffll;
   return p < q;
 }
-__device__ __forceinline__ bool finite(float x) { return isfinite(x); }
-__device__ __forceinline__ bool finite(double x) {
+__device__ __forceinline__ bool is_finite(float x) { return isfinite(x); }
+__device__ __forceinline__ bool is_finite(double x) {
   return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
 }
 

@@ -113,83 +113,22 @@ __global__ void step_end_kernel(Ctl *ctls, int nprob) {
   if (++ctl->nrej_run > 60) ctl->err_rate = 1;
 }
 
-// Checked steps leave U^n in its buffer and U^{n+1} in the stage buffer,
-// and the two buffers swap roles for the next step; where a step was
-// rejected, or a problem took no step (finished, stopped, or past its step
-// limit), U^n is copied into the stage buffer so that the next step starts
-// from it again.  Problem p (blockIdx.y) owns the 32-bit words [a0, a0 + n)
-// and [a1, a1 + n) of both buffers (FP64 values, or the FP32 hi and lo planes
-// of the mixed form).
-__global__ void restore_kernel(const unsigned int *src, unsigned int *dst, const ProbDesc *probs,
-                               long long nvals, int mixed, int nv, const Ctl *ctls) {
-  const int p = blockIdx.y;
-  const Ctl *ctl = ctls + p;
-  if (ctl->active && step_accepted(ctl)) return;
-  long long a0 = 0, a1 = nvals, n = nvals;   // single problem: everything
-  if (probs) {
-    const ProbDesc pd = probs[p];
-    n = (long long)nv * pd.ncell;
-    a0 = mixed ? pd.off : 2 * pd.off;
-    a1 = mixed ? nvals + pd.off : 2 * pd.off + n;
-  }
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    dst[a0 + i] = src[a0 + i];
-    dst[a1 + i] = src[a1 + i];
-  }
-}
-
-// Reductions of a state: min density, max rate, cells outside G.  The
-// state is FP64 planes (lo == nullptr) or FP32 hi / lo plane pairs.
+// Reductions of a state: min density, max rate, cells outside G.  The state
+// is FP64 planes (lo == nullptr) or FP32 hi / lo plane pairs.  Blocks (x)
+// stride over the cells of one problem (y; probs == nullptr: the single one).
+// Bound by the FP64 pipe (2 lanes per SM): about 30 FP64 instructions per
+// cell, with reciprocals instead of divisions and integer comparisons
+// (4096^2 FP64: 3.3 ms with divisions).  Batches take one block per 2048
+// cells of the longest problem: one block per problem left most SMs idle
+// (64 problems of up to 1024^2 cells: 23.7 ms).
 template <int NV>
-__global__ void state_reduce_kernel(const void *Uv, const float *lo, long long ncell, long long nx,
-                                    double dx, double dy, double gamma, Ctl *ctl) {
-  double mn = 1e300, mx = 0.0;
-  unsigned long long bad = 0, first = ~0ull;
-  auto at = [&](long long i) -> double {
-    if (lo) return (double)reinterpret_cast<const float *>(Uv)[i] + (double)lo[i];
-    return reinterpret_cast<const double *>(Uv)[i];
-  };
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
-       c += (long long)gridDim.x * blockDim.x) {
-    double rho = at(c), m1 = at(ncell + c), m2 = NV == 4 ? at(2 * ncell + c) : 0.0;
-    double E = at((NV - 1) * ncell + c);
-    double e = E / rho - 0.5 * (m1 * m1 + m2 * m2) / (rho * rho);
-    bool ok = rho > 0.0 && e > 0.0 && isfinite(E) && isfinite(m1) && isfinite(m2) && isfinite(rho);
-    if (!ok) {
-      ++bad;
-      first = (unsigned long long)c < first ? (unsigned long long)c : first;
-      continue;
-    }
-    mn = fmin(mn, rho);
-    double a = sqrt(gamma * (gamma - 1.0) * e);
-    double r = (fabs(m1 / rho) + a) / dx;
-    if (NV == 4) r += (fabs(m2 / rho) + a) / dy;
-    mx = fmax(mx, r);
-  }
-  for (int d = 16; d > 0; d >>= 1) {
-    mn = fmin(mn, __shfl_down_sync(0xffffffffu, mn, d));
-    mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, d));
-    bad += __shfl_down_sync(0xffffffffu, bad, d);
-    unsigned long long f = __shfl_down_sync(0xffffffffu, first, d);
-    first = f < first ? f : first;
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicMin(&ctl->minrho[2], dbits(mn));
-    atomicMax(&ctl->rate, dbits(mx));
-    if (bad) {
-      atomicAdd(&ctl->nviol, bad);
-      atomicMin(&ctl->first_bad, first);
-    }
-  }
-}
-
-// Batched form of the same reductions: one block per problem.
-template <int NV>
-__global__ void batch_reduce_kernel(const void *Uv, const float *lo, const ProbDesc *probs,
-                                    double gamma, Ctl *ctls) {
-  const ProbDesc pd = probs[blockIdx.x];
-  Ctl *ctl = ctls + blockIdx.x;
+__global__ void __launch_bounds__(256)
+    state_reduce_kernel(const void *Uv, const float *lo, const ProbDesc *probs, ProbDesc pd,
+                        double gamma, Ctl *ctls) {
+  if (probs) pd = probs[blockIdx.y];
+  Ctl *ctl = ctls + blockIdx.y;
+  const long long nc = pd.ncell;
+  const double gg1 = gamma * (gamma - 1.0);
   double mn = 1e300, mx = 0.0;
   unsigned long long bad = 0, first = ~0ull;
   auto at = [&](long long i) -> double {
@@ -197,33 +136,34 @@ __global__ void batch_reduce_kernel(const void *Uv, const float *lo, const ProbD
     if (lo) return (double)reinterpret_cast<const float *>(Uv)[i] + (double)lo[i];
     return reinterpret_cast<const double *>(Uv)[i];
   };
-  const long long nc = pd.ncell;
-  for (long long c = threadIdx.x; c < nc; c += blockDim.x) {
-    double rho = at(c), m1 = at(nc + c), m2 = NV == 4 ? at(2 * nc + c) : 0.0;
-    double E = at((NV - 1) * nc + c);
-    double e = E / rho - 0.5 * (m1 * m1 + m2 * m2) / (rho * rho);
-    bool ok = rho > 0.0 && e > 0.0 && isfinite(E) && isfinite(m1) && isfinite(m2) && isfinite(rho);
-    if (!ok) {
+  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nc;
+       c += (long long)gridDim.x * blockDim.x) {
+    const double rho = at(c), m1 = at(nc + c), m2 = NV == 4 ? at(2 * nc + c) : 0.0;
+    const double E = at((NV - 1) * nc + c);
+    const double ir = rcp(rho);
+    const double e = (E - 0.5 * (m1 * m1 + m2 * m2) * ir) * ir;
+    if (!(positive(rho) && positive(e) && is_finite(E) && is_finite(m1) && is_finite(m2) && is_finite(rho))) {
       ++bad;
       first = (unsigned long long)c < first ? (unsigned long long)c : first;
       continue;
     }
-    mn = fmin(mn, rho);
-    double a = sqrt(gamma * (gamma - 1.0) * e);
-    double r = (fabs(m1 / rho) + a) / pd.dx;
-    if (NV == 4) r += (fabs(m2 / rho) + a) / pd.dy;
-    mx = fmax(mx, r);
+    mn = less(rho, mn) ? rho : mn;
+    const double a = root(gg1 * e);
+    double r = (fabs(m1) * ir + a) * pd.idx;
+    if (NV == 4) r += (fabs(m2) * ir + a) * pd.idy;
+    mx = less(mx, r) ? r : mx;
   }
   for (int d = 16; d > 0; d >>= 1) {
-    mn = fmin(mn, __shfl_down_sync(0xffffffffu, mn, d));
-    mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, d));
+    const double omn = __shfl_down_sync(0xffffffffu, mn, d), omx = __shfl_down_sync(0xffffffffu, mx, d);
+    mn = less(omn, mn) ? omn : mn;
+    mx = less(mx, omx) ? omx : mx;
     bad += __shfl_down_sync(0xffffffffu, bad, d);
     unsigned long long f = __shfl_down_sync(0xffffffffu, first, d);
     first = f < first ? f : first;
   }
   if ((threadIdx.x & 31) == 0) {
-    atomicMin(&ctl->minrho[2], dbits(mn));
-    atomicMax(&ctl->rate, dbits(mx));
+    atomic_min_bits(&ctl->minrho[2], dbits(mn));
+    atomic_max_bits(&ctl->rate, dbits(mx));
     if (bad) {
       atomicAdd(&ctl->nviol, bad);
       atomicMin(&ctl->first_bad, first);
@@ -254,11 +194,7 @@ __device__ __forceinline__ void transpose_tile(const float *src, float *dst, int
   }
 }
 
-// gate (checked steps): transpose only when the step just taken was
-// rejected, restoring the transposed planes of U^n
-__global__ void transpose_planes_kernel(const float *in, float *out, int nx, int ny, long long ncell,
-                                        const Ctl *gate) {
-  if (gate && (!gate->active || step_accepted(gate))) return;
+__global__ void transpose_planes_kernel(const float *in, float *out, int nx, int ny, long long ncell) {
   const int v = blockIdx.z;
   transpose_tile(in + v * ncell, out + v * ncell, blockIdx.x * TT, blockIdx.y * TT, nx, ny);
 }
@@ -269,15 +205,50 @@ struct TileRef {
 };
 
 __global__ void transpose_planes_b_kernel(const float *in, float *out, const TileRef *tiles,
-                                          const ProbDesc *probs, long long nvals, int nv,
-                                          const Ctl *gates) {
+                                          const ProbDesc *probs, long long nvals, int nv) {
   const TileRef t = tiles[blockIdx.x];
-  if (gates && (!gates[t.prob].active || step_accepted(gates + t.prob))) return;
   const ProbDesc pd = probs[t.prob];
   // planes 0 .. nv-1: hi parts; nv .. 2 nv - 1: the lo parts nvals behind
   const int v = (int)blockIdx.y;
   const long long o = (v < nv ? 0 : nvals) + pd.off + (v % nv) * pd.ncell;
   transpose_tile(in + o, out + o, t.i0, t.j0, pd.nx, pd.ny);
+}
+
+// Checked steps leave U^n in its buffer and U^{n+1} in the stage buffer,
+// and the two buffers swap roles for the next step; where a step was
+// rejected, or a problem took no step (finished, stopped, or past its step
+// limit), U^n is copied into the stage buffer so that the next step starts
+// from it again, and after a rejection its transposed planes (UT, mixed 2-D
+// form) are formed again.  Problem p (blockIdx.y) owns the 32-bit words
+// [a0, a0 + n) and [a1, a1 + n) of both buffers (FP64 values, or the FP32 hi
+// and lo planes of the mixed form).  Nearly every step is accepted, so the
+// cost is that of blocks that find nothing to do: few blocks, each striding
+// over its problem (one block per 32 x 32 tile took 0.19 ms a step on
+// 4096^2, and 64 blocks per problem 0.39 ms on 4096 problems).
+__global__ void __launch_bounds__(256)
+    restore_kernel(const unsigned int *src, unsigned int *dst, float *UT, const ProbDesc *probs,
+                   ProbDesc pd, long long nvals, int mixed, int nv, const Ctl *ctls) {
+  const int p = blockIdx.y;
+  const Ctl *ctl = ctls + p;
+  if (ctl->active && step_accepted(ctl)) return;
+  if (probs) pd = probs[p];
+  const long long n = (long long)nv * pd.ncell;
+  const long long a0 = mixed ? pd.off : 2 * pd.off;
+  const long long a1 = mixed ? nvals + pd.off : 2 * pd.off + n;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  for (long long i = blockIdx.x * 256ll + tid; i < n; i += gridDim.x * 256ll) {
+    dst[a0 + i] = src[a0 + i];
+    dst[a1 + i] = src[a1 + i];
+  }
+  if (!UT || !ctl->active) return;
+  const float *in = reinterpret_cast<const float *>(src);
+  const int ntx = (pd.nx + TT - 1) / TT, nty = (pd.ny + TT - 1) / TT;
+  for (long long t = blockIdx.x; t < (long long)ntx * nty * 2 * nv; t += gridDim.x) {
+    const int v = (int)(t / ((long long)ntx * nty)), q = (int)(t % ((long long)ntx * nty));
+    const long long o = (v < nv ? 0 : nvals) + pd.off + (v % nv) * pd.ncell;
+    transpose_tile(in + o, UT + o, q % ntx * TT, q / ntx * TT, pd.nx, pd.ny);
+    __syncthreads();   // the tile's shared memory is read before the next one fills it
+  }
 }
 
 // The same stage combination with 16-byte accesses (nx, ny multiples of 4):
@@ -649,7 +620,8 @@ struct LineGroup {
   bool periodic;
   bool xdir;
   bool trans = false;         // y lines as rows of the transposed planes (mixed 2-D batches)
-  LineRef *lines = nullptr;   // device
+  LineRef *lines = nullptr;   // device: problem and line (the characteristic kernels)
+  LineDesc *descs = nullptr;  // device: the same lines resolved (the line kernels)
   long long nlines = 0;
   // characteristic-wise batches: the longest line of the group and the
   // group's own row and block-solve scratch (groups of a direction run
@@ -931,7 +903,7 @@ cudaError_t launch_char_group(const pp_cweno_s *h, const LineGroup &g, const Swe
   c.eps_weno = h->cfg.eps_weno;
   c.lines = g.lines;
   c.probs = h->probs;
-  c.xdir = a.xdir;
+  c.xdir = g.xdir ? 1 : (g.trans ? 2 : 0);
   cudaError_t e = cudaSuccess;
   if (h->char_tuning && is_mixed(h)) e = pick_char_layout(c, h->nv, g.periodic, st, &g.char_layout);
   c.layout = g.char_layout;
@@ -1012,13 +984,10 @@ cudaError_t launch_group(const pp_cweno_s *h, const LineGroup &g, int mode, cons
   a.Dout = Dout;
   a.Lout = Lout;
   a.R = g.R;
-  a.lines = g.lines;
-  a.probs = h->probs;
-  a.xdir = g.xdir ? 1 : (g.trans ? 2 : 0);
-  a.nvals = nvals(h);
+  a.lines = g.descs;
   if (g.trans) {   // rows of the transposed hi planes in, D_y transposed out
     a.Uh = h->UT;
-    a.Ul = nullptr;
+    a.Ul = h->UT + nvals(h);
     a.U0h = a.U0l = a.Uoh = a.Uol = nullptr;
     a.Din = nullptr;
     a.Dout = h->DT;
@@ -1120,21 +1089,33 @@ cudaError_t launch_combine_b(const pp_cweno_s *h, const void *Uin, void *Uout, i
   return cudaGetLastError();
 }
 
-// transposed hi planes of U^n; gated: only for the problems whose checked
-// step was just rejected
-cudaError_t transpose_state_hi(const pp_cweno_s *h, bool gated = false) {
-  const Ctl *gate = gated ? h->ctl : nullptr;
+// descriptor of a single problem in the layout of a batch's
+ProbDesc single_desc(const pp_cweno_s *h) {
+  ProbDesc d;
+  memset(&d, 0, sizeof(d));
+  d.nx = (int)h->nx;
+  d.ny = (int)h->ny;
+  d.ncell = h->ncell;
+  d.dx = h->dx;
+  d.dy = h->dy;
+  d.idx = 1.0 / h->dx;
+  d.idy = 1.0 / h->dy;
+  return d;
+}
+
+// transposed hi and lo planes of U^n
+cudaError_t transpose_state_hi(const pp_cweno_s *h) {
   if (h->btrans) {
     transpose_planes_b_kernel<<<dim3((unsigned)h->ntiles, (unsigned)(2 * h->nv)), dim3(TT, 8), 0,
                                 h->stream>>>(hi_of(h->U0), h->UT, h->tiles, h->probs, nvals(h),
-                                             h->nv, gate);
+                                             h->nv);
     return cudaGetLastError();
   }
   // the hi planes and the lo planes behind them, 2 nv planes in one launch
   dim3 grid((unsigned)((h->nx + TT - 1) / TT), (unsigned)((h->ny + TT - 1) / TT),
             (unsigned)(2 * h->nv));
   transpose_planes_kernel<<<grid, dim3(TT, 8), 0, h->stream>>>(hi_of(h->U0), h->UT, (int)h->nx,
-                                                               (int)h->ny, h->ncell, gate);
+                                                               (int)h->ny, h->ncell);
   return cudaGetLastError();
 }
 
@@ -1142,20 +1123,16 @@ cudaError_t transpose_state_hi(const pp_cweno_s *h, bool gated = false) {
 // stage buffer and its transposed planes back; then the per-problem
 // bookkeeping.  The caller swaps U0 and U1 afterwards.
 cudaError_t finish_checked_step(pp_cweno_s *h, const std::function<void()> &mark) {
-  const long long per = h->batch ? 0 : nvals(h);
-  long long longest = per;
-  if (h->batch)
-    for (const ProbDesc &d : h->probs_h) longest = std::max(longest, (long long)h->nv * d.ncell);
-  const unsigned bx = (unsigned)std::min<long long>(h->batch ? 64 : 4096, (longest + 255) / 256);
-  restore_kernel<<<dim3(std::max(1u, bx), (unsigned)h->nprob), 256, 0, h->stream>>>(
+  long long longest = h->batch ? 0 : nvals(h);
+  for (const ProbDesc &d : h->probs_h) longest = std::max(longest, (long long)h->nv * d.ncell);
+  // 64 words per thread and array; a single problem has the GPU to itself
+  const unsigned bx = (unsigned)std::min<long long>(h->batch ? 64 : 1216, (longest + 16383) / 16384);
+  restore_kernel<<<dim3(bx, (unsigned)h->nprob), dim3(TT, 8), 0, h->stream>>>(
       reinterpret_cast<const unsigned int *>(h->U0), reinterpret_cast<unsigned int *>(h->U1),
-      h->batch ? h->probs : nullptr, nvals(h), is_mixed(h) ? 1 : 0, h->nv, h->ctl);
+      h->ytrans || h->btrans ? h->UT : nullptr, h->batch ? h->probs : nullptr, single_desc(h),
+      nvals(h), is_mixed(h) ? 1 : 0, h->nv, h->ctl);
   cudaError_t e = cudaGetLastError();
   mark();
-  if (e == cudaSuccess && (h->ytrans || h->btrans)) {
-    e = transpose_state_hi(h, true);
-    mark();
-  }
   if (e != cudaSuccess) return e;
   step_end_kernel<<<(h->nprob + 127) / 128, 128, 0, h->stream>>>(h->ctl, h->nprob);
   e = cudaGetLastError();
@@ -1302,6 +1279,18 @@ int build_graph(pp_cweno_s *h) {
   return cuerr(e);
 }
 
+// the reduction's launch: a block per 2048 cells of the longest problem, at
+// most a full wave of blocks for a single one
+void launch_reduce(const pp_cweno_s *h, const void *U, const float *lo, const ProbDesc *probs, Ctl *ctl) {
+  long long longest = h->batch ? 0 : h->ncell;
+  for (const ProbDesc &d : h->probs_h) longest = std::max(longest, d.ncell);
+  const dim3 grid((unsigned)std::min<long long>(1216, (longest + 2047) / 2048), (unsigned)h->nprob);
+  if (h->nv == 4)
+    state_reduce_kernel<4><<<grid, 256, 0, h->stream>>>(U, lo, probs, single_desc(h), h->cfg.gamma, ctl);
+  else
+    state_reduce_kernel<3><<<grid, 256, 0, h->stream>>>(U, lo, probs, single_desc(h), h->cfg.gamma, ctl);
+}
+
 // reductions (min rho, max rate, violations) of a state into ctl[0..nprob)
 int reduce_state(pp_cweno_s *h, const void *U, Ctl *ctl, bool split_planes) {
   std::vector<Ctl> z((size_t)h->nprob);
@@ -1314,21 +1303,7 @@ int reduce_state(pp_cweno_s *h, const void *U, Ctl *ctl, bool split_planes) {
                                   h->stream);
   if (e != cudaSuccess) return PP_ERR_CUDA;
   const float *lo = split_planes ? lo_of(h, const_cast<void *>(U)) : nullptr;
-  if (h->batch) {
-    if (h->nv == 4)
-      batch_reduce_kernel<4><<<h->nprob, 256, 0, h->stream>>>(U, lo, h->probs, h->cfg.gamma, ctl);
-    else
-      batch_reduce_kernel<3><<<h->nprob, 256, 0, h->stream>>>(U, lo, h->probs, h->cfg.gamma, ctl);
-  } else {
-    int blocks = (int)fmin(1184.0, (double)((h->ncell + 255) / 256));
-    if (blocks < 1) blocks = 1;
-    if (h->nv == 4)
-      state_reduce_kernel<4><<<blocks, 256, 0, h->stream>>>(U, lo, h->ncell, h->nx, h->dx, h->dy,
-                                                            h->cfg.gamma, ctl);
-    else
-      state_reduce_kernel<3><<<blocks, 256, 0, h->stream>>>(U, lo, h->ncell, h->nx, h->dx, h->dy,
-                                                            h->cfg.gamma, ctl);
-  }
+  launch_reduce(h, U, lo, h->batch ? h->probs : nullptr, ctl);
   e = cudaStreamSynchronize(h->stream);   // z must outlive the copy
   if (e == cudaSuccess) e = cudaGetLastError();
   return cuerr(e);
@@ -1441,7 +1416,7 @@ int finish_create(pp_cweno_s *h) {
     const int chars = h->cfg.recon == PP_RECON_CHARACTERISTIC ? 2 * sweeps : 0;
     h->launches_per_step = 1 + 3 * ((h->ytrans ? 3 : sweeps) + chars);
   }
-  if (h->fcheck) h->launches_per_step += 2 + ((h->ytrans || h->btrans) ? 1 : 0);
+  if (h->fcheck) h->launches_per_step += 2;
   return PP_OK;
 }
 
@@ -1480,7 +1455,6 @@ int autotune_batch(pp_cweno_s *h) {
       memset(&a, 0, sizeof(a));
       fill_state(h, a, h->U0, h->U0, nullptr);
       fill_common(h, a, 0, 1e-13, h->ctl_scratch);
-      a.xdir = g.xdir ? 1 : (g.trans ? 2 : 0);
       a.vn = g.xdir ? 1 : 2;
       a.vt = h->nv == 4 ? (g.xdir ? 2 : 1) : -1;
       e = launch_char_group(h, g, a, g.trans ? (const void *)h->UT : (const void *)a.Uh, h->stream);
@@ -1743,6 +1717,35 @@ int pp_cweno_create_batch(const pp_cweno_config *cfgs, int64_t nprob, void *cuda
       const ProbDesc &d = h->probs_h[lr.prob];
       h->groups[g].nmax = std::max(h->groups[g].nmax, h->groups[g].xdir ? d.nx : d.ny);
     }
+    std::vector<LineDesc> descs;
+    descs.reserve(slines[g].size());
+    for (const LineRef &lr : slines[g]) {
+      const ProbDesc &d = h->probs_h[lr.prob];
+      LineDesc q;
+      memset(&q, 0, sizeof(q));
+      q.off = d.off;
+      q.ncell = d.ncell;
+      q.prob = lr.prob;
+      if (gx) {
+        q.n = d.nx; q.cs = 1; q.base = (long long)lr.line * d.nx;
+      } else if (h->groups[g].trans) {   // a row of the problem's transposed planes
+        q.n = d.ny; q.cs = 1; q.base = (long long)lr.line * d.ny;
+      } else {
+        q.n = d.ny; q.cs = d.nx; q.base = lr.line;
+      }
+      q.bclo = (short)d.bc[gx ? 0 : 2];
+      q.bchi = (short)d.bc[gx ? 1 : 3];
+      q.ih = gx ? d.idx : d.idy;
+      q.ih_other = h->nv == 4 ? (gx ? d.idy : d.idx) : 0.0;
+      q.ih_f = (float)q.ih;
+      q.ih_other_f = (float)q.ih_other;
+      descs.push_back(q);
+    }
+    e = cudaMalloc(&h->groups[g].descs, sizeof(LineDesc) * descs.size());
+    if (e == cudaSuccess)
+      e = cudaMemcpy(h->groups[g].descs, descs.data(), sizeof(LineDesc) * descs.size(),
+                     cudaMemcpyHostToDevice);
+    if (e != cudaSuccess || c0.recon != PP_RECON_CHARACTERISTIC) continue;
     e = cudaMalloc(&h->groups[g].lines, sizeof(LineRef) * slines[g].size());
     if (e == cudaSuccess)
       e = cudaMemcpy(h->groups[g].lines, slines[g].data(), sizeof(LineRef) * slines[g].size(),
@@ -2212,14 +2215,7 @@ int pp_cweno_operator_noalloc(const pp_cweno_config *cfg, const double *U_dev, d
 
   noalloc_ctl_reset<<<1, 32, 0, h.stream>>>(ctl);
   if (!(eps > 0.0)) {
-    h.nprob = 1;
-    const int blocks = (int)fmin(1184.0, (double)((h.ncell + 255) / 256));
-    if (nv == 4)
-      state_reduce_kernel<4><<<blocks < 1 ? 1 : blocks, 256, 0, h.stream>>>(
-          U_dev, nullptr, h.ncell, h.nx, h.dx, h.dy, cfg->gamma, ctl);
-    else
-      state_reduce_kernel<3><<<blocks < 1 ? 1 : blocks, 256, 0, h.stream>>>(
-          U_dev, nullptr, h.ncell, h.nx, h.dx, h.dy, cfg->gamma, ctl);
+    launch_reduce(&h, U_dev, nullptr, nullptr, ctl);
   }
   noalloc_ctl_arm<<<1, 32, 0, h.stream>>>(ctl, cfg->eps_pos, eps);
   noalloc_nan_fill<<<grid_for(nvals(&h)), 256, 0, h.stream>>>(L_dev, nvals(&h), ctl);
@@ -2260,6 +2256,7 @@ int pp_cweno_destroy(pp_cweno_t h) {
   if (h->yjoin) cudaEventDestroy(h->yjoin);
   for (auto &g : h->groups) {
     cudaFree(g.lines);
+    cudaFree(g.descs);
     cudaFree(g.cscr);
     cudaFree(g.crows);
   }
