@@ -280,9 +280,9 @@ def run_native(args, ws, rank, local):
             st = s.stats()
             launches = s.launches_per_step()
             s.close()
-            names = (["char_rows_x", "char_solve_x", "x_sweep", "char_rows_y", "char_solve_y",
+            names = (["char_solve_x", "x_sweep", "char_solve_y",
                       "y_sweep_transposed", "stage_combine"] if prec == 1 else
-                     ["char_rows_x", "char_solve_x", "x_sweep", "char_rows_y", "char_solve_y", "y_sweep"])
+                     ["char_solve_x", "x_sweep", "char_solve_y", "y_sweep"])
             per = prof[1:]           # prof[0]: the per-step dt kernel
             kms = {nm: sum(per[i::len(names)]) / max(1, len(per[i::len(names)]))
                    for i, nm in enumerate(names)}

@@ -14,13 +14,8 @@ struct ProbDesc {
   int bc[4];
 };
 
-// one line of a batched launch: problem index and line index inside it
-struct LineRef {
-  int prob, line;
-};
-
-// the same line as the line kernels read it, one record instead of a chain of
-// two: offset of its problem's block, first cell in a plane, cell stride,
+// one line of a batched launch, resolved (the kernels read one record instead
+// of a chain of two): offset of its problem's block, first cell in a plane, cell stride,
 // plane size, length, boundaries, inverse cell sizes along and across
 struct LineDesc {
   long long off, base, ncell;

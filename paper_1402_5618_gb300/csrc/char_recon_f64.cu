@@ -2,7 +2,7 @@
 #include "char_recon_kernel.cuh"
 
 namespace ppk {
-cudaError_t launch_char_recon_f64(const CharArgs &a, int nv, bool periodic, int part, cudaStream_t st) {
-  return chr::launch_char_recon_t<double>(a, nv, periodic, part, st);
+cudaError_t launch_char_recon_f64(const CharArgs &a, int nv, cudaStream_t st, bool attrs_only) {
+  return chr::launch_char_recon_t<double>(a, nv, st, attrs_only);
 }
 }  // namespace ppk

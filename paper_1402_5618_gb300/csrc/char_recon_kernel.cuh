@@ -1,14 +1,19 @@
 // char_recon_kernel.cuh -- kernel of the characteristic-wise reconstruction
 // (Sec. 2.3) in the arithmetic of the line: real = double is the plain
 // form; real = float the mixed form, reading the FP32 hi parts of the state.
-// The layout and the walk are described in char_recon.cuh.
+// The method and the layout are described in char_recon.cuh.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "char_recon.cuh"
+#include "compact_solve.cuh"
 #include "physics.cuh"
 
 namespace ppk {
 namespace chr {
+
+namespace cg = cooperative_groups;
 
 // Sec. 2.3: the Roe average of Ua and Ub, reduced to the four scalars the
 // left eigenvectors depend on: u, v (2-D), 1/a and c1 = (gamma - 1)/a^2
@@ -16,17 +21,21 @@ template <typename real, int NV>
 __device__ __forceinline__ void roe_scalars(const real *Ua, const real *Ub, real gamma,
                                             real (&rs)[4]) {
   const real one = real(1), half = real(0.5);
-  const real sa = sqrt(Ua[0]), sb = sqrt(Ub[0]);
-  const real isab = one / (sa + sb);
-  const real pa = pressure<real, NV>(Ua, gamma), pb = pressure<real, NV>(Ub, gamma);
-  const real u = (Ua[1] / sa + Ub[1] / sb) * isab;
-  const real v = NV == 4 ? (Ua[2] / sa + Ub[2] / sb) * isab : real(0);
-  const real H = ((Ua[NV - 1] + pa) / sa + (Ub[NV - 1] + pb) / sb) * isab;
-  const real a2 = (gamma - one) * (H - half * (u * u + v * v));
+  const real sa = root(Ua[0]), sb = root(Ub[0]);
+  const real isa = rcp(sa), isb = rcp(sb), isab = rcp(sa + sb);
+  const real ia = isa * isa, ib = isb * isb;   // 1 / rho
+  const real g1 = gamma - one;
+  const real pa = g1 * (Ua[NV - 1] - half * kin2<real, NV>(Ua) * ia);
+  const real pb = g1 * (Ub[NV - 1] - half * kin2<real, NV>(Ub) * ib);
+  const real u = (Ua[1] * isa + Ub[1] * isb) * isab;
+  const real v = NV == 4 ? (Ua[2] * isa + Ub[2] * isb) * isab : real(0);
+  const real H = ((Ua[NV - 1] + pa) * isa + (Ub[NV - 1] + pb) * isb) * isab;
+  const real a2 = g1 * (H - half * (u * u + v * v));
+  const real ia2 = rcp(a2);
   rs[0] = u;
   rs[1] = v;
-  rs[2] = one / sqrt(a2);
-  rs[3] = (gamma - one) / a2;
+  rs[2] = root(ia2);
+  rs[3] = g1 * ia2;
 }
 
 // rows l^(k) of L (eqs. (eigen), (leigenv)), ordered by the eigenvalues
@@ -57,6 +66,13 @@ __device__ __forceinline__ void left_from(const real (&rs)[4], real (&L)[NV][NV]
   }
 }
 
+// |a| > |b| for a pivot search; FP64 by the high words (an FP64 comparison
+// takes a slot of the FP64 pipe; a pivot within 2^-20 of the largest is as good)
+__device__ __forceinline__ bool larger(float a, float b) { return fabsf(a) > fabsf(b); }
+__device__ __forceinline__ bool larger(double a, double b) {
+  return (__double2hiint(a) & 0x7fffffff) > (__double2hiint(b) & 0x7fffffff);
+}
+
 // X <- M^{-1} X for an NV x NV block M and NCOL columns: Gaussian
 // elimination with partial pivoting, all indices fixed at compile time; the
 // pivots' reciprocals serve both passes (row c is final once column c is done)
@@ -65,12 +81,11 @@ __device__ __forceinline__ void gauss_solve(real (&M)[NV][NV], real (&X)[NV][NCO
   real inv[NV];
 #pragma unroll
   for (int c = 0; c < NV; ++c) {
-    real best = fabs(M[c][c]);
+    real best = M[c][c];
     int piv = c;
 #pragma unroll
     for (int r = c + 1; r < NV; ++r) {
-      const real m = fabs(M[r][c]);
-      if (m > best) { best = m; piv = r; }
+      if (larger(M[r][c], best)) { best = M[r][c]; piv = r; }
     }
 #pragma unroll
     for (int r = c + 1; r < NV; ++r) {
@@ -88,7 +103,7 @@ __device__ __forceinline__ void gauss_solve(real (&M)[NV][NV], real (&X)[NV][NCO
         X[r][j] = sw ? t : X[r][j];
       }
     }
-    inv[c] = real(1) / M[c][c];
+    inv[c] = rcp(M[c][c]);
 #pragma unroll
     for (int r = c + 1; r < NV; ++r) {
       const real f = M[r][c] * inv[c];
@@ -110,54 +125,8 @@ __device__ __forceinline__ void gauss_solve(real (&M)[NV][NV], real (&X)[NV][NCO
   }
 }
 
-// WENO-Z ratios of one characteristic field over its five-cell stencil v.
-// FP32: the scaled ratios with eps lifted to the rounding floor of the
-// indicators, FP32_BETA_FLOOR s^2 = 2^20 (u s)^2 with s = mag, the largest sum_m |l_m| |ubar_m|
-// over the stencil: the size of the terms the characteristic variable is
-// summed from, which bounds its rounding error even where the sum cancels
-// (the same floor as the component-wise mixed form, taken on those terms).
-template <typename real>
-__device__ __forceinline__ void char_ratios(const real (&v)[5], real mag, real eps, real &q0,
-                                            real &q1, real &q2, real &one) {
-  if constexpr (sizeof(real) == 4) {
-    const float c13 = 13.0f / 12.0f;
-    const float b0 = c13 * sqr(v[0] - 2.0f * v[1] + v[2]) + 0.25f * sqr(v[0] - 4.0f * v[1] + 3.0f * v[2]);
-    const float b1 = c13 * sqr(v[1] - 2.0f * v[2] + v[3]) + 0.25f * sqr(v[1] - v[3]);
-    const float b2 = c13 * sqr(v[2] - 2.0f * v[3] + v[4]) + 0.25f * sqr(3.0f * v[2] - 4.0f * v[3] + v[4]);
-    const float tau = fabsf(b2 - b0);
-    const float e = fmaf(FP32_BETA_FLOOR * mag, mag, eps);
-    const float d0 = b0 + e, d1 = b1 + e, d2 = b2 + e;
-    const float dmin = fminf(fminf(d0, d1), d2);
-    const float r = fminf(tau, dmin);
-    const float sc = dmin / tau;
-    one = tau <= dmin ? 1.0f : sc * sc;
-    q0 = sqr(r / d0);
-    q1 = sqr(r / d1);
-    q2 = sqr(r / d2);
-  } else {
-    zratios<real>(v[0], v[1], v[2], v[3], v[4], eps, q0, q1, q2);
-    one = real(1);
-  }
-}
-
-// asynchronous copies global -> shared (cp.async): a per-thread ring in
-// shared memory keeps several positions' loads of the serial walk in flight
-template <int B>
-__device__ __forceinline__ void cp_async(void *sdst, const void *gsrc) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(sdst);
-  if constexpr (B == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gsrc) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
 // geometry of one line: its first cell's offset in the planes, cell stride,
-// plane size, length and boundary kinds (a batched line from its problem)
+// plane size, length and boundary kinds
 struct LineGeo {
   long long base, cs, ncell;
   int n, bclo, bchi;
@@ -165,48 +134,40 @@ struct LineGeo {
 
 __device__ __forceinline__ LineGeo line_geo(const CharArgs &a, long long line) {
   LineGeo g;
-  if (!a.lines) {
-    g.base = line * a.line_stride;
-    g.cs = a.cell_stride;
-    g.ncell = a.ncell;
-    g.n = a.n;
-    g.bclo = a.bclo;
-    g.bchi = a.bchi;
+  if (a.lines) {   // a batched line
+    const LineDesc d = a.lines[line];
+    g.base = d.off + d.base;
+    g.cs = d.cs;
+    g.ncell = d.ncell;
+    g.n = d.n;
+    g.bclo = d.bclo;
+    g.bchi = d.bchi;
     return g;
   }
-  const LineRef lr = a.lines[line];
-  const ProbDesc pd = a.probs[lr.prob];
-  g.ncell = pd.ncell;
-  if (a.xdir == 1) {
-    g.n = pd.nx; g.cs = 1; g.base = pd.off + (long long)lr.line * pd.nx;
-    g.bclo = pd.bc[0]; g.bchi = pd.bc[1];
-  } else if (a.xdir == 2) {   // a row of the problem's transposed planes: a y line
-    g.n = pd.ny; g.cs = 1; g.base = pd.off + (long long)lr.line * pd.ny;
-    g.bclo = pd.bc[2]; g.bchi = pd.bc[3];
-  } else {
-    g.n = pd.ny; g.cs = pd.nx; g.base = pd.off + lr.line;
-    g.bclo = pd.bc[2]; g.bchi = pd.bc[3];
-  }
+  g.base = line * a.line_stride;
+  g.cs = a.cell_stride;
+  g.ncell = a.ncell;
+  g.n = a.n;
+  g.bclo = a.bclo;
+  g.bchi = a.bchi;
   return g;
 }
 
-// ghost-aware read of the line variables of line cell i (both kernels)
-template <typename real, int NV, bool PER>
+// ghost-aware read of the line variables of line cell i
+template <typename real, int NV>
 __device__ __forceinline__ void line_cell(const LineGeo &g, const real *U, const int (&gv)[NV],
                                           int i, real (&out)[NV]) {
   const int n = g.n;
   bool neg = false;
   if (i < 0 || i >= n) {
-    if (PER) {
-      i = (i % n + n) % n;
+    const int bc = i < 0 ? g.bclo : g.bchi;
+    if (bc == 0) {
+      i = i < 0 ? i + n : i - n;
+    } else if (bc == 1) {
+      i = i < 0 ? 0 : n - 1;
     } else {
-      const int bc = i < 0 ? g.bclo : g.bchi;
-      if (bc == 1) {
-        i = i < 0 ? 0 : n - 1;
-      } else {
-        i = i < 0 ? -i - 1 : 2 * n - 1 - i;
-        neg = true;
-      }
+      i = i < 0 ? -i - 1 : 2 * n - 1 - i;
+      neg = true;
     }
   }
   const real *src = U + g.base + (long long)i * g.cs;
@@ -215,754 +176,547 @@ __device__ __forceinline__ void line_cell(const LineGeo &g, const real *U, const
   if (neg) out[1] = -out[1];
 }
 
-template <int NV>
-__device__ __forceinline__ void grid_vars(const CharArgs &a, int (&gv)[NV]) {
+// ---------------------------------------------------------------- runs
+// A run of block rows by its two end unknowns (see compact_solve.cuh, with
+// blocks): end = a - B X_near - G X_far, X_near the unknown next to that end
+// outside the run, X_far the one at its other end.
+template <typename real, int NV>
+struct End {
+  real a[NV], B[NV][NV], G[NV][NV];
+};
+
+template <typename real, int NV>
+__device__ __forceinline__ void end_empty(End<real, NV> &e) {   // the unknown at the other end
 #pragma unroll
-  for (int k = 0; k < NV; ++k) gv[k] = k == 0 ? 0 : (k == NV - 1 ? NV - 1 : (k == 1 ? a.vn : a.vt));
+  for (int i = 0; i < NV; ++i) {
+    e.a[i] = real(0);
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      e.B[i][j] = real(0);
+      e.G[i][j] = i == j ? real(-1) : real(0);
+    }
+  }
+}
+template <typename real, int NV>
+__device__ __forceinline__ void end_select(bool c, const End<real, NV> &x, const End<real, NV> &y,
+                                           End<real, NV> &o) {
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    o.a[i] = c ? x.a[i] : y.a[i];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      o.B[i][j] = c ? x.B[i][j] : y.B[i][j];
+      o.G[i][j] = c ? x.G[i][j] : y.G[i][j];
+    }
+  }
+}
+template <typename real, int NV>
+__device__ __forceinline__ void end_xor(const End<real, NV> &x, int d, End<real, NV> &o) {
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    o.a[i] = __shfl_xor_sync(0xffffffffu, x.a[i], d);
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      o.B[i][j] = __shfl_xor_sync(0xffffffffu, x.B[i][j], d);
+      o.G[i][j] = __shfl_xor_sync(0xffffffffu, x.G[i][j], d);
+    }
+  }
 }
 
-// Steps 1-3 at every face, all in parallel.  One block takes a tile of 32
-// lines x 32 cells (plus the two-cell halo) into shared memory -- loaded
-// along whichever of the two axes is contiguous in memory -- and computes
-// the rows of both sides of every cell of the tile: the Roe scalars of the
-// row's face, the characteristic variables of its five-cell stencil (walk
-// order) and, per field k, the WENO-Z weights and the scalar row (a on the
-// previous unknown of the walk, b on this one, c on the next, r the
-// right-hand side; closure rows of bounded lines 0, 1, 0 and the explicit
-// WENO5-Z value).  Output per row: the 4 Roe scalars and 4 NV coefficients,
-// laid out [side][position][entry][line] so that both this kernel's stores
-// and the serial walk's loads are contiguous over the lines of a warp.
-constexpr int CT_L = 32, CT_C = 32;   // lines x cells of a tile
+// o <- e - M [x | r | -s] columnwise: the end e of a run whose far unknown is
+// u + r X_o - s X_o' (e.G multiplies it): a - G u, B + G r, -G s with B the
+// coefficient of X_o and the new far coefficient that of X_o'
+template <typename real, int NV>
+__device__ __forceinline__ void end_extend(const End<real, NV> &e, const real (&u)[NV],
+                                           const real (&r)[NV][NV], const real (&s)[NV][NV],
+                                           End<real, NV> &o) {
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    real t = e.a[i];
+#pragma unroll
+    for (int m = 0; m < NV; ++m) t -= e.G[i][m] * u[m];
+    o.a[i] = t;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      real p = e.B[i][j], q = real(0);
+#pragma unroll
+      for (int m = 0; m < NV; ++m) {
+        p += e.G[i][m] * r[m][j];
+        q -= e.G[i][m] * s[m][j];
+      }
+      o.B[i][j] = p;
+      o.G[i][j] = q;
+    }
+  }
+}
 
-template <typename real, int NV, bool PER>
-__global__ void __launch_bounds__(256) char_rows_kernel(const CharArgs a) {
+// One level of the butterfly over lanes d apart: F, L the run's first and last
+// unknown (walk order), later: this lane's run is the later of the two.  st
+// (u, r, s): the partner's facing unknown u + r X_o - s X_o' from the
+// unknowns outside the joined run (X_o on this lane's side), for the way down.
+template <typename real, int NV>
+struct BStep {
+  real u[NV], r[NV][NV], s[NV][NV];
+};
+
+template <typename real, int NV>
+__device__ __forceinline__ void block_up(int d, bool later, End<real, NV> &F, End<real, NV> &L,
+                                         BStep<real, NV> &st) {
+  End<real, NV> in, out, in2, out2;
+  end_select(later, F, L, in);
+  end_select(later, L, F, out);
+  end_xor(in, d, in2);
+  end_xor(out, d, out2);
+  // (I - b' b) [u | r | s] = [a' - b' a | b' g | g']
+  real M[NV][NV], X[NV][2 * NV + 1];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    real t = in2.a[i];
+#pragma unroll
+    for (int m = 0; m < NV; ++m) t -= in2.B[i][m] * in.a[m];
+    X[i][0] = t;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      real p = i == j ? real(1) : real(0), q = real(0);
+#pragma unroll
+      for (int m = 0; m < NV; ++m) {
+        p -= in2.B[i][m] * in.B[m][j];
+        q += in2.B[i][m] * in.G[m][j];
+      }
+      M[i][j] = p;
+      X[i][1 + j] = q;
+      X[i][1 + NV + j] = in2.G[i][j];
+    }
+  }
+  gauss_solve<real, NV, 2 * NV + 1>(M, X);
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    st.u[i] = X[i][0];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      st.r[i][j] = X[i][1 + j];
+      st.s[i][j] = X[i][1 + NV + j];
+    }
+  }
+  End<real, NV> o, o2;
+  end_extend(out, st.u, st.r, st.s, o);
+  // this lane's facing unknown a - b u - (g + b r) X_o + b s X_o', as u2 + r2
+  // X_o' - s2 X_o, extends the partner's outer end
+  real u2[NV], r2[NV][NV], s2[NV][NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    real t = in.a[i];
+#pragma unroll
+    for (int m = 0; m < NV; ++m) t -= in.B[i][m] * st.u[m];
+    u2[i] = t;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      real p = in.G[i][j], q = real(0);
+#pragma unroll
+      for (int m = 0; m < NV; ++m) {
+        p += in.B[i][m] * st.r[m][j];
+        q += in.B[i][m] * st.s[m][j];
+      }
+      s2[i][j] = p;
+      r2[i][j] = q;
+    }
+  }
+  end_extend(out2, u2, r2, s2, o2);
+  end_select(later, o2, o, F);
+  end_select(later, o, o2, L);
+}
+
+template <typename real, int NV>
+__device__ __forceinline__ void block_down(bool later, const BStep<real, NV> &st, real (&xl)[NV],
+                                           real (&xr)[NV]) {
+  real v[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    real t = st.u[i];
+#pragma unroll
+    for (int m = 0; m < NV; ++m) {
+      const real xo = later ? xr[m] : xl[m], xo2 = later ? xl[m] : xr[m];
+      t += st.r[i][m] * xo;
+      t -= st.s[i][m] * xo2;
+    }
+    v[i] = t;
+  }
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    if (later) xl[i] = v[i];
+    else xr[i] = v[i];
+  }
+}
+
+// the ring of a periodic line closed on itself, X_in = last and X_out = first:
+// (I + G_F) f + B_F l = a_F, B_L f + (I + G_L) l = a_L
+template <typename real, int NV>
+__device__ __forceinline__ void block_ring(const End<real, NV> &F, const End<real, NV> &L,
+                                           real (&xl)[NV], real (&xr)[NV]) {
+  real M[NV][NV], X[NV][NV + 1], N[NV][NV], Y[NV][1];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    X[i][0] = F.a[i];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      M[i][j] = F.G[i][j] + (i == j ? real(1) : real(0));
+      X[i][1 + j] = F.B[i][j];
+    }
+  }
+  gauss_solve<real, NV, NV + 1>(M, X);   // f = X_0 - X_1 l
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    real t = L.a[i];
+#pragma unroll
+    for (int m = 0; m < NV; ++m) t -= L.B[i][m] * X[m][0];
+    Y[i][0] = t;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      real p = L.G[i][j] + (i == j ? real(1) : real(0));
+#pragma unroll
+      for (int m = 0; m < NV; ++m) p -= L.B[i][m] * X[m][1 + j];
+      N[i][j] = p;
+    }
+  }
+  gauss_solve<real, NV, 1>(N, Y);
+#pragma unroll
+  for (int i = 0; i < NV; ++i) xl[i] = Y[i][0];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    real t = X[i][0];
+#pragma unroll
+    for (int m = 0; m < NV; ++m) t -= X[i][1 + m] * xl[m];
+    xr[i] = t;
+  }
+}
+
+// ---------------------------------------------------------------- rows
+// The block row of a cell, normalised by b: L y_p + diag(a) L y_{p-1} +
+// diag(c) L y_{p+1} = s in the deviations y from the cell averages, walk
+// order.  win: the five cells of the stencil in walk order.
+template <typename real, int NV>
+__device__ __forceinline__ void char_row(const real (&win)[5][NV], real gamma, real eps,
+                                         bool closure, real (&rs)[4], real (&ca)[NV],
+                                         real (&cc)[NV], real (&s)[NV]) {
   constexpr bool F32 = sizeof(real) == 4;
-  constexpr int RC = 4 * NV + 4;
-  constexpr int TW = CT_C + 4;        // cells of a tile row with the halo
-  __shared__ real tile[NV][CT_L][TW + 1];
-  __shared__ LineGeo sg[CT_L];
-  const int NMAX = a.n;               // position stride of the rows buffer
-  const long long NL = a.nlines;
-  const long long line0 = (long long)blockIdx.x * CT_L;
-  const int c0 = blockIdx.y * CT_C;
+  real L[NV][NV];
+  roe_scalars<real, NV>(win[2], win[3], gamma, rs);
+  left_from<real, NV>(rs, L);
+  real dU[4][NV], top[NV];
+#pragma unroll
+  for (int m = 0; m < NV; ++m) {
+#pragma unroll
+    for (int w = 0; w < 4; ++w) dU[w][m] = win[w + 1][m] - win[w][m];
+    if (F32) {
+      top[m] = fabs(win[0][m]);
+#pragma unroll
+      for (int w = 1; w < 5; ++w) top[m] = fmax(top[m], fabs(win[w][m]));
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    real D[4], mag = real(0);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      real t = L[k][0] * dU[w][0];
+#pragma unroll
+      for (int m = 1; m < NV; ++m) t += L[k][m] * dU[w][m];
+      D[w] = t;
+    }
+    const real k43 = real(4.0 / 3.0);
+    const real g0 = D[1] - D[0], g1 = D[2] - D[1], g2 = D[3] - D[2];
+    real e = eps;
+    if constexpr (F32) {
+      // the rounding floor of the indicators on the size of the terms the
+      // characteristic variable is summed from
+#pragma unroll
+      for (int m = 0; m < NV; ++m) mag += fabsf(L[k][m]) * top[m];
+      e = fmaf(FP32_BETA_FLOOR * mag, mag, eps);
+    }
+    const real d0 = fma(k43 * g0, g0, e) + D[1] * (D[1] + g0);
+    const real d1 = fma(k43 * g1, g1, e) + D[1] * D[2];
+    const real d2 = fma(k43 * g2, g2, e) + D[2] * (D[2] - g2);
+    real S0, S1, S2;
+    z_terms(d0, d1, d2, S0, S1, S2);
+    if (closure) {
+      const real a0 = real(0.1) * S0, a1 = real(0.6) * S1, a2 = real(0.3) * S2;
+      ca[k] = cc[k] = real(0);
+      s[k] = (a0 * (real(5) * D[1] - real(2) * D[0]) + a1 * (D[1] + real(2) * D[2]) +
+              a2 * (real(4) * D[2] - D[3])) * rcp(real(6) * (a0 + a1 + a2));
+    } else {
+      const real t2 = real(2.5) * S1, t4 = real(1.25) * S1;
+      const real ib = rcp(fma(real(3), S2, fma(real(2), t2, S0)));
+      ca[k] = fma(real(2), S0, t2) * ib;
+      cc[k] = real(1.5) * S2 * ib;
+      s[k] = (D[1] * fma(real(1.5), S0, t2) + D[2] * fma(real(2.25), S2, t4)) * ib;
+    }
+  }
+}
+
+// ---------------------------------------------------------------- kernel
+// One warp per (segment of 32 M cells, side); lane k holds the M cells of
+// chunk k; a cluster of R CTAs covers the line.  Shared memory: per row of
+// every lane the multipliers Y, F and g (x = g - F X_in - Y x_next).
+template <typename real, int NV>
+struct CharSmem {
+  static constexpr int E = 2 * NV * NV + NV;
+  End<real, NV> seg[2];   // this segment's first and last unknown
+  static size_t bytes(int M) { return sizeof(End<real, NV>) * 2 + sizeof(real) * 32 * E * (size_t)M; }
+};
+
+template <typename real, int NV>
+__global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
+  constexpr int E = CharSmem<real, NV>::E;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  End<real, NV> *seg = reinterpret_cast<End<real, NV> *>(smem_raw);
+  real *rows = reinterpret_cast<real *>(smem_raw + 2 * sizeof(End<real, NV>));
+  cg::cluster_group cluster = cg::this_cluster();
+  const int M = a.M, R = a.R;
+  const int rank = (int)cluster.block_rank(), lane = threadIdx.x, side = blockIdx.y;
+  const LineGeo geo = line_geo(a, blockIdx.x / R);
+  const int n = geo.n;
+  const bool per = geo.bclo == 0;
+  const int lo = rank * 32 * M, i0 = lo + lane * M;
+  const int cnt = max(0, min(M, n - i0));
+  const int dir = side == 0 ? 1 : -1;
+  const int first = side == 0 ? i0 : i0 + cnt - 1;   // the chunk's first cell in walk order
   const real *U = reinterpret_cast<const real *>(a.U);
   int gv[NV];
-  grid_vars<NV>(a, gv);
-  const int tid = threadIdx.x;
-  if (tid < CT_L && line0 + tid < NL) sg[tid] = line_geo(a, line0 + tid);
-  __syncthreads();
-  const bool along_cells = a.lines ? a.xdir != 0 : a.cell_stride == 1;
-  for (int idx = tid; idx < CT_L * TW; idx += blockDim.x) {
-    const int ll = along_cells ? idx / TW : idx % CT_L;
-    const int j = along_cells ? idx % TW : idx / CT_L;
-    const int i = c0 - 2 + j;
-    if (line0 + ll >= NL) continue;
-    const LineGeo g = sg[ll];
-    if (i < -2 || i > g.n + 1) continue;   // never read
-    real v[NV];
-    line_cell<real, NV, PER>(g, U, gv, i, v);
 #pragma unroll
-    for (int k = 0; k < NV; ++k) tile[k][ll][j] = v[k];
-  }
-  __syncthreads();
-  const int ll = tid % CT_L;
-  const long long line = line0 + ll;
-  if (line >= NL) return;
-  const int n = sg[ll].n;
-  real *rows = reinterpret_cast<real *>(a.rows);
+  for (int k = 0; k < NV; ++k) gv[k] = k == 0 ? 0 : (k == NV - 1 ? NV - 1 : (k == 1 ? a.vn : a.vt));
   const real gam = real(a.gamma), eps = real(a.eps_weno);
-  for (int q = tid / CT_L; q < 2 * CT_C; q += blockDim.x / CT_L) {
-    const int side = q / CT_C;
-    const int c = c0 + q % CT_C;
-    if (c >= n) continue;
-    const int dir = side == 0 ? 1 : -1;
-    const int p = side == 0 ? c : n - 1 - c;
-    const int jc = c - c0 + 2;        // the cell's column in the tile
-    real win[5][NV];
+  // entry e of row t of this lane
+  auto at = [&](int t, int e) -> real & { return rows[((long long)t * E + e) * 32 + lane]; };
+
+  // The chunk's rows first, their 4 + 3 NV numbers into the slots the
+  // multipliers take later: two loops whose bodies stay in the instruction
+  // caches instead of one that does not (the SM runs few warps of this kernel).
+  {
+    real win[5][NV], nxt[NV];
+    if (cnt > 0) {
 #pragma unroll
-    for (int w = 0; w < 5; ++w)
+      for (int w = 0; w < 4; ++w) line_cell<real, NV>(geo, U, gv, first + (w - 2) * dir, win[w + 1]);
+      line_cell<real, NV>(geo, U, gv, first + 2 * dir, nxt);
+    }
+#pragma unroll 1
+    for (int t = 0; t < cnt; ++t) {
+      const int c = first + t * dir;
 #pragma unroll
-      for (int k = 0; k < NV; ++k) win[w][k] = tile[k][ll][jc + (w - 2) * dir];
-    real rs[4], L[NV][NV];
-    roe_scalars<real, NV>(win[2], win[3], gam, rs);
-    left_from<real, NV>(rs, L);
-    const bool closure = !PER && (p == 0 || p == n - 1);
-    real *dst = rows + ((long long)side * NMAX + p) * RC * NL + line;
+      for (int w = 0; w < 4; ++w)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) dst[e * NL] = rs[e];
+        for (int k = 0; k < NV; ++k) win[w][k] = win[w + 1][k];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      real cv[5];
-      real mag = real(0);
+      for (int k = 0; k < NV; ++k) win[4][k] = nxt[k];
+      if (t + 1 < cnt) line_cell<real, NV>(geo, U, gv, c + 3 * dir, nxt);
+      real rs[4], ca[NV], cc[NV], s[NV];
+      char_row<real, NV>(win, gam, eps, !per && (c == 0 || c == n - 1), rs, ca, cc, s);
 #pragma unroll
-      for (int w = 0; w < 5; ++w) {
-        real s0 = real(0), s1 = real(0);
+      for (int i = 0; i < 4; ++i) at(t, i) = rs[i];
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        at(t, 4 + i) = ca[i];
+        at(t, 4 + NV + i) = cc[i];
+        at(t, 4 + 2 * NV + i) = s[i];
+      }
+    }
+  }
+  // elimination of the chunk: last = g - F X_in - Y x_next after every row,
+  // first = a - B X_in - G x_next folded along
+  End<real, NV> F, L;
+  end_empty(F);
+  end_empty(L);
+#pragma unroll 1
+  for (int t = 0; t < cnt; ++t) {
+    real Lk[NV][NV], ca[NV], cc[NV], s[NV];
+    {
+      real rs[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) rs[i] = at(t, i);
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        ca[i] = at(t, 4 + i);
+        cc[i] = at(t, 4 + NV + i);
+        s[i] = at(t, 4 + 2 * NV + i);
+      }
+      left_from<real, NV>(rs, Lk);
+    }
+    // (L - diag(a) L Y) [Y' | g' | F'] = [diag(c) L | s - diag(a) L g | -diag(a) L F]
+    real B[NV][NV], X[NV][2 * NV + 1];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      real tg = real(0);
+#pragma unroll
+      for (int m = 0; m < NV; ++m) tg += Lk[i][m] * L.a[m];
+      X[i][NV] = s[i] - ca[i] * tg;
+#pragma unroll
+      for (int j = 0; j < NV; ++j) {
+        real ty = real(0), tf = real(0);
 #pragma unroll
         for (int m = 0; m < NV; ++m) {
-          s0 += L[k][m] * win[w][m];
-          if (F32) s1 += fabs(L[k][m]) * fabs(win[w][m]);
+          ty += Lk[i][m] * L.B[m][j];
+          tf += Lk[i][m] * L.G[m][j];
         }
-        cv[w] = s0;
-        if (F32) mag = fmax(mag, s1);
+        B[i][j] = Lk[i][j] - ca[i] * ty;
+        X[i][j] = cc[i] * Lk[i][j];
+        X[i][NV + 1 + j] = -(ca[i] * tf);
       }
-      real q0, q1, q2, w0, w1, w2, one;
-      char_ratios<real>(cv, mag, eps, q0, q1, q2, one);
-      real fa, fb, fc, fr;
-      if (closure) {
-        zweights<real>(real(0.1), real(0.6), real(0.3), q0, q1, q2, w0, w1, w2, one);
-        const real p0 = real(2) * cv[0] - real(7) * cv[1] + real(11) * cv[2];
-        const real p1 = -cv[1] + real(5) * cv[2] + real(2) * cv[3];
-        const real p2 = real(2) * cv[2] + real(5) * cv[3] - cv[4];
-        fa = real(0);
-        fb = real(1);
-        fc = real(0);
-        fr = (w0 * p0 + w1 * p1 + w2 * p2) * real(1.0 / 6.0);
-      } else {
-        zweights<real>(real(0.2), real(0.5), real(0.3), q0, q1, q2, w0, w1, w2, one);
-        const Row<real> row = compact_row<real>(w0, w1, w2, cv[1], cv[2], cv[3]);
-        fa = row.a;
-        fb = row.b;
-        fc = row.c;
-        fr = row.r;
-      }
-      dst[(4 + 4 * k + 0) * NL] = fa;
-      dst[(4 + 4 * k + 1) * NL] = fb;
-      dst[(4 + 4 * k + 2) * NL] = fc;
-      dst[(4 + 4 * k + 3) * NL] = fr;
     }
-  }
-}
-
-// Step 4, the serial part: one thread per (line, side) walks the line in
-// the elimination order.  Position p of the walk is cell p (minus side,
-// left to right) or cell n-1-p (plus side, right to left); in walk order
-// both sides have the same rows (the plus row is the mirror image of the
-// minus row), so "previous" and "next" below are in walk order.  At each
-// position the thread rebuilds L from the four Roe scalars, takes the row
-// coefficients from char_rows_kernel, and runs one step of block Thomas.
-// The walk is bound by the latency of its own loads (few chains per SM), so
-// the row data of the next PD - 1 positions, and in the back substitution
-// their multipliers, are in flight in a per-thread shared-memory ring.
-// Periodic lines solve the cyclic system with the Woodbury correction
-// T = T' + U V^T, G = -B_0: T' has B_0 - G at the first position and
-// B_{n-1} - C_{n-1} G^{-1} A_0 at the last, U = (G, 0, .., 0, C_{n-1}),
-// V^T = (I, 0, .., 0, G^{-1} A_0); the NV columns of U ride along as extra
-// right-hand sides and x = y - Z (I + V^T Z)^{-1} V^T y at the end.
-template <typename real, int NV, bool PER>
-__global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
-  constexpr int NC = PER ? NV + 1 : 1;       // right-hand-side columns
-  constexpr int ROW = NV * NV + NV * NC;     // scratch values per row: Y, g
-  constexpr int RC = 4 * NV + 4;             // Roe scalars and row coefficients per position
-  const long long line = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (line >= a.nlines) return;
-  const int side = blockIdx.y;
-  const LineGeo geo = line_geo(a, line);
-  const int n = geo.n;
-  const int NMAX = a.n;   // position stride of rows and scratch
-  const long long NL = a.nlines;
-  const long long lbase = geo.base;
-  const real *rows = reinterpret_cast<const real *>(a.rows) + (long long)side * NMAX * RC * NL + line;
-  real *scr = reinterpret_cast<real *>(a.scr) + (long long)side * ((long long)NMAX * ROW + NV * NV) * NL + line;
-  auto slot = [&](int p, int e) -> real & { return scr[((long long)p * ROW + e) * NL]; };
-  auto wslot = [&](int e) -> real & { return scr[((long long)NMAX * ROW + e) * NL]; };
-  int gv[NV];
-  grid_vars<NV>(a, gv);
-  auto cidx = [&](int p) { return side == 0 ? p : n - 1 - p; };
-
-  // ring of PD positions: [slot][entry][thread], conflict-free; as deep as
-  // the 48 KB of static shared memory allows (periodic rows are longer)
-  constexpr int PD = sizeof(real) == 4 ? (PER ? 8 : 16) : 4;
-  constexpr int RING = RC > ROW ? RC : ROW;
-  __shared__ real ring[PD][RING][32];
-  const int tid = threadIdx.x;
-  auto issue_row = [&](int p) {
+    gauss_solve<real, NV, 2 * NV + 1>(B, X);
 #pragma unroll
-    for (int e = 0; e < RC; ++e)
-      cp_async<sizeof(real)>(&ring[p % PD][e][tid], &rows[((long long)p * RC + e) * NL]);
-  };
-#pragma unroll 1
-  for (int j = 0; j < PD - 1; ++j) {
-    if (j < n) issue_row(j);
-    cp_async_commit();
-  }
-
-  real co[RC];
-  real Yp[NV][NV], gp[NV][NC];   // the previous position's multipliers
-#pragma unroll 1
-  for (int p = 0; p < n; ++p) {
-    if (p + PD - 1 < n) issue_row(p + PD - 1);
-    cp_async_commit();
-    cp_async_wait<PD - 1>();   // the group of position p has landed
-#pragma unroll
-    for (int e = 0; e < RC; ++e) co[e] = ring[p % PD][e][tid];
-    real L[NV][NV];
-    {
-      const real rs[4] = {co[0], co[1], co[2], co[3]};
-      left_from<real, NV>(rs, L);
-    }
-    real ca[NV], cb[NV], cc[NV], cr[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      ca[k] = co[4 + 4 * k];
-      cb[k] = co[4 + 4 * k + 1];
-      cc[k] = co[4 + 4 * k + 2];
-      cr[k] = co[4 + 4 * k + 3];
-    }
-    // block row diag(ca, cb, cc) L, eliminated against the previous
-    // position: Bp = B - A Y_prev, X = [C | r - A g_prev]
-    real Bp[NV][NV], X[NV][NV + NC];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
+    for (int i = 0; i < NV; ++i) {
+      L.a[i] = X[i][NV];
+      at(t, i) = X[i][NV];
 #pragma unroll
       for (int j = 0; j < NV; ++j) {
-        Bp[k][j] = cb[k] * L[k][j];
-        X[k][j] = cc[k] * L[k][j];
-      }
-      X[k][NV] = cr[k];
-#pragma unroll
-      for (int j = 1; j < NC; ++j) X[k][NV + j] = real(0);
-    }
-    if constexpr (PER) {
-      if (p == 0) {
-        // G = -B_0: B'_0 = B_0 - G = 2 B_0, Woodbury columns U_0 = G, and
-        // G^{-1} A_0 for the last position and the final correction
-        real Gm[NV][NV], GiA[NV][NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-#pragma unroll
-          for (int j = 0; j < NV; ++j) {
-            Gm[k][j] = -Bp[k][j];
-            GiA[k][j] = ca[k] * L[k][j];
-            X[k][NV + 1 + j] = Gm[k][j];
-            Bp[k][j] = Bp[k][j] + Bp[k][j];
-          }
-        gauss_solve<real, NV, NV>(Gm, GiA);
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-#pragma unroll
-          for (int j = 0; j < NV; ++j) wslot(k * NV + j) = GiA[k][j];
+        L.B[i][j] = X[i][j];
+        L.G[i][j] = X[i][NV + 1 + j];
+        at(t, NV + i * NV + j) = X[i][j];
+        at(t, NV + NV * NV + i * NV + j) = X[i][NV + 1 + j];
       }
     }
-    if (p > 0) {
+    // first = a - B X_in - G x_p with x_p = g - F X_in - Y x_{p+1}
+    real G2[NV][NV];
 #pragma unroll
-      for (int k = 0; k < NV; ++k) {
+    for (int i = 0; i < NV; ++i) {
+      real p = F.a[i];
 #pragma unroll
-        for (int j = 0; j < NV; ++j) {
-          real t = real(0);
-#pragma unroll
-          for (int m = 0; m < NV; ++m) t += L[k][m] * Yp[m][j];
-          Bp[k][j] -= ca[k] * t;
-        }
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          real t = real(0);
-#pragma unroll
-          for (int m = 0; m < NV; ++m) t += L[k][m] * gp[m][c];
-          X[k][NV + c] -= ca[k] * t;
-        }
-      }
-    }
-    if constexpr (PER) {
-      if (p == n - 1) {
-        // B'_{n-1} = B_{n-1} - C_{n-1} G^{-1} A_0; the coupling to x_0 moves
-        // into the Woodbury columns (U_{n-1} = C_{n-1})
-        real GiA[NV][NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-#pragma unroll
-          for (int j = 0; j < NV; ++j) GiA[k][j] = wslot(k * NV + j);
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-#pragma unroll
-          for (int j = 0; j < NV; ++j) {
-            real t = real(0);
-#pragma unroll
-            for (int m = 0; m < NV; ++m) t += X[k][m] * GiA[m][j];
-            Bp[k][j] -= t;
-          }
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-#pragma unroll
-          for (int j = 0; j < NV; ++j) {
-            X[k][NV + 1 + j] += X[k][j];
-            X[k][j] = real(0);
-          }
-      }
-    }
-    gauss_solve<real, NV, NV + NC>(Bp, X);
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
+      for (int m = 0; m < NV; ++m) p -= F.G[i][m] * L.a[m];
+      F.a[i] = p;
 #pragma unroll
       for (int j = 0; j < NV; ++j) {
-        Yp[k][j] = X[k][j];
-        slot(p, k * NV + j) = X[k][j];
-      }
+        real q = F.B[i][j], r = real(0);
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        gp[k][c] = X[k][NV + c];
-        slot(p, NV * NV + k * NC + c) = X[k][NV + c];
+        for (int m = 0; m < NV; ++m) {
+          q -= F.G[i][m] * L.G[m][j];
+          r -= F.G[i][m] * L.B[m][j];
+        }
+        F.B[i][j] = q;
+        G2[i][j] = r;
       }
     }
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+#pragma unroll
+      for (int j = 0; j < NV; ++j) F.G[i][j] = G2[i][j];
   }
-  cp_async_wait<0>();
 
-  // back substitution x_p = g_p - Y_p x_{p+1}; step b = n-2-p reads the
-  // multipliers of position p through the same ring
+  // trees over the warp's chunks, then over the segments of the cluster
+  BStep<real, NV> st[5], sg[4];
+#pragma unroll 1
+  for (int h = 0; h < 5; ++h) {
+    const bool up = (lane >> h) & 1;
+    block_up(1 << h, side == 0 ? up : !up, F, L, st[h]);
+  }
+  real xl[NV], xr[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) xl[i] = xr[i] = real(0);
+  if (R > 1) {
+    if (lane == 0) {
+      seg[0] = F;
+      seg[1] = L;
+    }
+    cluster.sync();
+    const int q = lane & 15;
+    end_empty(F);
+    end_empty(L);
+    if (q < R) {
+      const End<real, NV> *o = cluster.map_shared_rank(seg, side == 0 ? q : R - 1 - q);
+      F = o[0];
+      L = o[1];
+    }
+#pragma unroll 1
+    for (int h = 0; (1 << h) < R; ++h) block_up(1 << h, (q >> h) & 1, F, L, sg[h]);
+    // Arrive now, wait before exit: a CTA's shared memory must outlive the
+    // reads of its run.  Only here, where every lane's reads have been used
+    // (the joins need them all): an arrival does not wait for loads in flight.
+    __syncwarp();
+    cluster_arrive_relaxed();
+  }
+  if (per) block_ring(F, L, xl, xr);
+  if (R > 1) {
+    const int q = lane & 15, own = side == 0 ? rank : R - 1 - rank;
+#pragma unroll 1
+    for (int h = 3; h >= 0; --h)
+      if ((1 << h) < R) block_down((q >> h) & 1, sg[h], xl, xr);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      xl[i] = __shfl_sync(0xffffffffu, xl[i], own);
+      xr[i] = __shfl_sync(0xffffffffu, xr[i], own);
+    }
+  }
+#pragma unroll 1
+  for (int h = 4; h >= 0; --h) {
+    const bool up = (lane >> h) & 1;
+    block_down(side == 0 ? up : !up, st[h], xl, xr);
+  }
+
+  // back substitution; the deviations overwrite g
+#pragma unroll 1
+  for (int t = cnt - 1; t >= 0; --t) {
+    real x[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      real p = at(t, i);
+#pragma unroll
+      for (int m = 0; m < NV; ++m) {
+        p -= at(t, NV + NV * NV + i * NV + m) * xl[m];
+        p -= at(t, NV + i * NV + m) * xr[m];
+      }
+      x[i] = p;
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      xr[i] = x[i];
+      at(t, i) = x[i];
+    }
+  }
+  __syncwarp();
+  // out: consecutive lanes on consecutive cells
   real *out = reinterpret_cast<real *>(side == 0 ? a.Um : a.Up);
-  real x[NV][NC];
-#pragma unroll
-  for (int k = 0; k < NV; ++k)
-#pragma unroll
-    for (int c = 0; c < NC; ++c) x[k][c] = gp[k][c];
-  auto issue_mult = [&](int b) {
-    const int p = n - 2 - b;
-#pragma unroll
-    for (int e = 0; e < ROW; ++e) cp_async<sizeof(real)>(&ring[b % PD][e][tid], &slot(p, e));
-  };
-#pragma unroll 1
-  for (int j = 0; j < PD - 1; ++j) {
-    if (j < n - 1) issue_mult(j);
-    cp_async_commit();
-  }
-#pragma unroll 1
-  for (int p = n - 1; p >= 0; --p) {
-    if (p < n - 1) {
-      const int b = n - 2 - p;
-      if (b + PD - 1 < n - 1) issue_mult(b + PD - 1);
-      cp_async_commit();
-      cp_async_wait<PD - 1>();
-      real Yc[ROW];
-#pragma unroll
-      for (int e = 0; e < ROW; ++e) Yc[e] = ring[b % PD][e][tid];
-      real xn[NV][NC];
-#pragma unroll
-      for (int k = 0; k < NV; ++k)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) xn[k][c] = x[k][c];
-#pragma unroll
-      for (int k = 0; k < NV; ++k)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          real s = Yc[NV * NV + k * NC + c];
-#pragma unroll
-          for (int j = 0; j < NV; ++j) s -= Yc[k * NV + j] * xn[j][c];
-          x[k][c] = s;
-        }
-    }
-    if (PER) {
-#pragma unroll
-      for (int k = 0; k < NV; ++k)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) slot(p, NV * NV + k * NC + c) = x[k][c];
-    } else {
-      real *dst = out + lbase + (long long)cidx(p) * geo.cs;
-#pragma unroll
-      for (int k = 0; k < NV; ++k) dst[gv[k] * geo.ncell] = x[k][0];
-    }
-  }
-  cp_async_wait<0>();
-  if constexpr (PER) {
-    // S = I + Z_0 + G^{-1} A_0 Z_{n-1}, t = y_0 + G^{-1} A_0 y_{n-1};
-    // x_p = y_p - Z_p S^{-1} t
-    real S[NV][NV], t[NV][1], GiA[NV][NV];
+  const int len = min(32 * M, n - lo);
+  for (int c = lane; c < len; c += 32) {
+    const int ch = c / M, j = c - ch * M;
+    const int t = side == 0 ? j : min(M, len - ch * M) - 1 - j;
+    const long long o = geo.base + (long long)(lo + c) * geo.cs;
 #pragma unroll
     for (int k = 0; k < NV; ++k)
-#pragma unroll
-      for (int j = 0; j < NV; ++j) GiA[k][j] = wslot(k * NV + j);
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-#pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        real s = (k == j ? real(1) : real(0)) + slot(0, NV * NV + k * NC + 1 + j);
-#pragma unroll
-        for (int m = 0; m < NV; ++m) s += GiA[k][m] * slot(n - 1, NV * NV + m * NC + 1 + j);
-        S[k][j] = s;
-      }
-      real s = slot(0, NV * NV + k * NC);
-#pragma unroll
-      for (int m = 0; m < NV; ++m) s += GiA[k][m] * slot(n - 1, NV * NV + m * NC);
-      t[k][0] = s;
-    }
-    gauss_solve<real, NV, 1>(S, t);
-#pragma unroll 1
-    for (int p = 0; p < n; ++p) {
-      real *dst = out + lbase + (long long)cidx(p) * geo.cs;
-#pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        real s = slot(p, NV * NV + k * NC);
-#pragma unroll
-        for (int j = 0; j < NV; ++j) s -= slot(p, NV * NV + k * NC + 1 + j) * t[j][0];
-        dst[gv[k] * geo.ncell] = s;
-      }
-    }
+      out[o + gv[k] * geo.ncell] = U[o + gv[k] * geo.ncell] + rows[((long long)t * E + k) * 32 + ch];
   }
+  if (R > 1) cluster_wait();
 }
 
-// ---------------------------------------------------------------- FP32, few walks
-// The same walk with four lanes per (line, side) chain, for launches with
-// few chains (batch groups of long 1-D lines: a few hundred walks of up to
-// 8192 positions, fewer than one warp per SM in the one-thread layout,
-// where the chain's latency is the whole cost).  Lane j holds column j of
-// the block being eliminated and the right-hand-side columns of unknown j:
-// column j of Y (and of the Woodbury block on periodic lines); the g
-// column is the same in every lane (every lane forms it from the same data
-// with the same multipliers).  Per position the lanes solve
-// B' [Y | g] = [C | r - A g_prev] together by Gaussian elimination with
-// partial pivoting: lane c finds the pivot of column c in its own column
-// and hands the exchange, the pivot's reciprocal and the multipliers to the
-// other lanes; the back substitution takes the upper triangle's entries
-// from their lanes.  A Y_prev needs column j of Y_prev only, which lane j
-// already holds.  With three fields lane 3 carries right-hand sides only.
-// The eight chains of a warp stay converged (full-warp shuffles over 4-lane
-// segments): the warp walks as many positions as its longest chain, and a
-// chain past its own end (a shorter batched line) computes on stale data
-// and stores nothing.  A position costs about twice the one-thread walk's
-// instructions per chain, so with many chains the one-thread walk is
-// faster; the launch picks by the number of chains.
-
-constexpr unsigned FULL = 0xffffffffu;
-constexpr int LW = 4;   // lanes per chain (shuffle segment width)
-
-// X <- M^{-1} X over the four lanes of a chain: M's column j and NR
-// columns X[s] in lane j (lane ids below are within the chain's segment)
-template <int NV, int NR>
-__device__ __forceinline__ void lanes_solve(float (&M)[NV], float (&X)[NR][NV]) {
-  float inv[NV];
-  float U[NV][NV];   // U[c][q], q > c: row c of the factor, from lane q
-#pragma unroll
-  for (int c = 0; c < NV; ++c) {
-    if (c < NV - 1) {
-      int piv = c;
-      float best = fabsf(M[c]);
-#pragma unroll
-      for (int r = c + 1; r < NV; ++r) {
-        const float m = fabsf(M[r]);
-        if (m > best) { best = m; piv = r; }
-      }
-      piv = __shfl_sync(FULL, piv, c, LW);
-#pragma unroll
-      for (int r = c + 1; r < NV; ++r) {
-        const bool sw = piv == r;
-        const float t = M[c];
-        M[c] = sw ? M[r] : t;
-        M[r] = sw ? t : M[r];
-#pragma unroll
-        for (int s = 0; s < NR; ++s) {
-          const float u = X[s][c];
-          X[s][c] = sw ? X[s][r] : u;
-          X[s][r] = sw ? u : X[s][r];
-        }
-      }
-    }
-    const float iv = __shfl_sync(FULL, 1.0f / M[c], c, LW);
-    inv[c] = iv;
-#pragma unroll
-    for (int r = c + 1; r < NV; ++r) {
-      const float f = __shfl_sync(FULL, M[r] * iv, c, LW);
-      M[r] -= f * M[c];
-#pragma unroll
-      for (int s = 0; s < NR; ++s) X[s][r] -= f * X[s][c];
-    }
-#pragma unroll
-    for (int q = c + 1; q < NV; ++q) U[c][q] = __shfl_sync(FULL, M[c], q, LW);
+template <typename real, int NV>
+cudaError_t launch_nv(const CharArgs &a, cudaStream_t st, bool attrs_only) {
+  auto kern = char_solve_kernel<real, NV>;
+  if (attrs_only) {
+    // (M = 16 rows per chunk at most)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)CharSmem<real, NV>::bytes(16));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                               (int)cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
   }
-#pragma unroll
-  for (int s = 0; s < NR; ++s)
-#pragma unroll
-    for (int c = NV - 1; c >= 0; --c) {
-      float x = X[s][c];
-#pragma unroll
-      for (int q = c + 1; q < NV; ++q) x -= U[c][q] * X[s][q];
-      X[s][c] = x * inv[c];
-    }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(a.nlines * a.R), 2, 1);
+  cfg.blockDim = dim3(32, 1, 1);
+  cfg.dynamicSmemBytes = CharSmem<real, NV>::bytes(a.M);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)a.R;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-template <int NV, bool PER>
-__global__ void __launch_bounds__(64) char_solve_lanes_kernel(const CharArgs a) {
-  constexpr int NC = PER ? NV + 1 : 1;       // right-hand-side columns of g
-  constexpr int ROW = NV * NV + NV * NC;     // scratch values per row: Y, g
-  constexpr int RC = 4 * NV + 4;             // Roe scalars and row coefficients per position
-  constexpr int CH = 16;                     // chains per block
-  constexpr int PD = 8;                      // positions in flight
-  constexpr int NR = PER ? 3 : 2;            // right-hand sides per lane: Y col, (Z col,) g
-  constexpr int SG = NR - 1;
-  constexpr int RING = RC > ROW ? RC : ROW;
-  // (a chain stride of 18 words instead of 16 takes the back substitution's
-  // 4-way bank conflicts away but measured slower: 120 against 95 ms per
-  // Riemann batch step)
-  __shared__ float ring[PD][RING][CH];
-  const int tid = threadIdx.x;
-  const int ch = tid >> 2, j = tid & 3;
-  const long long NL = a.nlines;
-  const long long line_ = (long long)blockIdx.x * CH + ch;
-  const bool live = line_ < NL;
-  const long long line = live ? line_ : NL - 1;   // idle chains repeat the last line, store nothing
-  const bool col = live && j < NV;                // lane owns a column of the block
-  const int side = blockIdx.y;
-  const LineGeo geo = line_geo(a, line);
-  const int n = geo.n;
-  const int nw = __reduce_max_sync(FULL, n);      // the warp's longest chain
-  const int NMAX = a.n;                           // position stride of rows and scratch
-  const long long lbase = geo.base;
-  const float *rows = reinterpret_cast<const float *>(a.rows) + (long long)side * NMAX * RC * NL + line;
-  float *scr = reinterpret_cast<float *>(a.scr) + (long long)side * ((long long)NMAX * ROW + NV * NV) * NL + line;
-  auto slot = [&](int p, int e) -> float & { return scr[((long long)p * ROW + e) * NL]; };
-  auto wslot = [&](int e) -> float & { return scr[((long long)NMAX * ROW + e) * NL]; };
-  int gv[NV];
-  grid_vars<NV>(a, gv);
-  auto cidx = [&](int p) { return side == 0 ? p : n - 1 - p; };
-  // lane j's entries of a row record, split four ways over the chain
-  auto issue_row = [&](int p) {
-#pragma unroll
-    for (int q = 0; q < RC / 4; ++q) {
-      const int e = j + 4 * q;
-      cp_async<4>(&ring[p % PD][e][ch], &rows[((long long)p * RC + e) * NL]);
-    }
-  };
-#pragma unroll 1
-  for (int i = 0; i < PD - 1; ++i) {
-    if (i < n) issue_row(i);
-    cp_async_commit();
-  }
-  // k-th entry of this lane's column of an NV x NV matrix (no dynamic register index)
-  auto colj = [&](const float (&Mk)[NV]) {
-    float v = Mk[0];
-#pragma unroll
-    for (int q = 1; q < NV; ++q) v = j == q ? Mk[q] : v;
-    return v;
-  };
-
-  float Yc[NV], Zc[NV], gc[NV], GiAc[NV];
-#pragma unroll
-  for (int k = 0; k < NV; ++k) Yc[k] = Zc[k] = gc[k] = GiAc[k] = 0.0f;
-#pragma unroll 1
-  for (int p = 0; p < nw; ++p) {
-    const bool act = live && p < n;
-    __syncwarp();   // slot (p - 1) % PD is read by every lane before it is refilled
-    if (p + PD - 1 < n) issue_row(p + PD - 1);
-    cp_async_commit();
-    cp_async_wait<PD - 1>();
-    __syncwarp();   // the chain's four lanes' copies of position p have landed
-    float co[RC];
-#pragma unroll
-    for (int e = 0; e < RC; ++e) co[e] = ring[p % PD][e][ch];
-    float L[NV][NV];
-    {
-      const float rs[4] = {co[0], co[1], co[2], co[3]};
-      left_from<float, NV>(rs, L);
-    }
-    float ca[NV], cb[NV], cc[NV], Lj[NV];
-    float M[NV], X[NR][NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      ca[k] = co[4 + 4 * k];
-      cb[k] = co[4 + 4 * k + 1];
-      cc[k] = co[4 + 4 * k + 2];
-      Lj[k] = colj(L[k]);
-      M[k] = cb[k] * Lj[k];
-      X[0][k] = cc[k] * Lj[k];
-      X[SG][k] = co[4 + 4 * k + 3];
-      if (PER) X[1][k] = 0.0f;
-    }
-    if constexpr (PER) {
-      if (p == 0) {
-        // G = -B_0: B'_0 = 2 B_0, Woodbury column j of U_0 = G, and column
-        // j of G^{-1} A_0 for the last position and the final correction
-        float Gm[NV], Aj[1][NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-          Gm[k] = -M[k];
-          Aj[0][k] = ca[k] * Lj[k];
-          X[1][k] = Gm[k];
-          M[k] += M[k];
-        }
-        lanes_solve<NV, 1>(Gm, Aj);
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-          GiAc[k] = Aj[0][k];
-          if (col) wslot(k * NV + j) = GiAc[k];
-        }
-      }
-    }
-    if (p > 0) {
-#pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        float tY = 0.0f, tg = 0.0f, tz = 0.0f;
-#pragma unroll
-        for (int m = 0; m < NV; ++m) {
-          tY += L[k][m] * Yc[m];
-          tg += L[k][m] * gc[m];
-          if (PER) tz += L[k][m] * Zc[m];
-        }
-        M[k] -= ca[k] * tY;
-        X[SG][k] -= ca[k] * tg;
-        if (PER) X[1][k] -= ca[k] * tz;
-      }
-    }
-    if constexpr (PER) {
-      if (p == n - 1) {
-        // B'_{n-1} = B_{n-1} - C_{n-1} G^{-1} A_0; the coupling to x_0 moves
-        // into the Woodbury columns (U_{n-1} = C_{n-1})
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-          float t = 0.0f;
-#pragma unroll
-          for (int m = 0; m < NV; ++m) t += cc[k] * L[k][m] * GiAc[m];
-          M[k] -= t;
-          X[1][k] += X[0][k];
-          X[0][k] = 0.0f;
-        }
-      }
-    }
-    lanes_solve<NV, NR>(M, X);
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      Yc[k] = X[0][k];
-      gc[k] = X[SG][k];
-      if (PER) Zc[k] = X[1][k];
-      if (col && act) {
-        slot(p, k * NV + j) = Yc[k];
-        if (PER) slot(p, NV * NV + k * NC + 1 + j) = Zc[k];
-      }
-    }
-    if (act && j == 0) {
-#pragma unroll
-      for (int k = 0; k < NV; ++k) slot(p, NV * NV + k * NC) = gc[k];
-    }
-  }
-  cp_async_wait<0>();
-  __syncwarp();   // the chain's scratch rows, written by all four lanes, are read below
-
-  // back substitution x_p = g_p - Y_p x_{p+1}; lane k (< NV) forms row k of
-  // x_p from row k of (Y_p, g_p) and all of x_{p+1}; step b is position
-  // n - 2 - b of each chain
-  const int k = j < NV ? j : NV - 1;
-  int gvk = gv[0];   // grid variable of field k, without a dynamic register index
-#pragma unroll
-  for (int q = 1; q < NV; ++q) gvk = k == q ? gv[q] : gvk;
-  float *out = reinterpret_cast<float *>(side == 0 ? a.Um : a.Up);
-  float x[NC];
-#pragma unroll
-  for (int c = 0; c < NC; ++c) x[c] = slot(n - 1, NV * NV + k * NC + c);
-  auto issue_mult = [&](int b) {
-    if (j >= NV) return;   // lane 3 of a three-field chain: nothing of its own
-    const int p = n - 2 - b;
-#pragma unroll
-    for (int q = 0; q < NV; ++q) cp_async<4>(&ring[b % PD][k * NV + q][ch], &slot(p, k * NV + q));
-#pragma unroll
-    for (int c = 0; c < NC; ++c)
-      cp_async<4>(&ring[b % PD][NV * NV + k * NC + c][ch], &slot(p, NV * NV + k * NC + c));
-  };
-  __syncwarp();
-#pragma unroll 1
-  for (int i = 0; i < PD - 1; ++i) {
-    if (i < n - 1) issue_mult(i);
-    cp_async_commit();
-  }
-  auto store_x = [&](int p) {
-    if (!col) return;
-    if (PER) {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) slot(p, NV * NV + k * NC + c) = x[c];
-    } else {
-      out[lbase + (long long)cidx(p) * geo.cs + (long long)gvk * geo.ncell] = x[0];
-    }
-  };
-  store_x(n - 1);
-#pragma unroll 1
-  for (int b = 0; b < nw - 1; ++b) {
-    const int p = n - 2 - b;
-    if (b + PD - 1 < n - 1) issue_mult(b + PD - 1);
-    cp_async_commit();
-    cp_async_wait<PD - 1>();   // this lane's own copies only: no exchange through the ring
-    float Yr[NV], gr[NC];   // (lane 3 of a three-field chain reads values it never uses)
-#pragma unroll
-    for (int q = 0; q < NV; ++q) Yr[q] = ring[b % PD][k * NV + q][ch];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) gr[c] = ring[b % PD][NV * NV + k * NC + c][ch];
-    float xn[NV][NC];
-#pragma unroll
-    for (int q = 0; q < NV; ++q)
-#pragma unroll
-      for (int c = 0; c < NC; ++c) xn[q][c] = __shfl_sync(FULL, x[c], q, LW);
-    if (p >= 0) {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        float s = gr[c];
-#pragma unroll
-        for (int q = 0; q < NV; ++q) s -= Yr[q] * xn[q][c];
-        x[c] = s;
-      }
-      store_x(p);
-    }
-  }
-  cp_async_wait<0>();
-  if constexpr (PER) {
-    __syncwarp();   // every lane's rows of y and Z are in the scratch
-    // S = I + Z_0 + G^{-1} A_0 Z_{n-1}, t = y_0 + G^{-1} A_0 y_{n-1};
-    // x_p = y_p - Z_p S^{-1} t, row k in lane k
-    float S[NV][NV], t[NV][1], GiA[NV][NV];
-#pragma unroll
-    for (int r = 0; r < NV; ++r)
-#pragma unroll
-      for (int q = 0; q < NV; ++q) GiA[r][q] = wslot(r * NV + q);
-#pragma unroll
-    for (int r = 0; r < NV; ++r) {
-#pragma unroll
-      for (int q = 0; q < NV; ++q) {
-        float s = (r == q ? 1.0f : 0.0f) + slot(0, NV * NV + r * NC + 1 + q);
-#pragma unroll
-        for (int m = 0; m < NV; ++m) s += GiA[r][m] * slot(n - 1, NV * NV + m * NC + 1 + q);
-        S[r][q] = s;
-      }
-      float s = slot(0, NV * NV + r * NC);
-#pragma unroll
-      for (int m = 0; m < NV; ++m) s += GiA[r][m] * slot(n - 1, NV * NV + m * NC);
-      t[r][0] = s;
-    }
-    gauss_solve<float, NV, 1>(S, t);
-    if (col) {
-#pragma unroll 4
-      for (int p = 0; p < n; ++p) {
-        float s = slot(p, NV * NV + k * NC);
-#pragma unroll
-        for (int q = 0; q < NV; ++q) s -= slot(p, NV * NV + k * NC + 1 + q) * t[q][0];
-        out[lbase + (long long)cidx(p) * geo.cs + (long long)gvk * geo.ncell] = s;
-      }
-    }
-  }
-}
-
-// Without a timed choice (CharArgs::layout < 0), FP32 launches with fewer
-// lines than this take the four-lane walk (2048 lines: 4096 chains, fewer
-// than one warp per SM in the one-thread layout; measured: the 4096^2
-// grid's 8192 chains walk faster one thread each, 3.41 against 4.17 ms, the
-// Riemann batch's groups of at most ~1700 chains faster four lanes each, 96
-// against 149 ms per step)
-constexpr long long LANES_BELOW = 2048;
-
-template <typename real, int NV, bool PER>
-cudaError_t launch_nv(const CharArgs &a, int part, cudaStream_t st) {
-  if (part == 0) {
-    const dim3 grid((unsigned)((a.nlines + CT_L - 1) / CT_L), (unsigned)((a.n + CT_C - 1) / CT_C), 1);
-    char_rows_kernel<real, NV, PER><<<grid, 256, 0, st>>>(a);
-  } else {
-    if constexpr (sizeof(real) == 4) {
-      if (a.layout == 1 || (a.layout < 0 && a.nlines < LANES_BELOW)) {
-        char_solve_lanes_kernel<NV, PER><<<dim3((unsigned)((a.nlines + 15) / 16), 2, 1), 64, 0, st>>>(a);
-        return cudaGetLastError();
-      }
-    }
-    char_solve_kernel<real, NV, PER><<<dim3((unsigned)((a.nlines + 31) / 32), 2, 1), 32, 0, st>>>(a);
-  }
-  return cudaGetLastError();
-}
-
-// part 0: the parallel rows kernel; part 1: the serial block solve
 template <typename real>
-cudaError_t launch_char_recon_t(const CharArgs &a, int nv, bool periodic, int part, cudaStream_t st) {
-  if (nv == 3) return periodic ? launch_nv<real, 3, true>(a, part, st) : launch_nv<real, 3, false>(a, part, st);
-  return periodic ? launch_nv<real, 4, true>(a, part, st) : launch_nv<real, 4, false>(a, part, st);
+cudaError_t launch_char_recon_t(const CharArgs &a, int nv, cudaStream_t st, bool attrs_only) {
+  return nv == 3 ? launch_nv<real, 3>(a, st, attrs_only) : launch_nv<real, 4>(a, st, attrs_only);
 }
 
 }  // namespace chr

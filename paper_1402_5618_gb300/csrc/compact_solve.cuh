@@ -36,6 +36,14 @@
 
 namespace ppk {
 
+// halves of a cluster barrier that publishes no data
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed;\n" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory");
+}
+
 // ---------------------------------------------------------------- pairs
 // .x belongs to the minus system, .y to the plus system.  FP32 pairs use the
 // paired instructions (one issue slot for two operations, each component
@@ -64,6 +72,32 @@ __device__ __forceinline__ double2 p_add(double2 a, double2 b) { return make_dou
 __device__ __forceinline__ double2 p_neg(double2 a) { return make_double2(-a.x, -a.y); }
 __device__ __forceinline__ float2 p_rcp(float2 a) { return make_float2(rcp(a.x), rcp(a.y)); }
 __device__ __forceinline__ double2 p_rcp(double2 a) { return make_double2(rcp(a.x), rcp(a.y)); }
+
+// scalars, for code written on either
+template <typename real>
+__device__ __forceinline__ real p_mul(real a, real b) { return a * b; }
+template <typename real>
+__device__ __forceinline__ real p_fma(real a, real b, real c) { return fma(a, b, c); }
+template <typename real>
+__device__ __forceinline__ real p_neg(real a) { return -a; }
+template <typename real>
+__device__ __forceinline__ real p_rcp(real a) { return rcp(a); }
+template <typename real>
+__device__ __forceinline__ real p_sel(bool c, bool, real a, real b) { return c ? a : b; }
+template <typename real>
+__device__ __forceinline__ real p_xor(real v, int d) { return __shfl_xor_sync(0xffffffffu, v, d); }
+__device__ __forceinline__ float2 p_sel(bool x, bool y, float2 a, float2 b) {
+  return make_float2(x ? a.x : b.x, y ? a.y : b.y);
+}
+__device__ __forceinline__ double2 p_sel(bool x, bool y, double2 a, double2 b) {
+  return make_double2(x ? a.x : b.x, y ? a.y : b.y);
+}
+__device__ __forceinline__ float2 p_xor(float2 v, int d) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, d), __shfl_xor_sync(0xffffffffu, v.y, d));
+}
+__device__ __forceinline__ double2 p_xor(double2 v, int d) {
+  return make_double2(__shfl_xor_sync(0xffffffffu, v.x, d), __shfl_xor_sync(0xffffffffu, v.y, d));
+}
 
 // ---------------------------------------------------------------- weights
 // power of two near 1/m (exact scaling): 2^-(exponent of m)
@@ -340,6 +374,80 @@ __device__ __forceinline__ void chunk_back(const real *u, real *dm, const real *
     dm[jm] = u[jm] + x.x;
     dp[jp] = u[jp] + x.y;
   }
+}
+
+// ---------------------------------------------------------------- trees
+// Runs of the lanes of a warp joined by a butterfly: 5 levels of a few dozen
+// instructions on every warp and no barrier.  The way of the FP32 form, and of
+// FP64 with short chunks, where a line has its SMs to itself and latency is
+// the cost; otherwise the FP64 pipe is, and one warp walks the chunks of the
+// segment with a fifth of the instructions.  At each level a lane sees its own run and its partner's
+// from the end that faces the other: inner (facing) and outer ends as
+// end = a - b X_near - g X_far.  With i = 1/(1 - b b'), the partner's inner
+// unknown is u + r X_o - s X_o' (X_o, X_o': outside the own and the
+// partner's outer end), kept for the way down.
+template <typename P>
+struct Ends {
+  P a, b, g;
+};
+template <typename P>
+struct Step {
+  P u, r, s;
+};
+
+// one level for one pair: own inner / outer ends in, the joined run's outer
+// ends out (own side in o, partner's side in o2)
+template <typename P>
+__device__ __forceinline__ void tree_join(const Ends<P> &in, const Ends<P> &out, const Ends<P> &in2,
+                                          const Ends<P> &out2, P one, Step<P> &st, Ends<P> &o,
+                                          Ends<P> &o2) {
+  const P i = p_rcp(p_fma(p_neg(in.b), in2.b, one));
+  const P gi = p_mul(in.g, i), gi2 = p_mul(in2.g, i);
+  st.u = p_mul(p_fma(p_neg(in2.b), in.a, in2.a), i);
+  st.r = p_mul(in2.b, gi);
+  st.s = gi2;
+  const P u2 = p_mul(p_fma(p_neg(in.b), in2.a, in.a), i);
+  const P nf = p_neg(out.g), nf2 = p_neg(out2.g);
+  o.a = p_fma(nf, st.u, out.a);
+  o.b = p_fma(out.g, st.r, out.b);
+  o.g = p_mul(nf, gi2);
+  o2.a = p_fma(nf2, u2, out2.a);
+  o2.b = p_fma(out2.g, p_mul(in.b, gi2), out2.b);
+  o2.g = p_mul(nf2, gi);
+}
+
+// F, L: the run's first and last unknown in walk order (L.b belongs to X_out,
+// L.g to X_in); rx, ry: this lane is the later of the two in walk order (for
+// the minus and the plus component)
+template <typename P>
+__device__ __forceinline__ void tree_up(int d, bool rx, bool ry, P one, Ends<P> &F, Ends<P> &L,
+                                        Step<P> &st) {
+  Ends<P> in, out, in2, out2, o, o2;
+  in.a = p_sel(rx, ry, F.a, L.a); in.b = p_sel(rx, ry, F.b, L.b); in.g = p_sel(rx, ry, F.g, L.g);
+  out.a = p_sel(rx, ry, L.a, F.a); out.b = p_sel(rx, ry, L.b, F.b); out.g = p_sel(rx, ry, L.g, F.g);
+  in2.a = p_xor(in.a, d); in2.b = p_xor(in.b, d); in2.g = p_xor(in.g, d);
+  out2.a = p_xor(out.a, d); out2.b = p_xor(out.b, d); out2.g = p_xor(out.g, d);
+  tree_join(in, out, in2, out2, one, st, o, o2);
+  F.a = p_sel(rx, ry, o2.a, o.a); F.b = p_sel(rx, ry, o2.b, o.b); F.g = p_sel(rx, ry, o2.g, o.g);
+  L.a = p_sel(rx, ry, o.a, o2.a); L.b = p_sel(rx, ry, o.b, o2.b); L.g = p_sel(rx, ry, o.g, o2.g);
+}
+template <typename P>
+__device__ __forceinline__ void tree_down(bool rx, bool ry, const Step<P> &st, P &xl, P &xr) {
+  const P xo = p_sel(rx, ry, xr, xl), xo2 = p_sel(rx, ry, xl, xr);
+  const P v = p_fma(p_neg(st.s), xo2, p_fma(st.r, xo, st.u));
+  xl = p_sel(rx, ry, v, xl);
+  xr = p_sel(rx, ry, xr, v);
+}
+
+// the ring of a periodic line closed on itself, X_in = last and X_out =
+// first: (1 + G) f + B l = A, C f + (1 + F) l = D, in FP64
+template <typename real>
+__device__ __forceinline__ void ring_close(const Ends<real> &F, const Ends<real> &L, real &xl,
+                                           real &xr) {
+  const double A = F.a, B = F.b, G = 1.0 + F.g, D = L.a, C = L.b, E = 1.0 + L.g;
+  const double idet = rcp(G * E - B * C);
+  xr = real((A * E - B * D) * idet);
+  xl = real((G * D - C * A) * idet);
 }
 
 }  // namespace ppk

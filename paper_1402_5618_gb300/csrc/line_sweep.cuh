@@ -144,40 +144,16 @@ __device__ __forceinline__ long long bind_line(SweepArgs &a, long long line) {
   return d.base;
 }
 
-// asynchronous copy of one value global -> shared: a thread's loads of a
-// segment are all in flight together, whatever the line's alignment
-template <typename real>
-__device__ __forceinline__ void load_async(real *dst, const real *src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  if constexpr (sizeof(real) == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void load_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
 template <typename real>
 __device__ __forceinline__ real shfl_down_r(real v, int d, int width = 32) {
   return __shfl_down_sync(0xffffffffu, v, d, width);
-}
-
-// split cluster barrier: arrive (release this CTA's shared-memory writes to
-// the cluster) and wait (acquire the other CTAs'), with independent work
-// between the two halves
-__device__ __forceinline__ void cluster_arrive() {
-  asm volatile("barrier.cluster.arrive.release;\n" ::: "memory");
-}
-__device__ __forceinline__ void cluster_arrive_relaxed() {   // publishes no data
-  asm volatile("barrier.cluster.arrive.relaxed;\n" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-  asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory");
 }
 
 // ---------------------------------------------------------------- smem
 template <typename real, int NV>
 struct Exch {
   Run<real> seg[2 * NV];         // this segment as a run, per variable and side
+  real xo[2 * NV];               // the unknown after the segment
   // mixed form, the line's reference state R (difference form): per
   // variable the hi / lo pair of the median of five sampled cells, R in
   // FP32, the reference fluxes F(R), (u_R, v_R, p_R, E_R + p_R), whether
@@ -186,6 +162,7 @@ struct Exch {
   int rgate[NV];
   float rspread[NV];             // largest |sample - R| per variable (hi parts)
   float epsf;                    // mixed form: the limiter epsilon of this stage
+  dfl dt;                        // mixed form: the time step
 };
 
 // Segment planes in shared memory carry one pad word per 128 bytes: segment
@@ -197,7 +174,10 @@ template <typename real, int NV, int M, int KCHUNK>
 struct Smem {
   static constexpr int KC = KCHUNK;       // chunks per conserved variable
   static constexpr int SEG = M * KC;      // cells per CTA segment
-  static constexpr int LPS = KC / 8;      // lanes that combine a system's chunks, eight each
+  // the chunks of a segment are joined by trees over the lanes (see
+  // compact_solve.cuh), or by LPS lanes of one warp per system, eight each
+  static constexpr bool TREE = sizeof(real) == 4 || M <= 4;
+  static constexpr int LPS = KC / 8;
   static constexpr int PSH = sizeof(real) == 4 ? 5 : 4;
   __host__ __device__ static constexpr int pad(int c) { return c + (c >> PSH); }
   static constexpr int UH = 3;                         // pad(-2) = -3
@@ -210,21 +190,25 @@ struct Smem {
   // per eight, so that lanes walking eight chunks each hit distinct banks
   static constexpr int KCP = KC + KC / 8;
   static constexpr int XP = KC + 1 + KC / 8;
+  static constexpr int FH = 2;                         // pad(-1) = -2
+  static constexpr int FWP = FH + pad(SEG) + 1;        // face values of cells -1 .. SEG
+  static constexpr int FLS = SEG + 4;                  // fluxes of a variable, rows on 16 bytes
+  static constexpr size_t up16(size_t x) { return (x + 15) / 16 * 16; }
   static constexpr size_t u_off = 0;                                     // real Us[NV][UWP]
-  static constexpr size_t fm_off = u_off + sizeof(real) * NV * UWP;      // real Fm, Fp[NV][WP]
-  static constexpr size_t fp_off = fm_off + sizeof(real) * NV * WP;
-  static constexpr size_t zm_off = fp_off + sizeof(real) * NV * WP;      // real Zm, Zp[NV][WP]
+  static constexpr size_t fm_off = u_off + sizeof(real) * NV * UWP;      // real Fm, Fp[NV][FWP]
+  static constexpr size_t fp_off = fm_off + sizeof(real) * NV * FWP;
+  static constexpr size_t zm_off = up16(fp_off + sizeof(real) * NV * FWP);   // real Zm, Zp[NV][WP]
   static constexpr size_t zp_off = zm_off + sizeof(real) * NV * WP;
-  static constexpr size_t fl_off = zm_off;     // real Fl[NV][SEG+2], after Zm and Zp are done with
-  static_assert(NV * (SEG + 2) <= 2 * NV * WP, "the fluxes must fit the two planes they reuse");
+  static constexpr size_t fl_off = zm_off;     // real Fl[NV][FLS], after Zm and Zp are done with
+  static_assert(FLS <= 2 * WP, "the fluxes must fit the two planes they reuse");
   static constexpr size_t cr_off = zp_off + sizeof(real) * NV * WP;      // real Cr[2 NV][6][KCP]
-  static constexpr size_t xs_off = cr_off + sizeof(real) * 2 * NV * 6 * KCP;   // real Xs[2 NV][XP]
-  static constexpr size_t ex_off = (xs_off + sizeof(real) * 2 * NV * XP + 15) / 16 * 16;
+  static constexpr size_t xs_off = cr_off + (TREE ? 0 : sizeof(real) * 2 * NV * 6 * KCP);   // real Xs[2 NV][XP]
+  static constexpr size_t ex_off = up16(xs_off + (TREE ? 0 : sizeof(real) * 2 * NV * XP));
   // mixed form: one byte per cell (its face values stored in full, not as
   // differences from R) and one per face (its flux stored as F - F(R))
   static constexpr size_t cf_off = ex_off + sizeof(Exch<real, NV>);
-  static constexpr size_t ff_off = cf_off + SEG;
-  static constexpr size_t bytes = (ff_off + SEG + 2 + 15) / 16 * 16;
+  static constexpr size_t ff_off = cf_off + SEG + 2;   // (flags of cells -1 .. SEG)
+  static constexpr size_t bytes = up16(ff_off + SEG + 2);
 };
 
 // line-variable k -> grid variable
@@ -259,8 +243,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
   using S = Smem<real, NV, M, KC>;
   constexpr int SEG = S::SEG;
   constexpr int T = NV * KC;
-  constexpr int UW = SEG + 4;            // cells -2 .. SEG+1
-  constexpr int UH = S::UH, UWP = S::UWP, WP = S::WP;
+  constexpr int UH = S::UH, UWP = S::UWP, WP = S::WP, FH = S::FH, FWP = S::FWP, FLS = S::FLS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   real *Us = reinterpret_cast<real *>(smem_raw + S::u_off);
   real *Fm = reinterpret_cast<real *>(smem_raw + S::fm_off);
@@ -298,6 +281,11 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
                  : (args.stage == 0 ? ctl->eps0
                                     : fmin(ctl->eps_pos, bits_double(ctl->minrho[args.stage - 1])));
       ex.epsf = (float)e;
+      if (MODE == MODE_FINAL) {
+        const double t = ctl->dt;
+        ex.dt.hi = (float)t;
+        ex.dt.lo = (float)(t - (double)ex.dt.hi);
+      }
     }
     eps_pos = real(0);   // set after the barrier
   } else {
@@ -307,9 +295,12 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
   }
 
   const long long cs = args.cell_stride;
-  unsigned char *cfull = smem_raw + S::cf_off;   // mixed: cell's faces stored in full
+  unsigned char *cfull = smem_raw + S::cf_off + 1;   // mixed: cell's faces stored in full
   unsigned char *fdel = smem_raw + S::ff_off;    // mixed: face flux stored as F - F(R)
 
+  if constexpr (MIXED && !PRE) {
+    for (int c = tid; c < SEG + 2; c += T) cfull[c - 1] = 0;
+  }
   // difference form possible: the reference samples and the lo parts load
   // with the hi parts
   const bool two = MIXED && !PRE && args.Ul != nullptr;
@@ -349,37 +340,71 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
     }
     return g * args.ncell + lbase + (long long)i * cs;
   };
-  // thread (v, k) brings in cells lo - 2 + k, + KC, ... of variable v; the
-  // lo parts go to the planes the face values take later
-  float *Ls = reinterpret_cast<float *>(Fm);
-  static_assert(!MIXED || UWP <= 2 * WP, "the lo parts must fit the face-value planes");
-  {
-    const long long plane = gvar(v, NV, args.vn, args.vt) * args.ncell + lbase;
-    const real *src;
-    if constexpr (MIXED) src = args.Uh + plane;
-    else src = args.U + plane;
-    const float *srl = two ? args.Ul + plane : nullptr;
-    real *dst = Us + v * UWP + UH;
-#pragma unroll 4
-    for (int j = k; j < UW; j += KC) {
-      const int i = lo - 2 + j, c = S::pad(j - 2);
-      if (i >= 0 && i < n) {
-        load_async(dst + c, src + (long long)i * cs);
-        if constexpr (MIXED) {
-          if (two) load_async(Ls + v * UWP + UH + c, srl + (long long)i * cs);
+  // Thread (v, k) brings in M cells of the segment of variable v, hi and lo
+  // parts, all its loads in flight together in registers until the reference
+  // state is known: (hi, lo) -> U or U - R on the way to shared memory, one
+  // pass.  Segments on 16-byte boundaries take float4 loads, others one value
+  // at a time, lanes on consecutive cells (a fixed stride per thread: no
+  // index arithmetic per value).  Threads k < 4 also take a halo cell, the
+  // next three a cell left over from the float4.
+  constexpr int NQ = (SEG / 4 + KC - 1) / KC;    // float4 of a thread
+  constexpr int NH = MIXED && 4 * NQ > M ? 4 * NQ : M;
+  real hv[NH], hr = real(0);
+  float lv[MIXED ? NH : 1], lr = 0.0f;
+  const int len = hi - lo;
+  const long long plane = gvar(v, NV, args.vn, args.vt) * args.ncell + lbase;
+  const real *src;
+  if constexpr (MIXED) src = args.Uh + plane;
+  else src = args.U + plane;
+  const float *srl = MIXED && two ? args.Ul + plane : nullptr;
+  const bool vec = MIXED && cs == 1 &&
+                   ((reinterpret_cast<unsigned long long>(src + lo) |
+                     reinterpret_cast<unsigned long long>(two ? srl + lo : nullptr)) & 15) == 0;
+  const int nq = len >> 2;               // whole float4 of the segment
+  // the extra cell of this thread: segment cell cx, or none (k >= 7 or past a tail)
+  const int cx = k < 2 ? k - 2 : (k < 4 ? len + k - 2 : 4 * nq + k - 4);
+  const bool extra = k < 4 || (vec && k < 7 && cx < len);
+  if (extra) {
+    const int i = lo + cx;
+    bool neg = false;
+    long long a = (long long)i * cs;
+    if (i < 0 || i >= n) a = cell_addr(v, i, neg) - plane;   // ghost cell
+    hr = src[a];
+    if (MIXED && two) lr = srl[a];
+    if (neg) { hr = -hr; lr = -lr; }
+  }
+  if (MIXED && vec) {
+    if constexpr (MIXED) {
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        if (k + q * KC < nq) {
+          const float4 x = *reinterpret_cast<const float4 *>(src + lo + 4 * (k + q * KC));
+          hv[4 * q] = x.x; hv[4 * q + 1] = x.y; hv[4 * q + 2] = x.z; hv[4 * q + 3] = x.w;
+          if (two) {
+            const float4 y = *reinterpret_cast<const float4 *>(srl + lo + 4 * (k + q * KC));
+            lv[4 * q] = y.x; lv[4 * q + 1] = y.y; lv[4 * q + 2] = y.z; lv[4 * q + 3] = y.w;
+          }
         }
-      } else if (i < hi + 2) {   // ghost cell
-        bool neg;
-        const long long a = cell_addr(v, i, neg) - plane;
-        dst[c] = neg ? -src[a] : src[a];
-        if constexpr (MIXED) {
-          if (two) Ls[v * UWP + UH + c] = neg ? -srl[a] : srl[a];
-        }
-      } else {
-        dst[c] = real(0);
-        if constexpr (MIXED) {
-          if (two) Ls[v * UWP + UH + c] = 0.0f;
-        }
+      }
+    }
+  } else if (cs == 1) {
+    const real *s1 = src + lo + k;
+    const float *s2 = MIXED && two ? srl + lo + k : nullptr;
+#pragma unroll
+    for (int q = 0; q < M; ++q) {
+      if (k + q * KC < len) {
+        hv[q] = s1[q * KC];
+        if constexpr (MIXED) lv[q] = two ? s2[q * KC] : 0.0f;
+      }
+    }
+  } else {
+    const long long step = KC * cs;
+    long long a = (lo + k) * cs;
+#pragma unroll
+    for (int q = 0; q < M; ++q, a += step) {
+      if (k + q * KC < len) {
+        hv[q] = src[a];
+        if constexpr (MIXED) lv[q] = two ? srl[a] : 0.0f;
       }
     }
   }
@@ -430,8 +455,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
       ex.rspread[kv] = spread;
     }
   }
-  load_async_wait();
-  __syncthreads();
+  if constexpr (MIXED) __syncthreads();   // the samples' verdict
   if constexpr (MIXED) eps_pos = ex.epsf;
   if constexpr (MIXED && !PRE) {
     if (two) {
@@ -461,19 +485,37 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
       ex.rp[2] = pr;
       ex.rp[3] = E + pr;
     }
-    if (dlt) {
-      // (hi - R_hi) + (lo - R_lo), exact where hi and R_hi are within a
-      // factor of two of each other
-      const float rh = ex.rh[v], rl = ex.rl[v];
-      real *dst = Us + v * UWP + UH;
-      const float *lsp = Ls + v * UWP + UH;
-      for (int j = k; j < UW; j += KC) {
-        const int c = S::pad(j - 2);
-        if (lo - 2 + j < hi + 2) dst[c] = (dst[c] - rh) + (lsp[c] - rl);
-      }
-      __syncthreads();
-    }
   }
+  {
+    real *dst = Us + v * UWP + UH;
+    float rh = 0.0f, rl = 0.0f;
+    if (dlt) { rh = ex.rh[v]; rl = ex.rl[v]; }
+    // (hi - R_hi) + (lo - R_lo), exact where hi and R_hi are within a
+    // factor of two of each other
+    auto val = [&](real x, float l) -> real {
+      if constexpr (MIXED) return dlt ? (x - rh) + (l - rl) : x;
+      else return x;
+    };
+    if (MIXED && vec) {
+      if constexpr (MIXED) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          if (k + q * KC < nq) {
+            float *d = dst + S::pad(4 * (k + q * KC));
+#pragma unroll
+            for (int e = 0; e < 4; ++e) d[e] = val(hv[4 * q + e], lv[4 * q + e]);
+          }
+        }
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < M; ++q)
+        if (k + q * KC < len) dst[S::pad(k + q * KC)] = val(hv[q], lv[MIXED ? q : 0]);
+    }
+    if (extra) dst[S::pad(cx)] = val(hr, lr);
+    for (int c = len + 2 + k; c < SEG + 2; c += KC) dst[S::pad(c)] = real(0);   // past the line
+  }
+  __syncthreads();
   (void)dlt;
   // epsilon of eq. (weight) for this thread's variable v.  The difference
   // form's indicators see U - R, but the rounding noise the FP32 stages
@@ -491,11 +533,12 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
   if constexpr (PRE) {
     const real *pm = reinterpret_cast<const real *>(args.Fm_pre);
     const real *pp = reinterpret_cast<const real *>(args.Fp_pre);
-    for (int idx = tid; idx < NV * (hi - lo); idx += T) {
-      const int kv = idx / (hi - lo), c = idx - kv * (hi - lo);
-      const long long o = gvar(kv, NV, args.vn, args.vt) * args.ncell + lbase + (long long)(lo + c) * cs;
-      Fm[kv * WP + S::pad(c)] = pm[o];
-      Fp[kv * WP + S::pad(c)] = pp[o];
+    const int c0 = lo > 0 || per ? -1 : 0, c1 = hi - lo + (hi < n || per ? 1 : 0);
+    for (int c = c0 + k; c < c1; c += KC) {
+      bool neg;
+      const long long o = cell_addr(v, lo + c, neg);
+      Fm[v * FWP + FH + S::pad(c)] = pm[o];
+      Fp[v * FWP + FH + S::pad(c)] = pp[o];
     }
   } else {
     // ---------------------------------------------------------------- solve
@@ -508,9 +551,11 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
     const int cb = S::pad(k * M);               // padded offset of the chunk's first cell
     const int w0 = lo + (k & ~31) * M;          // first cell of the warp's chunks
     const bool wlive = w0 < n;                  // (uniform over the warp)
-    typename Pair<real>::t cs[M - 1];
+    constexpr bool TREE = S::TREE;
+    using P = typename Pair<real>::t;
+    P cs[M - 1];
+    Run<real> rm = run_empty<real>(), rp = run_empty<real>();
     if (wlive) {
-      Run<real> rm, rp;
       {
         real D[M + 3], S0[M], S1[M], S2[M];
         {
@@ -524,7 +569,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
           chunk_weights<real, M>(win, eps_v, D, S0, S1, S2);
         }
         const EdgeInfo e = {lo + k * M, n, per};
-        real *dm = Fm + v * WP + cb, *dp = Fp + v * WP + cb;
+        real *dm = Fm + v * FWP + FH + cb, *dp = Fp + v * FWP + FH + cb;
         real *zm = Zm + v * WP + cb, *zp = Zp + v * WP + cb;
         // a warp without a line end skips the edge rows' tests
         if (w0 + 32 * M >= n || (w0 == 0 && !per))
@@ -532,14 +577,88 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
         else
           chunk_eliminate<real, M, false>(D, S0, S1, S2, e, dm, zm, dp, zp, cs, rm, rp);
       }
+      if constexpr (!TREE) {
       real *cm = Cr + (2 * v) * 6 * S::KCP + k + (k >> 3), *cp = cm + 6 * S::KCP;
       cm[0] = rm.A; cm[S::KCP] = rm.B; cm[2 * S::KCP] = rm.G;
       cm[3 * S::KCP] = rm.D; cm[4 * S::KCP] = rm.F; cm[5 * S::KCP] = rm.C;
       cp[0] = rp.A; cp[S::KCP] = rp.B; cp[2 * S::KCP] = rp.G;
       cp[3 * S::KCP] = rp.D; cp[4 * S::KCP] = rp.F; cp[5 * S::KCP] = rp.C;
+      }
     }
-    __syncthreads();
 
+    P xin, xown;   // the unknown before the chunk, its own last one
+    P xafter;      // the unknown after it (first and last chunk of the segment)
+    if constexpr (TREE) {
+      // ----------------------------------------- a warp per variable: trees
+      // over the warp's 32 chunks, then (16 lanes per side) over the
+      // segments of the cluster
+      Ends<P> F, L;
+      if (lo + k * M < n) {   // from first in terms of the chunk's own last to both ends
+        const P g = p_set(-rm.G, -rp.G);
+        const P f = p_set(rm.F, rp.F), c = p_set(rm.C, rp.C);
+        L.a = p_set(rm.D, rp.D); L.b = c; L.g = f;
+        F.a = p_fma(g, L.a, p_set(rm.A, rp.A));
+        F.b = p_fma(g, f, p_set(rm.B, rp.B));
+        F.g = p_mul(g, c);
+      } else {
+        F.a = F.b = L.a = L.b = p_set(real(0), real(0));
+        F.g = L.g = p_set(-real(1), -real(1));
+      }
+      const Ends<P> own = L;
+      const P one = p_set(real(1), real(1));
+      Step<P> st[5];
+#pragma unroll
+      for (int h = 0; h < 5; ++h) {
+        const bool r = lane & (1 << h);
+        tree_up(1 << h, r, !r, one, F, L, st[h]);
+      }
+      P xl = p_set(real(0), real(0)), xr = p_set(real(0), real(0));
+      if (R > 1) {
+        if (lane == 0) {
+          Run<real> &a = ex.seg[2 * v], &b = ex.seg[2 * v + 1];
+          a.A = F.a.x; a.B = F.b.x; a.G = F.g.x; a.D = L.a.x; a.C = L.b.x; a.F = L.g.x;
+          b.A = F.a.y; b.B = F.b.y; b.G = F.g.y; b.D = L.a.y; b.C = L.b.y; b.F = L.g.y;
+        }
+        cluster.sync();
+        // lane: side sd, walk position q among the segments
+        const int sd = lane >> 4, q = lane & 15;
+        Run<real> o = run_empty<real>();
+        if (q < R) o = cluster.map_shared_rank(&ex, sd ? R - 1 - q : q)->seg[2 * v + sd];
+        Ends<real> f, l;
+        f.a = o.A; f.b = o.B; f.g = o.G;
+        l.a = o.D; l.b = o.C; l.g = o.F;
+        Step<real> sg[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h)
+          if ((1 << h) < R) tree_up(1 << h, (q & (1 << h)) != 0, false, real(1), f, l, sg[h]);
+        real yl = real(0), yr = real(0);
+        if (per) ring_close(f, l, yl, yr);
+#pragma unroll
+        for (int h = 3; h >= 0; --h)
+          if ((1 << h) < R) tree_down((q & (1 << h)) != 0, false, sg[h], yl, yr);
+        const int lm = rank, lp = 16 + R - 1 - rank;
+        xl = p_set(__shfl_sync(0xffffffffu, yl, lm), __shfl_sync(0xffffffffu, yl, lp));
+        xr = p_set(__shfl_sync(0xffffffffu, yr, lm), __shfl_sync(0xffffffffu, yr, lp));
+      } else if (per) {
+        Ends<real> f, l;
+        const bool p = lane & 1;   // even lanes close the minus ring, odd lanes the plus ring
+        f.a = p ? F.a.y : F.a.x; f.b = p ? F.b.y : F.b.x; f.g = p ? F.g.y : F.g.x;
+        l.a = p ? L.a.y : L.a.x; l.b = p ? L.b.y : L.b.x; l.g = p ? L.g.y : L.g.x;
+        real yl, yr;
+        ring_close(f, l, yl, yr);
+        xl = p_set(__shfl_sync(0xffffffffu, yl, 0), __shfl_sync(0xffffffffu, yl, 1));
+        xr = p_set(__shfl_sync(0xffffffffu, yr, 0), __shfl_sync(0xffffffffu, yr, 1));
+      }
+#pragma unroll
+      for (int h = 4; h >= 0; --h) {
+        const bool r = lane & (1 << h);
+        tree_down(r, !r, st[h], xl, xr);
+      }
+      xin = xl;
+      xafter = xr;
+      xown = p_fma(p_neg(own.b), xr, p_fma(p_neg(own.g), xl, own.a));
+    } else {
+      __syncthreads();
     // ------------------------------------------- the segment's chunks
     // LPS lanes per system (variable and side), eight chunks each in walk
     // order.  Within a lane the chunks' last unknowns l_q are eliminated one
@@ -642,7 +761,10 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
         xl = fma(b1, a22, a12 * b2) * idet;
         xr = fma(a11, b2, a21 * b1) * idet;
       }
-      if (on && cl == 0) Xs[sys * S::XP] = xl;
+      if (on && cl == 0) {
+        Xs[sys * S::XP] = xl;
+        ex.xo[sys] = xr;
+      }
 #pragma unroll
       for (int h = 2; h >= 0; --h) {
         if ((1 << h) < LPS) {
@@ -662,67 +784,99 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
         if (on) xs[pos + (pos >> 3)] = x;
       }
     }
-    __syncthreads();
+      __syncthreads();
+      const real *xm = Xs + (2 * v) * S::XP, *xp = xm + S::XP;
+      const int m0 = k, m1 = k + 1, p0 = KC - 1 - k, p1 = KC - k;
+      xin = p_set(xm[m0 + (m0 >> 3)], xp[p0 + (p0 >> 3)]);
+      xown = p_set(xm[m1 + (m1 >> 3)], xp[p1 + (p1 >> 3)]);
+      xafter = p_set(ex.xo[2 * v], ex.xo[2 * v + 1]);
+    }
 
     // ------------------------------------------- back substitution
     if (wlive) {
-      const real *xm = Xs + (2 * v) * S::XP, *xp = xm + S::XP;
-      const int m0 = k, m1 = k + 1, p0 = KC - 1 - k, p1 = KC - k;
-      const typename Pair<real>::t xin = p_set(xm[m0 + (m0 >> 3)], xp[p0 + (p0 >> 3)]);
-      const typename Pair<real>::t xown = p_set(xm[m1 + (m1 >> 3)], xp[p1 + (p1 >> 3)]);
-      const int o = v * WP + cb, len = n - (lo + k * M);
+      const int o = v * WP + cb, of = v * FWP + FH + cb, mine = n - (lo + k * M);
       if (w0 + 32 * M > n)
-        chunk_back<real, M, true>(uv + cb, Fm + o, Zm + o, Fp + o, Zp + o, cs, xin, xown, len);
+        chunk_back<real, M, true>(uv + cb, Fm + of, Zm + o, Fp + of, Zp + o, cs, xin, xown, mine);
       else
-        chunk_back<real, M, false>(uv + cb, Fm + o, Zm + o, Fp + o, Zp + o, cs, xin, xown, len);
+        chunk_back<real, M, false>(uv + cb, Fm + of, Zm + o, Fp + of, Zp + o, cs, xin, xown, mine);
+      __syncwarp();   // (a lane past a ragged end may have written its idle slots)
+      // The face values of the two cells next to the segment are known here
+      // as well (the unknowns outside the segment's ends), so this CTA limits
+      // those cells itself and needs nothing more from its neighbours.
+      if (k == 0 && (lo > 0 || per)) {
+        const real u = uv[S::pad(-1)];
+        Fm[v * FWP + FH + S::pad(-1)] = u + xin.x;
+        Fp[v * FWP + FH + S::pad(-1)] = u + xafter.y;
+      }
+      if (k == (hi - lo - 1) / M && (hi < n || per)) {
+        const real u = uv[S::pad(hi - lo)];
+        Fm[v * FWP + FH + S::pad(hi - lo)] = u + xafter.x;
+        Fp[v * FWP + FH + S::pad(hi - lo)] = u + xin.y;
+      }
     }
+    // the neighbours read this CTA's run until here at the latest: arrive
+    // now, wait before exit (shared memory must outlive their reads)
+    if (R > 1) cluster_arrive_relaxed();
   }
   __syncthreads();
 
   // ---------------------------------------------------------------- limit
+  // Cells of the segment and, where the line goes on, the two next to it
+  // (their theta counts belong to the neighbours).
   unsigned int t1 = 0, t2 = 0;
-  const real inv12 = real(1) / (real(1) - real(2) * wgl);
+  const real inv12 = rcp(real(1) - real(2) * wgl);
   // difference form: the face values hold U - R until a cell is limited,
   // then the limited values in full (cfull[c] = 1)
   float rf[NV];
 #pragma unroll
   for (int kv = 0; kv < NV; ++kv) rf[kv] = dlt ? ex.rf[kv] : 0.0f;
   int anyfull = 0;   // this thread limited a cell (difference form)
-  if constexpr (MIXED) {
-    if (dlt)
-      for (int c = tid; c < hi - lo; c += T) cfull[c] = 0;
-  }
   if (args.limiter) {
     // FP32 pretest of every cell of this thread (a superset of the cells
     // the exact test limits: its thresholds carry twice the FP32 round-off
     // allowance, which covers the FP32 evaluation and, in the FP64 form, the
     // rounding of the inputs to FP32); the flagged cells (rare) are limited
     // exactly in a second loop, so the pretest loop carries no FP64 state
-    static_assert(SEG <= 32 * T, "one mask bit per cell of a thread");
+    static_assert(SEG + 2 <= 32 * T, "one mask bit per cell of a thread");
+    const int c0 = tid - (lo > 0 || per ? 1 : 0), c1 = hi - lo + (hi < n || per ? 1 : 0);
     unsigned int mask = 0;
     const float wgl_f = float(wgl), inv12_f = float(inv12), eps_f = float(eps_pos);
 #pragma unroll 1
-    for (int q = 0, c = tid; c < hi - lo; ++q, c += T) {
+    for (int q = 0, c = c0; c < c1; ++q, c += T) {
       float ub[NV], a[NV], b[NV];
+      const int pc = S::pad(c);
 #pragma unroll
       for (int kv = 0; kv < NV; ++kv) {
-        ub[kv] = to_f32(Us[kv * UWP + UH + S::pad(c)]) + rf[kv];
-        a[kv] = to_f32(Fm[kv * WP + S::pad(c)]) + rf[kv];
-        b[kv] = to_f32(Fp[kv * WP + S::pad(c)]) + rf[kv];
+        ub[kv] = to_f32(Us[kv * UWP + UH + pc]);
+        a[kv] = to_f32(Fm[kv * FWP + FH + pc]);
+        b[kv] = to_f32(Fp[kv * FWP + FH + pc]);
       }
-      if (limit_need_mixed<NV>(ub, a, b, wgl_f, inv12_f, eps_f)) mask |= 1u << q;
+      float full[NV], dm[NV], dp[NV];
+#pragma unroll
+      for (int kv = 0; kv < NV; ++kv) {
+        full[kv] = ub[kv] + rf[kv];
+        dm[kv] = a[kv] - ub[kv];
+        dp[kv] = b[kv] - ub[kv];
+      }
+      if (limit_box_free<NV>(full, dm, dp, wgl_f, eps_f)) continue;
+#pragma unroll
+      for (int kv = 0; kv < NV; ++kv) {
+        a[kv] += rf[kv];
+        b[kv] += rf[kv];
+      }
+      if (limit_need_mixed<NV>(full, a, b, wgl_f, inv12_f, eps_f)) mask |= 1u << q;
     }
 #pragma unroll 1
     while (mask) {
       const int q = __ffs(mask) - 1;
       mask &= mask - 1;
-      const int c = tid + q * T;
+      const int c = c0 + q * T, pc = S::pad(c);
       real ub[NV], a[NV], b[NV];
 #pragma unroll
       for (int kv = 0; kv < NV; ++kv) {
-        ub[kv] = Us[kv * UWP + UH + S::pad(c)];
-        a[kv] = Fm[kv * WP + S::pad(c)];
-        b[kv] = Fp[kv * WP + S::pad(c)];
+        ub[kv] = Us[kv * UWP + UH + pc];
+        a[kv] = Fm[kv * FWP + FH + pc];
+        b[kv] = Fp[kv * FWP + FH + pc];
       }
       if constexpr (MIXED) {
         if (dlt) {
@@ -731,7 +885,8 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
           // and the face values in full
 #pragma unroll
           for (int kv = 0; kv < NV; ++kv) {
-            ub[kv] = args.Uh[gvar(kv, NV, args.vn, args.vt) * args.ncell + lbase + (long long)(lo + c) * cs];
+            bool neg;   // (never a reflected cell: those beyond a wall are not limited)
+            ub[kv] = args.Uh[cell_addr(kv, lo + c, neg)];
             a[kv] += rf[kv];
             b[kv] += rf[kv];
           }
@@ -743,150 +898,88 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
       if (f) {
 #pragma unroll
         for (int kv = 0; kv < NV; ++kv) {
-          Fm[kv * WP + S::pad(c)] = a[kv];
-          Fp[kv * WP + S::pad(c)] = b[kv];
+          Fm[kv * FWP + FH + pc] = a[kv];
+          Fp[kv * FWP + FH + pc] = b[kv];
         }
         if constexpr (MIXED) {
           if (dlt) { cfull[c] = 1; anyfull = 1; }
         }
+        if (c >= 0 && c < hi - lo) {
+          t1 += f & 1;
+          t2 += (f >> 1) & 1;
+        }
       }
-      t1 += f & 1;
-      t2 += (f >> 1) & 1;
     }
   }
   // ---------------------------------------------------------------- flux
   // HLLC (or local Lax-Friedrichs) at face f (between cells f-1 and f): the
-  // left state is U^- of cell f-1, the right state U^+ of cell f; the two
-  // segment-end faces read a neighbour CTA's value.  fsmax: the largest
-  // |u| + a over this thread's face states
+  // left state is U^- of cell f-1, the right state U^+ of cell f, both in this
+  // CTA's shared memory; at the end of a bounded line the exterior state
+  // follows from the interior one.  fsmax: the largest |u| + a over this
+  // thread's face states; farface: a face of this thread is stored in full.
   real fsmax = real(0);
-  auto face = [&](int f) {
+  int farface = 0;
+  if constexpr (MIXED) anyfull = __syncthreads_or(anyfull);
+  else __syncthreads();
+#pragma unroll 1
+  for (int f = lo + tid; f <= hi; f += T) {
     real Ul[NV], Ur[NV], F[NV];
-    const real *srcL = nullptr;
-    const real *srcR = nullptr;
-    const unsigned char *cfL = cfull, *cfR = cfull;   // (difference form)
-    int il = 0, ir = 0;
-    // left state: U^- of cell f-1
-    if (f == 0) {
-      if (per) {
-        srcL = cluster.map_shared_rank(Fm, R - 1); il = (n - 1) - (R - 1) * SEG;
-        cfL = cluster.map_shared_rank(cfull, R - 1);
-      }
-    } else if (f - 1 < lo) {
-      srcL = cluster.map_shared_rank(Fm, rank - 1); il = f - 1 - (rank - 1) * SEG;
-      cfL = cluster.map_shared_rank(cfull, rank - 1);
-    } else { srcL = Fm; il = f - 1 - lo; }
-    // right state: U^+ of cell f
-    if (f == n) {
-      if (per) {
-        srcR = cluster.map_shared_rank(Fp, 0); ir = 0;
-        cfR = cluster.map_shared_rank(cfull, 0);
-      }
-    } else if (f >= hi) {
-      srcR = cluster.map_shared_rank(Fp, rank + 1); ir = f - (rank + 1) * SEG;
-      cfR = cluster.map_shared_rank(cfull, rank + 1);
-    } else { srcR = Fp; ir = f - lo; }
-    if (srcL) {
+    const int c = f - lo;   // the right cell
+    const bool bl = f == 0 && !per, br = f == n && !per;
+    {
+      const int il = FH + S::pad(c - 1), ir = FH + S::pad(c);
+      const real *L = bl ? Fp + ir : Fm + il, *Rr = br ? Fm + il : Fp + ir;
 #pragma unroll
-      for (int kv = 0; kv < NV; ++kv) Ul[kv] = srcL[kv * WP + S::pad(il)];
+      for (int kv = 0; kv < NV; ++kv) {
+        Ul[kv] = L[kv * FWP];
+        Ur[kv] = Rr[kv * FWP];
+      }
     }
-    if (srcR) {
-#pragma unroll
-      for (int kv = 0; kv < NV; ++kv) Ur[kv] = srcR[kv * WP + S::pad(ir)];
-    }
+    const bool wl = bl && args.bclo == 2, wr = br && args.bchi == 2;   // a wall's mirror state
     real sf;
+    bool near = false;
     if constexpr (MIXED) {
       if (dlt) {
         // stored values are U - R (or the limited U in full): both forms of
-        // each state, the exterior of a boundary face by its condition
+        // each state
         float dl[NV], dr[NV];
-        // flags of this CTA's cells only where one of them was limited
-        const bool fulL = srcL && (cfL != cfull || anyfull) && cfL[il];
-        const bool fulR = srcR && (cfR != cfull || anyfull) && cfR[ir];
-        if (srcL) {
+        const bool fulL = anyfull && cfull[bl ? c : c - 1], fulR = anyfull && cfull[br ? c - 1 : c];
 #pragma unroll
-          for (int kv = 0; kv < NV; ++kv) {
-            dl[kv] = fulL ? Ul[kv] - rf[kv] : Ul[kv];
-            Ul[kv] = fulL ? Ul[kv] : Ul[kv] + rf[kv];
-          }
+        for (int kv = 0; kv < NV; ++kv) {
+          dl[kv] = Ul[kv];
+          dr[kv] = Ur[kv];
+          Ul[kv] = fulL ? Ul[kv] : Ul[kv] + rf[kv];
+          Ur[kv] = fulR ? Ur[kv] : Ur[kv] + rf[kv];
         }
-        if (srcR) {
-#pragma unroll
-          for (int kv = 0; kv < NV; ++kv) {
-            dr[kv] = fulR ? Ur[kv] - rf[kv] : Ur[kv];
-            Ur[kv] = fulR ? Ur[kv] : Ur[kv] + rf[kv];
-          }
-        }
-        if (!srcL) {
-#pragma unroll
-          for (int kv = 0; kv < NV; ++kv) { Ul[kv] = Ur[kv]; dl[kv] = dr[kv]; }
-          if (args.bclo == 2) { Ul[1] = -Ul[1]; dl[1] = -dr[1] - 2.0f * rf[1]; }
-        }
-        if (!srcR) {
-#pragma unroll
-          for (int kv = 0; kv < NV; ++kv) { Ur[kv] = Ul[kv]; dr[kv] = dl[kv]; }
-          if (args.bchi == 2) { Ur[1] = -Ur[1]; dr[1] = -dl[1] - 2.0f * rf[1]; }
-        }
-        const bool near = !args.flux && !fulL && !fulR &&
-                          fabsf(dl[0]) <= 0.5f * rf[0] && fabsf(dr[0]) <= 0.5f * rf[0] &&
-                          fabsf(dl[NV - 1]) <= 0.5f * rf[NV - 1] &&
-                          fabsf(dr[NV - 1]) <= 0.5f * rf[NV - 1];
+        if (wl) { Ul[1] = -Ul[1]; dl[1] = -dl[1] - 2.0f * rf[1]; }
+        if (wr) { Ur[1] = -Ur[1]; dr[1] = -dr[1] - 2.0f * rf[1]; }
+        near = !args.flux && !fulL && !fulR &&
+               fabsf(dl[0]) <= 0.5f * rf[0] && fabsf(dr[0]) <= 0.5f * rf[0] &&
+               fabsf(dl[NV - 1]) <= 0.5f * rf[NV - 1] && fabsf(dr[NV - 1]) <= 0.5f * rf[NV - 1];
         if (near) hllc_delta<NV>(Ul, Ur, dl, dr, rf, ex.rp, gam, F, sf);
-        else if (args.flux) llf<real, NV>(Ul, Ur, gam, F, sf);
-        else hllc<real, NV>(Ul, Ur, gam, F, sf);
-        fdel[f - lo] = near ? 1 : 0;
-        if (sf > fsmax || sf != sf) fsmax = sf;   // a NaN speed stays
-#pragma unroll
-        for (int kv = 0; kv < NV; ++kv) Fl[kv * (SEG + 2) + (f - lo)] = F[kv];
-        return;
+        fdel[c] = near ? 1 : 0;
+        farface |= near ? 0 : 1;
+      } else {
+        if (wl) Ul[1] = -Ul[1];
+        if (wr) Ur[1] = -Ur[1];
       }
+    } else {
+      if (wl) Ul[1] = -Ul[1];
+      if (wr) Ur[1] = -Ur[1];
     }
-    if (!srcL) {  // boundary face 0: exterior = BC(interior)
-#pragma unroll
-      for (int kv = 0; kv < NV; ++kv) Ul[kv] = Ur[kv];
-      if (args.bclo == 2) Ul[1] = -Ul[1];
+    if (!near) {
+      if (args.flux) llf<real, NV>(Ul, Ur, gam, F, sf);
+      else hllc<real, NV>(Ul, Ur, gam, F, sf, MIXED || args.fcheck);
     }
-    if (!srcR) {
-#pragma unroll
-      for (int kv = 0; kv < NV; ++kv) Ur[kv] = Ul[kv];
-      if (args.bchi == 2) Ur[1] = -Ur[1];
-    }
-    if (args.flux) llf<real, NV>(Ul, Ur, gam, F, sf);
-    else hllc<real, NV>(Ul, Ur, gam, F, sf, MIXED || args.fcheck);
     if ((MIXED || args.fcheck) && (sf > fsmax || sf != sf)) fsmax = sf;   // a NaN speed stays
 #pragma unroll
-    for (int kv = 0; kv < NV; ++kv) Fl[kv * (SEG + 2) + (f - lo)] = F[kv];
-  };
-  if constexpr (MIXED) {
-    // faces with both states in this CTA first, then (after the cluster
-    // barrier completes) the two segment-end faces, on two warps; whether
-    // any of this CTA's cells holds its face values in full
-    anyfull = __syncthreads_or(anyfull);
-    cluster_arrive();   // this CTA's limited face values, for the neighbours
-    const bool lo_remote = per || lo > 0, hi_remote = per || hi < n;
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {   // one call site of the face code
-      int f, fend;
-      if (pass == 0) {
-        f = lo + (lo_remote ? 1 : 0) + tid;
-        fend = hi - (hi_remote ? 1 : 0);
-      } else {
-        cluster_wait();
-        f = (tid == 0 && lo_remote) ? lo : ((tid == 32 && hi_remote) ? hi : hi + 1);
-        fend = hi;
-      }
-      for (; f <= fend; f += T) face(f);
-    }
-  } else {
-    // the FP64 form (one CTA per SM, bound by the FP64 pipe): a plain
-    // barrier, then every face in one pass
-    cluster.sync();
-    for (int f = lo + tid; f <= hi; f += T) face(f);
+    for (int kv = 0; kv < NV; ++kv) Fl[kv * FLS + c] = F[kv];
   }
-  __syncthreads();
-  // the neighbours' face values are no longer read: arrive now, wait before
-  // exit (a CTA's shared memory must outlive the neighbours' reads of it)
-  cluster_arrive_relaxed();
+  // any face of the CTA in full form: only then the update compares the forms
+  bool mixedforms = false;
+  if constexpr (MIXED) mixedforms = __syncthreads_or(farface) && dlt;
+  else __syncthreads();
+  (void)mixedforms;
 
   // ---------------------------------------------------------------- update
   // the stage's extrema in the line's arithmetic (converted once per warp)
@@ -894,11 +987,41 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
   unsigned int nbad = 0;
   unsigned long long firstbad = ~0ull;
   const real ih = MIXED ? real(args.ih_f) : real(args.ih);
-  const double dt = (MODE == MODE_FINAL) ? ctl->dt : 0.0;
+  const double dt = (MODE == MODE_FINAL && !MIXED) ? ctl->dt : 0.0;
+  (void)dt;
   const double gg1 = MIXED ? 0.0 : args.gamma * (args.gamma - 1.0);
   (void)gg1;
   const real *Din = reinterpret_cast<const real *>(args.Din);
-  for (int c = tid; c < hi - lo; c += T) {
+  // x-sweep output: thread (v, k) writes cells of its own variable, four at a
+  // time on 16-byte boundaries
+  int cdone = 0;
+  if (MODE == MODE_XSWEEP && !mixedforms) {
+    real *D = reinterpret_cast<real *>(args.Dout) + plane + lo * cs;
+    const real *Fv = Fl + v * FLS;
+    bool vst = false;
+    if constexpr (MIXED) {
+      vst = cs == 1 && (reinterpret_cast<unsigned long long>(D) & 15) == 0;
+      if (vst) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          const int c = 4 * (k + q * KC);
+          if (c + 4 <= len) {
+            const float4 f = *reinterpret_cast<const float4 *>(Fv + c);
+            const float g = Fv[c + 4];
+            *reinterpret_cast<float4 *>(D + c) =
+                make_float4((f.x - f.y) * ih, (f.y - f.z) * ih, (f.z - f.w) * ih, (f.w - g) * ih);
+          }
+        }
+      }
+    }
+    const int c0 = vst ? len & ~3 : 0;
+    D += (c0 + k) * cs;
+    const long long step = KC * cs;
+    for (int c = c0 + k; c < len; c += KC, D += step) *D = (Fv[c] - Fv[c + 1]) * ih;
+    cdone = len;
+  }
+  if (MIXED && MODE == MODE_FINAL) cdone = len;
+  for (int c = cdone + tid; c < len; c += T) {
     int i = lo + c;
     long long addr = lbase + (long long)i * cs;
     real Lv[NV];
@@ -906,11 +1029,11 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
     // (a limited or distant face state) is put on the same footing
     int fmix = 0;   // 1: only the left face is F - F(R), 2: only the right one
     if constexpr (MIXED) {
-      if (dlt) fmix = (fdel[c] != fdel[c + 1]) ? (fdel[c] ? 2 : 1) : 0;
+      if (mixedforms) fmix = (fdel[c] != fdel[c + 1]) ? (fdel[c] ? 2 : 1) : 0;
     }
 #pragma unroll
     for (int kv = 0; kv < NV; ++kv) {
-      real fa = Fl[kv * (SEG + 2) + c], fb = Fl[kv * (SEG + 2) + c + 1];
+      real fa = Fl[kv * FLS + c], fb = Fl[kv * FLS + c + 1];
       if constexpr (MIXED) {
         if (fmix == 2) fb -= ex.rF[kv];
         else if (fmix == 1) fa -= ex.rF[kv];
@@ -963,56 +1086,60 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
         }
         mymax = less(mymax, rate) ? rate : mymax;
       }
-    } else {
-      // mixed form: compensated stage combination on hi + lo pairs
-      const dfl dtd = {float(dt), float(dt - double(float(dt)))};
-      const dfl third = {0.333333343f, -9.93410776e-09f};
-      const dfl two3 = {0.666666687f, -1.98682155e-08f};
-      float Th[NV], Tl[NV];
+    }
+  }
+  if constexpr (MIXED && MODE == MODE_FINAL) {
+    // mixed form in 1-D (2-D combines the two sweeps in a kernel of its own):
+    // compensated stage combination on hi + lo pairs; the states of a
+    // thread's next cell load while this one is combined
+    static_assert(NV == 3, "the 2-D mixed form has no final sweep");
+    const dfl third = {0.333333343f, -9.93410776e-09f};
+    const dfl two3 = {0.666666687f, -1.98682155e-08f};
+    const dfl dtd = ex.dt;
+    dfl nk[NV], n0[NV];
+    auto fetch = [&](int c) {
 #pragma unroll
       for (int kv = 0; kv < NV; ++kv) {
-        int g = gvar(kv, NV, args.vn, args.vt);
-        long long a = g * args.ncell + addr;
-        dfl uk = {args.Uh[a], args.Ul[a]};
-        dfl s = df_add(uk, df_mul_f(dtd, Lv[kv]));          // U_k + dt L
-        dfl un;
-        if (args.stage == 0) {
-          un = s;
-        } else {
-          dfl u0 = {args.U0h[a], args.U0l[a]};
-          if (args.stage == 1) un = df_add(df_mul_f(u0, 0.75f), df_mul_f(s, 0.25f));
-          else un = df_add(df_mul(u0, third), df_mul(s, two3));
-        }
-        args.Uoh[a] = un.hi;
-        args.Uol[a] = un.lo;
-        Th[kv] = un.hi;   // line-variable order (no run-time register index)
-        Tl[kv] = un.lo;
+        const long long a = kv * args.ncell + lbase + lo + c;
+        nk[kv] = {args.Uh[a], args.Ul[a]};
+        if (args.stage != 0) n0[kv] = {args.U0h[a], args.U0l[a]};
       }
-      float rho = Th[0], E = Th[NV - 1];
-      float mx = NV == 4 && args.vn != 1 ? Th[2] : Th[1];
-      float my = NV == 4 ? (args.vn != 1 ? Th[1] : Th[2]) : 0.0f;
+    };
+    if (tid < len) fetch(tid);
+    for (int c = tid; c < len; c += T) {
+      dfl uk[NV], u0[NV], un[NV];
+#pragma unroll
+      for (int kv = 0; kv < NV; ++kv) {
+        uk[kv] = nk[kv];
+        u0[kv] = n0[kv];
+      }
+      if (c + T < len) fetch(c + T);
+      const int fmix = mixedforms && fdel[c] != fdel[c + 1] ? (fdel[c] ? 2 : 1) : 0;
+#pragma unroll
+      for (int kv = 0; kv < NV; ++kv) {
+        float fa = Fl[kv * FLS + c], fb = Fl[kv * FLS + c + 1];
+        if (fmix == 2) fb -= ex.rF[kv];
+        else if (fmix == 1) fa -= ex.rF[kv];
+        const float L = (fa - fb) * ih;
+        const dfl s = df_add(uk[kv], df_mul_f(dtd, L));          // U_k + dt L
+        if (args.stage == 0) un[kv] = s;
+        else if (args.stage == 1) un[kv] = df_add(df_mul_f(u0[kv], 0.75f), df_mul_f(s, 0.25f));
+        else un[kv] = df_add(df_mul(u0[kv], third), df_mul(s, two3));
+        const long long a = kv * args.ncell + lbase + lo + c;
+        args.Uoh[a] = un[kv].hi;
+        args.Uol[a] = un[kv].lo;
+      }
+      const float rho = un[0].hi, mx = un[1].hi, E = un[2].hi;
       // g = rho E - |m|^2/2 with the compensated parts (its sign decides G)
-      dfl rE = df_mul({Th[0], Tl[0]}, {Th[NV - 1], Tl[NV - 1]});
-      dfl m2 = df_mul({Th[1], Tl[1]}, {Th[1], Tl[1]});
-      if (NV == 4) m2 = df_add(m2, df_mul({Th[2], Tl[2]}, {Th[2], Tl[2]}));
-      dfl gq = df_add(rE, {-0.5f * m2.hi, -0.5f * m2.lo});
-      bool ok = (rho > 0.0f) && (gq.hi > 0.0f) && isfinite(E) && isfinite(mx) && isfinite(my);
-      if (!ok) {
+      const dfl rE = df_mul(un[0], un[2]), m2 = df_mul(un[1], un[1]);
+      const dfl gq = df_add(rE, {-0.5f * m2.hi, -0.5f * m2.lo});
+      if (!((rho > 0.0f) && (gq.hi > 0.0f) && isfinite(E) && isfinite(mx))) {
         ++nbad;
-        firstbad = min(firstbad, (unsigned long long)addr);
+        firstbad = min(firstbad, (unsigned long long)(lbase + lo + c));
       } else {
         mymin = fminf(mymin, rho);
-        float e = gq.hi / (rho * rho);
-        float a = sqrtf(args.gg1_f * e);
-        float rate;
-        if (NV == 4) {
-          const float ihx = args.vn == 1 ? args.ih_f : args.ih_other_f;
-          const float ihy = args.vn == 1 ? args.ih_other_f : args.ih_f;
-          rate = (fabsf(mx / rho) + a) * ihx + (fabsf(my / rho) + a) * ihy;
-        } else {
-          rate = (fabsf(mx / rho) + a) * args.ih_f;
-        }
-        mymax = fmaxf(mymax, rate);
+        const float ir = rcp(rho);
+        mymax = fmaxf(mymax, (fabsf(mx) * ir + sqrtf(args.gg1_f * gq.hi) * ir) * ih);
       }
     }
   }
@@ -1052,7 +1179,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
       if (t1) atomicAdd(&ctl->theta1, (unsigned long long)t1);
       if (t2) atomicAdd(&ctl->theta2, (unsigned long long)t2);
     }
-  } else if (MODE == MODE_XSWEEP) {
+  } else if (MODE == MODE_XSWEEP && __any_sync(0xffffffffu, t1 | t2)) {
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
       t1 += __shfl_down_sync(0xffffffffu, t1, d);
@@ -1063,7 +1190,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
       if (t2) atomicAdd(&ctl->theta2, (unsigned long long)t2);
     }
   }
-  cluster_wait();
+  if (!PRE && R > 1) cluster_wait();
 }
 
 }  // namespace ppk

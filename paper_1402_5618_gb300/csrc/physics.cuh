@@ -333,16 +333,17 @@ __device__ __forceinline__ void hllc_delta(const float *Ul, const float *Ur, con
     dphys(dl, ul, dul, dpl, dF);
     return;
   }
-  const float den = rl * (SL - ul) - rr * (SR - ur);
+  const float Xl = rl * (SL - ul), Xr = rr * (SR - ur);
+  const float iden = rcp(Xl - Xr);
   const float dpn = dpr - dpl, dun = dur - dul;
-  const float sml = (dpn - rr * (SR - ur) * dun) / den;   // S_M - u_l
+  const float sml = (dpn - Xr * dun) * iden;   // S_M - u_l
   const float SM = ul + sml;
   const bool left = SM > 0.0f;
   if (!left && !(SR >= 0.0f)) {
     dphys(dr, ur, dur, dpr, dF);
     return;
   }
-  const float d = left ? sml : (dpn - rl * (SL - ul) * dun) / den;   // S_M - u_K
+  const float d = left ? sml : (dpn - Xl * dun) * iden;   // S_M - u_K
   const float rK = left ? rl : rr, uK = left ? ul : ur, pK = left ? pl : pr, SK = left ? SL : SR;
   const float vK = left ? vl : vr, EKr = left ? El * irl : Er * irr;
   float dK[NV];   // element-wise selects: no run-time indexing of the arrays
@@ -477,6 +478,33 @@ __device__ __forceinline__ int limit_cell(const real *ub, real *um, real *up, re
     flags |= 2;
   }
   return flags;
+}
+
+// A cell the limiter cannot touch, from the deviations of its two face values
+// from the average alone (FP32, both forms): with dk = max |face - average|
+// of component k, all three quadrature points of the limiter lie in the box
+// ub +- d (the interior one is ub - wgl/(1 - 2 wgl) (dm + dp), inside it for
+// wgl <= 1/4), so rho >= r = ub_0 - d_0 and g >= r (E - d_E) - |m|^2/2 at the
+// box's worst corner.  The thresholds are twice the FP32 allowances of
+// limiter_cell at the box's largest magnitudes, which leaves the evaluation's
+// own rounding (about a tenth of them) ample room.  NaN fails every comparison.  Smooth
+// cells pass, and skip the pretest below (a third of its instructions).
+template <int NV>
+__device__ __forceinline__ bool limit_box_free(const float *ub, const float *dm, const float *dp,
+                                               float wgl, float eps) {
+  const float uf = 5.9604645e-08f;
+  const float d0 = fmaxf(fabsf(dm[0]), fabsf(dp[0]));
+  const float dE = fmaxf(fabsf(dm[NV - 1]), fabsf(dp[NV - 1]));
+  float S = 0.0f;
+#pragma unroll
+  for (int k = 1; k < NV - 1; ++k) {
+    const float m = fabsf(ub[k]) + fmaxf(fabsf(dm[k]), fabsf(dp[k]));
+    S = fmaf(m, m, S);
+  }
+  const float r = ub[0] - d0, R = ub[0] + d0, E = ub[NV - 1] + dE;
+  const float g = fmaf(r, ub[NV - 1] - dE, -0.5f * S);
+  const float need = fmaf(eps * R, R, 128.0f * uf * fmaf(E, R, S));
+  return r > fmaf(32.0f * uf, R, 2.0f * eps) && g > need && need < 3.0e38f && wgl <= 0.25f;
 }
 
 // Mixed form: an FP32 test of the limiter's conditions with doubled

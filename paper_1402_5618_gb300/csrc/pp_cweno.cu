@@ -432,49 +432,65 @@ __device__ __forceinline__ void combine_tile(int i0, int j0, const float *Ukh, c
   float mymin = 3.0e38f, mymax = 0.0f;   // FP32 running extrema (converted once)
   unsigned int nbad = 0;
   unsigned long long firstbad = ~0ull;
+  // two rows at a time, all their loads before the first store (which the
+  // compiler may not move them across): 40 in flight per thread
+  constexpr int RP = 2;
+  static_assert(TT / RY % RP == 0, "row pairs");
+#pragma unroll 1
+  for (int r0 = 0; r0 < TT / RY; r0 += RP) {
+    float dx[RP][NV];
+    dfl uk[RP][NV], u0[RP][NV];
 #pragma unroll
-  for (int rr = 0; rr < TT / RY; ++rr) {
-    const int r = threadIdx.y + rr * RY;
-    const int j = j0 + r, i = i0 + threadIdx.x;
-    if (j >= ny || i >= nx) continue;
-    const long long addr = (long long)j * nx + i;
-    float Th[NV], Tl[NV];
+    for (int p = 0; p < RP; ++p) {
+      const int j = j0 + threadIdx.y + (r0 + p) * RY, i = i0 + threadIdx.x;
+      if (j >= ny || i >= nx) continue;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const long long a = v * ncell + addr;
-      const float L = Dx[a] + tile[v][r][threadIdx.x];
-      const dfl uk = {Ukh[a], Ukl[a]};
-      const dfl s = df_add(uk, df_mul_f(dtd, L));
-      dfl un;
-      if (stage == 0) {
-        un = s;
-      } else {
-        const dfl u0 = {U0h[a], U0l[a]};
-        if (stage == 1) un = df_add(df_mul_f(u0, 0.75f), df_mul_f(s, 0.25f));
-        else un = df_add(df_mul(u0, third), df_mul(s, two3));
+      for (int v = 0; v < NV; ++v) {
+        const long long a = v * ncell + (long long)j * nx + i;
+        dx[p][v] = Dx[a];
+        uk[p][v] = {Ukh[a], Ukl[a]};
+        if (stage != 0) u0[p][v] = {U0h[a], U0l[a]};
       }
-      Uoh[a] = un.hi;
-      Uol[a] = un.lo;
-      Th[v] = un.hi;
-      Tl[v] = un.lo;
-      tile[v][r][threadIdx.x] = un.hi;
-      tlo[v][r][threadIdx.x] = un.lo;
     }
-    const float rho = Th[0], mx = Th[1], my = Th[2], E = Th[NV - 1];
-    const dfl rE = df_mul({Th[0], Tl[0]}, {Th[NV - 1], Tl[NV - 1]});
-    const dfl m2 =
-        df_add(df_mul({Th[1], Tl[1]}, {Th[1], Tl[1]}), df_mul({Th[2], Tl[2]}, {Th[2], Tl[2]}));
-    const dfl gq = df_add(rE, {-0.5f * m2.hi, -0.5f * m2.lo});
-    const bool ok = rho > 0.0f && gq.hi > 0.0f && isfinite(E) && isfinite(mx) && isfinite(my);
-    if (!ok) {
-      ++nbad;
-      firstbad = min(firstbad, (unsigned long long)addr);
-    } else {
-      mymin = fminf(mymin, rho);
-      const float irho = 1.0f / rho;
-      const float a = sqrtf(gg1 * (gq.hi * irho * irho));
-      const float rate = (fabsf(mx * irho) + a) * ihx + (fabsf(my * irho) + a) * ihy;
-      mymax = fmaxf(mymax, rate);
+#pragma unroll
+    for (int p = 0; p < RP; ++p) {
+      const int r = threadIdx.y + (r0 + p) * RY;
+      const int j = j0 + r, i = i0 + threadIdx.x;
+      if (j >= ny || i >= nx) continue;
+      const long long addr = (long long)j * nx + i;
+      float Th[NV], Tl[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const long long a = v * ncell + addr;
+        const float L = dx[p][v] + tile[v][r][threadIdx.x];
+        const dfl s = df_add(uk[p][v], df_mul_f(dtd, L));
+        dfl un;
+        if (stage == 0) un = s;
+        else if (stage == 1) un = df_add(df_mul_f(u0[p][v], 0.75f), df_mul_f(s, 0.25f));
+        else un = df_add(df_mul(u0[p][v], third), df_mul(s, two3));
+        Uoh[a] = un.hi;
+        Uol[a] = un.lo;
+        Th[v] = un.hi;
+        Tl[v] = un.lo;
+        tile[v][r][threadIdx.x] = un.hi;
+        tlo[v][r][threadIdx.x] = un.lo;
+      }
+      const float rho = Th[0], mx = Th[1], my = Th[2], E = Th[NV - 1];
+      const dfl rE = df_mul({Th[0], Tl[0]}, {Th[NV - 1], Tl[NV - 1]});
+      const dfl m2 =
+          df_add(df_mul({Th[1], Tl[1]}, {Th[1], Tl[1]}), df_mul({Th[2], Tl[2]}, {Th[2], Tl[2]}));
+      const dfl gq = df_add(rE, {-0.5f * m2.hi, -0.5f * m2.lo});
+      const bool ok = rho > 0.0f && gq.hi > 0.0f && isfinite(E) && isfinite(mx) && isfinite(my);
+      if (!ok) {
+        ++nbad;
+        firstbad = min(firstbad, (unsigned long long)addr);
+      } else {
+        mymin = fminf(mymin, rho);
+        const float irho = 1.0f / rho;
+        const float a = sqrtf(gg1 * (gq.hi * irho * irho));
+        const float rate = (fabsf(mx * irho) + a) * ihx + (fabsf(my * irho) + a) * ihy;
+        mymax = fmaxf(mymax, rate);
+      }
     }
   }
   __syncthreads();
@@ -523,7 +539,7 @@ __device__ __forceinline__ void combine_tile(int i0, int j0, const float *Ukh, c
 }
 
 template <int NV, int RY>
-__global__ void __launch_bounds__(TT *RY, 6)
+__global__ void __launch_bounds__(TT *RY, 3)
     combine_t_kernel(const float *Ukh, const float *Ukl, const float *U0h, const float *U0l,
                      const float *Dx, const float *DyT, float *Uoh, float *Uol, float *UT, int nx,
                      int ny, long long ncell, int stage, float ihx, float ihy, float gg1,
@@ -535,7 +551,7 @@ __global__ void __launch_bounds__(TT *RY, 6)
 // batched problems: one block per tile of a problem, each problem at its
 // offset in every buffer, with its own grid and control block
 template <int NV, int RY>
-__global__ void __launch_bounds__(TT *RY, 6)
+__global__ void __launch_bounds__(TT *RY, 3)
     combine_tb_kernel(const float *Ukh, const float *Ukl, const float *U0h, const float *U0l,
                       const float *Dx, const float *DyT, float *Uoh, float *Uol, float *UT,
                       long long nvals_all, const TileRef *tiles, const ProbDesc *probs, int stage,
@@ -614,21 +630,21 @@ __global__ void noalloc_nan_fill(double *L, long long n, const Ctl *ctl) {
     L[i] = __longlong_as_double(0x7ff8000000000000ll);
 }
 
+// one line of a batch on the host: problem and line index inside it
+struct LineRef {
+  int prob, line;
+};
+
 // a batched launch group: lines of equal cluster size and boundary kind
 struct LineGroup {
   int R;
+  int m;                      // rows per thread chunk
   bool periodic;
   bool xdir;
   bool trans = false;         // y lines as rows of the transposed planes (mixed 2-D batches)
-  LineRef *lines = nullptr;   // device: problem and line (the characteristic kernels)
-  LineDesc *descs = nullptr;  // device: the same lines resolved (the line kernels)
+  LineDesc *descs = nullptr;  // device
   long long nlines = 0;
-  // characteristic-wise batches: the longest line of the group and the
-  // group's own row and block-solve scratch (groups of a direction run
-  // concurrently)
-  int nmax = 0;
-  void *cscr = nullptr, *crows = nullptr;
-  mutable int char_layout = -1;   // FP32 block-solve layout, timed at the first step
+  int nmax = 0;               // the longest line
 };
 
 struct pp_cweno_s {
@@ -659,21 +675,15 @@ struct pp_cweno_s {
   // cap): stage 3 writes the stage buffer, a commit kernel copies it over
   // U^n where the step was accepted
   bool fcheck = false;
-  // characteristic-wise reconstruction (single problem): U^- and U^+ planes
-  // of the current sweep direction and the block solver's scratch, in the
-  // line arithmetic (FP64, or FP32 for the mixed form)
-  void *UMP = nullptr, *cscr = nullptr, *crows = nullptr;
-  // mixed 2-D: the y direction's own planes and scratch, so that the y
-  // reconstruction (which reads only the stage input) runs on a side stream
-  // beside the x reconstruction and sweep: two sets of serial block walks
-  // in flight instead of one
-  void *UMPy = nullptr, *cscry = nullptr, *crowsy = nullptr;
+  // characteristic-wise reconstruction: U^- and U^+ planes of the current
+  // sweep direction in the line arithmetic (FP64, or FP32 for the mixed form)
+  void *UMP = nullptr;
+  // mixed 2-D: the y direction's own planes, so that the y reconstruction
+  // (which reads only the stage input) runs on a side stream beside the x
+  // reconstruction and sweep
+  void *UMPy = nullptr;
   cudaStream_t ystream = nullptr;
   cudaEvent_t yfork = nullptr, yjoin = nullptr;
-  // FP32 block-solve layout per direction (one thread or four lanes per
-  // walk), timed on the handle's own state at the first step; -1 until then
-  mutable int char_layout[2] = {-1, -1};
-  bool char_tuning = false;
   // per-kernel profiling: called after each reconstruction launch, so that
   // the reconstruction and the line kernel get separate events
   std::function<void()> mark_hook;
@@ -718,7 +728,31 @@ double bits_to_double(unsigned long long b) {
   return d;
 }
 
-int seg_count(long long n) { return (int)((n + SEG_CELLS - 1) / SEG_CELLS); }
+#ifndef PPK_CM
+#define PPK_CM 16
+#endif
+constexpr int MAX_CTAS = 16;   // CTAs (one cluster) per line
+
+// CTAs per line of n cells with M-row thread chunks
+int seg_count(long long n, int m) { return (int)((n + seg_cells(m) - 1) / seg_cells(m)); }
+
+// Rows per thread chunk of a launch of nlines lines of n cells: the handle's
+// choice (8 or 16), 16 where 8 would need more than 16 CTAs per line, halved
+// while one CTA still holds the line (fewer idle lanes) or while every CTA of
+// the launch gets an SM of its own (few lines: a line's FP64 work is bound by
+// the FP64 pipe of the SMs it runs on; GB300 has 152).
+int pick_m(int m, long long n, long long nlines) {
+#ifdef PPK_FORCE_M
+  m = PPK_FORCE_M;
+#endif
+  if (seg_count(n, m) > MAX_CTAS) m = 16;
+  while (m > 2) {
+    const int r = seg_count(n, m / 2);
+    if (r > 1 && (r > MAX_CTAS || nlines * r > 152)) break;
+    m /= 2;
+  }
+  return m;
+}
 
 bool bc_valid(int b) { return b == PP_BC_PERIODIC || b == PP_BC_TRANSMISSIVE || b == PP_BC_REFLECTIVE; }
 
@@ -739,7 +773,8 @@ int check_config(const pp_cweno_config *c) {
   if ((c->bc[0] == PP_BC_PERIODIC) != (c->bc[1] == PP_BC_PERIODIC)) return PP_ERR_ARG;
   if (c->ndim == 2 && (c->bc[2] == PP_BC_PERIODIC) != (c->bc[3] == PP_BC_PERIODIC)) return PP_ERR_ARG;
   // one line per cluster of at most 16 CTAs
-  if (seg_count(c->nx) > 16 || (c->ndim == 2 && seg_count(c->ny) > 16)) return PP_ERR_UNSUPPORTED;
+  if (seg_count(c->nx, 16) > MAX_CTAS || (c->ndim == 2 && seg_count(c->ny, 16) > MAX_CTAS))
+    return PP_ERR_UNSUPPORTED;
   return PP_OK;
 }
 
@@ -783,14 +818,14 @@ void fill_state(const pp_cweno_s *h, SweepArgs &a, const void *Uin, const void *
   }
 }
 
-cudaError_t dispatch(const pp_cweno_s *h, int mode, const SweepArgs &a,
-                     long long nlines, bool attrs_only, cudaStream_t st_override = nullptr) {
+cudaError_t dispatch(const pp_cweno_s *h, int mode, const SweepArgs &a, long long nlines, int m,
+                     cudaStream_t st_override = nullptr) {
   LaunchCfg c;
   c.precision = h->cfg.precision;
   c.nv = h->nv;
   c.mode = mode;
-  c.attrs_only = attrs_only;
-  c.m = h->m;
+  c.attrs_only = false;
+  c.m = m;
   SweepArgs b = a;
   b.ih = a.h > 0.0 ? 1.0 / a.h : 0.0;   // batched launches take it per problem
   b.ih_other = a.h_other > 0.0 ? 1.0 / a.h_other : 0.0;
@@ -804,42 +839,46 @@ cudaError_t dispatch(const pp_cweno_s *h, int mode, const SweepArgs &a,
   return launch_sweep(c, b, nlines, st_override ? st_override : h->stream);
 }
 
+// kernel attributes (dynamic shared memory, cluster size) of every line
+// kernel of a precision and dimension; never inside a stream capture
+cudaError_t set_sweep_attrs(int precision, int nv) {
+  const int modes[3] = {MODE_XSWEEP, MODE_FINAL, MODE_OPERATOR};
+  SweepArgs a;
+  memset(&a, 0, sizeof(a));
+  a.R = 1;
+  LaunchCfg c;
+  c.precision = precision;
+  c.nv = nv;
+  c.attrs_only = true;
+  for (c.m = 2; c.m <= 16; c.m *= 2)
+    for (int k = 0; k < 3; ++k) {
+      c.mode = modes[k];
+      if (nv == 3 && c.mode == MODE_XSWEEP) continue;
+      if (nv == 4 && c.mode == MODE_FINAL && precision == PP_PREC_MIXED) continue;
+      cudaError_t e = launch_sweep(c, a, 0, nullptr);
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
+}
+
+// Chunk length and CTAs per line and side of the characteristic solve: 16
+// rows, the fewest joins per row (2048^2 FP32: 1.64 ms per direction, 1.68 with
+// 12, 1.74 with 8); 8 for four FP64 fields, whose multipliers would fill the
+// shared memory of an SM with one warp; halved while every one-warp CTA still
+// gets an SM of its own (few lines: the chain of a chunk's rows is the cost).
+void char_layout(CharArgs &c, int nv, bool mixed) {
+  auto ctas = [&](int m) { return (c.n + 32 * m - 1) / (32 * m); };
+  int m = PPK_CM;
+  if (nv == 4 && !mixed && ctas(8) <= MAX_CTAS) m = 8;
+  while (m > 1 && ctas(m / 2) <= MAX_CTAS && 2 * c.nlines * ctas(m / 2) <= 152) m /= 2;
+  c.M = m;
+  c.R = ctas(m);
+}
+
 // Characteristic-wise handles: the face values of the sweep described by a
 // (line geometry, boundaries) from the planes U in the line arithmetic, into
 // the handle's U^- / U^+ planes (Sec. 2.3); the line kernel then limits them
 // and forms the fluxes and the update.  Nothing to do for other handles.
-// Autotuner of the FP32 block solve: with the rows of c computed, time the
-// solve in both layouts (one thread per walk, four lanes per walk; CUDA
-// events on the stream, the first launch of each a warm-up) and keep the
-// faster in *layout.  The solve writes only the face-value planes and its
-// scratch, which the step recomputes.
-cudaError_t pick_char_layout(CharArgs c, int nv, bool per, cudaStream_t st, int *layout) {
-  cudaError_t e = launch_char_recon_f32(c, nv, per, 0, st);
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (e == cudaSuccess) e = cudaEventCreate(&e0);
-  if (e == cudaSuccess) e = cudaEventCreate(&e1);
-  float best = 1e30f;
-  int best_l = 0;
-  for (int l = 0; l < 2 && e == cudaSuccess; ++l) {
-    c.layout = l;
-    float t_min = 1e30f;
-    for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {
-      e = cudaEventRecord(e0, st);
-      if (e == cudaSuccess) e = launch_char_recon_f32(c, nv, per, 1, st);
-      if (e == cudaSuccess) e = cudaEventRecord(e1, st);
-      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-      float t = 0.f;
-      if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
-      if (rep > 0 && t < t_min) t_min = t;
-    }
-    if (t_min < best) { best = t_min; best_l = l; }
-  }
-  if (e0) cudaEventDestroy(e0);
-  if (e1) cudaEventDestroy(e1);
-  if (e == cudaSuccess) *layout = best_l;
-  return e;
-}
-
 cudaError_t launch_char(const pp_cweno_s *h, const SweepArgs &a, const void *U, long long nlines,
                         cudaStream_t st = nullptr) {
   if (h->cfg.recon != PP_RECON_CHARACTERISTIC) return cudaSuccess;
@@ -848,9 +887,6 @@ cudaError_t launch_char(const pp_cweno_s *h, const SweepArgs &a, const void *U, 
   c.U = U;
   c.Um = const_cast<void *>(a.Fm_pre);
   c.Up = const_cast<void *>(a.Fp_pre);
-  const bool ybuf = h->UMPy && a.Fm_pre == h->UMPy;   // the y direction's own scratch
-  c.scr = ybuf ? h->cscry : h->cscr;
-  c.rows = ybuf ? h->crowsy : h->crows;
   c.ncell = h->ncell;
   c.nlines = nlines;
   c.cell_stride = a.cell_stride;
@@ -862,16 +898,10 @@ cudaError_t launch_char(const pp_cweno_s *h, const SweepArgs &a, const void *U, 
   c.bchi = a.bchi;
   c.gamma = h->cfg.gamma;
   c.eps_weno = h->cfg.eps_weno;
-  const bool per = a.bclo == PP_BC_PERIODIC;
-  cudaError_t e = cudaSuccess;
-  if (h->char_tuning && is_mixed(h))
-    e = pick_char_layout(c, h->nv, per, st ? st : h->stream, &h->char_layout[ybuf ? 1 : 0]);
-  c.layout = h->char_layout[ybuf ? 1 : 0];
-  for (int part = 0; part < 2 && e == cudaSuccess; ++part) {
-    e = is_mixed(h) ? launch_char_recon_f32(c, h->nv, per, part, st ? st : h->stream)
-                    : launch_char_recon_f64(c, h->nv, per, part, st ? st : h->stream);
-    if (e == cudaSuccess && h->mark_hook && !st) h->mark_hook();
-  }
+  char_layout(c, h->nv, is_mixed(h));
+  cudaError_t e = is_mixed(h) ? launch_char_recon_f32(c, h->nv, st ? st : h->stream, false)
+                              : launch_char_recon_f64(c, h->nv, st ? st : h->stream, false);
+  if (e == cudaSuccess && h->mark_hook && !st) h->mark_hook();
   return e;
 }
 
@@ -893,24 +923,16 @@ cudaError_t launch_char_group(const pp_cweno_s *h, const LineGroup &g, const Swe
   c.U = U;
   c.Um = const_cast<void *>(a.Fm_pre);
   c.Up = const_cast<void *>(a.Fp_pre);
-  c.scr = g.cscr;
-  c.rows = g.crows;
   c.nlines = g.nlines;
   c.n = g.nmax;
   c.vn = a.vn;
   c.vt = a.vt;
   c.gamma = h->cfg.gamma;
   c.eps_weno = h->cfg.eps_weno;
-  c.lines = g.lines;
-  c.probs = h->probs;
-  c.xdir = g.xdir ? 1 : (g.trans ? 2 : 0);
-  cudaError_t e = cudaSuccess;
-  if (h->char_tuning && is_mixed(h)) e = pick_char_layout(c, h->nv, g.periodic, st, &g.char_layout);
-  c.layout = g.char_layout;
-  for (int part = 0; part < 2 && e == cudaSuccess; ++part)
-    e = is_mixed(h) ? launch_char_recon_f32(c, h->nv, g.periodic, part, st)
-                    : launch_char_recon_f64(c, h->nv, g.periodic, part, st);
-  return e;
+  c.lines = g.descs;
+  char_layout(c, h->nv, is_mixed(h));
+  return is_mixed(h) ? launch_char_recon_f32(c, h->nv, st, false)
+                     : launch_char_recon_f64(c, h->nv, st, false);
 }
 
 // Single-problem launch.  Uin, U0, Uout are state buffers (FP64 planes or
@@ -944,7 +966,6 @@ long long fill_geometry(const pp_cweno_s *h, SweepArgs &a, bool xdir) {
     a.h = h->dy;
     a.h_other = h->dx;
   }
-  a.R = seg_count(a.n);
   return nlines;
 }
 
@@ -952,8 +973,7 @@ long long fill_geometry(const pp_cweno_s *h, SweepArgs &a, bool xdir) {
 // already computed (on the side stream)
 cudaError_t launch(const pp_cweno_s *h, int mode, bool xdir, const void *Uin, const void *U0,
                    const void *Din, void *Dout, void *Uout, int stage, double eps_fixed,
-                   Ctl *ctl, bool attrs_only = false, double *Lout = nullptr,
-                   bool char_done = false) {
+                   Ctl *ctl, double *Lout = nullptr, bool char_done = false) {
   SweepArgs a;
   memset(&a, 0, sizeof(a));
   fill_state(h, a, Uin, U0, Uout);
@@ -962,27 +982,27 @@ cudaError_t launch(const pp_cweno_s *h, int mode, bool xdir, const void *Uin, co
   a.Dout = Dout;
   a.Lout = Lout;
   const long long nlines = fill_geometry(h, a, xdir);
+  const int m = pick_m(h->m, a.n, nlines);
+  a.R = seg_count(a.n, m);
   if (!xdir) use_y_planes(h, a);
-  if (!attrs_only && !char_done) {
+  if (!char_done) {
     cudaError_t e = launch_char(h, a, is_mixed(h) ? (const void *)a.Uh : (const void *)a.U, nlines);
     if (e != cudaSuccess) return e;
   }
-  return dispatch(h, mode, a, nlines, attrs_only);
+  return dispatch(h, mode, a, nlines, m);
 }
 
 // Batched launch of one line group.  eps_fixed > 0 with ctl: a measurement
 // launch (the autotuner's) that reduces into a scratch control block array.
 cudaError_t launch_group(const pp_cweno_s *h, const LineGroup &g, int mode, const void *Uin,
                          const void *U0, const void *Din, void *Dout, void *Uout, int stage,
-                         bool attrs_only = false, double eps_fixed = 0.0, Ctl *ctl = nullptr,
-                         double *Lout = nullptr, cudaStream_t st = nullptr) {
+                         cudaStream_t st) {
   SweepArgs a;
   memset(&a, 0, sizeof(a));
   fill_state(h, a, Uin, U0, Uout);
-  fill_common(h, a, stage, eps_fixed, ctl ? ctl : h->ctl);
+  fill_common(h, a, stage, 0.0, h->ctl);
   a.Din = Din;
   a.Dout = Dout;
-  a.Lout = Lout;
   a.R = g.R;
   a.lines = g.descs;
   if (g.trans) {   // rows of the transposed hi planes in, D_y transposed out
@@ -995,12 +1015,12 @@ cudaError_t launch_group(const pp_cweno_s *h, const LineGroup &g, int mode, cons
   a.vn = g.xdir ? 1 : 2;
   a.vt = h->nv == 4 ? (g.xdir ? 2 : 1) : -1;
   a.fdir = g.xdir ? 0 : 1;
-  if (!attrs_only && h->cfg.recon == PP_RECON_CHARACTERISTIC) {
+  if (h->cfg.recon == PP_RECON_CHARACTERISTIC) {
     cudaError_t e = launch_char_group(h, g, a, is_mixed(h) ? (const void *)a.Uh : (const void *)a.U,
                                       st ? st : h->stream);
     if (e != cudaSuccess) return e;
   }
-  return dispatch(h, mode, a, g.nlines, attrs_only, st);
+  return dispatch(h, mode, a, g.nlines, g.m, st);
 }
 
 // y sweep of the mixed 2-D form over the transposed hi planes: a row sweep
@@ -1024,12 +1044,13 @@ cudaError_t launch_ysweep_t(const pp_cweno_s *h, int stage, bool char_done = fal
   a.h = h->dy;
   a.h_other = h->dx;
   a.fdir = 1;
-  a.R = seg_count(a.n);
+  const int m = pick_m(h->m, a.n, h->nx);
+  a.R = seg_count(a.n, m);
   if (!char_done) {
     cudaError_t e = launch_char(h, a, h->UT, h->nx);   // rows of the transposed planes
     if (e != cudaSuccess) return e;
   }
-  return dispatch(h, MODE_XSWEEP, a, h->nx, false);
+  return dispatch(h, MODE_XSWEEP, a, h->nx, m);
 }
 
 // the y direction's characteristic-wise face values of the stage input on
@@ -1152,7 +1173,7 @@ cudaError_t launch_groups(const pp_cweno_s *h, bool xdir, int mode, const void *
     cudaStream_t st = h->gstreams[i];
     e = cudaStreamWaitEvent(st, h->fork_ev, 0);
     if (e == cudaSuccess)
-      e = launch_group(h, g, mode, Uin, h->U0, Din, Dout, Uout, stage, false, 0.0, nullptr, nullptr, st);
+      e = launch_group(h, g, mode, Uin, h->U0, Din, Dout, Uout, stage, st);
     if (e == cudaSuccess) e = cudaEventRecord(h->gevents[i], st);
     ++used;
   }
@@ -1207,8 +1228,8 @@ cudaError_t enqueue_step_body(pp_cweno_s *h, cudaEvent_t *ev, int *nev) {
         mark();
         if (e == cudaSuccess && yside) e = cudaStreamWaitEvent(h->stream, h->yjoin, 0);
         if (e != cudaSuccess) return e;
-        e = launch(h, MODE_FINAL, false, Uin, h->U0, h->D, nullptr, Uout, s, 0.0, h->ctl, false,
-                   nullptr, yside);
+        e = launch(h, MODE_FINAL, false, Uin, h->U0, h->D, nullptr, Uout, s, 0.0, h->ctl, nullptr,
+                   yside);
         mark();
       } else {
         e = launch(h, MODE_FINAL, true, Uin, h->U0, nullptr, nullptr, Uout, s, 0.0, h->ctl);
@@ -1357,32 +1378,16 @@ int finish_create(pp_cweno_s *h) {
   // difference form reads both)
   if (e == cudaSuccess && tr) e = cudaMalloc(&h->UT, 2 * sizeof(float) * (size_t)nvals(h));
   if (e == cudaSuccess && tr) e = cudaMalloc(&h->DT, sizeof(float) * (size_t)nvals(h));
-  if (e == cudaSuccess && h->cfg.recon == PP_RECON_CHARACTERISTIC && h->batch) {
+  if (e == cudaSuccess && h->cfg.recon == PP_RECON_CHARACTERISTIC) {
     const size_t es = is_mixed(h) ? sizeof(float) : sizeof(double);
     e = cudaMalloc(&h->UMP, 2 * es * (size_t)nvals(h));
-    for (LineGroup &g : h->groups) {
-      if (e != cudaSuccess) break;
-      e = cudaMalloc(&g.cscr, es * (size_t)char_scratch_values(h->nv, g.periodic, g.nmax, g.nlines));
-      if (e == cudaSuccess) e = cudaMalloc(&g.crows, es * (size_t)char_rows_values(h->nv, g.nmax, g.nlines));
-    }
-  } else if (e == cudaSuccess && h->cfg.recon == PP_RECON_CHARACTERISTIC) {
-    const size_t es = is_mixed(h) ? sizeof(float) : sizeof(double);
-    e = cudaMalloc(&h->UMP, 2 * es * (size_t)nvals(h));
-    const long long sx = char_scratch_values(h->nv, h->cfg.bc[0] == PP_BC_PERIODIC, h->nx, h->ny);
-    const long long sy = h->nv == 4 ? char_scratch_values(h->nv, h->cfg.bc[2] == PP_BC_PERIODIC, h->ny, h->nx) : 0;
-    const long long rx = char_rows_values(h->nv, h->nx, h->ny);
-    const long long ry = h->nv == 4 ? char_rows_values(h->nv, h->ny, h->nx) : 0;
-    // the mixed 2-D form gives the y direction its own planes, scratch and
-    // stream (measured: 27.9 against 30.5 ms per 4096^2 step); in FP64 the
-    // two directions' kernels share the FP64 pipe and gain nothing (647
-    // against 581 ms), so the directions share one scratch and run in turn
-    const bool ysep = h->nv == 4 && is_mixed(h);
-    if (e == cudaSuccess) e = cudaMalloc(&h->cscr, es * (size_t)(ysep ? sx : std::max(sx, sy)));
-    if (e == cudaSuccess) e = cudaMalloc(&h->crows, es * (size_t)(ysep ? rx : std::max(rx, ry)));
-    if (ysep) {
+    CharArgs c;
+    memset(&c, 0, sizeof(c));
+    if (e == cudaSuccess)
+      e = is_mixed(h) ? launch_char_recon_f32(c, h->nv, nullptr, true)
+                      : launch_char_recon_f64(c, h->nv, nullptr, true);
+    if (h->nv == 4 && is_mixed(h) && !h->batch) {
       if (e == cudaSuccess) e = cudaMalloc(&h->UMPy, 2 * es * (size_t)nvals(h));
-      if (e == cudaSuccess) e = cudaMalloc(&h->cscry, es * (size_t)sy);
-      if (e == cudaSuccess) e = cudaMalloc(&h->crowsy, es * (size_t)ry);
       if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->ystream, cudaStreamNonBlocking);
       if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->yfork, cudaEventDisableTiming);
       if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->yjoin, cudaEventDisableTiming);
@@ -1390,30 +1395,15 @@ int finish_create(pp_cweno_s *h) {
   }
   if (e != cudaSuccess) return PP_ERR_CUDA;
   memset(h->hctl, 0, sizeof(Ctl) * h->nprob);
-  // kernel attributes (dynamic shared memory, cluster size) are set here,
-  // never inside a stream capture
-  const int modes[3] = {MODE_XSWEEP, MODE_FINAL, MODE_OPERATOR};
-  const int keep_m = h->m;
-  for (int mm = 8; mm <= 16 && e == cudaSuccess; mm += 8) {
-    h->m = mm;
-    for (int m = 0; m < 3 && e == cudaSuccess; ++m) {
-      if (h->nv == 3 && modes[m] == MODE_XSWEEP) continue;
-      SweepArgs a;
-      memset(&a, 0, sizeof(a));
-      a.R = 1;
-      e = dispatch(h, modes[m], a, 0, true);
-    }
-  }
-  h->m = keep_m;
-  if (e != cudaSuccess) return PP_ERR_CUDA;
+  if (set_sweep_attrs(h->cfg.precision, h->nv) != cudaSuccess) return PP_ERR_CUDA;
   if (h->batch) {
     h->launches_per_step = 1;
-    const long long per_group = h->cfg.recon == PP_RECON_CHARACTERISTIC ? 3 : 1;
+    const long long per_group = h->cfg.recon == PP_RECON_CHARACTERISTIC ? 2 : 1;
     for (int s = 0; s < 3; ++s)
       h->launches_per_step += per_group * (long long)h->groups.size() + (h->btrans ? 1 : 0);
   } else {
     const int sweeps = h->nv == 4 ? 2 : 1;
-    const int chars = h->cfg.recon == PP_RECON_CHARACTERISTIC ? 2 * sweeps : 0;
+    const int chars = h->cfg.recon == PP_RECON_CHARACTERISTIC ? sweeps : 0;
     h->launches_per_step = 1 + 3 * ((h->ytrans ? 3 : sweeps) + chars);
   }
   if (h->fcheck) h->launches_per_step += 2;
@@ -1437,89 +1427,13 @@ struct TuneKey {
 std::mutex g_tune_mu;
 std::vector<std::pair<TuneKey, int>> g_tune_cache;
 
-// Batches: the same choice, timed on one sweep over every x-line group of
-// the batch (the y groups run the same kernel), reducing into the scratch
-// control blocks and writing only scratch (the x-sweep output, or the stage
-// buffer as operator output).  Batches are not cached: their line mix is
-// their own.
-int autotune_batch(pp_cweno_s *h) {
-  if (h->cfg.recon == PP_RECON_CHARACTERISTIC) {   // its line kernels have no elimination to tune
-    h->m = 8;
-    if (!is_mixed(h)) return PP_OK;
-    // the block-solve layout of every line group, on the batch's own state
-    h->char_tuning = true;
-    cudaError_t e = cudaSuccess;
-    for (const LineGroup &g : h->groups) {
-      if (e != cudaSuccess) break;
-      SweepArgs a;
-      memset(&a, 0, sizeof(a));
-      fill_state(h, a, h->U0, h->U0, nullptr);
-      fill_common(h, a, 0, 1e-13, h->ctl_scratch);
-      a.vn = g.xdir ? 1 : 2;
-      a.vt = h->nv == 4 ? (g.xdir ? 2 : 1) : -1;
-      e = launch_char_group(h, g, a, g.trans ? (const void *)h->UT : (const void *)a.Uh, h->stream);
-    }
-    h->char_tuning = false;
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    return e == cudaSuccess ? PP_OK : PP_ERR_CUDA;
-  }
-  std::vector<Ctl> z((size_t)h->nprob);
-  memset(z.data(), 0, sizeof(Ctl) * z.size());
-  if (cudaMemcpyAsync(h->ctl_scratch, z.data(), sizeof(Ctl) * z.size(), cudaMemcpyHostToDevice,
-                      h->stream) != cudaSuccess)
-    return PP_ERR_CUDA;
-  cudaEvent_t e0, e1;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return PP_ERR_CUDA;
-  float best = 1e30f;
-  int best_m = 8;
-  cudaError_t e = cudaSuccess;
-  for (int mm = 8; mm <= 16 && e == cudaSuccess; mm += 8) {
-    h->m = mm;
-    float t_min = 1e30f;
-    for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {
-      cudaEventRecord(e0, h->stream);
-      for (const LineGroup &g : h->groups) {
-        if (!g.xdir || e != cudaSuccess) continue;
-        if (h->nv == 4)
-          e = launch_group(h, g, MODE_XSWEEP, h->U0, h->U0, nullptr, h->D, nullptr, 0, false, 1e-13,
-                           h->ctl_scratch);
-        else
-          e = launch_group(h, g, MODE_OPERATOR, h->U0, h->U0, nullptr, nullptr, nullptr, 0, false,
-                           1e-13, h->ctl_scratch, reinterpret_cast<double *>(h->U1));
-      }
-      cudaEventRecord(e1, h->stream);
-      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-      float t = 0.f;
-      if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
-      if (rep > 0 && t < t_min) t_min = t;   // first launch is a warm-up
-    }
-    if (t_min < best) { best = t_min; best_m = mm; }
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  h->m = best_m;
-  return e == cudaSuccess ? PP_OK : PP_ERR_CUDA;
-}
-
 int autotune(pp_cweno_s *h) {
   if (h->tuned) return PP_OK;
   h->tuned = true;
-  if (h->batch) return autotune_batch(h);
-  if (h->cfg.recon == PP_RECON_CHARACTERISTIC && is_mixed(h)) {
-    // the block-solve layout of each direction, on the handle's own state
-    // (the reconstruction writes only its planes and scratch)
-    pp_cweno_s *hm = h;
-    hm->char_tuning = true;
-    SweepArgs a;
-    memset(&a, 0, sizeof(a));
-    fill_state(h, a, h->U0, h->U0, nullptr);
-    fill_common(h, a, 0, 1e-13, h->ctl_scratch);
-    const long long nl = fill_geometry(h, a, true);
-    cudaError_t e = launch_char(h, a, a.Uh, nl);
-    if (e == cudaSuccess && h->nv == 4) e = launch_char_y(h, h->U0, h->stream);
-    hm->char_tuning = false;
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return PP_ERR_CUDA;
+  if (h->batch) {   // every line group has its own (pick_m); the longest is reported
+    h->m = 8;
+    for (const LineGroup &g : h->groups) h->m = std::max(h->m, g.m);
+    return PP_OK;
   }
   TuneKey key{h->cfg.precision, h->nv == 4 ? 2 : 1, h->nx, h->ny, h->cfg.bc[0] == PP_BC_PERIODIC};
   {
@@ -1547,7 +1461,7 @@ int autotune(pp_cweno_s *h) {
                    h->ctl_scratch);
       else
         e = launch(h, MODE_OPERATOR, true, h->U0, h->U0, nullptr, nullptr, nullptr, 0, 1e-13,
-                   h->ctl_scratch, false, reinterpret_cast<double *>(h->U1));
+                   h->ctl_scratch, reinterpret_cast<double *>(h->U1));
       cudaEventRecord(e1, h->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float t = 0.f;
@@ -1642,13 +1556,17 @@ int pp_cweno_create_batch(const pp_cweno_config *cfgs, int64_t nprob, void *cuda
   h->btrans = c0.precision == PP_PREC_MIXED && c0.ndim == 2;
   std::vector<TileRef> tiles;
   long long off = 0, cells = 0;
-  // line groups keyed by (direction, cluster size, periodic)
+  // line groups keyed by (direction, chunk length, cluster size, periodic)
   std::vector<std::vector<LineRef>> glines;
-  auto group_of = [&](bool xdir, int R, bool per) -> size_t {
+  auto group_of = [&](bool xdir, int n, bool per) -> size_t {
+    const int m = pick_m(16, n, 1 << 20), R = seg_count(n, m);
     for (size_t g = 0; g < h->groups.size(); ++g)
-      if (h->groups[g].xdir == xdir && h->groups[g].R == R && h->groups[g].periodic == per) return g;
+      if (h->groups[g].xdir == xdir && h->groups[g].m == m && h->groups[g].R == R &&
+          h->groups[g].periodic == per)
+        return g;
     LineGroup lg;
     lg.R = R;
+    lg.m = m;
     lg.periodic = per;
     lg.xdir = xdir;
     lg.trans = !xdir && h->btrans;
@@ -1673,10 +1591,10 @@ int pp_cweno_create_batch(const pp_cweno_config *cfgs, int64_t nprob, void *cuda
     h->probs_h.push_back(d);
     off += (long long)h->nv * d.ncell;
     cells += d.ncell;
-    size_t gx = group_of(true, seg_count(d.nx), c.bc[0] == PP_BC_PERIODIC);
+    size_t gx = group_of(true, d.nx, c.bc[0] == PP_BC_PERIODIC);
     for (int j = 0; j < d.ny; ++j) glines[gx].push_back({p, j});
     if (c.ndim == 2) {
-      size_t gy = group_of(false, seg_count(d.ny), c.bc[2] == PP_BC_PERIODIC);
+      size_t gy = group_of(false, d.ny, c.bc[2] == PP_BC_PERIODIC);
       for (int i = 0; i < d.nx; ++i) glines[gy].push_back({p, i});
       if (h->btrans)
         for (int j0 = 0; j0 < d.ny; j0 += TT)
@@ -1690,8 +1608,9 @@ int pp_cweno_create_batch(const pp_cweno_config *cfgs, int64_t nprob, void *cuda
   std::vector<size_t> order(h->groups.size());
   for (size_t g = 0; g < order.size(); ++g) order[g] = g;
   std::sort(order.begin(), order.end(), [&](size_t a, size_t b) {
-    if (h->groups[a].xdir != h->groups[b].xdir) return h->groups[a].xdir;
-    return h->groups[a].R > h->groups[b].R;
+    const LineGroup &p = h->groups[a], &q = h->groups[b];
+    if (p.xdir != q.xdir) return p.xdir;
+    return p.R * p.m > q.R * q.m;
   });
   std::vector<LineGroup> sorted;
   std::vector<std::vector<LineRef>> slines;
@@ -1744,11 +1663,6 @@ int pp_cweno_create_batch(const pp_cweno_config *cfgs, int64_t nprob, void *cuda
     e = cudaMalloc(&h->groups[g].descs, sizeof(LineDesc) * descs.size());
     if (e == cudaSuccess)
       e = cudaMemcpy(h->groups[g].descs, descs.data(), sizeof(LineDesc) * descs.size(),
-                     cudaMemcpyHostToDevice);
-    if (e != cudaSuccess || c0.recon != PP_RECON_CHARACTERISTIC) continue;
-    e = cudaMalloc(&h->groups[g].lines, sizeof(LineRef) * slines[g].size());
-    if (e == cudaSuccess)
-      e = cudaMemcpy(h->groups[g].lines, slines[g].data(), sizeof(LineRef) * slines[g].size(),
                      cudaMemcpyHostToDevice);
   }
   if (e == cudaSuccess && h->btrans) {
@@ -1998,10 +1912,10 @@ int pp_cweno_operator(pp_cweno_t h, const double *U_dev, double *L_dev, double e
     e = launch(h, MODE_XSWEEP, true, Uin, Uin, nullptr, h->D, nullptr, 0, eps, h->ctl_scratch);
     if (e == cudaSuccess)
       e = launch(h, MODE_OPERATOR, false, Uin, Uin, h->D, nullptr, nullptr, 0, eps, h->ctl_scratch,
-                 false, L_dev);
+                 L_dev);
   } else {
     e = launch(h, MODE_OPERATOR, true, Uin, Uin, nullptr, nullptr, nullptr, 0, eps, h->ctl_scratch,
-               false, L_dev);
+               L_dev);
   }
   if (e != cudaSuccess) return PP_ERR_CUDA;
   return cuerr(cudaStreamSynchronize(h->stream));
@@ -2191,20 +2105,8 @@ int pp_cweno_operator_noalloc(const pp_cweno_config *cfg, const double *U_dev, d
     if (!g_noalloc_ready[dev]) {
       void *ptr = nullptr;
       if (cudaGetSymbolAddress(&ptr, g_noalloc_scratch) != cudaSuccess || !ptr) return PP_ERR_CUDA;
-      const int modes[3] = {MODE_XSWEEP, MODE_FINAL, MODE_OPERATOR};
-      for (int ndim = 1; ndim <= 2; ++ndim) {
-        pp_cweno_s t;
-        t.cfg = *cfg;
-        t.cfg.precision = PP_PREC_FP64;
-        t.nv = ndim == 2 ? 4 : 3;
-        for (int m = 0; m < 3; ++m) {
-          if (t.nv == 3 && modes[m] == MODE_XSWEEP) continue;
-          SweepArgs a;
-          memset(&a, 0, sizeof(a));
-          a.R = 1;
-          if (dispatch(&t, modes[m], a, 0, true) != cudaSuccess) return PP_ERR_CUDA;
-        }
-      }
+      for (int k = 3; k <= 4; ++k)
+        if (set_sweep_attrs(PP_PREC_FP64, k) != cudaSuccess) return PP_ERR_CUDA;
       g_noalloc_ptr[dev] = ptr;
       g_noalloc_ready[dev] = true;
     }
@@ -2224,11 +2126,11 @@ int pp_cweno_operator_noalloc(const pp_cweno_config *cfg, const double *U_dev, d
   if (nv == 4) {
     e = launch(&h, MODE_XSWEEP, true, U_dev, U_dev, nullptr, D, nullptr, 0, 0.0, ctl);
     if (e == cudaSuccess)
-      e = launch(&h, MODE_OPERATOR, false, U_dev, U_dev, D, nullptr, nullptr, 0, 0.0, ctl, false,
+      e = launch(&h, MODE_OPERATOR, false, U_dev, U_dev, D, nullptr, nullptr, 0, 0.0, ctl,
                  L_dev);
   } else {
     e = launch(&h, MODE_OPERATOR, true, U_dev, U_dev, nullptr, nullptr, nullptr, 0, 0.0, ctl,
-               false, L_dev);
+               L_dev);
   }
   return cuerr(e);
 }
@@ -2246,19 +2148,12 @@ int pp_cweno_destroy(pp_cweno_t h) {
   cudaFree(h->UT);
   cudaFree(h->DT);
   cudaFree(h->UMP);
-  cudaFree(h->cscr);
-  cudaFree(h->crows);
   cudaFree(h->UMPy);
-  cudaFree(h->cscry);
-  cudaFree(h->crowsy);
   if (h->ystream) cudaStreamDestroy(h->ystream);
   if (h->yfork) cudaEventDestroy(h->yfork);
   if (h->yjoin) cudaEventDestroy(h->yjoin);
   for (auto &g : h->groups) {
-    cudaFree(g.lines);
     cudaFree(g.descs);
-    cudaFree(g.cscr);
-    cudaFree(g.crows);
   }
   for (cudaStream_t st : h->gstreams) cudaStreamDestroy(st);
   for (cudaEvent_t ev : h->gevents) cudaEventDestroy(ev);

@@ -8,14 +8,19 @@
 
 namespace ppk {
 
-constexpr int SEG_CELLS = 512;    // cells per CTA of a line's cluster
-
-// thread layout by chunk length: 512 cells per CTA, one warp per variable at
-// M = 16 and two at M = 8, and the resident CTAs per SM asked for
-template <typename real, int M>
+// Thread layout by chunk length M: a warp per variable, 32 chunks, 32 M cells
+// per CTA and at most 16 CTAs (a cluster) per line; and the resident CTAs per
+// SM asked for.
+constexpr int seg_cells(int m) { return 32 * m; }
+#ifndef PPK_C8
+#define PPK_C8 6
+#define PPK_C16 4
+#define PPK_D8 3
+#endif
+template <typename real, int NV, int M>
 struct Layout {
-  static constexpr int KC = SEG_CELLS / M;
-  static constexpr int CTAS = sizeof(real) == 4 ? (M == 8 ? 3 : 4) : (M == 8 ? 1 : 2);
+  static constexpr int KC = 32;
+  static constexpr int CTAS = sizeof(real) == 4 ? (M == 8 ? PPK_C8 : PPK_C16) : (M == 8 ? PPK_D8 : 2);
 };
 
 struct LaunchCfg {
@@ -23,35 +28,39 @@ struct LaunchCfg {
   int nv;          // 3 or 4
   int mode;        // MODE_*
   bool attrs_only; // set the kernel's attributes, launch nothing
-  int m;           // rows per thread chunk: 8 or 16 (picked by the autotuner)
+  int m;           // rows per thread chunk: 2, 4, 8 or 16
 };
 
 // Launch one sweep over nlines lines with R CTAs per line (cluster of R);
-// one entry per (precision, chunk length), each in its own translation unit.
+// one entry per (precision, chunk length), in its own translation unit except
+// the two short ones.
+cudaError_t launch_sweep_f64_short(const LaunchCfg &c, const SweepArgs &a, long long nlines,
+                                   cudaStream_t st);
 cudaError_t launch_sweep_f64_m8(const LaunchCfg &c, const SweepArgs &a, long long nlines,
                                 cudaStream_t st);
 cudaError_t launch_sweep_f64_m16(const LaunchCfg &c, const SweepArgs &a, long long nlines,
                                  cudaStream_t st);
+cudaError_t launch_sweep_f32_short(const LaunchCfg &c, const SweepArgs &a, long long nlines,
+                                   cudaStream_t st);
 cudaError_t launch_sweep_f32_m8(const LaunchCfg &c, const SweepArgs &a, long long nlines,
                                 cudaStream_t st);
 cudaError_t launch_sweep_f32_m16(const LaunchCfg &c, const SweepArgs &a, long long nlines,
                                  cudaStream_t st);
 
-// Launches with face values from another kernel (a.Fm_pre) use the M = 8
-// thread layout: their kernels contain no elimination for M to tune.
 inline cudaError_t launch_sweep(const LaunchCfg &c, const SweepArgs &a, long long nlines,
                                 cudaStream_t st) {
-  const bool m16 = c.m == 16 && !a.Fm_pre;
-  if (c.precision == 0) return m16 ? launch_sweep_f64_m16(c, a, nlines, st)
-                                   : launch_sweep_f64_m8(c, a, nlines, st);
-  return m16 ? launch_sweep_f32_m16(c, a, nlines, st) : launch_sweep_f32_m8(c, a, nlines, st);
+  if (c.precision == 0)
+    return c.m == 16 ? launch_sweep_f64_m16(c, a, nlines, st)
+         : c.m == 8 ? launch_sweep_f64_m8(c, a, nlines, st) : launch_sweep_f64_short(c, a, nlines, st);
+  return c.m == 16 ? launch_sweep_f32_m16(c, a, nlines, st)
+       : c.m == 8 ? launch_sweep_f32_m8(c, a, nlines, st) : launch_sweep_f32_short(c, a, nlines, st);
 }
 
 template <typename real, int NV, int M, int MODE, bool PRE>
 cudaError_t launch_m(const SweepArgs &a, long long nlines, cudaStream_t st, bool attrs_only) {
-  constexpr int KC = Layout<real, M>::KC;
+  constexpr int KC = Layout<real, NV, M>::KC;
   using S = Smem<real, NV, M, KC>;
-  auto kern = line_sweep<real, NV, M, KC, MODE, PRE, Layout<real, M>::CTAS>;
+  auto kern = line_sweep<real, NV, M, KC, MODE, PRE, Layout<real, NV, M>::CTAS>;
   if (attrs_only) {   // called at handle creation, outside any stream capture
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)S::bytes);
@@ -78,17 +87,14 @@ cudaError_t launch_m(const SweepArgs &a, long long nlines, cudaStream_t st, bool
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-// the reconstructing kernel, or (M = 8 only) the one taking precomputed
-// face values; attrs_only sets the attributes of both
+// the reconstructing kernel, or the one taking precomputed face values; attrs_only sets the attributes of both
 template <typename real, int NV, int M, int MODE>
 cudaError_t launch_pre(const LaunchCfg &c, const SweepArgs &a, long long nlines, cudaStream_t st) {
-  if constexpr (M == 8) {
-    if (c.attrs_only) {
-      cudaError_t e = launch_m<real, NV, M, MODE, true>(a, nlines, st, true);
-      if (e != cudaSuccess) return e;
-    } else if (a.Fm_pre) {
-      return launch_m<real, NV, M, MODE, true>(a, nlines, st, false);
-    }
+  if (c.attrs_only) {
+    cudaError_t e = launch_m<real, NV, M, MODE, true>(a, nlines, st, true);
+    if (e != cudaSuccess) return e;
+  } else if (a.Fm_pre) {
+    return launch_m<real, NV, M, MODE, true>(a, nlines, st, false);
   }
   return launch_m<real, NV, M, MODE, false>(a, nlines, st, c.attrs_only);
 }
@@ -106,8 +112,9 @@ cudaError_t launch_dispatch(const LaunchCfg &c, const SweepArgs &a, long long nl
   if (c.nv == 4) {
     if (c.mode == MODE_XSWEEP)
       return launch_pre<real, 4, M, MODE_XSWEEP>(c, a, nlines, st);
-    if (c.mode == MODE_FINAL)
-      return launch_pre<real, 4, M, MODE_FINAL>(c, a, nlines, st);
+    if constexpr (sizeof(real) == 8) {   // (the mixed form combines its two sweeps separately)
+      if (c.mode == MODE_FINAL) return launch_pre<real, 4, M, MODE_FINAL>(c, a, nlines, st);
+    }
     if (c.mode == MODE_OPERATOR)
       return launch_pre<real, 4, M, MODE_OPERATOR>(c, a, nlines, st);
   }
