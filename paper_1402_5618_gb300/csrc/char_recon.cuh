@@ -44,9 +44,16 @@ struct CharArgs {
   int vn, vt;               // grid index of the normal / tangential momentum (vt < 0 in 1-D)
   int bclo, bchi;
   int M, R;                 // rows per chunk, one-warp CTAs per line and side (n <= 32 M R)
+  void *scr;                // multipliers, char_scratch_values() values of the line's type, or
+                            // nullptr: in shared memory
   double gamma, eps_weno;
   const LineDesc *lines;    // batched launch: the group's lines (nullptr: one problem)
 };
+
+// scratch values: per row of every chunk the blocks Y and F and the vector g
+inline long long char_scratch_values(const CharArgs &a, int nv) {
+  return a.nlines * 2 * a.R * 32 * a.M * (2 * nv * nv + nv);
+}
 
 // one entry per precision, each in its own translation unit (the FP32 one
 // is compiled with the mixed form's fast division and square root);

@@ -38,33 +38,43 @@ __device__ __forceinline__ void roe_scalars(const real *Ua, const real *Ub, real
   rs[3] = g1 * ia2;
 }
 
-// rows l^(k) of L (eqs. (eigen), (leigenv)), ordered by the eigenvalues
-// u - a, u, (u,) u + a; in 2-D the third row is the shear field
-// (-v, 0, 1, 0) and v enters the acoustic rows through |u|^2 and -c1 v / 2
+// The rows l^(k) of L (eqs. (eigen), (leigenv)), ordered by the eigenvalues
+// u - a, u, (u,) u + a, with c1 = (gamma - 1)/a^2 and c2 = c1 |u|^2 / 2: the
+// acoustic rows are h + d and h - d, the entropy row e_0 - 2 h and in 2-D the
+// shear row (-v, 0, 1, 0), with h = (c2, -c1 u, [-c1 v,] c1)/2 and d = (u, -1,
+// [0,] 0)/(2 a).  L x from the two inner products takes 10 operations in 2-D.
 template <typename real, int NV>
-__device__ __forceinline__ void left_from(const real (&rs)[4], real (&L)[NV][NV]) {
-  const real one = real(1), half = real(0.5);
-  const real u = rs[0], v = rs[1], ia = rs[2], c1 = rs[3];
-  const real c2 = half * (u * u + v * v) * c1;
-  L[0][0] = half * (c2 + u * ia);
-  L[0][1] = -half * (c1 * u + ia);
-  L[0][NV - 1] = half * c1;
-  L[1][0] = one - c2;
-  L[1][1] = c1 * u;
-  L[1][NV - 1] = -c1;
-  L[NV - 1][0] = half * (c2 - u * ia);
-  L[NV - 1][1] = half * (ia - c1 * u);
-  L[NV - 1][NV - 1] = half * c1;
-  if constexpr (NV == 4) {
-    L[0][2] = -half * c1 * v;
-    L[1][2] = c1 * v;
-    L[3][2] = -half * c1 * v;
-    L[2][0] = -v;
-    L[2][1] = real(0);
-    L[2][2] = one;
-    L[2][3] = real(0);
+struct LeftEig {
+  real h[NV], d0, d1, v;
+  __device__ __forceinline__ explicit LeftEig(const real (&rs)[4]) {
+    const real half = real(0.5), hc = half * rs[3];
+    h[0] = half * (rs[0] * rs[0] + rs[1] * rs[1]) * hc;
+    h[1] = -hc * rs[0];
+    if (NV == 4) h[2] = -hc * rs[1];
+    h[NV - 1] = hc;
+    d1 = -half * rs[2];
+    d0 = -d1 * rs[0];
+    v = rs[1];
   }
-}
+  __device__ __forceinline__ void mul(const real (&x)[NV], real (&y)[NV]) const {
+    real H = h[0] * x[0];
+#pragma unroll
+    for (int m = 1; m < NV; ++m) H += h[m] * x[m];
+    const real D = d0 * x[0] + d1 * x[1];
+    y[0] = H + D;
+    y[1] = x[0] - real(2) * H;
+    if (NV == 4) y[2] = x[2] - v * x[0];
+    y[NV - 1] = H - D;
+  }
+  // entry (k, m) with k, m known at compile time
+  __device__ __forceinline__ real at(int k, int m) const {
+    const real d = m == 0 ? d0 : (m == 1 ? d1 : real(0));
+    if (k == 0) return h[m] + d;
+    if (k == NV - 1) return h[m] - d;
+    if (k == 1) return (m == 0 ? real(1) : real(0)) - real(2) * h[m];
+    return m == 0 ? -v : (m == 2 ? real(1) : real(0));
+  }
+};
 
 // |a| > |b| for a pivot search; FP64 by the high words (an FP64 comparison
 // takes a slot of the FP64 pipe; a pivot within 2^-20 of the largest is as good)
@@ -399,15 +409,19 @@ __device__ __forceinline__ void char_row(const real (&win)[5][NV], real gamma, r
                                          bool closure, real (&rs)[4], real (&ca)[NV],
                                          real (&cc)[NV], real (&s)[NV]) {
   constexpr bool F32 = sizeof(real) == 4;
-  real L[NV][NV];
   roe_scalars<real, NV>(win[2], win[3], gamma, rs);
-  left_from<real, NV>(rs, L);
-  real dU[4][NV], top[NV];
+  const LeftEig<real, NV> L(rs);
+  real dW[4][NV], top[NV];
 #pragma unroll
-  for (int m = 0; m < NV; ++m) {
+  for (int w = 0; w < 4; ++w) {
+    real dU[NV];
 #pragma unroll
-    for (int w = 0; w < 4; ++w) dU[w][m] = win[w + 1][m] - win[w][m];
-    if (F32) {
+    for (int m = 0; m < NV; ++m) dU[m] = win[w + 1][m] - win[w][m];
+    L.mul(dU, dW[w]);
+  }
+  if (F32) {
+#pragma unroll
+    for (int m = 0; m < NV; ++m) {
       top[m] = fabs(win[0][m]);
 #pragma unroll
       for (int w = 1; w < 5; ++w) top[m] = fmax(top[m], fabs(win[w][m]));
@@ -417,12 +431,7 @@ __device__ __forceinline__ void char_row(const real (&win)[5][NV], real gamma, r
   for (int k = 0; k < NV; ++k) {
     real D[4], mag = real(0);
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      real t = L[k][0] * dU[w][0];
-#pragma unroll
-      for (int m = 1; m < NV; ++m) t += L[k][m] * dU[w][m];
-      D[w] = t;
-    }
+    for (int w = 0; w < 4; ++w) D[w] = dW[w][k];
     const real k43 = real(4.0 / 3.0);
     const real g0 = D[1] - D[0], g1 = D[2] - D[1], g2 = D[3] - D[2];
     real e = eps;
@@ -430,7 +439,7 @@ __device__ __forceinline__ void char_row(const real (&win)[5][NV], real gamma, r
       // the rounding floor of the indicators on the size of the terms the
       // characteristic variable is summed from
 #pragma unroll
-      for (int m = 0; m < NV; ++m) mag += fabsf(L[k][m]) * top[m];
+      for (int m = 0; m < NV; ++m) mag += fabsf(L.at(k, m)) * top[m];
       e = fmaf(FP32_BETA_FLOOR * mag, mag, eps);
     }
     const real d0 = fma(k43 * g0, g0, e) + D[1] * (D[1] + g0);
@@ -455,13 +464,19 @@ __device__ __forceinline__ void char_row(const real (&win)[5][NV], real gamma, r
 
 // ---------------------------------------------------------------- kernel
 // One warp per (segment of 32 M cells, side); lane k holds the M cells of
-// chunk k; a cluster of R CTAs covers the line.  Shared memory: per row of
-// every lane the multipliers Y, F and g (x = g - F X_in - Y x_next).
+// chunk k; a cluster of R CTAs covers the line.  Kept per row of every lane
+// until the back substitution: the multipliers Y, F and g (x = g - F X_in - Y
+// x_next), in shared memory or, with many lines, in global scratch.
 template <typename real, int NV>
 struct CharSmem {
-  static constexpr int E = 2 * NV * NV + NV;
-  End<real, NV> seg[2];   // this segment's first and last unknown
-  static size_t bytes(int M) { return sizeof(End<real, NV>) * 2 + sizeof(real) * 32 * E * (size_t)M; }
+  static constexpr int E = 2 * NV * NV + NV;   // multipliers of a row
+  static constexpr int RC = 4 + 3 * NV;        // numbers of a row before its elimination
+  // this segment's first and last unknown, then per lane and row the
+  // multipliers, or only the row's numbers (scratch: the multipliers go to
+  // global memory)
+  static size_t bytes(int M, bool scratch) {
+    return sizeof(End<real, NV>) * 2 + sizeof(real) * 32 * (scratch ? RC : E) * (size_t)M;
+  }
 };
 
 template <typename real, int NV>
@@ -485,18 +500,43 @@ __global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
 #pragma unroll
   for (int k = 0; k < NV; ++k) gv[k] = k == 0 ? 0 : (k == NV - 1 ? NV - 1 : (k == 1 ? a.vn : a.vt));
   const real gam = real(a.gamma), eps = real(a.eps_weno);
-  // entry e of row t of this lane
-  auto at = [&](int t, int e) -> real & { return rows[((long long)t * E + e) * 32 + lane]; };
+  // a row's numbers, and its multipliers over them or in the scratch
+  const int RS = a.scr ? CharSmem<real, NV>::RC : E;
+  real *mult = rows;
+  if (a.scr)
+    mult = reinterpret_cast<real *>(a.scr) +
+           ((long long)blockIdx.y * gridDim.x + blockIdx.x) * ((long long)32 * E * M);
+  auto at = [&](int t, int e) -> real & { return rows[(t * RS + e) * 32 + lane]; };
+  auto mt = [&](int t, int e) -> real & { return mult[(t * E + e) * 32 + lane]; };
 
   // The chunk's rows first, their 4 + 3 NV numbers into the slots the
   // multipliers take later: two loops whose bodies stay in the instruction
   // caches instead of one that does not (the SM runs few warps of this kernel).
-  {
-    real win[5][NV], nxt[NV];
-    if (cnt > 0) {
+  // The cells come in with consecutive lanes on consecutive cells, each into
+  // its row's slots (read as a stencil cell before the row overwrites them);
+  // the two cells on either side of a chunk are a lane's own.
+  const int len = min(32 * M, n - lo);   // (<= 0: no cells)
+#pragma unroll 4
+  for (int c = lane; c < len; c += 32) {
+    const int ch = c / M, j = c - ch * M;
+    const int t = side == 0 ? j : min(M, len - ch * M) - 1 - j;
+    const long long o = geo.base + (long long)(lo + c) * geo.cs;
 #pragma unroll
-      for (int w = 0; w < 4; ++w) line_cell<real, NV>(geo, U, gv, first + (w - 2) * dir, win[w + 1]);
-      line_cell<real, NV>(geo, U, gv, first + 2 * dir, nxt);
+    for (int k = 0; k < NV; ++k) rows[(t * RS + k) * 32 + ch] = __ldg(U + o + gv[k] * geo.ncell);
+  }
+  __syncwarp();
+  {
+    real win[5][NV], after[2][NV];
+    if (cnt > 0) {
+      line_cell<real, NV>(geo, U, gv, first - 2 * dir, win[1]);
+      line_cell<real, NV>(geo, U, gv, first - dir, win[2]);
+      line_cell<real, NV>(geo, U, gv, first + cnt * dir, after[0]);
+      line_cell<real, NV>(geo, U, gv, first + (cnt + 1) * dir, after[1]);
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        win[3][k] = at(0, k);
+        win[4][k] = cnt > 1 ? at(1, k) : after[0][k];
+      }
     }
 #pragma unroll 1
     for (int t = 0; t < cnt; ++t) {
@@ -506,8 +546,8 @@ __global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) win[w][k] = win[w + 1][k];
 #pragma unroll
-      for (int k = 0; k < NV; ++k) win[4][k] = nxt[k];
-      if (t + 1 < cnt) line_cell<real, NV>(geo, U, gv, c + 3 * dir, nxt);
+      for (int k = 0; k < NV; ++k)
+        win[4][k] = t + 2 < cnt ? at(min(t + 2, M - 1), k) : (t + 2 == cnt ? after[0][k] : after[1][k]);
       real rs[4], ca[NV], cc[NV], s[NV];
       char_row<real, NV>(win, gam, eps, !per && (c == 0 || c == n - 1), rs, ca, cc, s);
 #pragma unroll
@@ -527,9 +567,8 @@ __global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
   end_empty(L);
 #pragma unroll 1
   for (int t = 0; t < cnt; ++t) {
-    real Lk[NV][NV], ca[NV], cc[NV], s[NV];
+    real ca[NV], cc[NV], s[NV], rs[4];
     {
-      real rs[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) rs[i] = at(t, i);
 #pragma unroll
@@ -538,40 +577,45 @@ __global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
         cc[i] = at(t, 4 + NV + i);
         s[i] = at(t, 4 + 2 * NV + i);
       }
-      left_from<real, NV>(rs, Lk);
     }
+    const LeftEig<real, NV> Lk(rs);
     // (L - diag(a) L Y) [Y' | g' | F'] = [diag(c) L | s - diag(a) L g | -diag(a) L F]
     real B[NV][NV], X[NV][2 * NV + 1];
+    {
+      real tg[NV];
+      Lk.mul(L.a, tg);
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      real tg = real(0);
+      for (int i = 0; i < NV; ++i) X[i][NV] = s[i] - ca[i] * tg[i];
+    }
 #pragma unroll
-      for (int m = 0; m < NV; ++m) tg += Lk[i][m] * L.a[m];
-      X[i][NV] = s[i] - ca[i] * tg;
+    for (int j = 0; j < NV; ++j) {
+      real y[NV], f[NV], ty[NV], tf[NV];
 #pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        real ty = real(0), tf = real(0);
+      for (int m = 0; m < NV; ++m) {
+        y[m] = L.B[m][j];
+        f[m] = L.G[m][j];
+      }
+      Lk.mul(y, ty);
+      Lk.mul(f, tf);
 #pragma unroll
-        for (int m = 0; m < NV; ++m) {
-          ty += Lk[i][m] * L.B[m][j];
-          tf += Lk[i][m] * L.G[m][j];
-        }
-        B[i][j] = Lk[i][j] - ca[i] * ty;
-        X[i][j] = cc[i] * Lk[i][j];
-        X[i][NV + 1 + j] = -(ca[i] * tf);
+      for (int i = 0; i < NV; ++i) {
+        const real l = Lk.at(i, j);
+        B[i][j] = l - ca[i] * ty[i];
+        X[i][j] = cc[i] * l;
+        X[i][NV + 1 + j] = -(ca[i] * tf[i]);
       }
     }
     gauss_solve<real, NV, 2 * NV + 1>(B, X);
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
       L.a[i] = X[i][NV];
-      at(t, i) = X[i][NV];
+      mt(t, i) = X[i][NV];
 #pragma unroll
       for (int j = 0; j < NV; ++j) {
         L.B[i][j] = X[i][j];
         L.G[i][j] = X[i][NV + 1 + j];
-        at(t, NV + i * NV + j) = X[i][j];
-        at(t, NV + NV * NV + i * NV + j) = X[i][NV + 1 + j];
+        mt(t, NV + i * NV + j) = X[i][j];
+        mt(t, NV + NV * NV + i * NV + j) = X[i][NV + 1 + j];
       }
     }
     // first = a - B X_in - G x_p with x_p = g - F X_in - Y x_{p+1}
@@ -650,17 +694,34 @@ __global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
     block_down(side == 0 ? up : !up, st[h], xl, xr);
   }
 
-  // back substitution; the deviations overwrite g
+  // back substitution, the multipliers of the two rows before the current one
+  // loading meanwhile; the deviations go where the row's numbers were
+  real nx[2][E];
+#pragma unroll
+  for (int d = 0; d < 2; ++d)
+    if (cnt > d) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) nx[d][e] = mt(cnt - 1 - d, e);
+    }
 #pragma unroll 1
   for (int t = cnt - 1; t >= 0; --t) {
-    real x[NV];
+    real m[E], x[NV];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      m[e] = nx[0][e];
+      nx[0][e] = nx[1][e];
+    }
+    if (t > 1) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) nx[1][e] = mt(t - 2, e);
+    }
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      real p = at(t, i);
+      real p = m[i];
 #pragma unroll
-      for (int m = 0; m < NV; ++m) {
-        p -= at(t, NV + NV * NV + i * NV + m) * xl[m];
-        p -= at(t, NV + i * NV + m) * xr[m];
+      for (int j = 0; j < NV; ++j) {
+        p -= m[NV + NV * NV + i * NV + j] * xl[j];
+        p -= m[NV + i * NV + j] * xr[j];
       }
       x[i] = p;
     }
@@ -673,14 +734,14 @@ __global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
   __syncwarp();
   // out: consecutive lanes on consecutive cells
   real *out = reinterpret_cast<real *>(side == 0 ? a.Um : a.Up);
-  const int len = min(32 * M, n - lo);
+#pragma unroll 4
   for (int c = lane; c < len; c += 32) {
     const int ch = c / M, j = c - ch * M;
     const int t = side == 0 ? j : min(M, len - ch * M) - 1 - j;
     const long long o = geo.base + (long long)(lo + c) * geo.cs;
 #pragma unroll
     for (int k = 0; k < NV; ++k)
-      out[o + gv[k] * geo.ncell] = U[o + gv[k] * geo.ncell] + rows[((long long)t * E + k) * 32 + ch];
+      out[o + gv[k] * geo.ncell] = __ldg(U + o + gv[k] * geo.ncell) + rows[(t * RS + k) * 32 + ch];
   }
   if (R > 1) cluster_wait();
 }
@@ -691,7 +752,7 @@ cudaError_t launch_nv(const CharArgs &a, cudaStream_t st, bool attrs_only) {
   if (attrs_only) {
     // (M = 16 rows per chunk at most)
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)CharSmem<real, NV>::bytes(16));
+                                         (int)CharSmem<real, NV>::bytes(16, false));
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                (int)cudaSharedmemCarveoutMaxShared);
@@ -702,7 +763,7 @@ cudaError_t launch_nv(const CharArgs &a, cudaStream_t st, bool attrs_only) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.nlines * a.R), 2, 1);
   cfg.blockDim = dim3(32, 1, 1);
-  cfg.dynamicSmemBytes = CharSmem<real, NV>::bytes(a.M);
+  cfg.dynamicSmemBytes = CharSmem<real, NV>::bytes(a.M, a.scr != nullptr);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -376,6 +376,65 @@ __device__ __forceinline__ void chunk_back(const real *u, real *dm, const real *
   }
 }
 
+// The same elimination of one system alone (SIDE 0 minus, 1 plus), d and f to
+// its two planes: a warp per side where a launch waits for its FP64
+// instructions one after another (short chunks).
+template <int SIDE, int M>
+__device__ __forceinline__ void side_eliminate(const double (&D)[M + 3], const double (&S0)[M],
+                                               const double (&S1)[M], const double (&S2)[M],
+                                               const EdgeInfo e, double *dd, double *ff,
+                                               double (&cs)[M - 1], Run<double> &r) {
+  double c = 0.0, d = 0.0, f = -1.0, A = 0.0, B = 0.0, G = -1.0;
+#pragma unroll
+  for (int j = 0; j < M; ++j) {
+    constexpr int L = M - 1;
+    const int jc = SIDE ? L - j : j, i = e.i0 + jc;
+    const double s0 = SIDE ? S2[jc] : S0[jc], s1 = S1[jc], s2 = SIDE ? S0[jc] : S2[jc];
+    // differences in walk order: before the previous cell, previous, next, after
+    const double e0 = SIDE ? -D[jc + 3] : D[jc], em = SIDE ? -D[jc + 2] : D[jc + 1];
+    const double ep = SIDE ? -D[jc + 1] : D[jc + 2], e3 = SIDE ? -D[jc] : D[jc + 3];
+    const double t2 = 2.5 * s1, t4 = 1.25 * s1;
+    double a = fma(2.0, s0, t2), b = fma(3.0, s2, fma(2.0, t2, s0)), cc = 1.5 * s2;
+    double s = fma(ep, fma(2.25, s2, t4), em * fma(1.5, s0, t2));
+    if (!e.periodic && (i == 0 || i == e.n - 1)) {   // closure
+      const double a0 = 0.1 * s0, a1 = 0.6 * s1, a2 = 0.3 * s2;
+      a = cc = 0.0;
+      b = 6.0 * (a0 + a1 + a2);
+      s = a0 * (5.0 * em - 2.0 * e0) + a1 * (em + 2.0 * ep) + a2 * (4.0 * ep - e3);
+    }
+    if (i < e.n) {
+      if (!(j == 0 || (SIDE && i == e.n - 1))) {
+        A = fma(-G, d, A);
+        B = fma(-G, f, B);
+        G = -(G * c);
+      }
+      const double inv = rcp(fma(-a, c, b));
+      d = fma(-a, d, s) * inv;
+      f = -(a * f) * inv;
+      c = cc * inv;
+    }
+    if (j < L) {
+      dd[jc] = d;
+      ff[jc] = f;
+      cs[j] = c;
+    }
+  }
+  r.A = A; r.B = B; r.G = G; r.D = d; r.F = f; r.C = c;
+}
+
+template <int SIDE, int M>
+__device__ __forceinline__ void side_back(const double *u, double *dd, const double *ff,
+                                          const double (&cs)[M - 1], double xin, double x, int len) {
+  dd[SIDE ? 0 : M - 1] = u[SIDE ? 0 : M - 1] + x;
+#pragma unroll
+  for (int j = M - 2; j >= 0; --j) {
+    const int jc = SIDE ? M - 1 - j : j;
+    const double y = fma(-cs[j], x, fma(-ff[jc], xin, dd[jc]));
+    x = SIDE || jc + 1 < len ? y : x;   // the minus system of a ragged chunk starts at its last cell
+    dd[jc] = u[jc] + x;
+  }
+}
+
 // ---------------------------------------------------------------- trees
 // Runs of the lanes of a warp joined by a butterfly: 5 levels of a few dozen
 // instructions on every warp and no barrier.  The way of the FP32 form, and of

@@ -33,6 +33,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "batch_lines.cuh"
 #include "compact_solve.cuh"
 #include "dfloat.cuh"
@@ -178,6 +180,10 @@ struct Smem {
   // compact_solve.cuh), or by LPS lanes of one warp per system, eight each
   static constexpr bool TREE = sizeof(real) == 4 || M <= 4;
   static constexpr int LPS = KC / 8;
+  // FP64 with short chunks: a warp per variable and side (a warp's FP64
+  // instructions take 64 cycles each, and these launches wait for them)
+  static constexpr int SIDES = sizeof(real) == 8 && M <= 4 ? 2 : 1;
+  static constexpr int THREADS = NV * KC * SIDES;
   static constexpr int PSH = sizeof(real) == 4 ? 5 : 4;
   __host__ __device__ static constexpr int pad(int c) { return c + (c >> PSH); }
   static constexpr int UH = 3;                         // pad(-2) = -3
@@ -238,11 +244,11 @@ __device__ __forceinline__ void atomic_min_bits(unsigned long long *w, unsigned 
 // PRE: the face values come from another kernel (args.Fm_pre / Fp_pre) and
 // the reconstruction phases are compiled out.
 template <typename real, int NV, int M, int KC, int MODE, bool PRE, int CTAS>
-__global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
+__global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_sweep(SweepArgs args_in) {
   constexpr bool MIXED = sizeof(real) == 4;
   using S = Smem<real, NV, M, KC>;
   constexpr int SEG = S::SEG;
-  constexpr int T = NV * KC;
+  constexpr int T = S::THREADS;
   constexpr int UH = S::UH, UWP = S::UWP, WP = S::WP, FH = S::FH, FWP = S::FWP, FLS = S::FLS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   real *Us = reinterpret_cast<real *>(smem_raw + S::u_off);
@@ -260,7 +266,8 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
   const int lo = rank * SEG;
   const int hi = min(lo + SEG, n);
   const int tid = threadIdx.x;
-  const int v = tid / KC;
+  const int v = tid / KC % NV;
+  const int sidew = tid / (NV * KC);   // (SIDES == 2: the system this warp solves)
   const int k = tid % KC;
   const int lane = tid & 31;
   const bool per = args.bclo == 0;
@@ -364,7 +371,8 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
   // the extra cell of this thread: segment cell cx, or none (k >= 7 or past a tail)
   const int cx = k < 2 ? k - 2 : (k < 4 ? len + k - 2 : 4 * nq + k - 4);
   const bool extra = k < 4 || (vec && k < 7 && cx < len);
-  if (extra) {
+  const bool loads = S::SIDES == 1 || sidew == 0;
+  if (loads && extra) {
     const int i = lo + cx;
     bool neg = false;
     long long a = (long long)i * cs;
@@ -387,7 +395,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
         }
       }
     }
-  } else if (cs == 1) {
+  } else if (loads && cs == 1) {
     const real *s1 = src + lo + k;
     const float *s2 = MIXED && two ? srl + lo + k : nullptr;
 #pragma unroll
@@ -397,7 +405,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
         if constexpr (MIXED) lv[q] = two ? s2[q * KC] : 0.0f;
       }
     }
-  } else {
+  } else if (loads) {
     const long long step = KC * cs;
     long long a = (lo + k) * cs;
 #pragma unroll
@@ -486,7 +494,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
       ex.rp[3] = E + pr;
     }
   }
-  {
+  if (loads) {
     real *dst = Us + v * UWP + UH;
     float rh = 0.0f, rl = 0.0f;
     if (dlt) { rh = ex.rh[v]; rl = ex.rl[v]; }
@@ -554,6 +562,83 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
     constexpr bool TREE = S::TREE;
     using P = typename Pair<real>::t;
     P cs[M - 1];
+    if constexpr (S::SIDES == 2) {
+      auto solve = [&](auto side_c) {
+        constexpr int SD = decltype(side_c)::value;
+        real *dd = (SD ? Fp : Fm) + v * FWP + FH, *ff = (SD ? Zp : Zm) + v * WP + cb;
+        double c1[M - 1];
+        Run<real> r = run_empty<real>();
+        if (wlive) {
+          real D[M + 3], S0[M], S1[M], S2[M], win[M + 4];
+          win[0] = uv[S::pad(k * M - 2)];
+          win[1] = uv[S::pad(k * M - 1)];
+#pragma unroll
+          for (int q = 0; q < M; ++q) win[q + 2] = uv[cb + q];
+          win[M + 2] = uv[S::pad(k * M + M)];
+          win[M + 3] = uv[S::pad(k * M + M + 1)];
+          chunk_weights<real, M>(win, eps_v, D, S0, S1, S2);
+          side_eliminate<SD, M>(D, S0, S1, S2, {lo + k * M, n, per}, dd + cb, ff, c1, r);
+        }
+        Ends<real> F, L;
+        if (lo + k * M < n) {
+          L.a = r.D; L.b = r.C; L.g = r.F;
+          F.a = fma(-r.G, L.a, r.A);
+          F.b = fma(-r.G, L.g, r.B);
+          F.g = -r.G * L.b;
+        } else {
+          F.a = F.b = L.a = L.b = real(0);
+          F.g = L.g = real(-1);
+        }
+        const Ends<real> own = L;
+        Step<real> st[5];
+#pragma unroll
+        for (int h = 0; h < 5; ++h) {
+          const bool up = lane & (1 << h);
+          tree_up(1 << h, SD ? !up : up, false, real(1), F, L, st[h]);
+        }
+        real xl = real(0), xr = real(0);
+        if (R > 1) {
+          if (lane == 0) {
+            Run<real> &a = ex.seg[2 * v + SD];
+            a.A = F.a; a.B = F.b; a.G = F.g; a.D = L.a; a.C = L.b; a.F = L.g;
+          }
+          cluster.sync();
+          const int q = lane & 15;
+          Run<real> o = run_empty<real>();
+          if (q < R) o = cluster.map_shared_rank(&ex, SD ? R - 1 - q : q)->seg[2 * v + SD];
+          F.a = o.A; F.b = o.B; F.g = o.G;
+          L.a = o.D; L.b = o.C; L.g = o.F;
+          Step<real> sg[4];
+#pragma unroll
+          for (int h = 0; h < 4; ++h)
+            if ((1 << h) < R) tree_up(1 << h, (q & (1 << h)) != 0, false, real(1), F, L, sg[h]);
+          if (per) ring_close(F, L, xl, xr);
+#pragma unroll
+          for (int h = 3; h >= 0; --h)
+            if ((1 << h) < R) tree_down((q & (1 << h)) != 0, false, sg[h], xl, xr);
+          const int at = SD ? R - 1 - rank : rank;
+          xl = __shfl_sync(0xffffffffu, xl, at);
+          xr = __shfl_sync(0xffffffffu, xr, at);
+        } else if (per) {
+          ring_close(F, L, xl, xr);
+        }
+#pragma unroll
+        for (int h = 4; h >= 0; --h) {
+          const bool up = lane & (1 << h);
+          tree_down(SD ? !up : up, false, st[h], xl, xr);
+        }
+        if (wlive) {
+          const real xo = fma(-own.b, xr, fma(-own.g, xl, own.a));
+          side_back<SD, M>(uv + cb, dd + cb, ff, c1, xl, xo, n - (lo + k * M));
+          __syncwarp();
+          // the cells next to the segment (below)
+          if (k == 0 && (lo > 0 || per)) dd[S::pad(-1)] = uv[S::pad(-1)] + (SD ? xr : xl);
+          if (k == (len - 1) / M && (hi < n || per)) dd[S::pad(len)] = uv[S::pad(len)] + (SD ? xl : xr);
+        }
+      };
+      if (sidew) solve(std::integral_constant<int, 1>());
+      else solve(std::integral_constant<int, 0>());
+    } else {
     Run<real> rm = run_empty<real>(), rp = run_empty<real>();
     if (wlive) {
       {
@@ -672,9 +757,12 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
     // any is the empty run.
     constexpr int LPS = S::LPS;
     constexpr int NCOMB = (2 * NV * LPS + 31) / 32 * 32;
-    const bool comb = tid < NCOMB;
-    const bool on = tid < 2 * NV * LPS;
-    const int sys = on ? tid / LPS : 0, cl = tid % LPS, sd = sys & 1;
+    // (which warps: in turn by CTA, as an FP64 instruction of a warp holds the
+    // FP64 unit of its SM quarter for 64 cycles, whatever the others do)
+    const int ct = (tid + T - (NCOMB == 32 ? (int)(blockIdx.x % NV) * 32 : 0)) % T;
+    const bool comb = ct < NCOMB;
+    const bool on = ct < 2 * NV * LPS;
+    const int sys = on ? ct / LPS : 0, cl = ct % LPS, sd = sys & 1;
     real Dt[7], Ft[7], Ct[7];
     Run<real> run = run_empty<real>(), seg;
     Cut<real> cut[3];
@@ -813,6 +901,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
         Fm[v * FWP + FH + S::pad(hi - lo)] = u + xafter.x;
         Fp[v * FWP + FH + S::pad(hi - lo)] = u + xin.y;
       }
+    }
     }
     // the neighbours read this CTA's run until here at the latest: arrive
     // now, wait before exit (shared memory must outlive their reads)
@@ -996,6 +1085,8 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
   // time on 16-byte boundaries
   int cdone = 0;
   if (MODE == MODE_XSWEEP && !mixedforms) {
+    cdone = len;
+    if (loads) {
     real *D = reinterpret_cast<real *>(args.Dout) + plane + lo * cs;
     const real *Fv = Fl + v * FLS;
     bool vst = false;
@@ -1018,7 +1109,7 @@ __global__ void __launch_bounds__(NV *KC, CTAS) line_sweep(SweepArgs args_in) {
     D += (c0 + k) * cs;
     const long long step = KC * cs;
     for (int c = c0 + k; c < len; c += KC, D += step) *D = (Fv[c] - Fv[c + 1]) * ih;
-    cdone = len;
+    }
   }
   if (MIXED && MODE == MODE_FINAL) cdone = len;
   for (int c = cdone + tid; c < len; c += T) {

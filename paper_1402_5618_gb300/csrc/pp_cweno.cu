@@ -113,6 +113,20 @@ __global__ void step_end_kernel(Ctl *ctls, int nprob) {
   if (++ctl->nrej_run > 60) ctl->err_rate = 1;
 }
 
+// whether a cell is in G, and its rate (|u| + a)/dx [+ (|v| + a)/dy]
+template <int NV>
+__device__ __forceinline__ bool cell_measure(double rho, double m1, double m2, double E, double gg1,
+                                             double idx, double idy, double &rate) {
+  const double ir = rcp(rho);
+  const double e = (E - 0.5 * (m1 * m1 + m2 * m2) * ir) * ir;
+  if (!(positive(rho) && positive(e) && is_finite(E) && is_finite(m1) && is_finite(m2) && is_finite(rho)))
+    return false;
+  const double a = root(gg1 * e);
+  rate = (fabs(m1) * ir + a) * idx;
+  if (NV == 4) rate += (fabs(m2) * ir + a) * idy;
+  return true;
+}
+
 // Reductions of a state: min density, max rate, cells outside G.  The state
 // is FP64 planes (lo == nullptr) or FP32 hi / lo plane pairs.  Blocks (x)
 // stride over the cells of one problem (y; probs == nullptr: the single one).
@@ -138,19 +152,15 @@ __global__ void __launch_bounds__(256)
   };
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nc;
        c += (long long)gridDim.x * blockDim.x) {
-    const double rho = at(c), m1 = at(nc + c), m2 = NV == 4 ? at(2 * nc + c) : 0.0;
-    const double E = at((NV - 1) * nc + c);
-    const double ir = rcp(rho);
-    const double e = (E - 0.5 * (m1 * m1 + m2 * m2) * ir) * ir;
-    if (!(positive(rho) && positive(e) && is_finite(E) && is_finite(m1) && is_finite(m2) && is_finite(rho))) {
+    const double rho = at(c);
+    double r;
+    if (!cell_measure<NV>(rho, at(nc + c), NV == 4 ? at(2 * nc + c) : 0.0, at((NV - 1) * nc + c), gg1,
+                          pd.idx, pd.idy, r)) {
       ++bad;
       first = (unsigned long long)c < first ? (unsigned long long)c : first;
       continue;
     }
     mn = less(rho, mn) ? rho : mn;
-    const double a = root(gg1 * e);
-    double r = (fabs(m1) * ir + a) * pd.idx;
-    if (NV == 4) r += (fabs(m2) * ir + a) * pd.idy;
     mx = less(mx, r) ? r : mx;
   }
   for (int d = 16; d > 0; d >>= 1) {
@@ -601,33 +611,87 @@ __global__ void fma_peak_kernel(T *out, int iters, T a, T b) {
 // lives for as long as the library is loaded, on every GPU that loads it.
 constexpr size_t NOALLOC_BYTES = size_t(32) << 20;   // 32 MiB
 constexpr size_t NOALLOC_CTL_BYTES = 256;
-static_assert(sizeof(Ctl) <= NOALLOC_CTL_BYTES, "control block must fit its slot");
+static_assert(sizeof(Ctl) <= NOALLOC_CTL_BYTES && sizeof(Ctl) % 8 == 0, "control block must fit its slot");
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
-// control block of a single operator evaluation: reductions reset, the
-// limiter epsilon min(eps_pos, min rho) taken from the preceding reduction
-// (or the caller's eps), active set
+// Control block of a single operator evaluation.  The limiter epsilon is the
+// caller's eps, or min(eps_pos, min rho) of a state inside G; on any other
+// state the operator is not evaluated (active = 0) and L gets NaN everywhere,
+// so the caller sees it in its own output.
+
+// where no grid-wide reduction is needed first: one block resets, reduces (eps
+// <= 0) and arms.  A 200-cell call waits for its launches: four small kernels
+// here were a fifth of its 43 us.
+template <int NV>
+__global__ void __launch_bounds__(1024)
+    noalloc_prepare(const double *U, double *L, long long nc, double gamma, double eps_pos,
+                    double eps, Ctl *ctl) {
+  __shared__ double smin[32];
+  __shared__ int sbad[32];
+  double mn = 1e300;
+  int bad = 0;
+  if (!(eps > 0.0)) {
+    const double gg1 = gamma * (gamma - 1.0);
+    for (long long c = threadIdx.x; c < nc; c += blockDim.x) {
+      const double rho = U[c];
+      double r;
+      if (cell_measure<NV>(rho, U[nc + c], NV == 4 ? U[2 * nc + c] : 0.0, U[(NV - 1) * nc + c], gg1, 1.0, 1.0, r))
+        mn = less(rho, mn) ? rho : mn;
+      else
+        bad = 1;
+    }
+    for (int d = 16; d > 0; d >>= 1) {
+      const double o = __shfl_down_sync(0xffffffffu, mn, d);
+      mn = less(o, mn) ? o : mn;
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    if ((threadIdx.x & 31) == 0) {
+      smin[threadIdx.x >> 5] = mn;
+      sbad[threadIdx.x >> 5] = bad;
+    }
+    __syncthreads();
+    mn = smin[0];
+    bad = sbad[0];
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) {
+      mn = less(smin[w], mn) ? smin[w] : mn;
+      bad |= sbad[w];
+    }
+  }
+  const double eps0 = eps > 0.0 ? eps : fmin(eps_pos, mn);
+  const bool active = !bad && eps0 > 0.0;
+  if (threadIdx.x == 0) {
+    unsigned char *b = reinterpret_cast<unsigned char *>(ctl);
+    for (size_t i = 0; i < sizeof(Ctl); i += 8) *reinterpret_cast<unsigned long long *>(b + i) = 0;
+    ctl->minrho[2] = dbits(mn);
+    ctl->nviol = bad;
+    ctl->first_bad = ~0ull;
+    ctl->eps0 = eps0;
+    ctl->active = active;
+  }
+  if (!active)
+    for (long long i = threadIdx.x; i < NV * nc; i += blockDim.x) L[i] = bitsd(0x7ff8000000000000ull);
+}
+
 __global__ void noalloc_ctl_reset(Ctl *ctl) {
   if (threadIdx.x != 0) return;
   unsigned char *b = reinterpret_cast<unsigned char *>(ctl);
-  for (size_t i = 0; i < sizeof(Ctl); ++i) b[i] = 0;
+  for (size_t i = 0; i < sizeof(Ctl); i += 8) *reinterpret_cast<unsigned long long *>(b + i) = 0;
   ctl->minrho[2] = 0x7ff0000000000000ull;
   ctl->first_bad = ~0ull;
 }
 
-__global__ void noalloc_ctl_arm(Ctl *ctl, double eps_pos, double eps) {
-  if (threadIdx.x != 0) return;
-  ctl->eps0 = eps > 0.0 ? eps : fmin(eps_pos, bitsd(ctl->minrho[2]));
-  ctl->active = ctl->nviol == 0 && ctl->eps0 > 0.0;
-}
-
-// a state the operator is not evaluated on (a cell outside G with eps <= 0)
-// gets L = NaN everywhere, so the caller sees it in its own output
-__global__ void noalloc_nan_fill(double *L, long long n, const Ctl *ctl) {
-  if (ctl->active) return;
+// after the grid-wide reduction
+__global__ void noalloc_arm(double *L, long long n, Ctl *ctl, double eps_pos) {
+  const double eps0 = fmin(eps_pos, bitsd(ctl->minrho[2]));
+  const bool active = ctl->nviol == 0 && eps0 > 0.0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    ctl->eps0 = eps0;
+    ctl->active = active;
+  }
+  if (active) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
-    L[i] = __longlong_as_double(0x7ff8000000000000ll);
+    L[i] = bitsd(0x7ff8000000000000ull);
 }
 
 // one line of a batch on the host: problem and line index inside it
@@ -645,6 +709,7 @@ struct LineGroup {
   LineDesc *descs = nullptr;  // device
   long long nlines = 0;
   int nmax = 0;               // the longest line
+  void *cscr = nullptr;       // characteristic solve: multipliers
 };
 
 struct pp_cweno_s {
@@ -682,6 +747,8 @@ struct pp_cweno_s {
   // (which reads only the stage input) runs on a side stream beside the x
   // reconstruction and sweep
   void *UMPy = nullptr;
+  // multipliers of the characteristic solve, x and (mixed 2-D) y direction
+  void *cscr = nullptr, *cscry = nullptr;
   cudaStream_t ystream = nullptr;
   cudaEvent_t yfork = nullptr, yjoin = nullptr;
   // per-kernel profiling: called after each reconstruction launch, so that
@@ -728,9 +795,6 @@ double bits_to_double(unsigned long long b) {
   return d;
 }
 
-#ifndef PPK_CM
-#define PPK_CM 16
-#endif
 constexpr int MAX_CTAS = 16;   // CTAs (one cluster) per line
 
 // CTAs per line of n cells with M-row thread chunks
@@ -742,9 +806,6 @@ int seg_count(long long n, int m) { return (int)((n + seg_cells(m) - 1) / seg_ce
 // the launch gets an SM of its own (few lines: a line's FP64 work is bound by
 // the FP64 pipe of the SMs it runs on; GB300 has 152).
 int pick_m(int m, long long n, long long nlines) {
-#ifdef PPK_FORCE_M
-  m = PPK_FORCE_M;
-#endif
   if (seg_count(n, m) > MAX_CTAS) m = 16;
   while (m > 2) {
     const int r = seg_count(n, m / 2);
@@ -862,17 +923,24 @@ cudaError_t set_sweep_attrs(int precision, int nv) {
 }
 
 // Chunk length and CTAs per line and side of the characteristic solve: 16
-// rows, the fewest joins per row (2048^2 FP32: 1.64 ms per direction, 1.68 with
-// 12, 1.74 with 8); 8 for four FP64 fields, whose multipliers would fill the
+// rows, the fewest joins per row (2048^2 FP32: 1.33 ms per direction, 1.86 with
+// 12, 1.95 with 8); 8 for four FP64 fields, whose multipliers would fill the
 // shared memory of an SM with one warp; halved while every one-warp CTA still
 // gets an SM of its own (few lines: the chain of a chunk's rows is the cost).
 void char_layout(CharArgs &c, int nv, bool mixed) {
   auto ctas = [&](int m) { return (c.n + 32 * m - 1) / (32 * m); };
-  int m = PPK_CM;
+  int m = 16;
   if (nv == 4 && !mixed && ctas(8) <= MAX_CTAS) m = 8;
   while (m > 1 && ctas(m / 2) <= MAX_CTAS && 2 * c.nlines * ctas(m / 2) <= 152) m /= 2;
   c.M = m;
   c.R = ctas(m);
+}
+
+// whether the solve keeps its multipliers in global scratch: four FP32 fields
+// and more one-warp CTAs than the GPU holds with them in shared memory (74 KB,
+// three per SM)
+bool char_uses_scratch(const CharArgs &c, int nv, bool mixed) {
+  return nv == 4 && mixed && 2 * c.nlines * c.R > 3 * 152;
 }
 
 // Characteristic-wise handles: the face values of the sweep described by a
@@ -899,6 +967,7 @@ cudaError_t launch_char(const pp_cweno_s *h, const SweepArgs &a, const void *U, 
   c.gamma = h->cfg.gamma;
   c.eps_weno = h->cfg.eps_weno;
   char_layout(c, h->nv, is_mixed(h));
+  c.scr = h->UMPy && a.Fm_pre == h->UMPy ? h->cscry : h->cscr;
   cudaError_t e = is_mixed(h) ? launch_char_recon_f32(c, h->nv, st ? st : h->stream, false)
                               : launch_char_recon_f64(c, h->nv, st ? st : h->stream, false);
   if (e == cudaSuccess && h->mark_hook && !st) h->mark_hook();
@@ -931,6 +1000,7 @@ cudaError_t launch_char_group(const pp_cweno_s *h, const LineGroup &g, const Swe
   c.eps_weno = h->cfg.eps_weno;
   c.lines = g.descs;
   char_layout(c, h->nv, is_mixed(h));
+  c.scr = g.cscr;
   return is_mixed(h) ? launch_char_recon_f32(c, h->nv, st, false)
                      : launch_char_recon_f64(c, h->nv, st, false);
 }
@@ -1386,6 +1456,19 @@ int finish_create(pp_cweno_s *h) {
     if (e == cudaSuccess)
       e = is_mixed(h) ? launch_char_recon_f32(c, h->nv, nullptr, true)
                       : launch_char_recon_f64(c, h->nv, nullptr, true);
+    auto scratch = [&](long long n, long long nlines, void **p) {
+      c.n = (int)n;
+      c.nlines = nlines;
+      char_layout(c, h->nv, is_mixed(h));
+      if (e == cudaSuccess && char_uses_scratch(c, h->nv, is_mixed(h)))
+        e = cudaMalloc(p, es * (size_t)char_scratch_values(c, h->nv));
+    };
+    if (h->batch) {
+      for (LineGroup &g : h->groups) scratch(g.nmax, g.nlines, &g.cscr);
+    } else {
+      scratch(h->nx, h->ny, &h->cscr);
+      if (h->nv == 4) scratch(h->ny, h->nx, &h->cscry);
+    }
     if (h->nv == 4 && is_mixed(h) && !h->batch) {
       if (e == cudaSuccess) e = cudaMalloc(&h->UMPy, 2 * es * (size_t)nvals(h));
       if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->ystream, cudaStreamNonBlocking);
@@ -1559,7 +1642,10 @@ int pp_cweno_create_batch(const pp_cweno_config *cfgs, int64_t nprob, void *cuda
   // line groups keyed by (direction, chunk length, cluster size, periodic)
   std::vector<std::vector<LineRef>> glines;
   auto group_of = [&](bool xdir, int n, bool per) -> size_t {
-    const int m = pick_m(16, n, 1 << 20), R = seg_count(n, m);
+    // 16 rows per chunk, 8 for four FP64 fields (three CTAs per SM instead of
+    // two: 64 problems of up to 1024^2 55.5 against 59.3 ms)
+    const int m = pick_m(c0.precision == PP_PREC_FP64 && c0.ndim == 2 ? 8 : 16, n, 1 << 20);
+    const int R = seg_count(n, m);
     for (size_t g = 0; g < h->groups.size(); ++g)
       if (h->groups[g].xdir == xdir && h->groups[g].m == m && h->groups[g].R == R &&
           h->groups[g].periodic == per)
@@ -2107,6 +2193,15 @@ int pp_cweno_operator_noalloc(const pp_cweno_config *cfg, const double *U_dev, d
       if (cudaGetSymbolAddress(&ptr, g_noalloc_scratch) != cudaSuccess || !ptr) return PP_ERR_CUDA;
       for (int k = 3; k <= 4; ++k)
         if (set_sweep_attrs(PP_PREC_FP64, k) != cudaSuccess) return PP_ERR_CUDA;
+      // load the kernels of either path now: a later call may be captured
+      cudaFuncAttributes fa;
+      if (cudaFuncGetAttributes(&fa, noalloc_prepare<3>) != cudaSuccess ||
+          cudaFuncGetAttributes(&fa, noalloc_prepare<4>) != cudaSuccess ||
+          cudaFuncGetAttributes(&fa, noalloc_ctl_reset) != cudaSuccess ||
+          cudaFuncGetAttributes(&fa, noalloc_arm) != cudaSuccess ||
+          cudaFuncGetAttributes(&fa, state_reduce_kernel<3>) != cudaSuccess ||
+          cudaFuncGetAttributes(&fa, state_reduce_kernel<4>) != cudaSuccess)
+        return PP_ERR_CUDA;
       g_noalloc_ptr[dev] = ptr;
       g_noalloc_ready[dev] = true;
     }
@@ -2115,12 +2210,17 @@ int pp_cweno_operator_noalloc(const pp_cweno_config *cfg, const double *U_dev, d
   Ctl *ctl = reinterpret_cast<Ctl *>(base);
   void *D = base + NOALLOC_CTL_BYTES;
 
-  noalloc_ctl_reset<<<1, 32, 0, h.stream>>>(ctl);
-  if (!(eps > 0.0)) {
+  if (eps > 0.0 || h.ncell <= 8192) {   // (eps given: nothing to reduce)
+    const int threads = eps > 0.0 ? 32 : (int)std::min<long long>(1024, (h.ncell + 31) / 32 * 32);
+    if (nv == 4)
+      noalloc_prepare<4><<<1, threads, 0, h.stream>>>(U_dev, L_dev, h.ncell, cfg->gamma, cfg->eps_pos, eps, ctl);
+    else
+      noalloc_prepare<3><<<1, threads, 0, h.stream>>>(U_dev, L_dev, h.ncell, cfg->gamma, cfg->eps_pos, eps, ctl);
+  } else {
+    noalloc_ctl_reset<<<1, 32, 0, h.stream>>>(ctl);
     launch_reduce(&h, U_dev, nullptr, nullptr, ctl);
+    noalloc_arm<<<grid_for(nvals(&h)), 256, 0, h.stream>>>(L_dev, nvals(&h), ctl, cfg->eps_pos);
   }
-  noalloc_ctl_arm<<<1, 32, 0, h.stream>>>(ctl, cfg->eps_pos, eps);
-  noalloc_nan_fill<<<grid_for(nvals(&h)), 256, 0, h.stream>>>(L_dev, nvals(&h), ctl);
   if (cudaGetLastError() != cudaSuccess) return PP_ERR_CUDA;
   cudaError_t e;
   if (nv == 4) {
@@ -2149,11 +2249,14 @@ int pp_cweno_destroy(pp_cweno_t h) {
   cudaFree(h->DT);
   cudaFree(h->UMP);
   cudaFree(h->UMPy);
+  cudaFree(h->cscr);
+  cudaFree(h->cscry);
   if (h->ystream) cudaStreamDestroy(h->ystream);
   if (h->yfork) cudaEventDestroy(h->yfork);
   if (h->yjoin) cudaEventDestroy(h->yjoin);
   for (auto &g : h->groups) {
     cudaFree(g.descs);
+    cudaFree(g.cscr);
   }
   for (cudaStream_t st : h->gstreams) cudaStreamDestroy(st);
   for (cudaEvent_t ev : h->gevents) cudaEventDestroy(ev);

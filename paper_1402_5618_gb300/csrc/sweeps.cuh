@@ -12,15 +12,23 @@ namespace ppk {
 // per CTA and at most 16 CTAs (a cluster) per line; and the resident CTAs per
 // SM asked for.
 constexpr int seg_cells(int m) { return 32 * m; }
-#ifndef PPK_C8
-#define PPK_C8 6
-#define PPK_C16 4
-#define PPK_D8 3
-#endif
+//
+// FP32 (issue and latency bound): registers of a 16-row chunk allow 4 CTAs of
+// four variables without spills (16 warps an SM; 5 CTAs: 2048^2 x sweep 0.32
+// against 0.29 ms), 5 of three (1-D Riemann batch step 2.2 against 2.4 ms with
+// 4).  FP64 (bound by the FP64 units, one per SM quarter, each held for 64
+// cycles by an instruction of one of its warps): warps in multiples of four.
+// Three variables with 16-row chunks would put two CTAs of three warps on an
+// SM, so they take 8-row chunks on two warps per variable instead (Riemann
+// batch 53.2 against 55.8 ms).
 template <typename real, int NV, int M>
 struct Layout {
-  static constexpr int KC = 32;
-  static constexpr int CTAS = sizeof(real) == 4 ? (M == 8 ? PPK_C8 : PPK_C16) : (M == 8 ? PPK_D8 : 2);
+  static constexpr bool F32 = sizeof(real) == 4;
+  static constexpr bool WIDE = !F32 && NV == 3 && M == 16;
+  static constexpr int MM = WIDE ? 8 : M;
+  static constexpr int KC = WIDE ? 64 : 32;
+  static constexpr int CTAS = F32 ? (M != 16 ? 6 : (NV == 4 ? 4 : 5))
+                                  : (M != 8 ? 2 : (NV == 4 ? 3 : 4));
 };
 
 struct LaunchCfg {
@@ -58,9 +66,9 @@ inline cudaError_t launch_sweep(const LaunchCfg &c, const SweepArgs &a, long lon
 
 template <typename real, int NV, int M, int MODE, bool PRE>
 cudaError_t launch_m(const SweepArgs &a, long long nlines, cudaStream_t st, bool attrs_only) {
-  constexpr int KC = Layout<real, NV, M>::KC;
-  using S = Smem<real, NV, M, KC>;
-  auto kern = line_sweep<real, NV, M, KC, MODE, PRE, Layout<real, NV, M>::CTAS>;
+  using Y = Layout<real, NV, M>;
+  using S = Smem<real, NV, Y::MM, Y::KC>;
+  auto kern = line_sweep<real, NV, Y::MM, Y::KC, MODE, PRE, Y::CTAS>;
   if (attrs_only) {   // called at handle creation, outside any stream capture
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)S::bytes);
@@ -74,7 +82,7 @@ cudaError_t launch_m(const SweepArgs &a, long long nlines, cudaStream_t st, bool
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(nlines * a.R), 1, 1);
-  cfg.blockDim = dim3(NV * S::KC, 1, 1);
+  cfg.blockDim = dim3(S::THREADS, 1, 1);
   cfg.dynamicSmemBytes = S::bytes;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
