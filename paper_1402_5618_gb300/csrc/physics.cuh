@@ -1,7 +1,6 @@
 // physics.cuh -- per-cell and per-face device arithmetic of the FVCW scheme
-// (Guo, Xiong & Shi): WENO-Z weights and compact rows (Sec. 2.2), the
-// explicit WENO5-Z closure of bounded lines, the Zhang-Shu limiter and the
-// HLLC flux with Batten's wave speeds (Sec. 2.4).
+// (Guo, Xiong & Shi): the Zhang-Shu limiter and the HLLC flux with Batten's
+// wave speeds (Sec. 2.4), and the arithmetic helpers the line code shares.
 //
 // Line variables are ordered (rho, m_n, [m_t,] E): m_n is the momentum
 // normal to the faces of the line, m_t (2-D only) the tangential one.
@@ -74,37 +73,12 @@ __device__ __forceinline__ float to_f32(double x) {
 }
 __device__ __forceinline__ float to_f32(float x) { return x; }
 
-// Sec. 2.2, eq. (weight): Jiang-Shu indicators of the three sub-stencils of
-// cell i and the WENO-Z ratios q_k = (tau5 / (beta_k + eps))^2 they feed.
-// The minus side (face i+1/2) uses (q0, q1, q2) with c = (0.2, 0.5, 0.3);
-// the mirrored plus side (face i-1/2) uses (q2, q1, q0).
-template <typename real>
-__device__ __forceinline__ void zratios(real um2, real um1, real u0, real up1, real up2,
-                                        real eps, real &q0, real &q1, real &q2) {
-  const real c13 = real(13.0) / real(12.0);
-  real b0 = c13 * sqr(um2 - real(2) * um1 + u0) + real(0.25) * sqr(um2 - real(4) * um1 + real(3) * u0);
-  real b1 = c13 * sqr(um1 - real(2) * u0 + up1) + real(0.25) * sqr(um1 - up1);
-  real b2 = c13 * sqr(u0 - real(2) * up1 + up2) + real(0.25) * sqr(real(3) * u0 - real(4) * up1 + up2);
-  real tau = fabs(b2 - b0);
-  real d0 = b0 + eps, d1 = b1 + eps, d2 = b2 + eps;
-  real ti = tau / (d0 * d1 * d2);   // one division for the three ratios
-  q0 = sqr(ti * d1 * d2);
-  q1 = sqr(ti * d0 * d2);
-  q2 = sqr(ti * d0 * d1);
-}
-
-// FP32 form of the same ratios, scaled so nothing overflows: with
-// d_k = beta_k + eps and dmin = min d_k, when tau > dmin the returned values
-// are (dmin/tau)^2 q_k = (dmin/d_k)^2 and the constant 1 of eq. (weight)
-// becomes s = (dmin/tau)^2; the normalised weights are unchanged
-// (near a jump of 3e6 the plain q_k reaches 1e52, beyond FP32's range).
-//
-// eps is lifted to the FP32 noise floor of the indicators.  The FP32
-// averages the indicators are computed from carry, besides their own
-// rounding (up to u max|ubar|, u = 2^-24), the rounding noise the FP32
+// FP32: eps of eq. (weight) is lifted to the FP32 noise floor of the
+// indicators.  The FP32 averages the indicators are computed from carry,
+// besides their own rounding (up to u max|ubar|, u = 2^-24), the rounding noise the FP32
 // fluxes leave in the state step after step: a random walk of about
 // cfl u |F| per step, tens to hundreds of u max|ubar| after 10^4 steps.
-// eps of eq. (weight), meant to sit above the indicators' zero level and
+// The eps, meant to sit above the indicators' zero level and
 // below every real one, becomes eps + 2^20 (u max|ubar|)^2 over the stencil:
 // above 33 (150 u max|ubar|)^2, the indicators of a flat stencil carrying
 // that noise, and still about 4e-9 max|ubar|^2, below the indicators of
@@ -116,87 +90,12 @@ __device__ __forceinline__ void zratios(real um2, real um1, real u0, real up1, r
 // 4096 (u max|ubar|)^2, 1.7e-6 at 2^20 (u max|ubar|)^2).
 constexpr float FP32_BETA_FLOOR = 1048576.0f * 5.9604645e-08f * 5.9604645e-08f;
 
-__device__ __forceinline__ void zratios_scaled(float um2, float um1, float u0, float up1, float up2,
-                                               float eps, float &q0, float &q1, float &q2,
-                                               float &one) {
-  const float c13 = 13.0f / 12.0f;
-  float b0 = c13 * sqr(um2 - 2.0f * um1 + u0) + 0.25f * sqr(um2 - 4.0f * um1 + 3.0f * u0);
-  float b1 = c13 * sqr(um1 - 2.0f * u0 + up1) + 0.25f * sqr(um1 - up1);
-  float b2 = c13 * sqr(u0 - 2.0f * up1 + up2) + 0.25f * sqr(3.0f * u0 - 4.0f * up1 + up2);
-  float tau = fabsf(b2 - b0);
-  const float umax = fmaxf(fmaxf(fmaxf(fabsf(um2), fabsf(um1)), fmaxf(fabsf(up1), fabsf(up2))),
-                           fabsf(u0));
-  eps = fmaf(FP32_BETA_FLOOR * umax, umax, eps);
-  float d0 = b0 + eps, d1 = b1 + eps, d2 = b2 + eps;
-  float dmin = fminf(fminf(d0, d1), d2);
-  // branch-free: the numerator is min(tau, dmin); the constant term is 1
-  // while tau <= dmin (no rescaling), else (dmin/tau)^2
-  const float r = fminf(tau, dmin);
-  const float sc = dmin / tau;
-  one = tau <= dmin ? 1.0f : sc * sc;
-  q0 = sqr(r / d0);
-  q1 = sqr(r / d1);
-  q2 = sqr(r / d2);
-}
-
-// normalised weights from linear weights (d0, d1, d2) and ratios (q0, q1, q2);
-// one is the scaled constant term (1 unless the ratios were rescaled)
-template <typename real>
-__device__ __forceinline__ void zweights(real d0, real d1, real d2, real q0, real q1, real q2,
-                                         real &w0, real &w1, real &w2, real one = real(1)) {
-  real a0 = d0 * (one + q0), a1 = d1 * (one + q1), a2 = d2 * (one + q2);
-  real is = real(1) / (a0 + a1 + a2);
-  w0 = a0 * is;
-  w1 = a1 * is;
-  w2 = a2 * is;
-}
-
-// ratios in the arithmetic of the line: plain in FP64, scaled in FP32
-template <typename real>
-__device__ __forceinline__ void zratios_any(real um2, real um1, real u0, real up1, real up2,
-                                            real eps, real &q0, real &q1, real &q2, real &one) {
-  if constexpr (sizeof(real) == 4) {
-    zratios_scaled(um2, um1, u0, up1, up2, eps, q0, q1, q2, one);
-  } else {
-    zratios(um2, um1, u0, up1, up2, eps, q0, q1, q2);
-    one = real(1);
-  }
-}
-
-// One tridiagonal row in elimination order: a on the previously eliminated
-// neighbour, b on the unknown, c on the next one, r the right-hand side.
-template <typename real>
-struct Row {
-  real a, b, c, r;
-};
-
-// eq. (CWENO-FV) with weights (w0, w1, w2): the row for the unknown u~ at
-// the face this cell reconstructs; uprev / unext are the neighbour averages
-// on the side of the previously / next eliminated unknown.  The plus side
-// is the mirror image, so the same formula serves both sides.
-template <typename real>
-__device__ __forceinline__ Row<real> compact_row(real w0, real w1, real w2, real uprev, real u0,
-                                                  real unext) {
-  const real third = real(1.0 / 3.0), sixth = real(1.0 / 6.0);
-  Row<real> row;
-  row.a = (real(2) * w0 + w1) * third;
-  row.b = (w0 + real(2) * (w1 + w2)) * third;
-  row.c = w2 * third;
-  row.r = (w0 * uprev + (real(5) * (w0 + w1) + w2) * u0 + (w1 + real(5) * w2) * unext) * sixth;
-  return row;
-}
-
 // ---------------------------------------------------------------- Euler
 template <typename real, int NV>
 __device__ __forceinline__ real kin2(const real *U) {  // |m|^2
   real m2 = U[1] * U[1];
   if (NV == 4) m2 += U[2] * U[2];
   return m2;
-}
-
-template <typename real, int NV>
-__device__ __forceinline__ real pressure(const real *U, real gamma) {
-  return (gamma - real(1)) * (U[NV - 1] - real(0.5) * kin2<real, NV>(U) / U[0]);
 }
 
 // physical flux from the normal velocity un = m_n / rho and the pressure
