@@ -74,17 +74,18 @@ typedef enum {
                                   in the line arithmetic of either precision.
                                   Single problems and batches
                                   (PP_ERR_UNSUPPORTED for
-                                  pp_cweno_operator_noalloc); needs
-                                  2 (n (nv^2 + nv) + nv^2) values per line of
-                                  scratch per sweep direction (periodic: nv^2 +
-                                  nv (nv+1) per row; FP64, or FP32 for the mixed
-                                  form), plus 2 (4 nv + 4) n values of row
-                                  data; a batch sizes both per group of lines
-                                  by the group's longest line; a mixed 2-D
-                                  problem keeps both directions' (and a
-                                  second set of face-value planes), its y
+                                  pp_cweno_operator_noalloc).  Needs
+                                  planes for the face values of one sweep
+                                  direction, U^- and U^+ in the line arithmetic.
+                                  A mixed 2-D problem keeps a second set, its y
                                   reconstruction running on a second stream
-                                  beside the x sweep */
+                                  beside the x sweep.  With many lines (more than
+                                  228 segments of 512 cells, of 256 for four FP64
+                                  fields) also scratch for the solve's
+                                  multipliers, 2 (2 nv^2 + nv) values per cell,
+                                  lines rounded up to the solve's chunks: mixed
+                                  2-D problems for each direction, batches for
+                                  each group of lines, FP64 problems once */
 } pp_recon_t;
 
 enum {
@@ -208,12 +209,14 @@ int pp_cweno_problem_stats(pp_cweno_t h, int64_t k, pp_cweno_stats_t *out);
 int pp_cweno_num_problems(pp_cweno_t h, int64_t *nprob);
 int pp_cweno_problem_cells(pp_cweno_t h, int64_t k, int64_t *ncell);
 
-/* Rows per thread chunk of the line kernels chosen for this handle (8 or
- * 16: the serial Thomas run of a thread against the depth of the parallel
- * scans).  The first set_state of a handle times one sweep with each choice
- * on the handle's own data and keeps the faster: single problems over the x
- * sweep (cached per precision, dimension, grid size and periodicity),
- * batches over every x-line group of the batch. */
+/* Rows per thread chunk of the line kernels chosen for this handle, 8 or 16
+ * (a thread's serial rows against the number of partial results to join).
+ * The first set_state of a single problem's handle times one x sweep with
+ * each choice on the handle's own data and keeps the faster (cached per
+ * precision, dimension, grid size and periodicity); a batch takes the choice
+ * of its line groups' sizes, the longest being reported here.  Lines short
+ * enough for fewer rows per chunk, and launches of so few lines that shorter
+ * segments still get an SM each, run with 2, 4 or 8 whatever the choice. */
 int pp_cweno_rows_per_chunk(pp_cweno_t h, int *m);
 
 /* Kernel launches enqueued per step (for launch accounting). */
@@ -222,8 +225,8 @@ int pp_cweno_launches_per_step(pp_cweno_t h, int64_t *n);
 /* Measurement: enqueue one step launch by launch with CUDA events on the
  * handle's stream between kernels, synchronise and return each kernel's
  * duration in ms (ms[0] the dt kernel, then the sweeps in launch order; a
- * characteristic-wise handle's sweep is preceded by its rows and block-solve
- * kernels, each timed on its own) in ms[0..*nk-1] (at most nmax entries). */
+ * characteristic-wise handle's sweep is preceded by its reconstruction kernel,
+ * timed on its own) in ms[0..*nk-1] (at most nmax entries). */
 int pp_cweno_profile_step(pp_cweno_t h, float *ms, int nmax, int *nk);
 
 /* Measurement: sustained fused multiply-add throughput of this GPU's CUDA

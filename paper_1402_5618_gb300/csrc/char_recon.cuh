@@ -16,11 +16,14 @@
 // and eliminates the M rows of a chunk in walk order (minus left to right,
 // plus right to left) as a function of the unknowns just outside it, the
 // chunks of a warp and the segments of a cluster are joined by trees, and
-// every thread substitutes back from the multipliers in shared memory.
-// Nothing but the state is read and nothing but the face values written.  A
-// walk of each line by one thread, the alternative with half the arithmetic,
-// is bound by its own chain: 2 x 800 positions in FP64 took 4.32 ms, and
-// 2048^2 lines in FP32, one warp per SM, 1.43 ms per direction.
+// every thread substitutes back from its rows' multipliers.  Nothing but the
+// state is read and nothing but the face values written, apart from the
+// multipliers of many lines.  A walk of each line by one thread, the alternative
+// with half the arithmetic, is bound by its own chain wherever the lines are
+// not many thousands: per pass, walk against this, 800 positions in FP64 (38
+// steps) 664 ms and 18.5, 512^2 FP64 38.4 and 6.9, 2048^2 FP64 207 and 92.5, 4096^2
+// mixed 35.5 and 28.8, 2048^2 mixed (three steps) 37.0 and 20.6, 4096 lines of
+// 256-8192 cells mixed 186 and 13.3.
 //
 // The output planes hold U^- and U^+ of every cell in the state's layout and
 // grid variable order; the line kernel limits them, evaluates the face
@@ -44,6 +47,8 @@ struct CharArgs {
   int vn, vt;               // grid index of the normal / tangential momentum (vt < 0 in 1-D)
   int bclo, bchi;
   int M, R;                 // rows per chunk, one-warp CTAs per line and side (n <= 32 M R)
+  int T;                    // rows of every chunk held in shared memory at a time: a power of
+                            // two that divides M, M itself without scratch (M <= 16)
   void *scr;                // multipliers, char_scratch_values() values of the line's type, or
                             // nullptr: in shared memory
   double gamma, eps_weno;

@@ -272,11 +272,10 @@ struct BStep {
 template <typename real, int NV>
 __device__ __forceinline__ void block_up(int d, bool later, End<real, NV> &F, End<real, NV> &L,
                                          BStep<real, NV> &st) {
-  End<real, NV> in, out, in2, out2;
+  End<real, NV> in, out, in2;
   end_select(later, F, L, in);
   end_select(later, L, F, out);
   end_xor(in, d, in2);
-  end_xor(out, d, out2);
   // (I - b' b) [u | r | s] = [a' - b' a | b' g | g']
   real M[NV][NV], X[NV][2 * NV + 1];
 #pragma unroll
@@ -308,30 +307,11 @@ __device__ __forceinline__ void block_up(int d, bool later, End<real, NV> &F, En
       st.s[i][j] = X[i][1 + NV + j];
     }
   }
+  // each lane extends its own outer end; the partner's comes back by shuffles
+  // (as many as its inputs would take, and 292 operations fewer in 2-D)
   End<real, NV> o, o2;
   end_extend(out, st.u, st.r, st.s, o);
-  // this lane's facing unknown a - b u - (g + b r) X_o + b s X_o', as u2 + r2
-  // X_o' - s2 X_o, extends the partner's outer end
-  real u2[NV], r2[NV][NV], s2[NV][NV];
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    real t = in.a[i];
-#pragma unroll
-    for (int m = 0; m < NV; ++m) t -= in.B[i][m] * st.u[m];
-    u2[i] = t;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      real p = in.G[i][j], q = real(0);
-#pragma unroll
-      for (int m = 0; m < NV; ++m) {
-        p += in.B[i][m] * st.r[m][j];
-        q += in.B[i][m] * st.s[m][j];
-      }
-      s2[i][j] = p;
-      r2[i][j] = q;
-    }
-  }
-  end_extend(out2, u2, r2, s2, o2);
+  end_xor(o, d, o2);
   end_select(later, o2, o, F);
   end_select(later, o, o2, L);
 }
@@ -466,16 +446,18 @@ __device__ __forceinline__ void char_row(const real (&win)[5][NV], real gamma, r
 // One warp per (segment of 32 M cells, side); lane k holds the M cells of
 // chunk k; a cluster of R CTAs covers the line.  Kept per row of every lane
 // until the back substitution: the multipliers Y, F and g (x = g - F X_in - Y
-// x_next), in shared memory or, with many lines, in global scratch.
+// x_next), in shared memory or, with many lines, in global scratch.  Bound by
+// FP64 instructions, in FP32 by instruction fetch and by latency (12 warps per
+// SM, 168 registers each).
 template <typename real, int NV>
 struct CharSmem {
   static constexpr int E = 2 * NV * NV + NV;   // multipliers of a row
   static constexpr int RC = 4 + 3 * NV;        // numbers of a row before its elimination
-  // this segment's first and last unknown, then per lane and row the
-  // multipliers, or only the row's numbers (scratch: the multipliers go to
-  // global memory)
-  static size_t bytes(int M, bool scratch) {
-    return sizeof(End<real, NV>) * 2 + sizeof(real) * 32 * (scratch ? RC : E) * (size_t)M;
+  // this segment's first and last unknown, then per lane the multipliers of
+  // every row, or (scratch: they go to global memory) the numbers of T rows
+  static size_t bytes(const CharArgs &a) {
+    return sizeof(End<real, NV>) * 2 +
+           sizeof(real) * 32 * (a.scr ? RC * (size_t)a.T : E * (size_t)a.M);
   }
 };
 
@@ -486,7 +468,7 @@ __global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
   End<real, NV> *seg = reinterpret_cast<End<real, NV> *>(smem_raw);
   real *rows = reinterpret_cast<real *>(smem_raw + 2 * sizeof(End<real, NV>));
   cg::cluster_group cluster = cg::this_cluster();
-  const int M = a.M, R = a.R;
+  const int M = a.M, R = a.R, T = a.T, shT = __ffs(T) - 1;
   const int rank = (int)cluster.block_rank(), lane = threadIdx.x, side = blockIdx.y;
   const LineGeo geo = line_geo(a, blockIdx.x / R);
   const int n = geo.n;
@@ -506,142 +488,156 @@ __global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
   if (a.scr)
     mult = reinterpret_cast<real *>(a.scr) +
            ((long long)blockIdx.y * gridDim.x + blockIdx.x) * ((long long)32 * E * M);
-  auto at = [&](int t, int e) -> real & { return rows[(t * RS + e) * 32 + lane]; };
-  auto mt = [&](int t, int e) -> real & { return mult[(t * E + e) * 32 + lane]; };
+  // (a lane's column moves with the row: lanes on consecutive cells of a chunk
+  // are then in different banks)
+  auto at = [&](int t, int e, int k) -> real & { return rows[(t * RS + e) * 32 + ((k + 4 * t) & 31)]; };
+  auto mt = [&](int t, int e) -> real & { return mult[(t * E + e) * 32 + ((lane + 4 * t) & 31)]; };
+  // the q-th cell of the rows [t0, t0 + T) of all chunks, consecutive q on
+  // consecutive cells: its chunk and row; false where the chunk has no such row
+  auto tile_cell = [&](int q, int t0, int &ch, int &t, long long &o) {
+    ch = q >> shT;
+    t = q & (T - 1);
+    const int c0 = lo + ch * M, m = min(M, n - c0);
+    o = geo.base + (long long)(c0 + (side == 0 ? t0 + t : m - 1 - t0 - t)) * geo.cs;
+    return t0 + t < m;
+  };
 
-  // The chunk's rows first, their 4 + 3 NV numbers into the slots the
-  // multipliers take later: two loops whose bodies stay in the instruction
-  // caches instead of one that does not (the SM runs few warps of this kernel).
-  // The cells come in with consecutive lanes on consecutive cells, each into
-  // its row's slots (read as a stencil cell before the row overwrites them);
-  // the two cells on either side of a chunk are a lane's own.
-  const int len = min(32 * M, n - lo);   // (<= 0: no cells)
+  End<real, NV> F, L;
+  end_empty(F);
+  end_empty(L);
+  // T rows at a time: first the 4 + 3 NV numbers of each, then their
+  // elimination -- two loops whose bodies stay in the instruction caches instead
+  // of one that does not.  The cells come in with consecutive lanes on
+  // consecutive cells, each into its row's slots (read as a stencil cell before
+  // the row overwrites them); the two cells on either side are a lane's own.
+#pragma unroll 1
+  for (int t0 = 0; t0 < M; t0 += T) {
+    __syncwarp();
 #pragma unroll 4
-  for (int c = lane; c < len; c += 32) {
-    const int ch = c / M, j = c - ch * M;
-    const int t = side == 0 ? j : min(M, len - ch * M) - 1 - j;
-    const long long o = geo.base + (long long)(lo + c) * geo.cs;
+    for (int q = lane; q < 32 * T; q += 32) {
+      int ch, t;
+      long long o;
+      if (tile_cell(q, t0, ch, t, o)) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) rows[(t * RS + k) * 32 + ch] = __ldg(U + o + gv[k] * geo.ncell);
-  }
-  __syncwarp();
-  {
+        for (int k = 0; k < NV; ++k) at(t, k, ch) = __ldg(U + o + gv[k] * geo.ncell);
+      }
+    }
+    __syncwarp();
+    const int tc = min(T, cnt - t0), f0 = first + t0 * dir;
     real win[5][NV], after[2][NV];
-    if (cnt > 0) {
-      line_cell<real, NV>(geo, U, gv, first - 2 * dir, win[1]);
-      line_cell<real, NV>(geo, U, gv, first - dir, win[2]);
-      line_cell<real, NV>(geo, U, gv, first + cnt * dir, after[0]);
-      line_cell<real, NV>(geo, U, gv, first + (cnt + 1) * dir, after[1]);
+    if (tc > 0) {
+      line_cell<real, NV>(geo, U, gv, f0 - 2 * dir, win[1]);
+      line_cell<real, NV>(geo, U, gv, f0 - dir, win[2]);
+      line_cell<real, NV>(geo, U, gv, f0 + tc * dir, after[0]);
+      line_cell<real, NV>(geo, U, gv, f0 + (tc + 1) * dir, after[1]);
 #pragma unroll
       for (int k = 0; k < NV; ++k) {
-        win[3][k] = at(0, k);
-        win[4][k] = cnt > 1 ? at(1, k) : after[0][k];
+        win[3][k] = at(0, k, lane);
+        win[4][k] = tc > 1 ? at(1, k, lane) : after[0][k];
       }
     }
 #pragma unroll 1
-    for (int t = 0; t < cnt; ++t) {
-      const int c = first + t * dir;
+    for (int t = 0; t < tc; ++t) {
+      const int c = f0 + t * dir;
 #pragma unroll
       for (int w = 0; w < 4; ++w)
 #pragma unroll
         for (int k = 0; k < NV; ++k) win[w][k] = win[w + 1][k];
 #pragma unroll
       for (int k = 0; k < NV; ++k)
-        win[4][k] = t + 2 < cnt ? at(min(t + 2, M - 1), k) : (t + 2 == cnt ? after[0][k] : after[1][k]);
+        win[4][k] = t + 2 < tc ? at(min(t + 2, T - 1), k, lane)
+                               : (t + 2 == tc ? after[0][k] : after[1][k]);
       real rs[4], ca[NV], cc[NV], s[NV];
       char_row<real, NV>(win, gam, eps, !per && (c == 0 || c == n - 1), rs, ca, cc, s);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) at(t, i) = rs[i];
+      for (int i = 0; i < 4; ++i) at(t, i, lane) = rs[i];
 #pragma unroll
       for (int i = 0; i < NV; ++i) {
-        at(t, 4 + i) = ca[i];
-        at(t, 4 + NV + i) = cc[i];
-        at(t, 4 + 2 * NV + i) = s[i];
+        at(t, 4 + i, lane) = ca[i];
+        at(t, 4 + NV + i, lane) = cc[i];
+        at(t, 4 + 2 * NV + i, lane) = s[i];
       }
     }
-  }
-  // elimination of the chunk: last = g - F X_in - Y x_next after every row,
-  // first = a - B X_in - G x_next folded along
-  End<real, NV> F, L;
-  end_empty(F);
-  end_empty(L);
+    // elimination of the chunk: last = g - F X_in - Y x_next after every row,
+    // first = a - B X_in - G x_next folded along
 #pragma unroll 1
-  for (int t = 0; t < cnt; ++t) {
-    real ca[NV], cc[NV], s[NV], rs[4];
-    {
+    for (int t = 0; t < tc; ++t) {
+      real ca[NV], cc[NV], s[NV], rs[4];
+      {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) rs[i] = at(t, i);
+        for (int i = 0; i < 4; ++i) rs[i] = at(t, i, lane);
 #pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        ca[i] = at(t, 4 + i);
-        cc[i] = at(t, 4 + NV + i);
-        s[i] = at(t, 4 + 2 * NV + i);
+        for (int i = 0; i < NV; ++i) {
+          ca[i] = at(t, 4 + i, lane);
+          cc[i] = at(t, 4 + NV + i, lane);
+          s[i] = at(t, 4 + 2 * NV + i, lane);
+        }
       }
-    }
-    const LeftEig<real, NV> Lk(rs);
-    // (L - diag(a) L Y) [Y' | g' | F'] = [diag(c) L | s - diag(a) L g | -diag(a) L F]
-    real B[NV][NV], X[NV][2 * NV + 1];
-    {
-      real tg[NV];
-      Lk.mul(L.a, tg);
+      const LeftEig<real, NV> Lk(rs);
+      // (L - diag(a) L Y) [Y' | g' | F'] = [diag(c) L | s - diag(a) L g | -diag(a) L F]
+      real B[NV][NV], X[NV][2 * NV + 1];
+      {
+        real tg[NV];
+        Lk.mul(L.a, tg);
 #pragma unroll
-      for (int i = 0; i < NV; ++i) X[i][NV] = s[i] - ca[i] * tg[i];
-    }
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      real y[NV], f[NV], ty[NV], tf[NV];
-#pragma unroll
-      for (int m = 0; m < NV; ++m) {
-        y[m] = L.B[m][j];
-        f[m] = L.G[m][j];
+        for (int i = 0; i < NV; ++i) X[i][NV] = s[i] - ca[i] * tg[i];
       }
-      Lk.mul(y, ty);
-      Lk.mul(f, tf);
-#pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        const real l = Lk.at(i, j);
-        B[i][j] = l - ca[i] * ty[i];
-        X[i][j] = cc[i] * l;
-        X[i][NV + 1 + j] = -(ca[i] * tf[i]);
-      }
-    }
-    gauss_solve<real, NV, 2 * NV + 1>(B, X);
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      L.a[i] = X[i][NV];
-      mt(t, i) = X[i][NV];
 #pragma unroll
       for (int j = 0; j < NV; ++j) {
-        L.B[i][j] = X[i][j];
-        L.G[i][j] = X[i][NV + 1 + j];
-        mt(t, NV + i * NV + j) = X[i][j];
-        mt(t, NV + NV * NV + i * NV + j) = X[i][NV + 1 + j];
-      }
-    }
-    // first = a - B X_in - G x_p with x_p = g - F X_in - Y x_{p+1}
-    real G2[NV][NV];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      real p = F.a[i];
-#pragma unroll
-      for (int m = 0; m < NV; ++m) p -= F.G[i][m] * L.a[m];
-      F.a[i] = p;
-#pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        real q = F.B[i][j], r = real(0);
+        real y[NV], f[NV], ty[NV], tf[NV];
 #pragma unroll
         for (int m = 0; m < NV; ++m) {
-          q -= F.G[i][m] * L.G[m][j];
-          r -= F.G[i][m] * L.B[m][j];
+          y[m] = L.B[m][j];
+          f[m] = L.G[m][j];
         }
-        F.B[i][j] = q;
-        G2[i][j] = r;
+        Lk.mul(y, ty);
+        Lk.mul(f, tf);
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+          const real l = Lk.at(i, j);
+          B[i][j] = l - ca[i] * ty[i];
+          X[i][j] = cc[i] * l;
+          X[i][NV + 1 + j] = -(ca[i] * tf[i]);
+        }
       }
+      gauss_solve<real, NV, 2 * NV + 1>(B, X);
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        L.a[i] = X[i][NV];
+        mt(t0 + t, i) = X[i][NV];
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+          L.B[i][j] = X[i][j];
+          L.G[i][j] = X[i][NV + 1 + j];
+          mt(t0 + t, NV + i * NV + j) = X[i][j];
+          mt(t0 + t, NV + NV * NV + i * NV + j) = X[i][NV + 1 + j];
+        }
+      }
+      // first = a - B X_in - G x_p with x_p = g - F X_in - Y x_{p+1}
+      real G2[NV][NV];
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        real p = F.a[i];
+#pragma unroll
+        for (int m = 0; m < NV; ++m) p -= F.G[i][m] * L.a[m];
+        F.a[i] = p;
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+          real q = F.B[i][j], r = real(0);
+#pragma unroll
+          for (int m = 0; m < NV; ++m) {
+            q -= F.G[i][m] * L.G[m][j];
+            r -= F.G[i][m] * L.B[m][j];
+          }
+          F.B[i][j] = q;
+          G2[i][j] = r;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < NV; ++i)
+#pragma unroll
+        for (int j = 0; j < NV; ++j) F.G[i][j] = G2[i][j];
     }
-#pragma unroll
-    for (int i = 0; i < NV; ++i)
-#pragma unroll
-      for (int j = 0; j < NV; ++j) F.G[i][j] = G2[i][j];
   }
 
   // trees over the warp's chunks, then over the segments of the cluster
@@ -703,45 +699,50 @@ __global__ void __launch_bounds__(32) char_solve_kernel(const CharArgs a) {
 #pragma unroll
       for (int e = 0; e < E; ++e) nx[d][e] = mt(cnt - 1 - d, e);
     }
-#pragma unroll 1
-  for (int t = cnt - 1; t >= 0; --t) {
-    real m[E], x[NV];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      m[e] = nx[0][e];
-      nx[0][e] = nx[1][e];
-    }
-    if (t > 1) {
-#pragma unroll
-      for (int e = 0; e < E; ++e) nx[1][e] = mt(t - 2, e);
-    }
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      real p = m[i];
-#pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        p -= m[NV + NV * NV + i * NV + j] * xl[j];
-        p -= m[NV + i * NV + j] * xr[j];
-      }
-      x[i] = p;
-    }
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      xr[i] = x[i];
-      at(t, i) = x[i];
-    }
-  }
-  __syncwarp();
-  // out: consecutive lanes on consecutive cells
   real *out = reinterpret_cast<real *>(side == 0 ? a.Um : a.Up);
-#pragma unroll 4
-  for (int c = lane; c < len; c += 32) {
-    const int ch = c / M, j = c - ch * M;
-    const int t = side == 0 ? j : min(M, len - ch * M) - 1 - j;
-    const long long o = geo.base + (long long)(lo + c) * geo.cs;
+#pragma unroll 1
+  for (int t0 = (M - 1) & ~(T - 1); t0 >= 0; t0 -= T) {
+    __syncwarp();
+#pragma unroll 1
+    for (int t = min(T, cnt - t0) - 1; t >= 0; --t) {
+      real m[E], x[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
-      out[o + gv[k] * geo.ncell] = __ldg(U + o + gv[k] * geo.ncell) + rows[(t * RS + k) * 32 + ch];
+      for (int e = 0; e < E; ++e) {
+        m[e] = nx[0][e];
+        nx[0][e] = nx[1][e];
+      }
+      if (t0 + t > 1) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) nx[1][e] = mt(t0 + t - 2, e);
+      }
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        real p = m[i];
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+          p -= m[NV + NV * NV + i * NV + j] * xl[j];
+          p -= m[NV + i * NV + j] * xr[j];
+        }
+        x[i] = p;
+      }
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        xr[i] = x[i];
+        at(t, i, lane) = x[i];
+      }
+    }
+    __syncwarp();
+    // out: consecutive lanes on consecutive cells
+#pragma unroll 4
+    for (int q = lane; q < 32 * T; q += 32) {
+      int ch, t;
+      long long o;
+      if (tile_cell(q, t0, ch, t, o)) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+          out[o + gv[k] * geo.ncell] = __ldg(U + o + gv[k] * geo.ncell) + at(t, k, ch);
+      }
+    }
   }
   if (R > 1) cluster_wait();
 }
@@ -750,9 +751,8 @@ template <typename real, int NV>
 cudaError_t launch_nv(const CharArgs &a, cudaStream_t st, bool attrs_only) {
   auto kern = char_solve_kernel<real, NV>;
   if (attrs_only) {
-    // (M = 16 rows per chunk at most)
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)CharSmem<real, NV>::bytes(16, false));
+                                         (int)(sizeof(End<real, NV>) * 2 + sizeof(real) * 32 * 16 * CharSmem<real, NV>::E));
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                (int)cudaSharedmemCarveoutMaxShared);
@@ -763,7 +763,7 @@ cudaError_t launch_nv(const CharArgs &a, cudaStream_t st, bool attrs_only) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.nlines * a.R), 2, 1);
   cfg.blockDim = dim3(32, 1, 1);
-  cfg.dynamicSmemBytes = CharSmem<real, NV>::bytes(a.M, a.scr != nullptr);
+  cfg.dynamicSmemBytes = CharSmem<real, NV>::bytes(a);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;

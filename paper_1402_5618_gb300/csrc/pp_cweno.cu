@@ -922,25 +922,36 @@ cudaError_t set_sweep_attrs(int precision, int nv) {
   return cudaSuccess;
 }
 
-// Chunk length and CTAs per line and side of the characteristic solve: 16
-// rows, the fewest joins per row (2048^2 FP32: 1.33 ms per direction, 1.86 with
-// 12, 1.95 with 8); 8 for four FP64 fields, whose multipliers would fill the
-// shared memory of an SM with one warp; halved while every one-warp CTA still
-// gets an SM of its own (few lines: the chain of a chunk's rows is the cost).
-void char_layout(CharArgs &c, int nv, bool mixed) {
+// Rows per chunk (M), one-warp CTAs per line and side (R) and rows in shared
+// memory at a time (T) of the characteristic solve; returns whether the
+// multipliers go to global scratch.
+// Few lines: multipliers in shared memory, M = 16 (8 for four FP64 fields,
+// whose multipliers would fill an SM with one warp), halved while every CTA
+// still gets an SM of its own (the chain of a chunk's rows is the cost).
+// More CTAs than three per SM, what shared memory holds: scratch, and chunks as
+// long as leave six warps per SM, up to 128 rows: a level of joins costs as
+// much as 0.6 rows, and there are five and more per chunk.  M is a multiple of
+// T, not a power of two, so that lines of any length use the lanes of their
+// segments.  T = 8 (FP64: 4) lets the registers, not shared memory, set the
+// number of warps.  Per SSP-RK3 step, against M = 16 (8) with at most six (three)
+// warps per SM: 2048^2 mixed 6.9 ms (9.8), 4096^2 mixed 28.8 (40.1), 4096^2 FP64
+// 372 (1195).  Three mixed steps on 2048^2: T = 16 24.1 ms, T = 4 21.6, T = 8
+// 20.6; M up to 32 22.5, up to 64 21.4, up to 256 20.6.
+bool char_layout(CharArgs &c, int nv, bool mixed) {
   auto ctas = [&](int m) { return (c.n + 32 * m - 1) / (32 * m); };
   int m = 16;
   if (nv == 4 && !mixed && ctas(8) <= MAX_CTAS) m = 8;
   while (m > 1 && ctas(m / 2) <= MAX_CTAS && 2 * c.nlines * ctas(m / 2) <= 152) m /= 2;
-  c.M = m;
+  c.M = c.T = m;
   c.R = ctas(m);
-}
-
-// whether the solve keeps its multipliers in global scratch: four FP32 fields
-// and more one-warp CTAs than the GPU holds with them in shared memory (74 KB,
-// three per SM)
-bool char_uses_scratch(const CharArgs &c, int nv, bool mixed) {
-  return nv == 4 && mixed && 2 * c.nlines * c.R > 3 * 152;
+  if (2 * c.nlines * c.R <= 3 * 152) return false;
+  const int T = mixed ? 8 : 4;
+  c.R = ctas(128);
+  auto rows = [&](int r) { return (c.n + 32 * T * r - 1) / (32 * T * r) * T; };
+  while (2 * c.nlines * c.R < 6 * 152 && rows(c.R + 1) >= 16 && c.R < MAX_CTAS) ++c.R;
+  c.M = rows(c.R);
+  c.T = T;
+  return true;
 }
 
 // Characteristic-wise handles: the face values of the sweep described by a
@@ -966,8 +977,9 @@ cudaError_t launch_char(const pp_cweno_s *h, const SweepArgs &a, const void *U, 
   c.bchi = a.bchi;
   c.gamma = h->cfg.gamma;
   c.eps_weno = h->cfg.eps_weno;
-  char_layout(c, h->nv, is_mixed(h));
-  c.scr = h->UMPy && a.Fm_pre == h->UMPy ? h->cscry : h->cscr;
+  c.scr = !char_layout(c, h->nv, is_mixed(h)) ? nullptr
+          : h->UMPy && a.Fm_pre == h->UMPy    ? h->cscry
+                                              : h->cscr;
   cudaError_t e = is_mixed(h) ? launch_char_recon_f32(c, h->nv, st ? st : h->stream, false)
                               : launch_char_recon_f64(c, h->nv, st ? st : h->stream, false);
   if (e == cudaSuccess && h->mark_hook && !st) h->mark_hook();
@@ -999,8 +1011,7 @@ cudaError_t launch_char_group(const pp_cweno_s *h, const LineGroup &g, const Swe
   c.gamma = h->cfg.gamma;
   c.eps_weno = h->cfg.eps_weno;
   c.lines = g.descs;
-  char_layout(c, h->nv, is_mixed(h));
-  c.scr = g.cscr;
+  c.scr = char_layout(c, h->nv, is_mixed(h)) ? g.cscr : nullptr;
   return is_mixed(h) ? launch_char_recon_f32(c, h->nv, st, false)
                      : launch_char_recon_f64(c, h->nv, st, false);
 }
@@ -1456,18 +1467,27 @@ int finish_create(pp_cweno_s *h) {
     if (e == cudaSuccess)
       e = is_mixed(h) ? launch_char_recon_f32(c, h->nv, nullptr, true)
                       : launch_char_recon_f64(c, h->nv, nullptr, true);
+    size_t have = 0;   // bytes behind *p
     auto scratch = [&](long long n, long long nlines, void **p) {
       c.n = (int)n;
       c.nlines = nlines;
-      char_layout(c, h->nv, is_mixed(h));
-      if (e == cudaSuccess && char_uses_scratch(c, h->nv, is_mixed(h)))
-        e = cudaMalloc(p, es * (size_t)char_scratch_values(c, h->nv));
+      if (!char_layout(c, h->nv, is_mixed(h))) return;
+      const size_t bytes = es * (size_t)char_scratch_values(c, h->nv);
+      if (bytes <= have || e != cudaSuccess) return;
+      cudaFree(*p);
+      *p = nullptr;
+      have = bytes;
+      e = cudaMalloc(p, bytes);
     };
     if (h->batch) {
-      for (LineGroup &g : h->groups) scratch(g.nmax, g.nlines, &g.cscr);
+      for (LineGroup &g : h->groups) {
+        have = 0;
+        scratch(g.nmax, g.nlines, &g.cscr);
+      }
     } else {
       scratch(h->nx, h->ny, &h->cscr);
-      if (h->nv == 4) scratch(h->ny, h->nx, &h->cscry);
+      if (is_mixed(h)) have = 0;   // (FP64: one direction at a time, one scratch)
+      if (h->nv == 4) scratch(h->ny, h->nx, is_mixed(h) ? &h->cscry : &h->cscr);
     }
     if (h->nv == 4 && is_mixed(h) && !h->batch) {
       if (e == cudaSuccess) e = cudaMalloc(&h->UMPy, 2 * es * (size_t)nvals(h));
