@@ -155,13 +155,13 @@ def replica_value(ws: int, ncell: int, steps: int, ms_max: float) -> float:
 #   y sweep  reads U_k and D_x, U^n in stages 2-3 (2/3 on average),
 #            writes U_{k+1}                                          117.3 B
 # Mixed form (3 kernels per stage):
-#   x sweep  reads the FP32 hi parts of U_k, writes D_x (FP32)        32 B
-#   y sweep  reads the transposed hi parts, writes D_y transposed     32 B
+#   x sweep  reads the hi and lo parts of U_k, writes D_x (FP32)      48 B
+#   y sweep  reads the transposed parts, writes D_y transposed        48 B
 #   combine  reads U_k, U^n (2/3), D_x, D_y; writes U_{k+1} and its
 #            transposed hi and lo parts                              149.3 B
 KERNEL_BYTES = {
     0: [("x_sweep", 64.0), ("y_sweep", 32 + 32 + 32 * 2.0 / 3.0 + 32)],
-    1: [("x_sweep", 32.0), ("y_sweep_transposed", 32.0),
+    1: [("x_sweep", 48.0), ("y_sweep_transposed", 48.0),
         ("stage_combine", 32 + 32 * 2.0 / 3.0 + 16 + 16 + 32 + 32)],
 }
 
@@ -189,16 +189,15 @@ ALU_PEAK_TFLOPS = {1: 152 * 128 * 2 * 2.07e9 / 1e12, 0: 1.25}
 # was taken on (their SHA-256 below); any change to them voids it.
 # Captured on the 3072^2 blast (`bench.py --profile-only mixed|fp64 --n 3072`,
 # the first x sweep of the first step, `-s 6 -c 1` past the autotuner's
-# trials): reads are the algorithmic bytes of a plain-form line (the blast's
-# lines are flat to FP32 precision at that step); writes fall short of them by
-# what is still dirty in L2 when the kernel ends.  The FP64 form's dominant
+# trials): reads are the algorithmic bytes; writes fall short of them by what
+# is still dirty in L2 when the kernel ends.  The FP64 form's dominant
 # kernel is its y sweep, for which no capture of these sources exists.
 TRAFFIC_PER_CELL = {            # {(precision, kernel): bytes per cell}
-    (1, "x_sweep"): 28.33,
-    (0, "x_sweep"): 59.64,
+    (1, "x_sweep"): 45.01,
+    (0, "x_sweep"): 59.86,
 }
-TRAFFIC_SRC_SHA256 = "125b6e168b43838d09caa6c191c5d38175b8c94383bd35a6e8e9d3d6b2b84e5a"
-KERNEL_SOURCES = ("line_sweep.cuh", "physics.cuh", "dfloat.cuh", "batch_lines.cuh")
+TRAFFIC_SRC_SHA256 = "03bb5b96c0a25d10ff27c4d3018930dc616d3701503e118473d320a1da8ae69f"
+KERNEL_SOURCES = ("line_sweep.cuh", "compact_solve.cuh", "physics.cuh", "dfloat.cuh", "batch_lines.cuh")
 
 
 def _kernel_src_sha256() -> str:
@@ -385,8 +384,8 @@ def _roofline(r, prec, ncell, hbm_peak, peak_kind):
     import numpy as np
     prof = np.array(r["prof"])          # [steps, launches]: dt kernel, then per stage
     kinds = KERNEL_BYTES[prec]
-    # then (checked steps) the commit copy, the transposed-plane restore of
-    # the mixed form and the step-end bookkeeping
+    # then (checked steps) the restore of a rejected step and the step-end
+    # bookkeeping
     per = prof[:, 1:1 + 3 * len(kinds)].reshape(prof.shape[0], 3, len(kinds))
     tot = per.sum(axis=(0, 1))
     table = {}

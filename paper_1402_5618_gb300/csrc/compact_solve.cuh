@@ -26,8 +26,9 @@
 // of the unknowns just outside it (X_in before, X_out after):
 //   first = A - B X_in - G X_out,   last = D - F X_in - C X_out.
 // The order of elimination is free: b_i 2^i >= a_i 2^(i-1) + c_i 2^(i+1) in
-// every row (b - a/2 - 2c = 15/4 S1 >= 0), so the matrix scaled by 2^i is diagonally dominant and every pivot and every 1 - C B of a
-// composition stays positive, as in the serial elimination.
+// every row (b - a/2 - 2c = 15/4 S1 >= 0), so the matrix scaled by 2^i is
+// diagonally dominant and every pivot and every 1 - C B of a composition stays
+// positive, as in the serial elimination.
 #pragma once
 
 #include <cuda_runtime.h>

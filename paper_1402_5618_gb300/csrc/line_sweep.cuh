@@ -8,15 +8,14 @@
 //   solve    for each conserved variable the minus and plus compact-WENO
 //            systems (eq. (CWENO-FV)), exactly and in partitioned form
 //            (compact_solve.cuh): every thread eliminates a chunk of M rows of
-//            one variable in both systems, one or two warps combine the
-//            chunks of the segment, eight to a lane and then across lanes,
-//            and the segments of the cluster through distributed shared
-//            memory; the solution at the run ends goes back the same way and
-//            every thread substitutes back in its chunk.  A periodic line is
-//            the same with the ring closed where the segments combine.
+//            one variable in both systems as a function of the unknowns
+//            outside it, the chunks of the segment are joined within a warp,
+//            the segments of the cluster through distributed shared memory,
+//            and every thread substitutes back in its chunk.  A periodic line
+//            is the same with the ring closed where the segments are joined;
 //   limit    Zhang-Shu limiter per cell (Sec. 2.4);
-//   flux     HLLC at every face of the segment (the two segment-end faces
-//            read the neighbour CTA's limited face value);
+//   flux     HLLC at every face of the segment (the CTA limits the cell on
+//            either side of its segment itself: no exchange of faces);
 //   update   flux difference (eq. (1DEulerFV-b)) and either the x-sweep
 //            output D = L_x, or the SSP-RK3 stage combination (eq. (RK3))
 //            with L = D + L_y (2-D) / L (1-D), plus the grid-wide reductions
@@ -26,7 +25,15 @@
 // real = float: the mixed form -- FP32 line arithmetic, the state stored as
 // FP32 hi + lo pairs combined with compensated (double-float) arithmetic,
 // FP64 only for the limiter factors of cells that need limiting and for the
-// Sherman-Morrison scalars.
+// closing of a periodic ring.
+//
+// What bounds it: in FP64 the FP64 pipe (72-76% busy on large grids; a line
+// alone waits for its own chain of FP64 instructions), in the mixed form
+// instruction issue (47%) and fixed latencies, barriers and instruction
+// fetch, with 16 warps per SM; HBM is at 14%.  Per sweep of 4096^2 cells (corner
+// blast), against a scan over projective chunk maps with divisions in every
+// row and an exchange of limited faces: mixed 1.63 -> 0.84 ms, FP64 48.0 -> 16.0
+// (x) and 51.6 -> 18.3 ms (y with the stage update).
 #pragma once
 
 #include <cooperative_groups.h>

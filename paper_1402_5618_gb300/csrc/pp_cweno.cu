@@ -934,8 +934,8 @@ cudaError_t set_sweep_attrs(int precision, int nv) {
 // T, not a power of two, so that lines of any length use the lanes of their
 // segments.  T = 8 (FP64: 4) lets the registers, not shared memory, set the
 // number of warps.  Per SSP-RK3 step, against M = 16 (8) with at most six (three)
-// warps per SM: 2048^2 mixed 6.9 ms (9.8), 4096^2 mixed 28.8 (40.1), 4096^2 FP64
-// 372 (1195).  Three mixed steps on 2048^2: T = 16 24.1 ms, T = 4 21.6, T = 8
+// warps per SM: 2048^2 mixed 6.9 ms (9.8), 4096^2 mixed 27.3 (40.1), 4096^2 FP64
+// 360 (1195).  Three mixed steps on 2048^2: T = 16 24.1 ms, T = 4 21.6, T = 8
 // 20.6; M up to 32 22.5, up to 64 21.4, up to 256 20.6.
 bool char_layout(CharArgs &c, int nv, bool mixed) {
   auto ctas = [&](int m) { return (c.n + 32 * m - 1) / (32 * m); };
@@ -1513,10 +1513,10 @@ int finish_create(pp_cweno_s *h) {
   return PP_OK;
 }
 
-// Autotuner: the rows per thread chunk (M = 8: more threads and a deeper
-// parallel scan; M = 16: longer serial elimination runs, one warp per
-// variable) is picked per handle by timing the first sweep of a stage on the
-// handle's own state, with CUDA events on its stream.  The sweep writes only
+// Autotuner: the rows per thread chunk (M = 8: more threads and partial results
+// to join; M = 16: longer serial runs) of a single problem is picked by timing
+// the first sweep of a stage on the handle's own state, with CUDA events on
+// its stream; batches take it by rule (pick_m).  The sweep writes only
 // scratch (the x-sweep output buffer, or the stage buffer as an operator
 // output), and the choice is cached per (precision, ndim, nx, ny, periodic).
 struct TuneKey {
