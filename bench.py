@@ -196,7 +196,7 @@ TRAFFIC_PER_CELL = {            # {(precision, kernel): bytes per cell}
     (1, "x_sweep"): 45.01,
     (0, "x_sweep"): 59.86,
 }
-TRAFFIC_SRC_SHA256 = "03bb5b96c0a25d10ff27c4d3018930dc616d3701503e118473d320a1da8ae69f"
+TRAFFIC_SRC_SHA256 = "df84695ac674e64df2d4dfbfa8ae895904b113d530ba3f08194a9a01841d7333"
 KERNEL_SOURCES = ("line_sweep.cuh", "compact_solve.cuh", "physics.cuh", "dfloat.cuh", "batch_lines.cuh")
 
 

@@ -27,7 +27,7 @@
 // FP64 only for the limiter factors of cells that need limiting and for the
 // closing of a periodic ring.
 //
-// What bounds it: in FP64 the FP64 pipe (72-76% busy on large grids; a line
+// What bounds it: in FP64 the FP64 pipe (71-76% busy on large grids; a line
 // alone waits for its own chain of FP64 instructions), in the mixed form
 // instruction issue (47%) and fixed latencies, barriers and instruction
 // fetch, with 16 warps per SM; HBM is at 14%.  Per sweep of 4096^2 cells (corner
