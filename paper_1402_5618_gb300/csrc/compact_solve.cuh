@@ -37,7 +37,10 @@
 
 namespace ppk {
 
-// halves of a cluster barrier that publishes no data
+// halves of a cluster barrier; the relaxed arrival publishes no data
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release;\n" ::: "memory");
+}
 __device__ __forceinline__ void cluster_arrive_relaxed() {
   asm volatile("barrier.cluster.arrive.relaxed;\n" ::: "memory");
 }

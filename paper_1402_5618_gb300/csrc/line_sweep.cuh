@@ -546,6 +546,10 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
   // face values computed outside (the characteristic-wise reconstruction):
   // U^- and U^+ of the segment's cells in the state's layout
   if constexpr (PRE) {
+    // A stage may update the state in place, and the halo cells loaded above are
+    // the neighbours' cells: no CTA of the line writes before all have loaded
+    // (arrive here, wait before the update; the other kernels meet at the joins).
+    if (MODE != MODE_XSWEEP && R > 1) cluster_arrive();
     const real *pm = reinterpret_cast<const real *>(args.Fm_pre);
     const real *pp = reinterpret_cast<const real *>(args.Fp_pre);
     const int c0 = lo > 0 || per ? -1 : 0, c1 = hi - lo + (hi < n || per ? 1 : 0);
@@ -1078,6 +1082,7 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
   (void)mixedforms;
 
   // ---------------------------------------------------------------- update
+  if (PRE && MODE != MODE_XSWEEP && R > 1) cluster_wait();
   // the stage's extrema in the line's arithmetic (converted once per warp)
   real mymin = real(sizeof(real) == 4 ? 3.0e38 : 1.0e300), mymax = real(0);
   unsigned int nbad = 0;
