@@ -170,6 +170,7 @@ struct Exch {
   float rh[NV], rl[NV], rf[NV], rF[NV], rp[4];
   int rgate[NV];
   float rspread[NV];             // largest |sample - R| per variable (hi parts)
+  float hend[2][NV];             // hi parts of the cells before and after the segment
   float epsf;                    // mixed form: the limiter epsilon of this stage
   dfl dt;                        // mixed form: the time step
 };
@@ -528,6 +529,9 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
         if (k + q * KC < len) dst[S::pad(k + q * KC)] = val(hv[q], lv[MIXED ? q : 0]);
     }
     if (extra) dst[S::pad(cx)] = val(hr, lr);
+    if constexpr (MIXED && !PRE) {
+      if (k == 1 || k == 2) ex.hend[k - 1][v] = hr;
+    }
     for (int c = len + 2 + k; c < SEG + 2; c += KC) dst[S::pad(c)] = real(0);   // past the line
   }
   __syncthreads();
@@ -982,11 +986,14 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
         if (dlt) {
           // the average as the plain form has it (the FP32 hi part, not
           // R + (ubar - R): exact relative to ubar however far it is from R)
-          // and the face values in full
+          // and the face values in full.  A neighbour's cell comes from the
+          // load phase: its owner may have updated it in place by now.
+          const long long o = lbase + (long long)(lo + c) * cs;
 #pragma unroll
           for (int kv = 0; kv < NV; ++kv) {
-            bool neg;   // (never a reflected cell: those beyond a wall are not limited)
-            ub[kv] = args.Uh[cell_addr(kv, lo + c, neg)];
+            ub[kv] = c < 0 ? ex.hend[0][kv]
+                     : c >= len ? ex.hend[1][kv]
+                                : args.Uh[gvar(kv, NV, args.vn, args.vt) * args.ncell + o];
             a[kv] += rf[kv];
             b[kv] += rf[kv];
           }
