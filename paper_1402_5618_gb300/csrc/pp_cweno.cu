@@ -128,8 +128,9 @@ __device__ __forceinline__ bool cell_measure(double rho, double m1, double m2, d
 }
 
 // Reductions of a state: min density, max rate, cells outside G.  The state
-// is FP64 planes (lo == nullptr) or FP32 hi / lo plane pairs.  Blocks (x)
-// stride over the cells of one problem (y; probs == nullptr: the single one).
+// is FP64 planes (lo == nullptr) or FP32 hi / lo plane pairs.  Blocks (y)
+// stride over the cells of one problem (x, the axis that takes more than
+// 65 535; probs == nullptr: the single one).
 // Bound by the FP64 pipe (2 lanes per SM): about 30 FP64 instructions per
 // cell, with reciprocals instead of divisions and integer comparisons
 // (4096^2 FP64: 3.3 ms with divisions).  Batches take one block per 2048
@@ -139,8 +140,8 @@ template <int NV>
 __global__ void __launch_bounds__(256)
     state_reduce_kernel(const void *Uv, const float *lo, const ProbDesc *probs, ProbDesc pd,
                         double gamma, Ctl *ctls) {
-  if (probs) pd = probs[blockIdx.y];
-  Ctl *ctl = ctls + blockIdx.y;
+  if (probs) pd = probs[blockIdx.x];
+  Ctl *ctl = ctls + blockIdx.x;
   const long long nc = pd.ncell;
   const double gg1 = gamma * (gamma - 1.0);
   double mn = 1e300, mx = 0.0;
@@ -150,8 +151,8 @@ __global__ void __launch_bounds__(256)
     if (lo) return (double)reinterpret_cast<const float *>(Uv)[i] + (double)lo[i];
     return reinterpret_cast<const double *>(Uv)[i];
   };
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nc;
-       c += (long long)gridDim.x * blockDim.x) {
+  for (long long c = blockIdx.y * (long long)blockDim.x + threadIdx.x; c < nc;
+       c += (long long)gridDim.y * blockDim.x) {
     const double rho = at(c);
     double r;
     if (!cell_measure<NV>(rho, at(nc + c), NV == 4 ? at(2 * nc + c) : 0.0, at((NV - 1) * nc + c), gg1,
@@ -229,7 +230,7 @@ __global__ void transpose_planes_b_kernel(const float *in, float *out, const Til
 // rejected, or a problem took no step (finished, stopped, or past its step
 // limit), U^n is copied into the stage buffer so that the next step starts
 // from it again, and after a rejection its transposed planes (UT, mixed 2-D
-// form) are formed again.  Problem p (blockIdx.y) owns the 32-bit words
+// form) are formed again.  Problem p (blockIdx.x) owns the 32-bit words
 // [a0, a0 + n) and [a1, a1 + n) of both buffers (FP64 values, or the FP32 hi
 // and lo planes of the mixed form).  Nearly every step is accepted, so the
 // cost is that of blocks that find nothing to do: few blocks, each striding
@@ -238,7 +239,7 @@ __global__ void transpose_planes_b_kernel(const float *in, float *out, const Til
 __global__ void __launch_bounds__(256)
     restore_kernel(const unsigned int *src, unsigned int *dst, float *UT, const ProbDesc *probs,
                    ProbDesc pd, long long nvals, int mixed, int nv, const Ctl *ctls) {
-  const int p = blockIdx.y;
+  const int p = blockIdx.x;
   const Ctl *ctl = ctls + p;
   if (ctl->active && step_accepted(ctl)) return;
   if (probs) pd = probs[p];
@@ -246,14 +247,14 @@ __global__ void __launch_bounds__(256)
   const long long a0 = mixed ? pd.off : 2 * pd.off;
   const long long a1 = mixed ? nvals + pd.off : 2 * pd.off + n;
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  for (long long i = blockIdx.x * 256ll + tid; i < n; i += gridDim.x * 256ll) {
+  for (long long i = blockIdx.y * 256ll + tid; i < n; i += gridDim.y * 256ll) {
     dst[a0 + i] = src[a0 + i];
     dst[a1 + i] = src[a1 + i];
   }
   if (!UT || !ctl->active) return;
   const float *in = reinterpret_cast<const float *>(src);
   const int ntx = (pd.nx + TT - 1) / TT, nty = (pd.ny + TT - 1) / TT;
-  for (long long t = blockIdx.x; t < (long long)ntx * nty * 2 * nv; t += gridDim.x) {
+  for (long long t = blockIdx.y; t < (long long)ntx * nty * 2 * nv; t += gridDim.y) {
     const int v = (int)(t / ((long long)ntx * nty)), q = (int)(t % ((long long)ntx * nty));
     const long long o = (v < nv ? 0 : nvals) + pd.off + (v % nv) * pd.ncell;
     transpose_tile(in + o, UT + o, q % ntx * TT, q / ntx * TT, pd.nx, pd.ny);
@@ -1228,8 +1229,8 @@ cudaError_t finish_checked_step(pp_cweno_s *h, const std::function<void()> &mark
   long long longest = h->batch ? 0 : nvals(h);
   for (const ProbDesc &d : h->probs_h) longest = std::max(longest, (long long)h->nv * d.ncell);
   // 64 words per thread and array; a single problem has the GPU to itself
-  const unsigned bx = (unsigned)std::min<long long>(h->batch ? 64 : 1216, (longest + 16383) / 16384);
-  restore_kernel<<<dim3(bx, (unsigned)h->nprob), dim3(TT, 8), 0, h->stream>>>(
+  const unsigned by = (unsigned)std::min<long long>(h->batch ? 64 : 1216, (longest + 16383) / 16384);
+  restore_kernel<<<dim3((unsigned)h->nprob, by), dim3(TT, 8), 0, h->stream>>>(
       reinterpret_cast<const unsigned int *>(h->U0), reinterpret_cast<unsigned int *>(h->U1),
       h->ytrans || h->btrans ? h->UT : nullptr, h->batch ? h->probs : nullptr, single_desc(h),
       nvals(h), is_mixed(h) ? 1 : 0, h->nv, h->ctl);
@@ -1386,7 +1387,7 @@ int build_graph(pp_cweno_s *h) {
 void launch_reduce(const pp_cweno_s *h, const void *U, const float *lo, const ProbDesc *probs, Ctl *ctl) {
   long long longest = h->batch ? 0 : h->ncell;
   for (const ProbDesc &d : h->probs_h) longest = std::max(longest, d.ncell);
-  const dim3 grid((unsigned)std::min<long long>(1216, (longest + 2047) / 2048), (unsigned)h->nprob);
+  const dim3 grid((unsigned)h->nprob, (unsigned)std::min<long long>(1216, (longest + 2047) / 2048));
   if (h->nv == 4)
     state_reduce_kernel<4><<<grid, 256, 0, h->stream>>>(U, lo, probs, single_desc(h), h->cfg.gamma, ctl);
   else
