@@ -56,6 +56,11 @@ __device__ __forceinline__ bool less(double a, double b) {
   q ^= (q >> 63) & 0x7fffffffffffffffll;
   return p < q;
 }
+// a NaN an FP64 operation returned (quiet)
+__device__ __forceinline__ bool is_nan(double x) {
+  return (__double2hiint(x) & 0x7ff80000) == 0x7ff80000;
+}
+__device__ __forceinline__ bool is_nan(float x) { return x != x; }
 __device__ __forceinline__ bool is_finite(float x) { return isfinite(x); }
 __device__ __forceinline__ bool is_finite(double x) {
   return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
@@ -148,10 +153,13 @@ __device__ __forceinline__ void hllc(const real *Ul, const real *Ur, real gamma,
   const real a2 = g1 * (Ht - real(0.5) * (ut * ut + vt * vt));
   const real at = root(a2);
   real SL = ul - al, SR = ur + ar;
-  if (a2 >= real(0)) {   // rounding may leave no real Roe sound speed: then the face states' own
+  // The smaller and the larger of two speeds, of which either may be NaN:
+  // rounding may leave no real Roe sound speed, and a face state of negative
+  // pressure (limiter off) has none of its own.
+  if (a2 >= real(0)) {
     const real tl = ut - at, tr = ut + at;
-    SL = less(tl, SL) ? tl : SL;
-    SR = less(SR, tr) ? tr : SR;
+    SL = less(tl, SL) || is_nan(SL) ? tl : SL;
+    SR = less(SR, tr) || is_nan(SR) ? tr : SR;
   }
   if (positive(SL)) {
     phys_flux_u<real, NV>(Ul, ul, pl, F);
