@@ -15,7 +15,8 @@
 //            is the same with the ring closed where the segments are joined;
 //   limit    Zhang-Shu limiter per cell (Sec. 2.4);
 //   flux     HLLC at every face of the segment (the CTA limits the cell on
-//            either side of its segment itself: no exchange of faces);
+//            either side of its segment itself: no exchange of faces; both
+//            CTAs at a seam come to the same bits, see Exch::ends);
 //   update   flux difference (eq. (1DEulerFV-b)) and either the x-sweep
 //            output D = L_x, or the SSP-RK3 stage combination (eq. (RK3))
 //            with L = D + L_y (2-D) / L (1-D), plus the grid-wide reductions
@@ -162,7 +163,13 @@ __device__ __forceinline__ real shfl_down_r(real v, int d, int width = 32) {
 template <typename real, int NV>
 struct Exch {
   Run<real> seg[2 * NV];         // this segment as a run, per variable and side
-  real xo[2 * NV];               // the unknown after the segment
+  // Per variable and side, for every segment of the line the unknowns before
+  // (x) and after it (y, walk order); the own segment's first and last are the
+  // one after the previous and the one before the next.  A face between two
+  // segments is evaluated by both CTAs, and the line's flux differences
+  // telescope only if they get the same number: every CTA computes the entries
+  // at its ends by the same operations on the same runs.
+  typename Pair<real>::t ends[2 * NV][16];
   // mixed form, the line's reference state R (difference form): per
   // variable the hi / lo pair of the median of five sampled cells, R in
   // FP32, the reference fluxes F(R), (u_R, v_R, p_R, E_R + p_R), whether
@@ -577,6 +584,25 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
     constexpr bool TREE = S::TREE;
     using P = typename Pair<real>::t;
     P cs[M - 1];
+    // The last segment of a periodic line may hold one cell, whose unknown is
+    // its first and its last: both seams then take the one of the ring's closure.
+    const bool lone = per && R > 1 && n % SEG == 1;
+    // After the back substitution: the face values of the two cells next to the
+    // segment are known here as well (the unknowns outside its ends), so this CTA
+    // limits those cells itself and needs nothing more from its neighbours; and
+    // the segment's own end cells take the same numbers as there.  A lane per
+    // value (out: the cell outside, right: that end, plus: that system).
+    auto seam_faces = [&](bool act, bool out, bool right, bool plus) {
+      if (KC > 32 && (k & ~31) != (right ? ((len - 1) / M & ~31) : 0)) return;
+      if (!act || !(per || (right ? hi < n : lo > 0))) return;
+      int r = rank;
+      if (!out) r = right ? (rank == R - 1 ? 0 : rank + 1) : (rank == 0 ? R - 1 : rank - 1);
+      bool y = (right == plus) != out;
+      if (TREE && lone && r == R - 2 && y != plus) { r = 0; y = plus; }
+      const real *x = reinterpret_cast<const real *>(&ex.ends[2 * v + plus][r]);
+      const int at = S::pad((right ? len - 1 : 0) + (out ? (right ? 1 : -1) : 0));
+      (plus ? Fp : Fm)[v * FWP + FH + at] = uv[at] + x[y];
+    };
     if constexpr (S::SIDES == 2) {
       auto solve = [&](auto side_c) {
         constexpr int SD = decltype(side_c)::value;
@@ -631,11 +657,14 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
 #pragma unroll
           for (int h = 3; h >= 0; --h)
             if ((1 << h) < R) tree_down((q & (1 << h)) != 0, false, sg[h], xl, xr);
-          const int at = SD ? R - 1 - rank : rank;
-          xl = __shfl_sync(0xffffffffu, xl, at);
-          xr = __shfl_sync(0xffffffffu, xr, at);
+          if (lane < R) ex.ends[2 * v + SD][SD ? R - 1 - q : q] = p_set(xl, xr);
+          __syncwarp();
+          const P x = ex.ends[2 * v + SD][rank];
+          xl = x.x;
+          xr = x.y;
         } else if (per) {
           ring_close(F, L, xl, xr);
+          if (lane == 0) ex.ends[2 * v + SD][0] = p_set(xl, xr);
         }
 #pragma unroll
         for (int h = 4; h >= 0; --h) {
@@ -646,9 +675,7 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
           const real xo = fma(-own.b, xr, fma(-own.g, xl, own.a));
           side_back<SD, M>(uv + cb, dd + cb, ff, c1, xl, xo, n - (lo + k * M));
           __syncwarp();
-          // the cells next to the segment (below)
-          if (k == 0 && (lo > 0 || per)) dd[S::pad(-1)] = uv[S::pad(-1)] + (SD ? xr : xl);
-          if (k == (len - 1) / M && (hi < n || per)) dd[S::pad(len)] = uv[S::pad(len)] + (SD ? xl : xr);
+          seam_faces(lane < 4, lane & 1, lane & 2, SD);
         }
       };
       if (sidew) solve(std::integral_constant<int, 1>());
@@ -687,7 +714,6 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
     }
 
     P xin, xown;   // the unknown before the chunk, its own last one
-    P xafter;      // the unknown after it (first and last chunk of the segment)
     if constexpr (TREE) {
       // ----------------------------------------- a warp per variable: trees
       // over the warp's 32 chunks, then (16 lanes per side) over the
@@ -736,9 +762,11 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
 #pragma unroll
         for (int h = 3; h >= 0; --h)
           if ((1 << h) < R) tree_down((q & (1 << h)) != 0, false, sg[h], yl, yr);
-        const int lm = rank, lp = 16 + R - 1 - rank;
-        xl = p_set(__shfl_sync(0xffffffffu, yl, lm), __shfl_sync(0xffffffffu, yl, lp));
-        xr = p_set(__shfl_sync(0xffffffffu, yr, lm), __shfl_sync(0xffffffffu, yr, lp));
+        if (q < R) ex.ends[2 * v + sd][sd ? R - 1 - q : q] = p_set(yl, yr);
+        __syncwarp();
+        const P xm = ex.ends[2 * v][rank], xp = ex.ends[2 * v + 1][rank];
+        xl = p_set(xm.x, xp.x);
+        xr = p_set(xm.y, xp.y);
       } else if (per) {
         Ends<real> f, l;
         const bool p = lane & 1;   // even lanes close the minus ring, odd lanes the plus ring
@@ -746,6 +774,7 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
         l.a = p ? L.a.y : L.a.x; l.b = p ? L.b.y : L.b.x; l.g = p ? L.g.y : L.g.x;
         real yl, yr;
         ring_close(f, l, yl, yr);
+        if (lane < 2) ex.ends[2 * v + lane][0] = p_set(yl, yr);
         xl = p_set(__shfl_sync(0xffffffffu, yl, 0), __shfl_sync(0xffffffffu, yl, 1));
         xr = p_set(__shfl_sync(0xffffffffu, yr, 0), __shfl_sync(0xffffffffu, yr, 1));
       }
@@ -755,7 +784,6 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
         tree_down(r, !r, st[h], xl, xr);
       }
       xin = xl;
-      xafter = xr;
       xown = p_fma(p_neg(own.b), xr, p_fma(p_neg(own.g), xl, own.a));
     } else {
       __syncthreads();
@@ -823,50 +851,65 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
         seg = run_join(rt ? o : seg, rt ? seg : o, cut[h]);
       }
       if (on && cl == 0) ex.seg[sys] = seg;
+      __syncwarp();
     }
     if (R > 1) cluster.sync();
     if (comb) {
-      // the rest of the line as seen from this segment: l_rest = Dr - Fr
-      // X_last - Cr X_first before it, f_rest = Ar - Br X_last - Gr X_first
-      // after it.  Bounded: lane 0 joins the segments before, lane 1 those
-      // after; periodic: lane 0 joins all others around the ring.
-      Run<real> rest = run_empty<real>();
+      // The seams at either end of the segment: the runs before and after a
+      // seam from the ends of the line, lane 0 joining the segments forwards,
+      // lane 1 backwards, so that the neighbour comes to the same two runs.
+      // Kept of them, without (e) and with this segment (w), is the end at the
+      // seam: its value, the coefficient of the line's far end and that of the
+      // unknown across the seam.  Periodic: lane 0 goes on to the whole line,
+      // whose ring gives the unknowns at its two ends.
+      const int wpos = sd ? R - 1 - rank : rank;
+      real e1 = real(0), e2 = real(-1), e3 = real(0), w1 = e1, w2 = e2, w3 = e3;
+      real el = real(0), er = real(0);   // before the first and after the last cell (bounded: no weight)
       {
-        const int wpos = sd ? R - 1 - rank : rank;
-        const int cnt = per ? (cl == 0 ? R - 1 : 0) : (cl == 0 ? wpos : (cl == 1 ? R - 1 - wpos : 0));
-        int at = (per || cl) ? wpos + 1 : 0;
+        Run<real> rest = run_empty<real>();
+        const int cnt = cl == 0 ? (per ? R : wpos + 1) : (cl == 1 ? R - wpos : 0);
         Cut<real> unused;
 #pragma unroll 1
-        for (int q = 0; q < cnt; ++q, ++at) {
-          if (at >= R) at -= R;
-          const Exch<real, NV> *rx = cluster.map_shared_rank(&ex, sd ? R - 1 - at : at);
-          const Run<real> o = rx->seg[sys];
-          rest = run_join(rest, o, unused);
+        for (int q = 0; q < cnt; ++q) {
+          const int at = cl == 0 ? q : R - 1 - q;
+          const Run<real> o = cluster.map_shared_rank(&ex, sd ? R - 1 - at : at)->seg[sys];
+          if (at == wpos) {
+            e1 = cl == 0 ? rest.D : rest.A; e2 = cl == 0 ? rest.F : rest.G; e3 = cl == 0 ? rest.C : rest.B;
+          }
+          if (q == 0) rest = o;
+          else rest = run_join(cl == 0 ? rest : o, cl == 0 ? o : rest, unused);
+          if (at == wpos) {
+            w1 = cl == 0 ? rest.D : rest.A; w2 = cl == 0 ? rest.F : rest.G; w3 = cl == 0 ? rest.C : rest.B;
+          }
+        }
+        if (per) {
+          const Run<real> w = run_shfl(rest, 0, LPS);
+          Ends<real> f, l;
+          f.a = w.A; f.b = w.B; f.g = w.G;
+          l.a = w.D; l.b = w.C; l.g = w.F;
+          ring_close(f, l, el, er);
         }
       }
-      const Run<real> r0 = run_shfl(rest, 0, LPS), r1 = run_shfl(rest, 1, LPS);
-      real xl, xr;   // the unknowns before and after the segment
-      if (per) {
-        // the ring's closure in FP64 (both forms): 2 x 2
-        const double A = seg.A, B = seg.B, G = seg.G, D = seg.D, F = seg.F, C = seg.C;
-        const double Ar = r0.A, Br = r0.B, Gr = r0.G, Dr = r0.D, Fr = r0.F, Cq = r0.C;
-        const double a11 = 1.0 - Fr * F - Cq * B, a12 = Fr * C + Cq * G;
-        const double a21 = Br * F + Gr * B, a22 = 1.0 - Br * C - Gr * G;
-        const double b1 = Dr - Fr * D - Cq * A, b2 = Ar - Br * D - Gr * A;
-        const double idet = rcp(a11 * a22 - a12 * a21);
-        xl = real((b1 * a22 + a12 * b2) * idet);
-        xr = real((a11 * b2 + a21 * b1) * idet);
-      } else {
-        const real a11 = fma(-r0.C, seg.B, real(1)), a12 = r0.C * seg.G;
-        const real a21 = r1.B * seg.F, a22 = fma(-r1.B, seg.C, real(1));
-        const real b1 = fma(-r0.C, seg.A, r0.D), b2 = fma(-r1.B, seg.D, r1.A);
-        const real idet = rcp(fma(a11, a22, -(a12 * a21)));
-        xl = fma(b1, a22, a12 * b2) * idet;
-        xr = fma(a11, b2, a21 * b1) * idet;
+      // lane 0: the seam before the segment, lane 1: the one after it; (o) the
+      // run across it; last of the earlier run and first of the later one
+      const real o1 = __shfl_xor_sync(0xffffffffu, w1, 1, LPS), o2 = __shfl_xor_sync(0xffffffffu, w2, 1, LPS);
+      const real o3 = __shfl_xor_sync(0xffffffffu, w3, 1, LPS);
+      const real ea = fma(-e2, cl == 0 ? el : er, e1), oa = fma(-o2, cl == 0 ? er : el, o1);
+      const real i1 = rcp(fma(-e3, o3, real(1)));
+      const real ye = fma(-e3, oa, ea) * i1, yo = fma(-o3, ea, oa) * i1;
+      real sl = cl == 0 ? ye : yo, sf = cl == 0 ? yo : ye;
+      if (wpos == (cl == 0 ? 0 : R - 1)) { sl = el; sf = er; }
+      // a last segment of one cell (see lone)
+      if (lone) {
+        if (sd == 0 && wpos == (cl == 0 ? R - 1 : R - 2)) sf = el;
+        if (sd == 1 && wpos == (cl == 0 ? 1 : 0)) sl = er;
       }
-      if (on && cl == 0) {
-        Xs[sys * S::XP] = xl;
-        ex.xo[sys] = xr;
+      real xl = __shfl_sync(0xffffffffu, sl, 0, LPS), xr = __shfl_sync(0xffffffffu, sf, 1, LPS);
+      if (on && cl < 2) {
+        const int w = (cl == 0) == (sd != 0) ? rank + 1 : rank - 1, rw = w < 0 ? R - 1 : (w == R ? 0 : w);
+        ex.ends[sys][cl == 0 ? rank : rw].x = sl;
+        ex.ends[sys][cl == 0 ? rw : rank].y = sf;
+        if (cl == 0) Xs[sys * S::XP] = xl;
       }
 #pragma unroll
       for (int h = 2; h >= 0; --h) {
@@ -892,7 +935,6 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
       const int m0 = k, m1 = k + 1, p0 = KC - 1 - k, p1 = KC - k;
       xin = p_set(xm[m0 + (m0 >> 3)], xp[p0 + (p0 >> 3)]);
       xown = p_set(xm[m1 + (m1 >> 3)], xp[p1 + (p1 >> 3)]);
-      xafter = p_set(ex.xo[2 * v], ex.xo[2 * v + 1]);
     }
 
     // ------------------------------------------- back substitution
@@ -903,19 +945,7 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
       else
         chunk_back<real, M, false>(uv + cb, Fm + of, Zm + o, Fp + of, Zp + o, cs, xin, xown, mine);
       __syncwarp();   // (a lane past a ragged end may have written its idle slots)
-      // The face values of the two cells next to the segment are known here
-      // as well (the unknowns outside the segment's ends), so this CTA limits
-      // those cells itself and needs nothing more from its neighbours.
-      if (k == 0 && (lo > 0 || per)) {
-        const real u = uv[S::pad(-1)];
-        Fm[v * FWP + FH + S::pad(-1)] = u + xin.x;
-        Fp[v * FWP + FH + S::pad(-1)] = u + xafter.y;
-      }
-      if (k == (hi - lo - 1) / M && (hi < n || per)) {
-        const real u = uv[S::pad(hi - lo)];
-        Fm[v * FWP + FH + S::pad(hi - lo)] = u + xafter.x;
-        Fp[v * FWP + FH + S::pad(hi - lo)] = u + xin.y;
-      }
+      if (R > 1 || per) seam_faces(lane < 8, lane & 1, lane & 4, lane & 2);
     }
     }
     // the neighbours read this CTA's run until here at the latest: arrive
