@@ -213,10 +213,11 @@ int pp_cweno_problem_cells(pp_cweno_t h, int64_t k, int64_t *ncell);
  * (a thread's serial rows against the number of partial results to join).
  * The first set_state of a single problem's handle times one x sweep with
  * each choice on the handle's own data and keeps the faster (cached per
- * precision, dimension, grid size and periodicity); a batch takes the choice
- * of its line groups' sizes, the longest being reported here.  Lines short
- * enough for fewer rows per chunk, and launches of so few lines that shorter
- * segments still get an SM each, run with 2, 4 or 8 whatever the choice. */
+ * device, precision, dimension, grid size, periodicity, reconstruction and
+ * flux); a batch takes the choice of its line groups' sizes, the longest
+ * being reported here.  Lines short enough for fewer rows per chunk, and
+ * launches of so few lines that shorter segments still get an SM each, run
+ * with 2, 4 or 8 whatever the choice. */
 int pp_cweno_rows_per_chunk(pp_cweno_t h, int *m);
 
 /* Kernel launches enqueued per step (for launch accounting). */

@@ -1519,13 +1519,15 @@ int finish_create(pp_cweno_s *h) {
 // the first sweep of a stage on the handle's own state, with CUDA events on
 // its stream; batches take it by rule (pick_m).  The sweep writes only
 // scratch (the x-sweep output buffer, or the stage buffer as an operator
-// output), and the choice is cached per (precision, ndim, nx, ny, periodic).
+// output), and the choice is cached per (device, precision, ndim, nx, ny,
+// periodic, reconstruction, flux).
 struct TuneKey {
-  int prec, ndim;
+  int dev, prec, ndim;
   long long nx, ny;
-  int per;
+  int per, recon, flux;   // other kernels behind another reconstruction or flux
   bool operator==(const TuneKey &o) const {
-    return prec == o.prec && ndim == o.ndim && nx == o.nx && ny == o.ny && per == o.per;
+    return dev == o.dev && prec == o.prec && ndim == o.ndim && nx == o.nx && ny == o.ny &&
+           per == o.per && recon == o.recon && flux == o.flux;
   }
 };
 std::mutex g_tune_mu;
@@ -1539,7 +1541,10 @@ int autotune(pp_cweno_s *h) {
     for (const LineGroup &g : h->groups) h->m = std::max(h->m, g.m);
     return PP_OK;
   }
-  TuneKey key{h->cfg.precision, h->nv == 4 ? 2 : 1, h->nx, h->ny, h->cfg.bc[0] == PP_BC_PERIODIC};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return PP_ERR_CUDA;
+  const TuneKey key{dev, h->cfg.precision, h->nv == 4 ? 2 : 1, h->nx, h->ny,
+                    h->cfg.bc[0] == PP_BC_PERIODIC, h->cfg.recon, h->cfg.flux};
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     for (auto &kv : g_tune_cache)
@@ -1559,13 +1564,16 @@ int autotune(pp_cweno_s *h) {
     h->m = mm;
     float t_min = 1e30f;
     for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {
+      // (a characteristic handle's face values, which do not depend on M, come
+      // with the very first launch and are not timed)
+      const bool char_done = mm > 8 || rep > 0;
       cudaEventRecord(e0, h->stream);
       if (h->nv == 4)
         e = launch(h, MODE_XSWEEP, true, h->U0, h->U0, nullptr, h->D, nullptr, 0, 1e-13,
-                   h->ctl_scratch);
+                   h->ctl_scratch, nullptr, char_done);
       else
         e = launch(h, MODE_OPERATOR, true, h->U0, h->U0, nullptr, nullptr, nullptr, 0, 1e-13,
-                   h->ctl_scratch, reinterpret_cast<double *>(h->U1));
+                   h->ctl_scratch, reinterpret_cast<double *>(h->U1), char_done);
       cudaEventRecord(e1, h->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float t = 0.f;
