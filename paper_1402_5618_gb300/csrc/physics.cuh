@@ -394,8 +394,9 @@ __device__ __forceinline__ int limit_cell(const real *ub, real *um, real *up, re
 // wgl <= 1/4), so rho >= r = ub_0 - d_0 and g >= r (E - d_E) - |m|^2/2 at the
 // box's worst corner.  The thresholds are twice the FP32 allowances of
 // limiter_cell at the box's largest magnitudes, which leaves the evaluation's
-// own rounding (about a tenth of them) ample room.  NaN fails every comparison.  Smooth
-// cells pass, and skip the pretest below (a third of its instructions).
+// own rounding (about a tenth of them) ample room.  NaN fails every comparison,
+// and a threshold within reach of the products' underflow fails.  Smooth cells
+// pass, and skip the pretest below (a third of its instructions).
 template <int NV>
 __device__ __forceinline__ bool limit_box_free(const float *ub, const float *dm, const float *dp,
                                                float wgl, float eps) {
@@ -411,7 +412,8 @@ __device__ __forceinline__ bool limit_box_free(const float *ub, const float *dm,
   const float r = ub[0] - d0, R = ub[0] + d0, E = ub[NV - 1] + dE;
   const float g = fmaf(r, ub[NV - 1] - dE, -0.5f * S);
   const float need = fmaf(eps * R, R, 128.0f * uf * fmaf(E, R, S));
-  return r > fmaf(32.0f * uf, R, 2.0f * eps) && g > need && need < 3.0e38f && wgl <= 0.25f;
+  return r > fmaf(32.0f * uf, R, 2.0f * eps) && g > need && need < 3.0e38f && need > 1.0e-36f &&
+         wgl <= 0.25f;
 }
 
 // Mixed form: an FP32 test of the limiter's conditions with doubled
@@ -446,9 +448,10 @@ __device__ __forceinline__ bool limit_need_mixed(const float *ub, const float *u
       32.0f * uf * ((fabsf(ub[NV - 1]) + emx) * (fabsf(ub[0]) + rmx) + sm);
   need = need | (energy_form<float, NV>(um, eps) < eta2) |
          (energy_form<float, NV>(up, eps) < eta2) | (energy_form<float, NV>(w3, eps) < eta2);
-  // magnitudes beyond FP32's range (or NaN) make the allowance non-finite:
+  // magnitudes beyond FP32's range (or NaN) make the allowance non-finite, and
+  // below 1e-36 the products' underflow (1e-38) is no longer small against it:
   // such a cell always goes to the exact test
-  return need | !(eta2 <= 3.0e38f);
+  return need | !(eta2 <= 3.0e38f && eta2 >= 1.0e-36f);
 }
 
 // The FP64 limiter of a flagged cell of the mixed form, on FP32 face values
