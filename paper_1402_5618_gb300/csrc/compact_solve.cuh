@@ -139,8 +139,8 @@ __device__ __forceinline__ void z_terms(double d0, double d1, double d2, double 
 }
 
 // FP32: S_k = 1 + (tau/d_k)^2 by reciprocals (cheap here).  d_k >= 2^-28
-// umax^2 (the rounding floor of the indicators) and tau <= ~10 umax^2, so
-// S_k stays below 2^65.
+// umax^2 (the rounding floor of the indicators) and tau <= 33.4 umax^2 (cells of
+// alternating sign: beta <= 13/12 4^2 + 8^2/4), so S_k stays below 2^67.
 __device__ __forceinline__ void z_terms(float d0, float d1, float d2, float &S0, float &S1, float &S2) {
   const float tau = d2 - d0;
   const float t0 = tau * rcp(d0), t1 = tau * rcp(d1), t2 = tau * rcp(d2);
@@ -448,8 +448,8 @@ __device__ __forceinline__ void side_back(const double *u, double *dd, const dou
 // partner's inner unknown is u + r X_o - s X_o' (X_o, X_o': outside the own
 // and the partner's outer end), kept for the way down.  A lane extends its own
 // outer end only and receives the partner's: as many shuffles as reading the
-// partner's inputs, six operations fewer (a 200-cell FP64 line on 16 CTAs
-// 0.0258 ms instead of 0.0288).
+// partner's inputs, six operations fewer (a 200-cell FP64 line, four CTAs of
+// two-row chunks, 0.0258 ms instead of 0.0288).
 template <typename P>
 struct Ends {
   P a, b, g;

@@ -28,7 +28,7 @@
 // FP64 only for the limiter factors of cells that need limiting and for the
 // closing of a periodic ring.
 //
-// What bounds it: in FP64 the FP64 pipe (71-76% busy on large grids; a line
+// What bounds it: in FP64 the FP64 pipe (71% busy on large grids; a line
 // alone waits for its own chain of FP64 instructions), in the mixed form
 // instruction issue (47%) and fixed latencies, barriers and instruction
 // fetch, with 16 warps per SM; HBM is at 14%.  Per sweep of 4096^2 cells (corner
@@ -948,8 +948,11 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
       if (R > 1 || per) seam_faces(lane < 8, lane & 1, lane & 4, lane & 2);
     }
     }
-    // the neighbours read this CTA's run until here at the latest: arrive
-    // now, wait before exit (shared memory must outlive their reads)
+    // This CTA has read its neighbours' runs: arrive now, wait before exit (a
+    // CTA's shared memory must outlive the reads of its run).  A relaxed arrival
+    // does not wait for loads in flight, so it has to follow the use of every
+    // value read from another CTA: each passes a join's shuffle or arithmetic
+    // above, whose result the back substitution has consumed.
     if (R > 1) cluster_arrive_relaxed();
   }
   __syncthreads();

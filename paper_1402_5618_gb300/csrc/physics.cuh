@@ -20,9 +20,16 @@ __device__ __forceinline__ real sqr(real x) { return x * x; }
 // with as few as the result needs: the hardware's approximation (about 20
 // bits) and one third-order step, y (1 + e + e^2) with e = 1 - x y for 1/x and
 // y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 for x^(-1/2) (the truncated
-// binomial series), whose error e^3 is below FP64's.  3 FP64 instructions for
-// 1/x and 6 for a square root; the operators take 5.3 and 9 instruction times
-// (measured).  Arguments the approximations flush (zeros, subnormals) take the operators.
+// binomial series), whose error e^3 is below FP64's: at most one unit in the last
+// place from the rounded value.  3 FP64 instructions for 1/x and 6 for a square
+// root; the operators take 5.3 and 9 instruction times (measured).
+// root() leaves what the approximation flushes (zeros, subnormals) to the
+// operator.  rcp() wants a normal, finite argument: zeros, subnormals and
+// infinities give NaN where 1/x is infinite or zero, and so does root() of an
+// infinity.  Its arguments are densities of limited face states and of cells (a
+// cell of any other density is outside G, which a NaN energy says too), sums of
+// weights (z_terms keeps them normal), pivots 1 - c b > 0, and differences of
+// wave speeds, zero only where no sound speed is left and the flux has no value.
 __device__ __forceinline__ float rcp(float x) { return 1.0f / x; }
 __device__ __forceinline__ double rcp(double x) {
   double y;

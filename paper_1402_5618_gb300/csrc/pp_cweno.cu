@@ -1074,8 +1074,7 @@ cudaError_t launch(const pp_cweno_s *h, int mode, bool xdir, const void *Uin, co
   return dispatch(h, mode, a, nlines, m);
 }
 
-// Batched launch of one line group.  eps_fixed > 0 with ctl: a measurement
-// launch (the autotuner's) that reduces into a scratch control block array.
+// Batched launch of one line group on stream st.
 cudaError_t launch_group(const pp_cweno_s *h, const LineGroup &g, int mode, const void *Uin,
                          const void *U0, const void *Din, void *Dout, void *Uout, int stage,
                          cudaStream_t st) {
