@@ -858,35 +858,41 @@ __global__ void __launch_bounds__(Smem<real, NV, M, KC>::THREADS, CTAS) line_swe
       // The seams at either end of the segment: the runs before and after a
       // seam from the ends of the line, lane 0 joining the segments forwards,
       // lane 1 backwards, so that the neighbour comes to the same two runs.
-      // Kept of them, without (e) and with this segment (w), is the end at the
-      // seam: its value, the coefficient of the line's far end and that of the
-      // unknown across the seam.  Periodic: lane 0 goes on to the whole line,
-      // whose ring gives the unknowns at its two ends.
+      // Needed of them is the end at the seam alone (t: its value, the
+      // coefficient of the line's far end and of the unknown across the seam),
+      // without (e) and with this segment (w).  Periodic: both lanes go on to the
+      // whole line, whose ring gives the unknowns at its two ends.
       const int wpos = sd ? R - 1 - rank : rank;
       real e1 = real(0), e2 = real(-1), e3 = real(0), w1 = e1, w2 = e2, w3 = e3;
       real el = real(0), er = real(0);   // before the first and after the last cell (bounded: no weight)
       {
-        Run<real> rest = run_empty<real>();
-        const int cnt = cl == 0 ? (per ? R : wpos + 1) : (cl == 1 ? R - wpos : 0);
-        Cut<real> unused;
+        real t1 = e1, t2 = e2, t3 = e3;
+        const int cnt = cl > 1 ? 0 : (per ? R : (cl == 0 ? wpos + 1 : R - wpos));
 #pragma unroll 1
         for (int q = 0; q < cnt; ++q) {
           const int at = cl == 0 ? q : R - 1 - q;
-          const Run<real> o = cluster.map_shared_rank(&ex, sd ? R - 1 - at : at)->seg[sys];
-          if (at == wpos) {
-            e1 = cl == 0 ? rest.D : rest.A; e2 = cl == 0 ? rest.F : rest.G; e3 = cl == 0 ? rest.C : rest.B;
+          const Run<real> &o = cluster.map_shared_rank(&ex, sd ? R - 1 - at : at)->seg[sys];
+          if (at == wpos) { e1 = t1; e2 = t2; e3 = t3; }
+          // the next segment's end facing the seam, a - b (across) - g (beyond),
+          // and its other one, a2 - f (across) - c (beyond)
+          const real a2 = cl == 0 ? o.D : o.A, f = cl == 0 ? o.F : o.G, c = cl == 0 ? o.C : o.B;
+          if (q == 0) {
+            t1 = a2; t2 = f; t3 = c;
+          } else {
+            const real a = cl == 0 ? o.A : o.D, b = cl == 0 ? o.B : o.C, g = cl == 0 ? o.G : o.F;
+            const real i = rcp(fma(-t3, b, real(1))), fi = f * i;
+            t1 = fma(-fi, fma(-t3, a, t1), a2);
+            t2 = -(fi * t2);
+            t3 = fma(fi, t3 * g, c);
           }
-          if (q == 0) rest = o;
-          else rest = run_join(cl == 0 ? rest : o, cl == 0 ? o : rest, unused);
-          if (at == wpos) {
-            w1 = cl == 0 ? rest.D : rest.A; w2 = cl == 0 ? rest.F : rest.G; w3 = cl == 0 ? rest.C : rest.B;
-          }
+          if (at == wpos) { w1 = t1; w2 = t2; w3 = t3; }
         }
         if (per) {
-          const Run<real> w = run_shfl(rest, 0, LPS);
           Ends<real> f, l;
-          f.a = w.A; f.b = w.B; f.g = w.G;
-          l.a = w.D; l.b = w.C; l.g = w.F;
+          l.a = __shfl_sync(0xffffffffu, t1, 0, LPS); l.g = __shfl_sync(0xffffffffu, t2, 0, LPS);
+          l.b = __shfl_sync(0xffffffffu, t3, 0, LPS);
+          f.a = __shfl_sync(0xffffffffu, t1, 1, LPS); f.g = __shfl_sync(0xffffffffu, t2, 1, LPS);
+          f.b = __shfl_sync(0xffffffffu, t3, 1, LPS);
           ring_close(f, l, el, er);
         }
       }
