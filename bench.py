@@ -193,10 +193,10 @@ ALU_PEAK_TFLOPS = {1: 152 * 128 * 2 * 2.07e9 / 1e12, 0: 1.25}
 # is still dirty in L2 when the kernel ends.  The FP64 form's dominant
 # kernel is its y sweep, for which no capture of these sources exists.
 TRAFFIC_PER_CELL = {            # {(precision, kernel): bytes per cell}
-    (1, "x_sweep"): 45.01,
-    (0, "x_sweep"): 59.86,
+    (1, "x_sweep"): 45.02,
+    (0, "x_sweep"): 59.69,
 }
-TRAFFIC_SRC_SHA256 = "df84695ac674e64df2d4dfbfa8ae895904b113d530ba3f08194a9a01841d7333"
+TRAFFIC_SRC_SHA256 = "52f369643a21602e0a81537e2d179ce7a5ac34af536de0334abc2f1e05c4ff68"
 KERNEL_SOURCES = ("line_sweep.cuh", "compact_solve.cuh", "physics.cuh", "dfloat.cuh", "batch_lines.cuh")
 
 

@@ -28,13 +28,13 @@
 // FP64 only for the limiter factors of cells that need limiting and for the
 // closing of a periodic ring.
 //
-// What bounds it: in FP64 the FP64 pipe (71% busy on large grids; a line
+// What bounds it: in FP64 the FP64 pipe (70-77% busy on large grids; a line
 // alone waits for its own chain of FP64 instructions), in the mixed form
 // instruction issue (47%) and fixed latencies, barriers and instruction
 // fetch, with 16 warps per SM; HBM is at 14%.  Per sweep of 4096^2 cells (corner
 // blast), against a scan over projective chunk maps with divisions in every
-// row and an exchange of limited faces: mixed 1.63 -> 0.84 ms, FP64 48.0 -> 16.0
-// (x) and 51.6 -> 18.3 ms (y with the stage update).
+// row and an exchange of limited faces: mixed 1.63 -> 0.83 ms, FP64 48.0 -> 16.4
+// (x) and 51.6 -> 18.1 ms (y with the stage update).
 #pragma once
 
 #include <cooperative_groups.h>
